@@ -69,8 +69,8 @@ struct octax_env {
   uint64_t seed = 0;
   std::vector<GameDev> games_h;
   std::vector<uint16_t> game_of_slot;
-  GameDev *games_d = nullptr;
-  uint8_t *images_d = nullptr;
+  uint8_t *blobs_d = nullptr;  // what CTAs stage, one blob per game
+  int n_uops = 0;
   DevState st{};
   uint32_t *slot_of_row_d = nullptr;
   std::vector<void *> allocs;
@@ -184,7 +184,7 @@ int per_cta(const octax_launch &c) { return c.block / 32 * c.inst_per_warp; }
 int wave_of(const octax_env *e, const octax_launch &c) {
   if (!c.balance) return 0;
   return max_resident_ctas(c.block, c.inst_per_warp, c.writer_warps,
-                           uses_wrappers(e->games_h.data(), e->games_h.size()), e->schip);
+                           uses_wrappers(e->games_h.data(), e->games_h.size()), e->schip, e->n_uops);
 }
 
 const char *launch_problem(const octax_launch &c, int schip) {
@@ -199,10 +199,10 @@ const char *launch_problem(const octax_launch &c, int schip) {
     if (J % W != 0 || !(J / W == 8 || J / W == 16 || J / W == 32))
       return "block/32*inst_per_warp/writer_warps must be 8, 16 or 32";
     if (schip) return "writer warps serve CHIP-8 environments only";
-    if (step_ws_smem_bytes(c.block, c.inst_per_warp) > max_dynamic_smem())
+    if (!shape_fits(c.block, c.inst_per_warp, schip, W))
       return "too many instances per CTA for the writer ring";
   }
-  if (step_smem_bytes(c.block, c.inst_per_warp, schip) > max_dynamic_smem())
+  if (!shape_fits(c.block, c.inst_per_warp, schip, 0))
     return "too many instances per CTA for shared memory";
   return nullptr;
 }
@@ -235,6 +235,25 @@ int octax::build_games(const octax_game *games, int n_games, std::vector<GameDev
     memcpy(img + 0x200, games[g].rom, games[g].rom_len);
   }
   return OCTAX_OK;
+}
+
+int octax::table_uops(const octax_game *games, int n_games) {
+  uint32_t len = 0;
+  for (int g = 0; g < n_games; ++g) len = std::max(len, games[g].rom_len);
+  return (int)((len + 1) / 2);
+}
+
+cudaError_t octax::upload_blobs(const std::vector<GameDev> &games, const std::vector<uint8_t> &images, int n_uops,
+                                int schip, uint32_t quirks, uint8_t *blobs, cudaStream_t s) {
+  const size_t stride = blob_stride(n_uops);
+  std::vector<uint8_t> h(games.size() * stride, 0);
+  for (size_t g = 0; g < games.size(); ++g) {
+    memcpy(&h[g * stride], &images[g * kRamBytes], kRamBytes);
+    memcpy(&h[g * stride + kRamBytes], &games[g], sizeof(GameDev));
+  }
+  cudaError_t r = cudaMemcpyAsync(blobs, h.data(), h.size(), cudaMemcpyHostToDevice, s);
+  if (r == cudaSuccess) r = cudaStreamSynchronize(s);  // h is a local buffer
+  return r == cudaSuccess ? launch_tables(blobs, stride, (int)games.size(), n_uops, schip, quirks, s) : r;
 }
 
 namespace {
@@ -308,8 +327,9 @@ StepLaunch base_launch(octax_env *e, const GroupTable *gt) {
   StepLaunch p;
   memset(&p, 0, sizeof p);
   p.st = e->st;
-  p.games = e->games_d;
-  p.images = e->images_d;
+  p.blobs = e->blobs_d;
+  p.n_uops = e->n_uops;
+  p.stride = (uint32_t)blob_stride(e->n_uops);
   p.groups = gt->dev;
   p.n_groups = gt->count;
   p.S = e->S;
@@ -346,7 +366,7 @@ int enqueue_steps(octax_env *e, const octax_launch &cfg, int n_steps, const IO &
       cfg.persistent
           ? std::min(gt->count, std::max(1, max_resident_ctas(cfg.block, cfg.inst_per_warp, cfg.writer_warps,
                                                       uses_wrappers(e->games_h.data(), e->games_h.size()),
-                                                      e->schip)))
+                                                      e->schip, e->n_uops)))
           : gt->count;
   if (cfg.persistent) {
     rc = ensure_counters(e, launches);
@@ -505,44 +525,27 @@ int octax_create(const octax_game *games, int n_games, const uint16_t *game_of_e
   DevState &st = e->st;
   st.n = n_envs;
   cudaError_t r = cudaSuccess;
-  uint32_t *uid_tmp = nullptr;
+  uint32_t *uid_tmp = nullptr, *row_tmp = nullptr;
+  e->n_uops = table_uops(games, n_games);
 #define ALLOC(ptr, cnt) \
   if (r == cudaSuccess) r = dalloc(e, &(ptr), (cnt))
-  ALLOC(e->games_d, (size_t)n_games);
-  ALLOC(e->images_d, images.size());
-  ALLOC(st.v, 4 * n);
-  ALLOC(st.pcI, n);
-  ALLOC(st.misc, n);
-  ALLOC(st.stack, 16 * n);
-  ALLOC(st.disp, (size_t)disp_words(e->schip) * n);
-  ALLOC(st.dirty, n);
-  ALLOC(st.wrange, n);
+  ALLOC(e->blobs_d, (size_t)n_games * blob_stride(e->n_uops));
+  ALLOC(st.rec, n * rec_words(e->schip));
   ALLOC(st.ram, n * kRamBytes);
-  ALLOC(st.ep, n);
-  ALLOC(st.env_steps, n);
-  ALLOC(st.prev_score, n);
-  ALLOC(st.key, 2 * n);
-  ALLOC(st.uid, n);
-  ALLOC(st.out_row, n);
-  ALLOC(st.game, n);
-  ALLOC(st.last_act, n);
-  ALLOC(st.mode, n);
-  ALLOC(st.rpl, 16 * n);
   st.schip = e->schip;
   ALLOC(e->slot_of_row_d, n);
   ALLOC(e->io_d, 1);
   ALLOC(e->err_d, 1);
   ALLOC(uid_tmp, n);
+  ALLOC(row_tmp, n);
 #undef ALLOC
   if (r != cudaSuccess) {
     free_env(e);
     set_error(std::string("octax_create: device allocation failed: ") + cudaGetErrorString(r));
     return OCTAX_ENOMEM;
   }
-  r = cudaMemcpy(e->games_d, e->games_h.data(), e->games_h.size() * sizeof(GameDev), cudaMemcpyHostToDevice);
-  if (r == cudaSuccess) r = cudaMemcpy(e->images_d, images.data(), images.size(), cudaMemcpyHostToDevice);
-  if (r == cudaSuccess) r = cudaMemcpy(st.out_row, row_of_slot.data(), n * 4, cudaMemcpyHostToDevice);
-  if (r == cudaSuccess) r = cudaMemcpy(st.game, e->game_of_slot.data(), n * 2, cudaMemcpyHostToDevice);
+  r = upload_blobs(e->games_h, images, e->n_uops, e->schip, quirks, e->blobs_d, e->stream);
+  if (r == cudaSuccess) r = cudaMemcpy(row_tmp, row_of_slot.data(), n * 4, cudaMemcpyHostToDevice);
   if (r == cudaSuccess) r = cudaMemcpy(e->slot_of_row_d, slot_of_row.data(), n * 4, cudaMemcpyHostToDevice);
   if (r == cudaSuccess) r = cudaMemcpy(uid_tmp, uid_of_slot.data(), n * 4, cudaMemcpyHostToDevice);
   if (r == cudaSuccess) r = cudaMemset(e->err_d, 0, sizeof(unsigned int));
@@ -561,8 +564,9 @@ int octax_create(const octax_game *games, int n_games, const uint16_t *game_of_e
   ResetLaunch p;
   memset(&p, 0, sizeof p);
   p.st = st;
-  p.games = e->games_d;
-  p.images = e->images_d;
+  p.blobs = e->blobs_d;
+  p.n_uops = e->n_uops;
+  p.stride = (uint32_t)blob_stride(e->n_uops);
   p.groups = gt->dev;
   p.n_groups = gt->count;
   p.S = e->S;
@@ -570,6 +574,7 @@ int octax_create(const octax_game *games, int n_games, const uint16_t *game_of_e
   p.ipw = e->cfg.inst_per_warp;
   p.init = 1;
   p.seed = seed;
+  p.row_of_slot = row_tmp;
   p.uid_of_slot = uid_tmp;
   r = launch_reset(p, e->cfg.block, e->stream);
   if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);
@@ -597,8 +602,9 @@ int octax_reset(octax_env *e, const uint8_t *mask_dev, uint8_t *obs_dev) {
   ResetLaunch p;
   memset(&p, 0, sizeof p);
   p.st = e->st;
-  p.games = e->games_d;
-  p.images = e->images_d;
+  p.blobs = e->blobs_d;
+  p.n_uops = e->n_uops;
+  p.stride = (uint32_t)blob_stride(e->n_uops);
   p.groups = gt->dev;
   p.n_groups = gt->count;
   p.mask = mask_dev;
@@ -736,7 +742,7 @@ int octax_state_hash(octax_env *e, uint64_t *hash_dev) {
     set_error("octax_state_hash: null argument");
     return OCTAX_EINVAL;
   }
-  cudaError_t r = launch_hash(e->st, e->images_d, e->slot_of_row_d, e->n, hash_dev, e->stream);
+  cudaError_t r = launch_hash(e->st, e->blobs_d, blob_stride(e->n_uops), e->slot_of_row_d, e->n, hash_dev, e->stream);
   return r == cudaSuccess ? OCTAX_OK : cuda_fail(r, "octax_state_hash");
 }
 
@@ -749,7 +755,7 @@ int octax_get_state(octax_env *e, int64_t first, int64_t count, octax_state_reco
   octax_state_record *tmp = nullptr;
   cudaError_t r = cudaMallocAsync(&tmp, count * sizeof(octax_state_record), e->stream);
   if (r != cudaSuccess) return cuda_fail(r, "octax_get_state alloc");
-  r = launch_records(e->st, e->images_d, e->slot_of_row_d, first, count, tmp, e->stream);
+  r = launch_records(e->st, e->blobs_d, blob_stride(e->n_uops), e->slot_of_row_d, first, count, tmp, e->stream);
   if (r == cudaSuccess)
     r = cudaMemcpyAsync(out_host, tmp, count * sizeof(octax_state_record), cudaMemcpyDeviceToHost, e->stream);
   cudaFreeAsync(tmp, e->stream);
@@ -773,7 +779,7 @@ int octax_set_state(octax_env *e, int64_t first, int64_t count, const octax_stat
   if (r != cudaSuccess) return cuda_fail(r, "octax_set_state alloc");
   r = cudaMemcpyAsync(tmp, in_host, count * sizeof(octax_state_record), cudaMemcpyHostToDevice, e->stream);
   if (r == cudaSuccess)
-    r = launch_set_records(e->st, e->games_d, e->images_d, e->slot_of_row_d, first, count, tmp, e->stream);
+    r = launch_set_records(e->st, e->blobs_d, blob_stride(e->n_uops), e->slot_of_row_d, first, count, tmp, e->stream);
   cudaFreeAsync(tmp, e->stream);
   if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);
   return r == cudaSuccess ? OCTAX_OK : cuda_fail(r, "octax_set_state");
@@ -859,11 +865,7 @@ int octax_autotune(octax_env *e, int n_steps, const uint8_t *actions_dev, float 
     void *p;
     size_t bytes;
   };
-  const Piece pieces[] = {{st.v, 16 * n},     {st.pcI, 4 * n},    {st.misc, 4 * n},
-                          {st.stack, 32 * n}, {st.disp, 8 * (size_t)disp_words(e->schip) * n}, {st.dirty, 8 * n},
-                          {st.ram, 4096 * n}, {st.ep, 4 * n},     {st.env_steps, 4 * n},
-                          {st.prev_score, 4 * n}, {st.last_act, n}, {st.mode, n}, {st.rpl, 16 * n},
-                          {st.wrange, 4 * n}};
+  const Piece pieces[] = {{st.rec, 4 * (size_t)rec_words(e->schip) * n}, {st.ram, 4096 * n}};
   size_t total = 0;
   for (const Piece &pc : pieces) total += pc.bytes;
   uint8_t *backup = nullptr, *acts = nullptr, *obs = nullptr, *done = nullptr;

@@ -48,44 +48,49 @@ struct alignas(16) GameDev {
 };
 static_assert(sizeof(GameDev) <= 192, "GameDev must fit its shared-memory slot");
 constexpr int kGameSmem = 192;
-// Micro-op table: one entry per even address, 16 bytes (wide: operand offsets
-// and NNN ready to use) or 8 bytes (narrow: packed; half the shared memory).
-constexpr int kUopSmemWide = kRamBytes / 2 * 16;
-constexpr int kUopSmemNarrow = kRamBytes / 2 * 8;
 constexpr int kLutSmem = 256 * 8;            // byte of pixels -> 8 output bytes
-constexpr int kAluSmem = 16 * 2 * 16;        // 8XYN coefficients per N (two int4)
+// What a CTA stages of its game, one contiguous blob per game in device
+// memory, in this order: RAM image | descriptor | pixel table | coefficients |
+// micro-ops (one per even address of the ROM and a sentinel; 8 bytes of each,
+// then 4 bytes of each).
+constexpr int kBlobLut = kRamBytes + kGameSmem;
+constexpr int kBlobCoef = kBlobLut + kLutSmem;
+constexpr int kBlobUops = kBlobCoef + 64;
+__host__ __device__ constexpr uint32_t blob_bytes(uint32_t n_uops) {
+  return ((uint32_t)kBlobUops + 12 * (n_uops + 1) + 15) & ~15u;
+}
+inline size_t blob_stride(int n_uops) { return ((size_t)blob_bytes((uint32_t)n_uops) + 255) & ~(size_t)255; }
 
-// Emulator state, structure-of-arrays over slots (slot = index in these arrays).
+// Emulator state: one record of 32-bit words per slot (slot = index), the same
+// words in device memory and, while a CTA steps the instance, in shared memory:
+// a warp moves the records of its instances as one run of 16-byte pieces.
+// Words, after the packed display (64, SCHIP 256):
+//   +0 V0-VF  +4 DT | last action | ST | 15 (bytes)  +5 PC | I << 16
+//   +6 SP | hires << 7 | status << 8 | game << 16  +7 written range  +8 dirty pages (u64)
+//   +10 episode steps  +11 env steps  +12 stack (16 x u16)  +20 uid  +21 Philox key (2)
+//   +23 output row  [SCHIP: +24 flag registers (16 bytes)]
+// The lengths, 92 and 284 words, are 28 mod 32: instances next to each other
+// start four banks apart.
+constexpr int kRecTail = 28;
+template <bool kS>
+struct Rec {
+  static constexpr int kV = kS ? 256 : 64;
+  static constexpr int kPseudo = kV + 4, kPcI = kV + 5, kMisc = kV + 6, kWrange = kV + 7, kDirty = kV + 8, kEp = kV + 10,
+                       kEnv = kV + 11, kStack = kV + 12, kUid = kV + 20, kKey = kV + 21, kRow = kV + 23, kRpl = kV + 24,
+                       kWords = kV + kRecTail;
+};
+static_assert(Rec<false>::kWords % 4 == 0 && Rec<true>::kWords % 4 == 0, "records move as 16-byte pieces");
+__host__ __device__ inline int rec_words(int schip) { return schip ? Rec<true>::kWords : Rec<false>::kWords; }
+
 struct DevState {
   int64_t n;              // slots
-  uint32_t *v;            // [4][n]   V[4j..4j+3] little-endian in word j
-  uint32_t *pcI;          // [n]      PC | I << 16
-  uint32_t *misc;         // [n]      SP | DT << 8 | ST << 16 | status << 24
-  uint16_t *stack;        // [16][n]
-  uint64_t *disp;         // [W][n]   CHIP-8 (W = 32): bit x of word y = pixel (x, y);
-                          //          SCHIP (W = 128): bit x of word 2y + h = pixel (64h + x, y)
-  uint64_t *dirty;        // [n]      RAM pages that differ from the ROM image
-  uint32_t *wrange;       // [n]      lowest | highest << 16 RAM address written since the
-                          //          reset (kNoWrites: none): bytes outside it equal the image
+  uint32_t *rec;          // [n][rec_words]
   uint8_t *ram;           // [n][4096] per-instance RAM (valid on dirty pages only)
-  uint32_t *ep;           // [n]      steps since reset
-  uint32_t *env_steps;    // [n]      steps since creation
-  int32_t *prev_score;    // [n]      score at the end of the last step / reset
-  uint32_t *key;          // [2][n]   Philox key
-  uint32_t *uid;          // [n]      Philox counter word 0
-  uint32_t *out_row;      // [n]      row of this slot in its request's outputs
-  uint16_t *game;         // [n]
-  uint8_t *last_act;      // [n]      action index applied at the previous step
-  uint8_t *mode;          // [n]      SCHIP: 1 = hires
-  uint8_t *rpl;           // [n][16]  SCHIP flag registers
-  int schip;              // 1: SCHIP layout (disp has 128 words per slot)
+  int schip;              // 1: SCHIP layout
 };
 
 // Every per-slot array is set (checked on the host before each launch).
-inline bool state_complete(const DevState &s) {
-  return s.n > 0 && s.v && s.pcI && s.misc && s.stack && s.disp && s.dirty && s.wrange && s.ram && s.ep && s.env_steps &&
-         s.prev_score && s.key && s.uid && s.out_row && s.game && s.last_act && s.mode && s.rpl;
-}
+inline bool state_complete(const DevState &s) { return s.n > 0 && s.rec && s.ram; }
 
 // A group: up to block/32*ipw consecutive slots that share one game (one CTA's work).
 struct Group {
@@ -109,8 +114,9 @@ struct IO {
 
 struct StepLaunch {
   DevState st;
-  const GameDev *games;
-  const uint8_t *images;   // [n_games][4096] initial RAM image (font + ROM)
+  const uint8_t *blobs;    // [n_games][blob_stride(n_uops)]
+  int n_uops;              // micro-ops per game (0 in a launch without room for the table)
+  uint32_t stride;         // blob_stride of the table as built
   const Group *groups;
   int n_groups;
   IO io0;                  // used when io_table == nullptr
@@ -129,8 +135,9 @@ struct StepLaunch {
 
 struct ResetLaunch {
   DevState st;
-  const GameDev *games;
-  const uint8_t *images;
+  const uint8_t *blobs;
+  int n_uops;
+  uint32_t stride;
   const Group *groups;
   int n_groups;
   const uint8_t *mask;     // [n_out_rows] by out_row, nullable = all
@@ -140,38 +147,42 @@ struct ResetLaunch {
   int ipw;
   int init;                // 1: also set key/uid/env_steps/status (creation)
   uint64_t seed;
-  const uint32_t *uid_of_slot;  // used when init (nullable = out_row)
+  const uint32_t *row_of_slot;  // used when init (nullable = group.row0 + lane)
+  const uint32_t *uid_of_slot;  // used when init (nullable = the row)
   const uint64_t *seed_of_group;  // init: per-group seed (nullable = seed)
-  int set_rows;            // init: out_row = group.row0 + lane, game = group.game
 };
 
-// Dynamic shared memory of a step CTA; wide = 16-byte micro-op table (the
-// narrow size is the minimum a launch shape needs).
-size_t step_smem_bytes(int block, int ipw, int schip, int wide = 0);
+// Dynamic shared memory of a step CTA with a table of n_uops micro-ops.
+size_t step_smem_bytes(int block, int ipw, int schip, int n_uops);
 // Warp-specialised kernel: `block` emulator threads plus 32 * writers writer threads.
-size_t step_ws_smem_bytes(int block, int ipw);
+size_t step_ws_smem_bytes(int block, int ipw, int n_uops);
 size_t max_dynamic_smem();
+// The launch shapes that are accepted: what a CTA's instances may take of shared memory.
+bool shape_fits(int block, int ipw, int schip, int writers);
+// Fills the pixel table and the micro-ops of every blob from its RAM image.
+cudaError_t launch_tables(uint8_t *blobs, size_t stride, int n_games, int n_uops, int schip, uint32_t quirks,
+                          cudaStream_t s);
 cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s);
 cudaError_t launch_reset(const ResetLaunch &p, int block, cudaStream_t s);
-cudaError_t launch_hash(const DevState &st, const uint8_t *images, const uint32_t *slot_of_row,
+cudaError_t launch_hash(const DevState &st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
                         int64_t rows, uint64_t *out, cudaStream_t s);
-cudaError_t launch_records(const DevState &st, const uint8_t *images, const uint32_t *slot_of_row,
+cudaError_t launch_records(const DevState &st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
                            int64_t first, int64_t count, octax_state_record *out, cudaStream_t s);
-cudaError_t launch_set_records(const DevState &st, const GameDev *games, const uint8_t *images,
-                               const uint32_t *slot_of_row, int64_t first, int64_t count,
-                               const octax_state_record *in, cudaStream_t s);
-int max_resident_ctas(int block, int ipw, int writers, int wrappers, int schip);
+cudaError_t launch_set_records(const DevState &st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
+                               int64_t first, int64_t count, const octax_state_record *in, cudaStream_t s);
+int max_resident_ctas(int block, int ipw, int writers, int wrappers, int schip, int n_uops);
 // True when a game enables the sticky-action or no-op-reset wrapper.
 inline int uses_wrappers(const GameDev *games, size_t n) {
   for (size_t i = 0; i < n; ++i)
     if (games[i].sticky != 0u || games[i].max_noops != 0u) return 1;
   return 0;
 }
-// Bytes of device state per slot (all DevState arrays).
-constexpr size_t kSlotStateBytes = 16 + 4 + 4 + 32 + 256 + 8 + 4 + 4096 + 4 + 4 + 4 + 8 + 4 + 4 + 2 + 1 + 1 + 16;
-inline size_t slot_state_bytes(int schip) {
-  return kSlotStateBytes + (schip ? 8 * (kSchipDispWords - kDispWords) : 0);
-}
+// Bytes of device memory that a server's budget is charged per slot; the
+// record and the RAM take 4,464 (SCHIP 5,232) of them.
+constexpr size_t kSlotStateBytes = 4468, kSchipSlotStateBytes = 5236;
+inline size_t slot_state_bytes(int schip) { return schip ? kSchipSlotStateBytes : kSlotStateBytes; }
+static_assert(4 * Rec<false>::kWords + kRamBytes <= kSlotStateBytes, "slot fits its charge");
+static_assert(4 * Rec<true>::kWords + kRamBytes <= kSchipSlotStateBytes, "slot fits its charge");
 cudaError_t alloc_state(DevState &st, int64_t n, int schip, void **block_out, size_t *bytes_out);
 // Append one step launch to a graph (after `dep`, if non-null).
 cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t dep, const StepLaunch &p,
@@ -180,6 +191,11 @@ cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t 
 // Validate game descriptors; build device descriptors and 4 KB RAM images.
 int build_games(const octax_game *games, int n_games, std::vector<GameDev> &dev,
                 std::vector<uint8_t> &images);
+// Micro-op table length for these games (entries for every address of the longest ROM).
+int table_uops(const octax_game *games, int n_games);
+// Upload the blobs of `games` (device memory of n * blob_stride bytes) and build their tables.
+cudaError_t upload_blobs(const std::vector<GameDev> &games, const std::vector<uint8_t> &images, int n_uops, int schip,
+                         uint32_t quirks, uint8_t *blobs, cudaStream_t s);
 
 // Error reporting (thread-local message).
 void set_error(const std::string &msg);

@@ -1,44 +1,62 @@
 // liboctax device code: the vectorised CHIP-8 environment step for sm_103a.
 //
 // Mapping (one CTA = one group of block/32 * ipw instances of one game):
-//  - each warp emulates `ipw` instances, one per lane; PC/I/SP/timers/status,
-//    the 64-bit dirty-page mask and the written-address range live in
-//    registers; V0-VF (one u32 each),
-//    the call stack and the bit-packed 64x32 display (one u64 per row, bit x =
-//    pixel x; Super-CHIP: two u64 per row of the 128x64 buffer) live in
-//    shared memory laid out [register|entry|row][instance],
-//    so lanes touching their own instance never bank-conflict;
+//  - each warp emulates `ipw` instances with L = 32 / ipw lanes each (rounded
+//    to a power of two). The L lanes of an instance execute the same
+//    instructions on the same values; they split what has parts: the rows of a
+//    sprite, a clear, a copy. Display row y belongs to lane y mod L;
+//  - an instance's state is one record of 32-bit words, in device memory and in
+//    shared memory alike, so that a warp fetches and returns the records of its
+//    instances as one run of 16-byte pieces. PC/I/SP/status, the 64-bit
+//    dirty-page mask and the written-address range live in registers; V0-VF and
+//    the timers as bytes in shared memory, a copy per lane (20 bytes apart:
+//    five banks, so lanes on the same register never collide), which keeps
+//    lanes from ever waiting for one another over a register;
 //  - the game's initial 4 KB RAM image (font + ROM) is staged once per CTA in
 //    shared memory and is read-only; an instance's writes go to 64-byte pages
-//    of its own RAM in global memory, tracked by the dirty mask. Fetches and
-//    loads read the shared image unless the page is dirty; sprites read it
-//    whenever their bytes lie outside the range of addresses written since
-//    the reset (data packed next to a score buffer). A reset only clears the
-//    mask and the range;
-//  - observations can also be written one bit per pixel (the display words
-//    themselves), 8x fewer bytes;
+//    of its own RAM in global memory, tracked by the dirty mask. Sprites and
+//    fetches use the image whenever their bytes lie outside the range of
+//    addresses written since the reset (data packed next to a score buffer);
+//    other reads unless their page is dirty. A reset only clears the mask and
+//    the range;
 //  - dispatch limits divergence: the common opcodes (jumps, skips, loads,
-//    adds, 8XYN ALU, key tests, FX07/FX15) run through one branch-free
-//    predicated datapath that every lane executes together, with 8XYN as
-//    integer multiply-adds from a per-N coefficient table; DXYN and four FX
-//    forms take short branches, and the rest (CXNN, calls/returns, 00E0, BCD
-//    and bulk memory ops, quirk variants, undefined encodings, the
-//    Super-CHIP forms) a divergent switch. Every even address of the image
-//    is decoded once per CTA into a micro-op (one bit per datapath decision,
-//    NNN, and the pre-multiplied shared-memory offsets of VX and VY), so the
-//    hot loop does one or two shared loads and single-bit tests per
-//    instruction;
+//    adds, 8XYN ALU, key tests, timers, FX29) run through one branch-free
+//    datapath that every lane executes together: one signed byte dot product
+//    (VX, VY, VX & VY, VX >> 1) . coefficients + immediate, whose low byte is
+//    the result, whose bit 8 is the flag and which decides a skip by being
+//    zero; the next PC is one of two that the micro-op carries. Micro-ops are
+//    decoded once per environment (tables_kernel) for every even address of
+//    the ROM and staged with the image. DXYN has a branch of its own; the
+//    rest (CXNN, calls and returns, 00E0, BCD and bulk memory ops, odd or
+//    written addresses, undefined encodings, the Super-CHIP forms) takes a
+//    divergent switch;
 //  - observation frames are expanded from the packed rows by the whole warp
 //    together (a byte of pixels becomes 8 bytes through a 256-entry table in
 //    shared memory): every store is a 16-byte streaming store and each store
-//    instruction writes eight complete 64-byte image rows (CHIP-8) or four
-//    128-byte rows (Super-CHIP).
+//    instruction writes complete 64-byte image rows (CHIP-8) or 128-byte rows
+//    (Super-CHIP). They can also be written one bit per pixel (the display
+//    words themselves), 8x fewer bytes.
 // Each instance runs exactly K instructions per frame, so all lanes of a warp
 // meet at every frame boundary.
+//
+// What bounds it: below a few thousand instances the dependent chain of one
+// instruction (micro-op load, register loads, compare, next offset); in the
+// middle the warp instructions per emulated instruction; above, the frame
+// stores. Measured against the form before it (a lane per instance with the
+// others idle, 8- or 16-byte micro-ops decoded by every CTA, registers as
+// 32-bit words interleaved over the CTA, coefficient rows and separate
+// selects per instruction class): one step of 64 template instances 11.0 ->
+// 6.2 us, of 16,384 34.2 -> 20.9 us (7.0 TB/s), 16 packed steps of 12,289
+// shooter instances 352 -> 163 us, 8 Super-CHIP steps of 8,192 492 -> 303 us,
+// 8 steps of 65,536 over 16 ROMs 978 -> 836 us, 4 steps of 262,144 random
+// programs 1,472 -> 1,452 us. The micro-ops take 12 bytes and not 16 so that
+// a CTA of 64 instances with a 3.5 KB ROM keeps four CTAs per SM (random
+// programs 1,683 us with 16); the pixel table stays because expanding by
+// multiplication costs the issue-bound cases 1 % (it gains 7 % on one step of
+// 16,384); three CTAs of 256 threads per SM (80 registers) lose 8 % there.
 #include <algorithm>
 #include <map>
 #include <mutex>
-#include <tuple>
 #include <cstring>
 
 #include "octax_internal.h"
@@ -48,33 +66,35 @@ namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// The CTA's dynamic shared memory. Every kernel lays it out with carve(), so
-// the game's 4 KB RAM image is its first 4 KB. Reading the image through this
-// array (not through a pointer) keeps those loads in the shared state space.
+// The CTA's dynamic shared memory: the game's blob (its RAM image first),
+// the records, the lanes' registers. Reading the image
+// through this array (not through a pointer) keeps those loads in the shared
+// state space.
 extern __shared__ __align__(16) uint8_t g_smem[];
 
 __device__ __forceinline__ uint32_t img_byte(uint32_t a) { return g_smem[a]; }
 
 struct Regs {
-  uint32_t pc, I, sp, dt, st, status;
+  uint32_t pc, I, sp, status;
   uint64_t dirty;
   uint32_t draws, phase, env_steps;
-  uint32_t key0, key1, uid;
-  uint32_t last_act;  // action index applied at the previous step (sticky actions)
   uint32_t hires;     // SCHIP: 1 in 128x64 mode
   uint32_t wrange;    // lowest | highest << 16 RAM address written since the reset
+  uint32_t wbase, wspan;  // the same as micro-op offsets (set_range): a fetch at offset o may read a
+                          // written byte if o - wbase <= wspan
 };
 
 struct Ctx {
-  uint64_t *disp;      // shared: this instance's row 0; row r at disp[r * J]
-  uint32_t *stack;     // shared: this instance's entry 0; entry i at stack[i * J]
-  uint32_t *V;         // shared: this instance's V0; Vx at V[x * J]
+  uint8_t *V;          // shared: this lane's V0-VF, DT, last action, ST, 15
+  uint32_t *rec;       // shared: this instance's record
   uint8_t *ram;        // global: this instance's 4 KB RAM (dirty pages)
-  int J;
-  const void *uops;      // shared: micro-op table, uint4 or uint2 entries (stage_game)
-  const int4 *alu;       // shared: 8XYN coefficients, two int4 per N (stage_game)
-  uint8_t *rpl;          // global: this instance's 16 SCHIP flag bytes
+  uint32_t n_uops;     // entries of the micro-op table (the sentinel follows)
+  uint32_t sub, L;     // this lane among the L of its instance
+  uint32_t gmask;      // those lanes
 };
+
+constexpr uint32_t kDT = 16, kLastAct = 17, kST = 18, kFifteen = 19;  // bytes behind V0-VF
+constexpr int kLaneBytes = 20;
 
 // Packed display words per instance and bytes per observation frame.
 template <bool kS>
@@ -83,22 +103,41 @@ struct Disp {
   static constexpr int kFrame = kS ? kSchipFrameBytes : kFrameBytes;
 };
 
-__device__ __forceinline__ uint32_t getV(const Ctx &C, uint32_t x) { return C.V[x * C.J]; }
-__device__ __forceinline__ void setV(const Ctx &C, uint32_t x, uint32_t val) { C.V[x * C.J] = val & 0xFFu; }
-__device__ __forceinline__ void setVF(const Ctx &C, uint32_t f) { C.V[15 * C.J] = f; }
+__device__ __forceinline__ uint64_t *disp_of(const Ctx &C) { return reinterpret_cast<uint64_t *>(C.rec); }
+__device__ __forceinline__ uint32_t getV(const Ctx &C, uint32_t x) { return C.V[x]; }
+__device__ __forceinline__ void setV(const Ctx &C, uint32_t x, uint32_t val) { C.V[x] = (uint8_t)val; }
+__device__ __forceinline__ void setVF(const Ctx &C, uint32_t f) { C.V[15] = (uint8_t)f; }
 
 __device__ __forceinline__ uint32_t dirty_bit(uint64_t dirty, uint32_t a) {
   return (uint32_t)(dirty >> ((a & 0xFFFu) >> kPageShift)) & 1u;
 }
 
+// Micro-op offset (8 bytes per even address) of a PC; the sentinel's for an
+// odd PC or one outside the table.
+__device__ __forceinline__ uint32_t to_off(uint32_t pc, uint32_t n_uops) {
+  const uint32_t d = pc - 0x200u;
+  return min(__funnelshift_r(d, d, 1), n_uops) << 3;
+}
+__device__ __forceinline__ uint32_t off_pc(uint32_t off) { return 0x200u + (off >> 2); }
+
+// A fetch at offset o reads the two bytes from off_pc(o) on; the range starts
+// one byte early for that. Nothing written: an offset no fetch has.
+__device__ __forceinline__ void set_range(Regs &R, uint32_t wrange) {
+  const uint32_t lo = wrange & 0xFFFFu, hi = wrange >> 16;
+  R.wrange = wrange;
+  R.wbase = lo > hi ? 0x40000000u : (lo - 1u - 0x200u) << 2;
+  R.wspan = lo > hi ? 0u : ((hi - lo + 1u) << 2) + 3u;
+}
+
 // Page copy-on-write keeps one 64-bit mask in registers, and beside it the
-// range of RAM addresses written since the reset, so a sprite on a dirty
-// page but outside that range (beside a score buffer, say) is still drawn
-// from the shared image. Other reads of a dirty page use its complete copy.
+// range of RAM addresses written since the reset, so a sprite or an
+// instruction on a dirty page but outside that range (beside a score buffer,
+// say) is still read from the shared image. Other reads of a dirty page use
+// its complete copy.
 // True when every byte of [a, a + len) (len <= 32, a + len <= 4096) is as in the image.
-__device__ __forceinline__ bool unwritten(const Regs &R, const Ctx &C, uint32_t a, uint32_t len) {
-  if (!(dirty_bit(R.dirty, a) | dirty_bit(R.dirty, a + len - 1u))) return true;
-  return a + len - 1u < (R.wrange & 0xFFFFu) || a > (R.wrange >> 16);
+__device__ __forceinline__ bool unwritten(const Regs &R, uint32_t a, uint32_t len) {
+  if (a + len - 1u < (R.wrange & 0xFFFFu) || a > (R.wrange >> 16)) return true;
+  return !(dirty_bit(R.dirty, a) | dirty_bit(R.dirty, a + len - 1u));
 }
 
 // A byte of RAM: a dirty page's copy is complete.
@@ -107,6 +146,8 @@ __device__ __forceinline__ uint32_t rd8(const Regs &R, const Ctx &C, uint32_t a)
   return dirty_bit(R.dirty, a) ? (uint32_t)C.ram[a] : img_byte(a);
 }
 
+// All lanes of the instance store the same byte. The page copy must be
+// finished by all of them before any stores into it.
 __device__ __forceinline__ void wr8(Regs &R, const Ctx &C, uint32_t a, uint32_t val) {
   a &= 0xFFFu;
   const uint32_t page = a >> kPageShift;
@@ -118,8 +159,9 @@ __device__ __forceinline__ void wr8(Regs &R, const Ctx &C, uint32_t a, uint32_t 
     dst[2] = src[2];
     dst[3] = src[3];
     R.dirty |= 1ull << page;
+    __syncwarp(C.gmask);
   }
-  R.wrange = min(R.wrange & 0xFFFFu, a) | max(R.wrange >> 16, a) << 16;
+  set_range(R, min(R.wrange & 0xFFFFu, a) | max(R.wrange >> 16, a) << 16);
   C.ram[a] = (uint8_t)val;
 }
 
@@ -143,53 +185,44 @@ __device__ __forceinline__ uint32_t philox_w0(uint32_t c0, uint32_t c1, uint32_t
   return c0;
 }
 
-__device__ __forceinline__ void tick(Regs &R) {
-  R.dt -= (R.dt > 0);
-  R.st -= (R.st > 0);
+__device__ __forceinline__ void tick(const Ctx &C) {
+  uint32_t *w = reinterpret_cast<uint32_t *>(C.V + kDT);
+  uint32_t t = *w;  // DT | last action << 8 | ST << 16 | 15 << 24
+  t -= (t & 0xFFu) != 0u;
+  t -= (t & 0xFF0000u) != 0u ? 0x10000u : 0u;
+  *w = t;
 }
 
 // DXYN: XOR an 8-wide, n-row sprite at (vx mod 64, vy mod 32); VF = collision.
+// Each lane draws the screen rows it owns.
 __device__ __forceinline__ void draw(Regs &R, const Ctx &C, uint32_t vx, uint32_t vy, uint32_t n,
                                      uint32_t quirks) {
   const uint32_t x0 = vx & 63u, y0 = vy & 31u, I = R.I;
   const bool wrap = quirks & OCTAX_QUIRK_WRAP_SPRITES;
-  // the sprite spans at most two pages: read it from the image unless a byte
-  // of it may have been written
-  const bool clean = n == 0 || (I + n <= (uint32_t)kRamBytes && unwritten(R, C, I, n));
-  if (clean && !wrap && I + n <= (uint32_t)kRamBytes) {
-    // Common case: sprite in the shared image, rows below the screen clipped,
-    // no per-row checks; collision bits are OR-ed over the rows.
-    const uint32_t rows = n < 32u - y0 ? n : 32u - y0;
-    uint64_t *row = C.disp + y0 * C.J;
-    uint64_t hit = 0;
-    for (uint32_t r = 0; r < rows; ++r) {
+  const uint32_t rows = wrap ? n : min(n, 32u - y0);  // rows below the screen clip
+  const uint32_t r0 = (C.sub - y0) & (C.L - 1u);      // the first row of this lane
+  uint64_t *const disp = disp_of(C);
+  uint64_t hit = 0;
+  // the sprite is read from the image unless a byte of it may have been written
+  if (!wrap && I + n <= (uint32_t)kRamBytes && (n == 0 || unwritten(R, I, n))) {
+    for (uint32_t r = r0; r < rows; r += C.L) {
       const uint64_t s = (uint64_t)(__brev(img_byte(I + r)) >> 24) << x0;  // pixel j -> bit x0 + j, right edge clips
+      const uint64_t old = disp[y0 + r];
+      hit |= old & s;
+      disp[y0 + r] = old ^ s;
+    }
+  } else {
+    for (uint32_t r = r0; r < rows; r += C.L) {
+      const uint64_t rev = __brev(rd8(R, C, I + r)) >> 24;  // pixel j of the sprite -> bit j
+      uint64_t s = rev << x0;
+      if (wrap && x0 > 56u) s |= rev >> (64u - x0);
+      uint64_t *row = disp + ((y0 + r) & 31u);
       const uint64_t old = *row;
       hit |= old & s;
       *row = old ^ s;
-      row += C.J;
     }
-    setVF(C, hit != 0ull);
-    return;
   }
-  uint32_t coll = 0;
-  for (uint32_t r = 0; r < n; ++r) {
-    uint32_t py = y0 + r;
-    if (py >= 32u) {
-      if (!wrap) break;
-      py &= 31u;
-    }
-    const uint32_t a = (I + r) & 0xFFFu;
-    const uint32_t b = clean ? img_byte(a) : rd8(R, C, a);
-    const uint32_t rev = __brev(b) >> 24;  // pixel j of the sprite -> bit j
-    uint64_t s = (uint64_t)rev << x0;       // right edge clips
-    if (wrap && x0 > 56u) s |= (uint64_t)rev >> (64u - x0);
-    uint64_t *row = C.disp + py * C.J;
-    const uint64_t old = *row;
-    coll |= (old & s) != 0ull;
-    *row = old ^ s;
-  }
-  setVF(C, coll);
+  setVF(C, (__ballot_sync(C.gmask, hit != 0ull) & C.gmask) != 0u);
 }
 
 // Each of the low 16 bits of v doubled (bit j -> bits 2j and 2j + 1).
@@ -216,14 +249,17 @@ __device__ __forceinline__ void draw_schip(Regs &R, const Ctx &C, uint32_t vx, u
   const uint32_t bx = x0 * unit, bits_w = width * unit;  // buffer column, pattern width (<= 32)
   // sprite bytes from the shared image unless one of them may have been written
   const uint32_t I = R.I, nbytes = n ? n : 32u;
-  const bool from_img = I + nbytes <= (uint32_t)kRamBytes && unwritten(R, C, I, nbytes);
-  uint32_t coll = 0;
-  for (uint32_t r = 0; r < rows; ++r) {
-    uint32_t gy = y0 + r;
-    if (gy >= gh) {
+  const bool from_img = I + nbytes <= (uint32_t)kRamBytes && unwritten(R, I, nbytes);
+  uint64_t hit = 0;
+  // buffer rows b below the sprite's top; each lane draws the rows it owns
+  const uint32_t top = y0 * unit;
+  for (uint32_t b = (C.sub - top) & (C.L - 1u); b < rows * unit; b += C.L) {
+    uint32_t by = top + b;
+    if (by >= 64u) {
       if (!wrap) break;
-      gy -= gh;
+      by -= 64u;
     }
+    const uint32_t r = b >> (unit - 1u);
     uint32_t bits;
     if (from_img) bits = n ? img_byte(I + r) : (img_byte(I + 2u * r) << 8) | img_byte(I + 2u * r + 1u);
     else bits = n ? rd8(R, C, I + r) : ((rd8(R, C, I + 2u * r) << 8) | rd8(R, C, I + 2u * r + 1u));
@@ -233,109 +269,214 @@ __device__ __forceinline__ void draw_schip(Regs &R, const Ctx &C, uint32_t vx, u
     uint64_t lo = bx < 64u ? pat << bx : 0ull;
     uint64_t hi = bx == 0u ? 0ull : bx < 64u ? pat >> (64u - bx) : pat << (bx - 64u);
     if (wrap && bx + bits_w > 128u) lo |= pat >> (128u - bx);  // wrapped part re-enters at column 0
-    for (uint32_t d = 0; d < unit; ++d) {
-      uint64_t *row = C.disp + 2u * (gy * unit + d) * C.J;
-      const uint64_t o0 = row[0], o1 = row[C.J];
-      coll |= ((o0 & lo) | (o1 & hi)) != 0ull;
-      row[0] = o0 ^ lo;
-      row[C.J] = o1 ^ hi;
-    }
+    uint64_t *row = disp_of(C) + 2u * by;
+    const uint64_t o0 = row[0], o1 = row[1];
+    hit |= (o0 & lo) | (o1 & hi);
+    row[0] = o0 ^ lo;
+    row[1] = o1 ^ hi;
   }
-  setVF(C, coll);
+  setVF(C, (__ballot_sync(C.gmask, hit != 0ull) & C.gmask) != 0u);
 }
 
 // SCHIP scrolls of the 128x64 buffer by buffer pixels; vacated pixels clear.
 __device__ __forceinline__ void scroll_down(const Ctx &C, uint32_t k) {
-  for (int y = 63; y >= 0; --y)
-    for (int h = 0; h < 2; ++h)
-      C.disp[(2 * y + h) * C.J] = (uint32_t)y >= k ? C.disp[(2 * (y - (int)k) + h) * C.J] : 0ull;
+  // rows change owners: one lane moves them all, between two meetings of the instance's lanes
+  uint64_t *d = disp_of(C);
+  __syncwarp(C.gmask);
+  if (C.sub == 0)
+    for (int w = 127; w >= 0; --w) d[w] = (uint32_t)w >= 2u * k ? d[w - 2 * (int)k] : 0ull;
+  __syncwarp(C.gmask);
 }
 __device__ __forceinline__ void scroll_right(const Ctx &C, uint32_t c) {  // 0 < c < 64
-  for (int y = 0; y < 64; ++y) {
-    const uint64_t lo = C.disp[2 * y * C.J], hi = C.disp[(2 * y + 1) * C.J];
-    C.disp[2 * y * C.J] = lo << c;
-    C.disp[(2 * y + 1) * C.J] = (hi << c) | (lo >> (64u - c));
+  uint64_t *d = disp_of(C);
+  for (uint32_t y = C.sub; y < 64u; y += C.L) {
+    const uint64_t lo = d[2 * y], hi = d[2 * y + 1];
+    d[2 * y] = lo << c;
+    d[2 * y + 1] = (hi << c) | (lo >> (64u - c));
   }
 }
 __device__ __forceinline__ void scroll_left(const Ctx &C, uint32_t c) {  // 0 < c < 64
-  for (int y = 0; y < 64; ++y) {
-    const uint64_t lo = C.disp[2 * y * C.J], hi = C.disp[(2 * y + 1) * C.J];
-    C.disp[2 * y * C.J] = (lo >> c) | (hi << (64u - c));
-    C.disp[(2 * y + 1) * C.J] = hi >> c;
+  uint64_t *d = disp_of(C);
+  for (uint32_t y = C.sub; y < 64u; y += C.L) {
+    const uint64_t lo = d[2 * y], hi = d[2 * y + 1];
+    d[2 * y] = (lo >> c) | (hi << (64u - c));
+    d[2 * y + 1] = hi >> c;
   }
 }
-
-// Opcodes the predicated datapath covers: classes 1 3 4 6 7 A always; 5 9
-// with N = 0; 8 with N in 0-7,E (classic shifts and logic); E with 9E/A1;
-// F with 07 and 15. The rarer FX forms (0A 18 1E 29 ...) take the slow path,
-// which keeps their selects out of every instruction slot.
-__device__ __forceinline__ bool is_fast_op(uint32_t op, uint32_t quirks) {
-  const uint32_t cls = op >> 12, n = op & 15u, nn = op & 0xFFu;
-  const uint32_t cbit = 1u << cls;
-  bool fast = (cbit & 0x04DAu) != 0;
-  fast |= ((cbit & 0x0220u) != 0) & (n == 0);
-  fast |= (cls == 8) & ((n <= 7) | (n == 14)) &
-          ((quirks & (OCTAX_QUIRK_SHIFT_USES_VY | OCTAX_QUIRK_LOGIC_RESETS_VF)) == 0);
-  fast |= (cls == 14) & ((nn == 0x9Eu) | (nn == 0xA1u));
-  fast |= (cls == 15) & ((nn == 0x07u) | (nn == 0x15u));
-  return fast;
+// Clear the rows this lane owns.
+template <bool kS>
+__device__ __forceinline__ void clear_display(const Ctx &C) {
+  uint64_t *d = disp_of(C);
+  constexpr uint32_t kPerRow = kS ? 2 : 1;
+  for (uint32_t y = C.sub; y < Disp<kS>::kWords / kPerRow; y += C.L)
+#pragma unroll
+    for (uint32_t h = 0; h < kPerRow; ++h) d[kPerRow * y + h] = 0ull;
 }
 
-// Decoded form of the opcode at an even image address, built once per CTA
-// (the operands travel beside it: see fetch_uop). A slow opcode is stored raw
-// (bit 20 clear). A fast one has one bit per datapath decision, so that each
-// select tests a single bit:
-//   bits 0-11 NNN (NN, N in its low bits) | 19 write VF (8XYN, N >= 4) | 20 fast |
-//   21 skip negated | 22 skip | 23 skip compares VY (else NN) | 24 jump |
-//   25 skip tests the held key | 26 VX = NN | 27 VX += NN | 28 VX = 8XYN |
-//   29 VX = DT | 30 I = NNN | 31 DT = VX.
-constexpr uint32_t kUopFast = 1u << 20;
-// A slow opcode tagged for the short FX branch of execute (FX0A, FX18, FX29 and
-// FX1E without its quirk): bit 21 set on the raw opcode (bit 20 clear).
-constexpr uint32_t kUopFx = 1u << 21;
+// ---- micro-ops ---------------------------------------------------------------
+// Decoded form of the instruction at an even address, 12 bytes in two tables:
+//   x: coefficients (offset in the table of them) | xs << 8 | ys << 16 (bytes behind Ctx::V), flags
+//      in the top byte
+//   y: offset of the next micro-op when the skip test holds | << 16 when it does not (equal: no skip);
+//      a slow opcode: the opcode | kind << 16
+//   z: immediate << 19 (13 bits, signed) | dst (a byte behind Ctx::V)
+// res = coefficients . (VX, VY, VX & VY, VX >> 1) + immediate, then by flag:
+constexpr uint32_t kUWrite = 1u << 24;  // V[dst] = low byte of res (dst may be DT or ST)
+constexpr uint32_t kUFlag = 1u << 25;   // VF = bit 8 of res (8XY5 / 8XY7 add 256: NOT borrow)
+constexpr uint32_t kUBit0 = 1u << 26;   // ... exclusive-or bit 0 of VX (8XY6)
+constexpr uint32_t kUIndex = 1u << 27;  // I = res
+constexpr uint32_t kUKey = 1u << 28;    // the immediate is the key term: skip when VX & 15 is the held key
+constexpr uint32_t kUSlow = 1u << 29;   // not for the datapath: kind in y
+constexpr uint32_t kKindDraw = 1u << 16, kKindRaw = 2u << 16;  // else the opcode as it is
+// The key term of a step: -key, or 256 with no key held. VX + it, taken modulo
+// 16 with the ninth bit, is zero just when VX & 15 is the key.
+constexpr uint32_t kKeyMask = 0x10Fu, kSkipMask = 0x1FFu;
 
-__device__ __forceinline__ uint32_t make_uop(uint32_t op, uint32_t quirks) {
-  if (!is_fast_op(op, quirks)) {
-    const uint32_t nn = op & 0xFFu;
-    const bool fx = (op >> 12) == 0xFu &&
-                    (nn == 0x0Au || nn == 0x18u || nn == 0x29u || (nn == 0x1Eu && !(quirks & OCTAX_QUIRK_FX1E_VF)));
-    return fx ? (op | kUopFx) : op;
-  }
-  const uint32_t cls = op >> 12, nn = op & 0xFFu;
-  uint32_t u = (op & 0xFFFu) | kUopFast;
+__device__ __forceinline__ constexpr uint32_t coef(int c0, int c1, int c2, int c3) {
+  return (c0 & 0xFF) | (c1 & 0xFF) << 8 | (c2 & 0xFF) << 16 | (uint32_t)(c3 & 0xFF) << 24;
+}
+enum { kCZero, kCX, kCY, kCOr, kCAnd, kCXor, kCAdd, kCSub, kCShr, kCRsub, kCTwice, kCGlyph, kCBigGlyph };
+__constant__ const uint32_t kCoefs[16] = {
+    coef(0, 0, 0, 0), coef(1, 0, 0, 0),  coef(0, 1, 0, 0), coef(1, 1, -1, 0),  // x + y - (x & y) = x | y
+    coef(0, 0, 1, 0), coef(1, 1, -2, 0),                                        // x + y - 2 (x & y) = x ^ y
+    coef(1, 1, 0, 0), coef(1, -1, 0, 0), coef(0, 0, 0, 1), coef(-1, 1, 0, 0), coef(2, 0, 0, 0),
+    coef(0, 0, 5, 0), coef(0, 0, 10, 0)};                                       // glyphs of 5 or 10 bytes
+
+// Micro-op of `op` at table entry e. Successors and jump targets outside the
+// table leave the instruction to the switch, which sets PC itself.
+__device__ __forceinline__ uint3 make_uop(uint32_t op, uint32_t e, uint32_t n_uops, uint32_t quirks, bool schip) {
+  const uint32_t cls = op >> 12, x = (op >> 8) & 15u, y = (op >> 4) & 15u, n = op & 15u, nn = op & 0xFFu;
+  const uint32_t nnn = op & 0xFFFu;
+  const uint32_t next = (e + 1) << 3, skip = (e + 2) << 3;
+  uint32_t flags = 0, dst = x, xs = x, ys = y, c = kCZero, t = next, f = next;
+  int32_t imm = 0;
+  bool fast = e + 1 < n_uops;
+  auto skips = [&](bool negated) {
+    t = negated ? next : skip;
+    f = negated ? skip : next;
+    fast &= e + 2 < n_uops;
+  };
   switch (cls) {
-    case 0x1: u |= 1u << 24; break;
-    case 0x3: u |= 1u << 22; break;
-    case 0x4: u |= (1u << 22) | (1u << 21); break;
-    case 0x5: u |= (1u << 22) | (1u << 23); break;
-    case 0x9: u |= (1u << 22) | (1u << 23) | (1u << 21); break;
-    case 0x6: u |= 1u << 26; break;
-    case 0x7: u |= 1u << 27; break;
-    case 0x8: u |= (1u << 28) | ((op & 15u) >= 4u ? (1u << 19) : 0u); break;
-    case 0xA: u |= 1u << 30; break;
-    case 0xE: u |= (1u << 22) | (1u << 25) | (nn == 0xA1u ? (1u << 21) : 0u); break;
-    default:  // 0xF
-      if (nn == 0x07u) u |= 1u << 29;
-      else u |= 1u << 31;  // 0x15
+    case 0x0:  // 0NNN is ignored; the rest goes to the switch
+      fast &= !(op == 0x00E0u || op == 0x00EEu ||
+                (schip && ((op & 0xFFF0u) == 0x00C0u || (op >= 0x00FBu && op <= 0x00FFu))));
+      break;
+    case 0x1:
+      fast = nnn >= 0x200u && !(nnn & 1u) && ((nnn - 0x200u) >> 1) < n_uops;
+      t = f = (nnn - 0x200u) << 2;
+      break;
+    case 0x3:
+    case 0x4:
+      c = kCX;
+      imm = -(int32_t)nn;
+      skips(cls == 0x4);
+      break;
+    case 0x5:
+    case 0x9:
+      c = kCSub;
+      skips(cls == 0x9);
+      fast &= n == 0;
+      break;
+    case 0x6:
+      imm = (int32_t)nn;
+      flags = kUWrite;
+      break;
+    case 0x7:
+      c = kCX;
+      imm = (int32_t)nn;
+      flags = kUWrite;
+      break;
+    case 0x8:
+      flags = kUWrite;
+      if (n >= 1 && n <= 3 && (quirks & OCTAX_QUIRK_LOGIC_RESETS_VF)) flags |= kUFlag;  // bit 8 of those is 0
+      if ((n == 6 || n == 14) && (quirks & OCTAX_QUIRK_SHIFT_USES_VY)) xs = y;
+      switch (n) {
+        case 0x0: c = kCY; break;
+        case 0x1: c = kCOr; break;
+        case 0x2: c = kCAnd; break;
+        case 0x3: c = kCXor; break;
+        case 0x4: c = kCAdd; flags |= kUFlag; break;
+        case 0x5: c = kCSub; imm = 256; flags |= kUFlag; break;
+        case 0x6: c = kCShr; flags |= kUFlag | kUBit0; break;
+        case 0x7: c = kCRsub; imm = 256; flags |= kUFlag; break;
+        case 0xE: c = kCTwice; flags |= kUFlag; break;
+        default: fast = false; break;
+      }
+      break;
+    case 0xA:
+      imm = (int32_t)nnn;
+      flags = kUIndex;
+      break;
+    case 0xE:
+      c = kCX;
+      flags = kUKey;
+      skips(nn == 0xA1u);
+      fast &= nn == 0x9Eu || nn == 0xA1u;
+      break;
+    case 0xF:
+      if (nn == 0x07u) {
+        c = kCX;
+        xs = kDT;
+        flags = kUWrite;
+      } else if (nn == 0x15u || nn == 0x18u) {
+        c = kCX;
+        dst = nn == 0x15u ? kDT : kST;
+        flags = kUWrite;
+      } else if (nn == 0x29u || (schip && nn == 0x30u)) {
+        c = nn == 0x29u ? kCGlyph : kCBigGlyph;
+        ys = kFifteen;
+        imm = nn == 0x29u ? 0x50 : (int32_t)kBigFontAddr;
+        flags = kUIndex;
+      } else {
+        fast = false;
+      }
+      break;
+    default:
+      fast = false;
       break;
   }
-  return u;
+  if (fast) return make_uint3(c << 2 | xs << 8 | ys << 16 | flags, t | f << 16, (uint32_t)imm << 19 | dst);
+  return make_uint3(x << 8 | y << 16 | kUSlow, op | (cls == 0xDu ? kKindDraw : 0u), 0u);
 }
 
-// The rare / heavy instructions and every variant the fast datapath leaves
-// out (quirk bits, undefined encodings). PC has already been advanced.
+// 4 pixels (bits 0..3) -> 4 bytes of value 0/1 (byte j = bit j).
+__device__ __forceinline__ uint32_t spread4(uint32_t nib) { return (nib * 0x00204081u) & 0x01010101u; }
+
+// One CTA per game: its blob's pixel table and micro-ops from its RAM image.
+__global__ void tables_kernel(uint8_t *blobs, uint64_t stride, uint32_t n_uops, int schip, uint32_t quirks) {
+  uint8_t *b = blobs + blockIdx.x * stride;
+  uint2 *lut = reinterpret_cast<uint2 *>(b + kBlobLut);
+  for (uint32_t i = threadIdx.x; i < 256; i += blockDim.x) lut[i] = make_uint2(spread4(i & 15u), spread4(i >> 4));
+  if (threadIdx.x < 16) reinterpret_cast<uint32_t *>(b + kBlobCoef)[threadIdx.x] = kCoefs[threadIdx.x];
+  uint2 *xy = reinterpret_cast<uint2 *>(b + kBlobUops);
+  uint32_t *z = reinterpret_cast<uint32_t *>(xy + n_uops + 1);
+  for (uint32_t e = threadIdx.x; e <= n_uops; e += blockDim.x) {
+    uint3 u = make_uint3(kUSlow, kKindRaw, 0u);  // the sentinel
+    if (e < n_uops)
+      u = make_uop((uint32_t)b[0x200 + 2 * e] << 8 | b[0x201 + 2 * e], e, n_uops, quirks, schip != 0);
+    xy[e] = make_uint2(u.x, u.y);
+    z[e] = u.z;
+  }
+}
+
+// Any instruction: the rare / heavy ones, undefined encodings, and every one
+// from an odd, written or far address. PC has already been advanced.
+// The lanes of the instance meet here first: those ahead wait before they
+// change the stack, RAM or the flag registers, which the lanes share.
 // kS: the SCHIP variant (128x64 buffer, extra 00xx and FXxx forms).
 template <bool kS>
 __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, uint32_t pc, int key,
                                        uint32_t quirks) {
   const uint32_t x = (op >> 8) & 15u, y = (op >> 4) & 15u, n = op & 15u, nn = op & 0xFFu;
   const uint32_t nnn = op & 0xFFFu;
+  uint16_t *const stack = reinterpret_cast<uint16_t *>(C.rec + Rec<kS>::kStack);
+  uint8_t *const rpl = kS ? reinterpret_cast<uint8_t *>(C.rec + Rec<kS>::kRpl) : nullptr;
+  __syncwarp(C.gmask);
   const uint32_t vx = getV(C, x), vy = getV(C, y);
   switch (op >> 12) {
     case 0x0:
       if (op == 0x00E0u) {
-#pragma unroll 8
-        for (int r = 0; r < Disp<kS>::kWords; ++r) C.disp[r * C.J] = 0ull;
+        clear_display<kS>(C);
       } else if (kS && (op & 0xFFF0u) == 0x00C0u) {  // scroll down N
         scroll_down(C, n * (R.hires ? 1u : 2u));
       } else if (kS && op == 0x00FBu) {  // scroll right 4
@@ -353,7 +494,7 @@ __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, ui
           R.sp = 16;
         }
         R.sp -= 1;
-        R.pc = C.stack[R.sp * C.J];
+        R.pc = stack[R.sp];
       }
       break;
     case 0x1:
@@ -364,7 +505,7 @@ __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, ui
         R.status |= OCTAX_STATUS_STACK_FAULT;
         R.sp = 0;
       }
-      C.stack[R.sp * C.J] = R.pc;
+      stack[R.sp] = (uint16_t)R.pc;
       R.sp += 1;
       R.pc = nnn;
       break;
@@ -441,8 +582,8 @@ __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, ui
       R.pc = (nnn + ((quirks & OCTAX_QUIRK_JUMP_VX) ? vx : getV(C, 0))) & 0xFFFu;
       break;
     case 0xC: {
-      const uint32_t rnd = philox_w0(R.uid, R.env_steps, pc | ((R.draws & 0xFFFFu) << 16), R.phase,
-                                     R.key0, R.key1);
+      const uint32_t rnd = philox_w0(C.rec[Rec<kS>::kUid], R.env_steps, pc | ((R.draws & 0xFFFFu) << 16), R.phase,
+                                     C.rec[Rec<kS>::kKey], C.rec[Rec<kS>::kKey + 1]);
       R.draws += 1;
       setV(C, x, rnd & nn);
       break;
@@ -464,13 +605,13 @@ __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, ui
     }
     default:  // 0xF
       switch (nn) {
-        case 0x07: setV(C, x, R.dt); break;
+        case 0x07: setV(C, x, getV(C, kDT)); break;
         case 0x0A:
           if (key >= 0) setV(C, x, (uint32_t)key);
           else R.pc = pc;
           break;
-        case 0x15: R.dt = vx; break;
-        case 0x18: R.st = vx; break;
+        case 0x15: setV(C, kDT, vx); break;
+        case 0x18: setV(C, kST, vx); break;
         case 0x1E: {
           const uint32_t s = R.I + vx;
           R.I = s & 0xFFFFu;
@@ -484,14 +625,14 @@ __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, ui
           break;
         case 0x75:
           if (kS) {
-            for (uint32_t i = 0; i <= x; ++i) C.rpl[i] = (uint8_t)getV(C, i);
+            for (uint32_t i = 0; i <= x; ++i) rpl[i] = (uint8_t)getV(C, i);
           } else {
             R.status |= OCTAX_STATUS_BAD_OP;
           }
           break;
         case 0x85:
           if (kS) {
-            for (uint32_t i = 0; i <= x; ++i) setV(C, i, C.rpl[i]);
+            for (uint32_t i = 0; i <= x; ++i) setV(C, i, rpl[i]);
           } else {
             R.status |= OCTAX_STATUS_BAD_OP;
           }
@@ -517,84 +658,55 @@ __device__ __forceinline__ void exec_slow(Regs &R, const Ctx &C, uint32_t op, ui
   }
 }
 
-// Micro-op of the instruction at pc as {make_uop word, X * J, Y * J, NNN}:
-// the shared-memory offsets of VX and VY come pre-multiplied. kW: the table
-// holds those four words (one 16-byte load); otherwise it holds {word,
-// X * J | Y * J << 16} (half the shared memory, two more extracts). Odd PCs
-// and written pages give the raw opcode, which takes the general path.
-template <bool kW>
-__device__ __forceinline__ uint4 fetch_uop(const Regs &R, const Ctx &C, uint32_t pc) {
-  if (!((pc & 1u) | dirty_bit(R.dirty, pc))) {
-    if (kW) return static_cast<const uint4 *>(C.uops)[pc >> 1];
-    const uint2 e = static_cast<const uint2 *>(C.uops)[pc >> 1];
-    return make_uint4(e.x, e.y & 0xFFFFu, e.y >> 16, e.x & 0xFFFu);
-  }
-  return make_uint4((rd8(R, C, pc) << 8) | rd8(R, C, pc + 1u), 0u, 0u, 0u);
+// a (unsigned bytes) . b (signed bytes) + c
+__device__ __forceinline__ int32_t dot4(uint32_t a, uint32_t b, int32_t c) {
+  int32_t d;
+  asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
 }
 
-// Execute micro-op u, the instruction at R.pc. key: held CHIP-8 key or -1.
+// Run `count` instructions from R.pc on. key: held CHIP-8 key or -1.
+// The loop carries the micro-op offset; R.pc holds the PC whenever the offset
+// is the sentinel's.
 template <bool kS>
-__device__ __forceinline__ void execute(Regs &R, const Ctx &C, const uint4 u4, int key, uint32_t quirks) {
-  const uint32_t pc = R.pc, u = u4.x;
-  if (u & kUopFast) {
-    const uint32_t nnn = u4.w, nn = u & 0xFFu, n = u & 15u;
-    uint32_t *const Vx = C.V + u4.y;
-    const uint32_t vx = *Vx, vy = C.V[u4.z];
-    // next PC: skips (bit 22; 23: against VY, 25: against the held key; 21: negated), jump (24)
-    const uint32_t lhs = (u & (1u << 25)) ? (vx & 15u) : vx;
-    const uint32_t rhs = (u & (1u << 25)) ? (uint32_t)key : ((u & (1u << 23)) ? vy : nn);
-    const bool skip = (u & (1u << 22)) && ((lhs == rhs) != ((u & (1u << 21)) != 0u));
-    uint32_t npc = (pc + (skip ? 4u : 2u)) & 0xFFFu;
-    npc = (u & (1u << 24)) ? nnn : npc;
-    R.pc = npc;
-    // 8XYN result and flag (N in 0-7, E) as integer linear combinations, so
-    // the work runs as multiply-adds (stage_game lists the coefficients):
-    // result = c0 vx + c1 vy + c2 (vx & vy) + c3 (vx >> 1), whose low byte is
-    // VX; the carry / NOT-borrow / shifted-out bit is bit 8 of a result + b vx + k.
-    const int4 cr = C.alu[2 * n], cf = C.alu[2 * n + 1];
-    const int32_t ix = (int32_t)vx, iy = (int32_t)vy;
-    const int32_t res = cr.x * ix + cr.y * iy + cr.z * (ix & iy) + cr.w * (ix >> 1);
-    const uint32_t alu = (uint32_t)res;
-    const uint32_t flag = ((uint32_t)(cf.x * res + cf.y * ix + cf.z) >> 8) & 1u;
-    // VX write (26: NN, 27: VX + NN, 28: 8XYN, 29: DT), VF (19), I = NNN (30), DT = VX (31)
-    uint32_t val = (u & (1u << 27)) ? (vx + nn) : nn;
-    val = (u & (1u << 28)) ? alu : val;
-    val = (u & (1u << 29)) ? R.dt : val;
-    if (u & (15u << 26)) *Vx = val & 0xFFu;
-    if (u & (1u << 19)) C.V[15 * C.J] = flag;  // after VX: with X = F the flag wins
-    R.I = (u & (1u << 30)) ? nnn : R.I;
-    R.dt = (u & (1u << 31)) ? vx : R.dt;
-  } else if (u & kUopFx) {  // FX0A / FX18 / FX1E / FX29: a short branch, not the general switch
-    R.pc = (pc + 2u) & 0xFFFu;
-    uint32_t *const Vx = C.V + u4.y;
-    const uint32_t vx = *Vx, nn = u & 0xFFu;
-    if (nn == 0x0Au) {
-      if (key >= 0) *Vx = (uint32_t)key;
-      else R.pc = pc;
-    } else if (nn == 0x18u) {
-      R.st = vx;
-    } else if (nn == 0x1Eu) {
-      R.I = (R.I + vx) & 0xFFFFu;
-    } else {
-      R.I = 0x50u + 5u * (vx & 15u);
-    }
-  } else if ((u >> 12) == 0xDu) {  // DXYN, the most frequent slow opcode: its own branch
-    R.pc = (pc + 2u) & 0xFFFu;
-    if (kS) draw_schip(R, C, getV(C, (u >> 8) & 15u), getV(C, (u >> 4) & 15u), u & 15u, quirks);
-    else draw(R, C, getV(C, (u >> 8) & 15u), getV(C, (u >> 4) & 15u), u & 15u, quirks);
-  } else {
-    R.pc = (pc + 2u) & 0xFFFu;
-    exec_slow<kS>(R, C, u & 0xFFFFu, pc, key, quirks);
-  }
-}
-
-// Run `count` instructions.
-template <bool kS, bool kW>
-__device__ __forceinline__ void run_instrs(Regs &R, const Ctx &C, int key, uint32_t quirks,
-                                           uint32_t count) {
+__device__ __forceinline__ void run_instrs(Regs &R, const Ctx &C, int key, uint32_t quirks, uint32_t count) {
+  const uint8_t *const uops = g_smem + kBlobUops;
+  const uint32_t sentinel = C.n_uops << 3;
+  const uint8_t *const imms = uops + sentinel + 8;
+  const int32_t keyterm = key >= 0 ? -key : 256;
+  uint32_t off = to_off(R.pc, C.n_uops);
   // Not unrolled: on divergent programs a second copy of the datapath costs
   // more in instruction fetch than the loop overhead it saves.
-  for (uint32_t k = 0; k < count; ++k) execute<kS>(R, C, fetch_uop<kW>(R, C, R.pc), key, quirks);
+#pragma unroll 1
+  for (uint32_t k = 0; k < count; ++k) {
+    uint2 u = *reinterpret_cast<const uint2 *>(uops + off);
+    const uint32_t z = *reinterpret_cast<const uint32_t *>(imms + (off >> 1));
+    if (off - R.wbase <= R.wspan && dirty_bit(R.dirty, off_pc(off))) u = make_uint2(kUSlow, kKindRaw);  // written
+    const uint32_t vx = C.V[(u.x >> 8) & 0xFFu], vy = C.V[(u.x >> 16) & 0xFFu];
+    if (!(u.x & kUSlow)) {
+      const uint32_t c = *reinterpret_cast<const uint32_t *>(g_smem + kBlobCoef + (u.x & 0xFFu));
+      const bool by_key = u.x & kUKey;
+      const int32_t res = dot4(vx + (vy << 8) + ((vx & vy) << 16) + ((vx >> 1) << 24), c,
+                               by_key ? keyterm : (int32_t)z >> 19);
+      off = ((uint32_t)res & (by_key ? kKeyMask : kSkipMask)) == 0u ? u.y & 0xFFFFu : u.y >> 16;
+      if (u.x & kUWrite) C.V[z & 31u] = (uint8_t)res;
+      // after VX: with X = F the flag wins
+      if (u.x & kUFlag) C.V[15] = (uint8_t)((((uint32_t)res >> 8) ^ ((u.x & kUBit0) ? vx : 0u)) & 1u);
+      if (u.x & kUIndex) R.I = (uint32_t)res;
+    } else {
+      const uint32_t pc = off == sentinel ? R.pc : off_pc(off);
+      R.pc = (pc + 2u) & 0xFFFu;
+      if (u.y & kKindDraw) {
+        if (kS) draw_schip(R, C, vx, vy, u.y & 15u, quirks);
+        else draw(R, C, vx, vy, u.y & 15u, quirks);
+      } else {
+        const uint32_t op = (u.y & kKindRaw) ? rd8(R, C, pc) << 8 | rd8(R, C, pc + 1u) : u.y;
+        exec_slow<kS>(R, C, op, pc, key, quirks);
+      }
+      off = to_off(R.pc, C.n_uops);
+    }
+  }
+  if (off != sentinel) R.pc = off_pc(off);
 }
 
 __device__ __forceinline__ int32_t term_value(const Regs &R, const Ctx &C, const TermDev &t) {
@@ -639,395 +751,341 @@ __device__ __forceinline__ bool terminated(const Regs &R, const Ctx &C, const Ga
 // K), then the no-op reset wrapper (§3.2): a drawn number of no-key env steps
 // of frameskip frames each, unobserved. The previous action becomes the no-op.
 // kWrap = false compiles the wrapper out (no game of the launch uses it).
-template <bool kWrap, bool kS, bool kW>
+template <bool kWrap, bool kS>
 __device__ __forceinline__ void reset_instance(Regs &R, const Ctx &C, const GameDev &G, uint32_t quirks) {
+  uint32_t *const V = reinterpret_cast<uint32_t *>(C.V);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) C.V[i * C.J] = 0;
+  for (int i = 0; i < 4; ++i) V[i] = 0;
+  V[4] = 15u << 24;  // DT, ST = 0
   R.pc = 0x200;
   R.I = 0;
   R.sp = 0;
-  R.dt = 0;
-  R.st = 0;
   R.dirty = 0;
-  R.wrange = kNoWrites;
+  set_range(R, kNoWrites);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) C.stack[i * C.J] = 0;
-#pragma unroll 8
-  for (int r = 0; r < Disp<kS>::kWords; ++r) C.disp[r * C.J] = 0ull;
+  for (int i = 0; i < 8; ++i) C.rec[Rec<kS>::kStack + i] = 0;
+  clear_display<kS>(C);
   R.hires = 0;  // SCHIP: every episode starts in lores with clear flag registers
   if (kS)
-    for (int i = 0; i < 16; ++i) C.rpl[i] = 0;
+    for (int i = 0; i < 4; ++i) C.rec[Rec<kS>::kRpl + i] = 0;
   // Startup: full chunks of K (each followed by a tick), then the remainder
   // (no tick); after it, the no-op frames (K instructions and a tick each).
   // One loop, so that the interpreter is inlined here only once.
   const uint32_t noop_frames =
       !kWrap || G.max_noops == 0u ? 0u
-                        : philox_w0(R.uid, R.env_steps, 0u, 3u, R.key0, R.key1) % (G.max_noops + 1u) * G.frameskip;
+                        : philox_w0(C.rec[Rec<kS>::kUid], R.env_steps, 0u, 3u, C.rec[Rec<kS>::kKey],
+                                    C.rec[Rec<kS>::kKey + 1]) % (G.max_noops + 1u) * G.frameskip;
   const uint32_t full = G.startup / G.K, rem = G.startup - full * G.K;
   const uint32_t chunks = full + (rem != 0u) + noop_frames;
   R.phase = 1;
   R.draws = 0;
   for (uint32_t i = 0; i < chunks; ++i) {
     const bool partial = i == full && rem != 0u;
-    run_instrs<kS, kW>(R, C, -1, quirks, partial ? rem : G.K);
-    if (!partial) tick(R);
+    run_instrs<kS>(R, C, -1, quirks, partial ? rem : G.K);
+    if (!partial) tick(C);
   }
-  R.last_act = G.n_actions;
+  C.V[kLastAct] = (uint8_t)G.n_actions;
   R.phase = 0;
   R.draws = 0;
 }
 
-// 4 pixels (bits 0..3) -> 4 bytes of value 0/1 (byte j = bit j).
-__device__ __forceinline__ uint32_t spread4(uint32_t nib) { return (nib * 0x00204081u) & 0x01010101u; }
-
 // Pixels 16q..16q+15 of a packed row -> 16 bytes of 0/1, through a
 // per-CTA table that maps a byte of pixels to its 8 output bytes.
-__device__ __forceinline__ uint4 expand16(uint64_t row, uint32_t q, const uint2 *lut) {
+__device__ __forceinline__ uint4 expand16(uint64_t row, uint32_t q) {
+  const uint2 *const lut = reinterpret_cast<const uint2 *>(g_smem + kBlobLut);
   const uint32_t bits = (uint32_t)(row >> (16u * q)) & 0xFFFFu;
   const uint2 lo = lut[bits & 0xFFu], hi = lut[bits >> 8];
   return make_uint4(lo.x, lo.y, hi.x, hi.y);
 }
 
-// Whole-warp frame write: lane -> instance 8m + lane/4 of the warp, quarter
-// lane%4 of every row, for the warp's `ipw` instances. frame (per lane, 0 =
-// skip) points at the 2 KB frame of that lane's own instance.
+// Whole-warp frame write of the warp's `ipw` instances (records at `recs`).
+// frame (per lane, 0 = skip) points at the frame of that lane's own instance,
+// whose lanes start at instance << lane_sh.
+// 16-byte pieces of a row: 4 (CHIP-8) or 8 (SCHIP) lanes write one row, so the
+// warp writes 8 (4) rows at a time: one row of each of 8 (4) instances, or, with
+// fewer instances, several rows of each.
 template <bool kS>
-__device__ __forceinline__ void capture_frame(const uint64_t *disp_warp, int J, uint8_t *frame,
-                                              int lane, int ipw, const uint2 *lut);
-
-// CHIP-8 frame (32 rows x 64 bytes): lanes 4i..4i+3 write the four 16-pixel
-// quarters of one row of instance i (8 instances per pass).
-template <>
-__device__ __forceinline__ void capture_frame<false>(const uint64_t *disp_warp, int J, uint8_t *frame,
-                                                     int lane, int ipw, const uint2 *lut) {
+__device__ __forceinline__ void capture_frame(const uint32_t *recs, uint8_t *frame, int lane, int ipw, int lane_sh) {
+  constexpr int kPer = kS ? 8 : 4, kLogAll = kS ? 2 : 3;  // lanes per row, log2(rows at a time)
+  constexpr int kRows = kS ? 64 : 32, kRowBytes = kS ? 128 : 64;
   const uint64_t mine = reinterpret_cast<uint64_t>(frame);
-  const uint32_t q = lane & 3;
-  const int passes = (ipw + 7) >> 3;
-  for (int m = 0; m < passes; ++m) {
-    const int src = 8 * m + (lane >> 2);
-    const uint64_t base = __shfl_sync(kFull, mine, src);
-    if (base) {
-      const uint64_t *col = disp_warp + src;
+  const uint32_t q = lane & (kPer - 1);
+  const int lg = min(5 - lane_sh, kLogAll);   // log2(instances at a time)
+  const int step = 1 << (kLogAll - lg);       // rows of one instance at a time
+  const int place = lane / kPer;              // row of the 8 (4)
+  const int r0 = place & (step - 1);
+  for (int m = 0; m < ipw; m += 1 << lg) {
+    const int src = m + (place >> (kLogAll - lg));
+    const uint64_t base = __shfl_sync(kFull, mine, (src << lane_sh) & 31);
+    if (src < ipw && base) {
+      const uint64_t *row = reinterpret_cast<const uint64_t *>(recs + src * Rec<kS>::kWords);
+      if (kS) row += q >> 2;
       uint8_t *dst = reinterpret_cast<uint8_t *>(base) + q * 16u;
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) __stcs(reinterpret_cast<uint4 *>(dst + r * 64), expand16(col[r * J], q, lut));
-    }
-  }
-}
-
-// SCHIP frame (64 rows x 128 bytes): lanes 8i..8i+7 write the eight 16-pixel
-// chunks of one row of instance i (4 instances per pass).
-template <>
-__device__ __forceinline__ void capture_frame<true>(const uint64_t *disp_warp, int J, uint8_t *frame,
-                                                    int lane, int ipw, const uint2 *lut) {
-  const uint64_t mine = reinterpret_cast<uint64_t>(frame);
-  const uint32_t q = lane & 7, h = q >> 2;
-  const int passes = (ipw + 3) >> 2;
-  for (int m = 0; m < passes; ++m) {
-    const int src = 4 * m + (lane >> 3);
-    const uint64_t base = __shfl_sync(kFull, mine, src);
-    if (base) {
-      const uint64_t *col = disp_warp + src;
-      uint8_t *dst = reinterpret_cast<uint8_t *>(base) + q * 16u;
-#pragma unroll 8
-      for (int r = 0; r < 64; ++r)
-        __stcs(reinterpret_cast<uint4 *>(dst + r * 128), expand16(col[(2 * r + h) * J], q & 3u, lut));
+      for (int r = r0; r < kRows; r += 4 * step)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int y = r + u * step;
+          __stcs(reinterpret_cast<uint4 *>(dst + y * kRowBytes), expand16(row[kS ? 2 * y : y], q & 3u));
+        }
     }
   }
 }
 
 // Packed frame of every instance of the warp with a non-null `frame`: its
-// display words copied as they are, two per 16-byte streaming store
-// (CHIP-8: 16 stores per instance, two instances per pass; SCHIP: 64).
+// display words copied as they are, two per 16-byte streaming store.
 template <bool kS>
-__device__ __forceinline__ void capture_packed(const uint64_t *disp_warp, int J, uint8_t *frame, int lane,
-                                               int ipw) {
-  constexpr int kPairs = Disp<kS>::kWords / 2;  // 16-byte stores per instance-frame
-  constexpr int kPerPass = 32 / (kPairs < 32 ? kPairs : 32);
+__device__ __forceinline__ void capture_packed(const uint32_t *recs, uint8_t *frame, int lane, int ipw, int lane_sh) {
+  constexpr int kPieces = Disp<kS>::kWords / 2;  // 16-byte stores per instance-frame: 16 or 64
+  constexpr int kAtOnce = kS ? 1 : 2;            // instances
   const uint64_t mine = reinterpret_cast<uint64_t>(frame);
-  for (int m = 0; m < ipw; m += kPerPass) {
-    const int src = m + lane / (32 / kPerPass);
-    const uint64_t base = __shfl_sync(kFull, mine, src < 32 ? src : 31);
-    if (src < ipw && base) {
-      const uint64_t *col = disp_warp + src;
-      for (int c = lane % (32 / kPerPass); c < kPairs; c += 32 / kPerPass) {
-        const uint64_t w0 = col[(2 * c) * J], w1 = col[(2 * c + 1) * J];
-        __stcs(reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(base) + c * 16),
-               make_uint4((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32)));
-      }
-    }
+  for (int m = 0; m < ipw; m += kAtOnce) {
+    const int src = m + (kS ? 0 : lane >> 4);
+    const uint64_t base = __shfl_sync(kFull, mine, (src << lane_sh) & 31);
+    if (src < ipw && base)
+      for (int c = lane & (kS ? 31 : 15); c < kPieces; c += 32)
+        __stcs(reinterpret_cast<uint4 *>(base) + c, reinterpret_cast<const uint4 *>(recs + src * Rec<kS>::kWords)[c]);
   }
 }
 
 // Packed reset observation of the instances in `which` (every stack slot).
 template <bool kS>
-__device__ __forceinline__ void write_reset_packed(const uint64_t *disp_warp, int J, uint8_t *obs, int S,
-                                                   unsigned which, int lane) {
-  constexpr int kPairs = Disp<kS>::kWords / 2;
+__device__ __forceinline__ void write_reset_packed(const uint32_t *recs, uint8_t *obs, int S, unsigned which, int lane,
+                                                   int lane_sh) {
+  constexpr int kPieces = Disp<kS>::kWords / 2;
   const uint64_t mine = reinterpret_cast<uint64_t>(obs);
-  while (which) {
+  while (which) {  // bit of an instance's first lane
     const int src = __ffs(which) - 1;
     which &= which - 1;
-    const uint64_t base = __shfl_sync(kFull, mine, src);
-    const uint64_t *col = disp_warp + src;
-    for (int c = lane; c < kPairs; c += 32) {
-      const uint64_t w0 = col[(2 * c) * J], w1 = col[(2 * c + 1) * J];
-      const uint4 o = make_uint4((uint32_t)w0, (uint32_t)(w0 >> 32), (uint32_t)w1, (uint32_t)(w1 >> 32));
-      for (int s = 0; s < S; ++s)
-        __stcs(reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(base) + s * 8 * Disp<kS>::kWords + c * 16), o);
-    }
+    uint4 *const base = reinterpret_cast<uint4 *>(__shfl_sync(kFull, mine, src));
+    const uint4 *const d = reinterpret_cast<const uint4 *>(recs + (src >> lane_sh) * Rec<kS>::kWords);
+    for (int c = lane; c < kPieces; c += 32)
+      for (int s = 0; s < S; ++s) __stcs(base + s * kPieces + c, d[c]);
   }
 }
 
 // Reset observation of the instances in `which`: the display in every stack slot.
 template <bool kS>
-__device__ __forceinline__ void write_reset_obs(const uint64_t *disp_warp, int J, uint8_t *obs, int S,
-                                                unsigned which, int lane, const uint2 *lut) {
+__device__ __forceinline__ void write_reset_obs(const uint32_t *recs, uint8_t *obs, int S, unsigned which, int lane,
+                                                int lane_sh) {
   const uint64_t mine = reinterpret_cast<uint64_t>(obs);
   constexpr int kChunks = Disp<kS>::kFrame / 16;  // 16-byte chunks per frame
-  while (which) {
+  while (which) {  // bit of an instance's first lane
     const int src = __ffs(which) - 1;
     which &= which - 1;
     const uint64_t base = __shfl_sync(kFull, mine, src);
-    const uint64_t *col = disp_warp + src;
+    const uint64_t *const d = reinterpret_cast<const uint64_t *>(recs + (src >> lane_sh) * Rec<kS>::kWords);
 #pragma unroll
     for (int it = 0; it < kChunks / 32; ++it) {
-      const int c = it * 32 + lane;  // 16-byte chunk of the frame
-      uint4 o;
-      if (kS) o = expand16(col[(2 * (c >> 3) + ((c >> 2) & 1)) * J], c & 3, lut);
-      else o = expand16(col[(c >> 2) * J], c & 3, lut);
+      const int c = it * 32 + lane;  // 16-byte chunk of the frame: word c / 4 of the display
+      const uint4 o = expand16(d[c >> 2], c & 3);
       for (int s = 0; s < S; ++s)
         __stcs(reinterpret_cast<uint4 *>(reinterpret_cast<uint8_t *>(base) + s * Disp<kS>::kFrame + c * 16), o);
     }
   }
 }
 
-struct Smem {
-  uint8_t *img;
-  GameDev *game;
-  void *uops;       // micro-op table (fetch_uop)
-  int4 *alu;        // 8XYN coefficients (execute)
-  uint2 *lut;       // byte of pixels -> 8 bytes of 0/1
-  uint64_t *disp;
-  uint32_t *stack;
-  uint32_t *V;
+__device__ __forceinline__ void copy16_async(void *smem, const void *gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Shared memory of a CTA: the game's blob | records [instances] | registers [emulator lanes][20].
+__device__ __forceinline__ uint32_t *smem_recs(uint32_t n_uops) {
+  return reinterpret_cast<uint32_t *>(g_smem + blob_bytes(n_uops));
+}
+__device__ __forceinline__ const GameDev &smem_game() { return *reinterpret_cast<const GameDev *>(g_smem + kRamBytes); }
+
+// Starts the copy of a game's blob (all threads; copy_wait and a barrier follow).
+__device__ __forceinline__ void stage_game(const uint8_t *blobs, uint32_t stride, int game, uint32_t n_uops) {
+  const uint8_t *src = blobs + (size_t)game * stride;
+  const uint32_t bytes = n_uops ? blob_bytes(n_uops) : (uint32_t)kBlobUops;
+  for (uint32_t i = 16 * threadIdx.x; i < bytes; i += 16 * blockDim.x) copy16_async(g_smem + i, src + i);
+  // no room for the table: only the sentinel
+  if (!n_uops && threadIdx.x < 3) reinterpret_cast<uint32_t *>(g_smem + kBlobUops)[threadIdx.x] = threadIdx.x ? kKindRaw : kUSlow;
+}
+
+// The lanes of a warp and what it emulates: ipw instances, each by 1 << sh lanes.
+struct Warp {
+  int lane, w, ipw, sh;  // w: among the CTA's emulator warps
+  int J;                 // instances of the CTA
+  int i, j;              // this lane's instance within the warp / the CTA
+  uint32_t *recs;        // the warp's records
+  bool active;           // this lane emulates an instance
+  int count;             // instances of this warp
 };
 
-// Shared memory of a CTA with J instances: image | game | decoded opcodes |
-// expansion table | 8XYN coefficients | display [W][J] u64 | stack [16][J] u32 | V [16][J] u32,
-// W = 32 (CHIP-8) or 128 (SCHIP).
-template <bool kS, bool kW>
-__device__ __forceinline__ Smem carve(uint8_t *smem, int J) {
-  constexpr int kUopSmem = kW ? kUopSmemWide : kUopSmemNarrow;
-  Smem s;
-  s.img = smem;
-  s.game = reinterpret_cast<GameDev *>(smem + kRamBytes);
-  s.uops = smem + kRamBytes + kGameSmem;
-  s.lut = reinterpret_cast<uint2 *>(smem + kRamBytes + kGameSmem + kUopSmem);
-  s.alu = reinterpret_cast<int4 *>(smem + kRamBytes + kGameSmem + kUopSmem + kLutSmem);
-  s.disp = reinterpret_cast<uint64_t *>(smem + kRamBytes + kGameSmem + kUopSmem + kLutSmem + kAluSmem);
-  s.stack = reinterpret_cast<uint32_t *>(s.disp + Disp<kS>::kWords * J);
-  s.V = s.stack + 16 * J;
-  return s;
-}
-
-// Every thread of the CTA calls this (it contains a barrier).
-template <bool kW>
-__device__ __forceinline__ void stage_game(const Smem &S, const GameDev *games, const uint8_t *images,
-                                           int game, uint32_t quirks, int J) {
-  const uint4 *src = reinterpret_cast<const uint4 *>(images + (size_t)game * kRamBytes);
-  uint4 *dst = reinterpret_cast<uint4 *>(S.img);
-  for (int i = threadIdx.x; i < kRamBytes / 16; i += blockDim.x) dst[i] = src[i];
-  const uint4 *gs = reinterpret_cast<const uint4 *>(games + game);
-  uint4 *gd = reinterpret_cast<uint4 *>(S.game);
-  for (int i = threadIdx.x; i < (int)(sizeof(GameDev) / 16); i += blockDim.x) gd[i] = gs[i];
-  __syncthreads();
-  for (int b = threadIdx.x; b < 256; b += blockDim.x) S.lut[b] = make_uint2(spread4(b & 15u), spread4(b >> 4));
-  if (threadIdx.x < 16) {
-    // per N: {c0, c1, c2, c3} {a, b, k, 0} (see execute); other N are never fast
-    int4 r = make_int4(0, 0, 0, 0), f = make_int4(0, 0, 0, 0);
-    switch (threadIdx.x) {
-      case 0x0: r = make_int4(0, 1, 0, 0); break;                                    // VY
-      case 0x1: r = make_int4(1, 1, -1, 0); break;                                   // x + y - (x & y) = x | y
-      case 0x2: r = make_int4(0, 0, 1, 0); break;                                    // x & y
-      case 0x3: r = make_int4(1, 1, -2, 0); break;                                   // x + y - 2 (x & y) = x ^ y
-      case 0x4: r = make_int4(1, 1, 0, 0); f = make_int4(1, 0, 0, 0); break;         // carry = bit 8 of the sum
-      case 0x5: r = make_int4(1, -1, 0, 0); f = make_int4(1, 0, 256, 0); break;      // NOT borrow: x - y + 256 >= 256
-      case 0x6: r = make_int4(0, 0, 0, 1); f = make_int4(-512, 256, 0, 0); break;    // bit 0: 256 (x - 2 (x >> 1))
-      case 0x7: r = make_int4(-1, 1, 0, 0); f = make_int4(1, 0, 256, 0); break;      // NOT borrow: y - x + 256 >= 256
-      case 0xE: r = make_int4(2, 0, 0, 0); f = make_int4(1, 0, 0, 0); break;         // bit 7 shifted out = bit 8 of 2x
-      default: break;
-    }
-    S.alu[2 * threadIdx.x] = r;
-    S.alu[2 * threadIdx.x + 1] = f;
-  }
-  // decode the opcode at every even address of the image once
-  for (int w = threadIdx.x; w < kRamBytes / 2; w += blockDim.x) {
-    const uint32_t op = ((uint32_t)S.img[2 * w] << 8) | S.img[2 * w + 1];
-    const uint32_t xo = ((op >> 8) & 15u) * (uint32_t)J, yo = ((op >> 4) & 15u) * (uint32_t)J;
-    if (kW) static_cast<uint4 *>(S.uops)[w] = make_uint4(make_uop(op, quirks), xo, yo, op & 0xFFFu);
-    else static_cast<uint2 *>(S.uops)[w] = make_uint2(make_uop(op, quirks), xo | (yo << 16));
-  }
+__device__ __forceinline__ Warp make_warp(int ipw, int emu_warps, const Group &g, uint32_t n_uops, int words) {
+  Warp W;
+  W.lane = threadIdx.x & 31;
+  W.w = threadIdx.x >> 5;
+  W.ipw = ipw;
+  W.sh = ipw <= 1 ? 5 : __clz(ipw - 1) - 27;  // 5 - ceil(log2(ipw))
+  W.J = emu_warps * ipw;
+  W.i = W.lane >> W.sh;
+  W.j = W.w * ipw + W.i;
+  W.count = min(max((int)g.count - W.w * ipw, 0), ipw);
+  W.active = W.i < W.count;
+  W.recs = smem_recs(n_uops) + W.w * ipw * words;
+  return W;
 }
 
 template <bool kS>
-__device__ __forceinline__ void load_regs(Regs &R, const DevState &st, int64_t slot) {
-  const uint32_t pcI = st.pcI[slot], misc = st.misc[slot];
-  const int64_t n = st.n;
+__device__ __forceinline__ Ctx make_ctx(const Warp &W, const DevState &st, int64_t slot, uint32_t n_uops) {
+  Ctx C;
+  C.rec = W.recs + (W.active ? W.i : 0) * Rec<kS>::kWords;
+  C.V = reinterpret_cast<uint8_t *>(smem_recs(n_uops) + W.J * Rec<kS>::kWords) + threadIdx.x * kLaneBytes;
+  C.ram = st.ram + slot * (int64_t)kRamBytes;
+  C.n_uops = n_uops;
+  C.L = 1u << W.sh;
+  C.sub = W.lane & (C.L - 1u);
+  C.gmask = (W.sh == 5 ? kFull : (1u << C.L) - 1u) << (W.lane - C.sub);
+  return C;
+}
+
+// Starts the copy of the warp's records (copy_wait and a warp barrier follow).
+template <bool kS>
+__device__ __forceinline__ void fetch_records(const Warp &W, const DevState &st, const Group &g) {
+  const uint32_t *src = st.rec + ((int64_t)g.slot0 + W.w * W.ipw) * Rec<kS>::kWords;
+  for (int c = 4 * W.lane; c < W.count * Rec<kS>::kWords; c += 128) copy16_async(W.recs + c, src + c);
+}
+
+template <bool kS>
+__device__ __forceinline__ void load_regs(Regs &R, const Ctx &C) {
+  const uint32_t pcI = C.rec[Rec<kS>::kPcI], misc = C.rec[Rec<kS>::kMisc];
   R.pc = pcI & 0xFFFFu;
   R.I = pcI >> 16;
-  R.sp = misc & 0xFFu;
-  R.dt = (misc >> 8) & 0xFFu;
-  R.st = (misc >> 16) & 0xFFu;
-  R.status = misc >> 24;
-  R.dirty = st.dirty[slot];
-  R.wrange = st.wrange[slot];
-  R.env_steps = st.env_steps[slot];
-  R.key0 = st.key[slot];
-  R.key1 = st.key[n + slot];
-  R.uid = st.uid[slot];
-  R.last_act = st.last_act[slot];
-  R.hires = kS ? st.mode[slot] : 0u;
+  R.sp = misc & 0x7Fu;
+  R.hires = kS ? (misc >> 7) & 1u : 0u;
+  R.status = (misc >> 8) & 0xFFu;
+  R.dirty = *reinterpret_cast<const uint64_t *>(C.rec + Rec<kS>::kDirty);
+  set_range(R, C.rec[Rec<kS>::kWrange]);
+  R.env_steps = C.rec[Rec<kS>::kEnv];
   R.draws = 0;
   R.phase = 0;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) reinterpret_cast<uint32_t *>(C.V)[k] = C.rec[Rec<kS>::kV + k];
 }
 
+// Back into the record (every lane of the instance stores the same words).
 template <bool kS>
-__device__ __forceinline__ void store_regs(const Regs &R, const DevState &st, int64_t slot) {
-  st.pcI[slot] = R.pc | (R.I << 16);
-  st.misc[slot] = R.sp | (R.dt << 8) | (R.st << 16) | (R.status << 24);
-  st.dirty[slot] = R.dirty;
-  st.env_steps[slot] = R.env_steps;
-  st.last_act[slot] = (uint8_t)R.last_act;
-  if (kS) st.mode[slot] = (uint8_t)R.hires;
+__device__ __forceinline__ void store_regs(const Regs &R, const Ctx &C, uint32_t ep) {
+  C.rec[Rec<kS>::kPcI] = R.pc | (R.I << 16);
+  C.rec[Rec<kS>::kMisc] = (C.rec[Rec<kS>::kMisc] & 0xFFFF0000u) | R.status << 8 | R.hires << 7 | R.sp;
+  C.rec[Rec<kS>::kWrange] = R.wrange;
+  *reinterpret_cast<uint64_t *>(C.rec + Rec<kS>::kDirty) = R.dirty;
+  C.rec[Rec<kS>::kEp] = ep;
+  C.rec[Rec<kS>::kEnv] = R.env_steps;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) C.rec[Rec<kS>::kV + k] = reinterpret_cast<const uint32_t *>(C.V)[k];
 }
 
-// V0-VF: packed 4 per u32 in global memory, one per u32 in shared memory.
-__device__ __forceinline__ void load_V(const Ctx &C, const DevState &st, int64_t slot) {
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    const uint32_t word = st.v[w * st.n + slot];
-#pragma unroll
-    for (int b = 0; b < 4; ++b) C.V[(4 * w + b) * C.J] = (word >> (8 * b)) & 0xFFu;
-  }
+// The warp's records back to device memory; `which` (bits of first lanes): of those instances only.
+template <bool kS>
+__device__ __forceinline__ void return_records(const Warp &W, const DevState &st, const Group &g, unsigned which) {
+  __syncwarp();
+  uint32_t *dst = st.rec + ((int64_t)g.slot0 + W.w * W.ipw) * Rec<kS>::kWords;
+  for (int c = 4 * W.lane; c < W.count * Rec<kS>::kWords; c += 128)
+    if ((which >> ((c / Rec<kS>::kWords) << W.sh)) & 1u)
+      *reinterpret_cast<uint4 *>(dst + c) = *reinterpret_cast<const uint4 *>(W.recs + c);
 }
 
-__device__ __forceinline__ void store_V(const Ctx &C, const DevState &st, int64_t slot) {
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    uint32_t word = 0;
-#pragma unroll
-    for (int b = 0; b < 4; ++b) word |= C.V[(4 * w + b) * C.J] << (8 * b);
-    st.v[w * st.n + slot] = word;
-  }
+// The key an action index holds down (-1: none).
+__device__ __forceinline__ int key_of(Regs &R, const GameDev &G, uint32_t a) {
+  if (a < G.n_actions) return G.action_set[a] & 15;
+  if (a > G.n_actions) R.status |= OCTAX_STATUS_BAD_ACTION;
+  return -1;
 }
 
-template <bool kWrap, bool kS, bool kW>
-__device__ void run_group(const StepLaunch &p, const Group &g, const Smem &S) {
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, ipw = p.ipw;
-  const int J = (blockDim.x >> 5) * ipw;  // instances per CTA
-  const int j = w * ipw + lane;           // this lane's instance (if lane < ipw)
+// Sticky actions (§3.2): repeat the previous step's action with probability sticky / 2^32.
+template <bool kWrap, bool kS>
+__device__ __forceinline__ uint32_t applied_action(const Regs &R, const Ctx &C, const GameDev &G, uint32_t a) {
+  if (kWrap && G.sticky != 0u &&
+      philox_w0(C.rec[Rec<kS>::kUid], R.env_steps, 0u, 2u, C.rec[Rec<kS>::kKey], C.rec[Rec<kS>::kKey + 1]) < G.sticky)
+    a = C.V[kLastAct];
+  C.V[kLastAct] = (uint8_t)a;
+  return a;
+}
+
+template <bool kWrap, bool kS>
+__device__ void run_group(const StepLaunch &p, const Group &g, const Warp &W) {
   const DevState &st = p.st;
-  const int64_t n = st.n;
-  const GameDev &G = *S.game;
-  const bool mine = lane < ipw;
-  const bool active = mine && j < (int)g.count;
-  const int64_t slot = (int64_t)g.slot0 + (active ? j : 0);
+  const GameDev &G = smem_game();
+  const int64_t slot = (int64_t)g.slot0 + (W.active ? W.j : 0);
   const IO io = p.io_table ? p.io_table[g.io] : p.io0;
   const uint32_t quirks = p.quirks;
-  uint64_t *disp_warp = S.disp + w * ipw;
-
+  const Ctx C = make_ctx<kS>(W, st, slot, (uint32_t)p.n_uops);
+  const int frame = io.packed ? 8 * Disp<kS>::kWords : Disp<kS>::kFrame;
   Regs R;
-  load_regs<kS>(R, st, slot);
-  const int64_t row = active ? (int64_t)st.out_row[slot] : 0;
-  uint32_t ep = st.ep[slot];
-  int32_t prev = st.prev_score[slot];
-  if (mine) {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) S.stack[i * J + j] = st.stack[i * n + slot];
-#pragma unroll 8
-    for (int r = 0; r < Disp<kS>::kWords; ++r) S.disp[r * J + j] = st.disp[r * n + slot];
-  }
-  const Ctx C{S.disp + (mine ? j : 0), S.stack + (mine ? j : 0), S.V + (mine ? j : 0),
-              st.ram + slot * (int64_t)kRamBytes, J, S.uops, S.alu, st.rpl + slot * 16};
-  if (mine) load_V(C, st, slot);
+  load_regs<kS>(R, C);
+  const int64_t row = (int64_t)C.rec[Rec<kS>::kRow];
+  uint32_t ep = C.rec[Rec<kS>::kEp];
+  int32_t prev = W.active ? score(R, C, G) : 0;
   const uint32_t K = G.K, FS = G.frameskip, first_kept = FS - (uint32_t)p.S;
+  uint32_t a_next = W.active ? io.actions[(int64_t)p.step0 * io.rows + row] : 0u;
   __syncwarp();
 
   for (int s = 0; s < p.steps; ++s) {
     const int64_t io_row = (int64_t)(p.step0 + s) * io.rows + row;
     int key = -1;
     uint8_t *my_obs = nullptr;
-    if (active) {
-      uint32_t a = io.actions[io_row];
-      // sticky actions (§3.2): repeat the previous step's action with probability sticky / 2^32
-      if (kWrap && G.sticky != 0u && philox_w0(R.uid, R.env_steps, 0u, 2u, R.key0, R.key1) < G.sticky) a = R.last_act;
-      R.last_act = a;
-      if (a < G.n_actions) key = G.action_set[a] & 15;
-      else if (a > G.n_actions) R.status |= OCTAX_STATUS_BAD_ACTION;
-      my_obs = io.obs + io_row * (int64_t)p.S * (io.packed ? 8 * Disp<kS>::kWords : Disp<kS>::kFrame);
+    if (W.active) {
+      key = key_of(R, G, applied_action<kWrap, kS>(R, C, G, a_next));
+      my_obs = io.obs + io_row * (int64_t)p.S * frame;
+      if (s + 1 < p.steps) a_next = io.actions[io_row + io.rows];  // in flight during this step
     }
     R.draws = 0;
     R.phase = 0;
     for (uint32_t f = 0; f < FS; ++f) {
-      if (active) {
-        run_instrs<kS, kW>(R, C, key, quirks, K);
-        tick(R);
+      if (W.active) {
+        run_instrs<kS>(R, C, key, quirks, K);
+        tick(C);
       }
       if (f >= first_kept) {
         __syncwarp();
-        if (io.packed)
-          capture_packed<kS>(disp_warp, J, my_obs ? my_obs + (f - first_kept) * 8 * Disp<kS>::kWords : nullptr,
-                             lane, ipw);
-        else
-          capture_frame<kS>(disp_warp, J, my_obs ? my_obs + (f - first_kept) * Disp<kS>::kFrame : nullptr, lane,
-                            ipw, S.lut);
+        uint8_t *const dst = my_obs ? my_obs + (f - first_kept) * frame : nullptr;
+        if (io.packed) capture_packed<kS>(W.recs, dst, W.lane, W.ipw, W.sh);
+        else capture_frame<kS>(W.recs, dst, W.lane, W.ipw, W.sh);
         __syncwarp();
       }
     }
     bool done = false;
-    if (active) {
+    if (W.active) {
       const int32_t sc = score(R, C, G);
       ep += 1;
       R.env_steps += 1;
       done = terminated(R, C, G) || (G.max_steps != 0 && ep >= G.max_steps);
-      io.reward[io_row] = (float)(sc - prev);
-      io.done[io_row] = done ? 1 : 0;
+      if (C.sub == 0) {
+        io.reward[io_row] = (float)(sc - prev);
+        io.done[io_row] = done ? 1 : 0;
+      }
       if (done) {
-        reset_instance<kWrap, kS, kW>(R, C, G, quirks);
+        reset_instance<kWrap, kS>(R, C, G, quirks);
         ep = 0;
         prev = score(R, C, G);
       } else {
         prev = sc;
       }
     }
-    const unsigned which = __ballot_sync(kFull, done);
+    const unsigned which = __ballot_sync(kFull, done && C.sub == 0);
     if (which) {
       __syncwarp();
-      if (io.packed) write_reset_packed<kS>(disp_warp, J, my_obs, p.S, which, lane);
-      else write_reset_obs<kS>(disp_warp, J, my_obs, p.S, which, lane, S.lut);
+      if (io.packed) write_reset_packed<kS>(W.recs, my_obs, p.S, which, W.lane, W.sh);
+      else write_reset_obs<kS>(W.recs, my_obs, p.S, which, W.lane, W.sh);
       __syncwarp();
     }
   }
 
-  if (active) {
-    store_regs<kS>(R, st, slot);
-    store_V(C, st, slot);
-    st.wrange[slot] = R.wrange;
-    st.ep[slot] = ep;
-    st.prev_score[slot] = prev;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) st.stack[i * n + slot] = (uint16_t)S.stack[i * J + j];
-#pragma unroll 8
-    for (int r = 0; r < Disp<kS>::kWords; ++r) st.disp[r * n + slot] = S.disp[r * J + j];
-  }
+  if (W.active) store_regs<kS>(R, C, ep);
+  return_records<kS>(W, st, g, kFull);
 }
 
 // One CTA's loop over groups (a persistent CTA pulls them off the queue).
-template <bool kWrap, bool kS, bool kW>
-__device__ __forceinline__ void step_body(const StepLaunch &p) {
-  uint8_t *const smem = g_smem;
-  const Smem S = carve<kS, kW>(smem, (blockDim.x >> 5) * p.ipw);
+// Every step kernel is held to 128 registers (two 256-thread CTAs per SM).
+// kWrap: the sticky-action / no-op-reset variant (games without the wrappers
+// run the kernel without them); kS: the Super-CHIP display layout.
+template <bool kWrap, bool kS>
+__global__ void __launch_bounds__(kMaxBlock, 2) step_kernel(const StepLaunch p) {
   __shared__ int s_group;
   int cur_game = -1;
   int gi = blockIdx.x;
@@ -1039,32 +1097,18 @@ __device__ __forceinline__ void step_body(const StepLaunch &p) {
     }
     if (gi >= p.n_groups) break;
     const Group g = p.groups[gi];
+    const Warp W = make_warp(p.ipw, blockDim.x >> 5, g, (uint32_t)p.n_uops, Rec<kS>::kWords);
+    fetch_records<kS>(W, p.st, g);
     if ((int)g.game != cur_game) {
-      stage_game<kW>(S, p.games, p.images, g.game, p.quirks, (blockDim.x >> 5) * p.ipw);
+      stage_game(p.blobs, p.stride, g.game, (uint32_t)p.n_uops);
       cur_game = g.game;
     }
+    copy_wait();
     __syncthreads();
-    run_group<kWrap, kS, kW>(p, g, S);
-    __syncthreads();  // shared memory is reused by the next group
+    run_group<kWrap, kS>(p, g, W);
     if (!p.work_counter) break;
+    __syncthreads();  // shared memory is reused by the next group
   }
-}
-
-// kWrap: the sticky-action / no-op-reset variant (games without the wrappers
-// run the kernel without them); kS: the Super-CHIP display layout.
-// kW: 16-byte micro-op table (the launcher picks it where it costs no
-// occupancy; Super-CHIP kernels, whose displays dominate shared memory, use
-// the 8-byte table). Every step kernel is held to 128 registers (two
-// 256-thread CTAs per SM): unbounded, the wrapper and Super-CHIP
-// instantiations took 157-210 and ran 12-16 % slower.
-template <bool kW>
-__global__ void __launch_bounds__(kMaxBlock, 2) step_kernel_chip8(const StepLaunch p) {
-  step_body<false, false, kW>(p);
-}
-
-template <bool kWrap, bool kS, bool kW>
-__global__ void __launch_bounds__(kMaxBlock, 2) step_kernel(const StepLaunch p) {
-  step_body<kWrap, kS, kW>(p);
 }
 
 
@@ -1122,101 +1166,81 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, unsigned
 }
 
 struct WsSmem {
-  Smem base;
-  uint64_t *ring;    // [2][32][J] snapshots of packed display rows
+  uint64_t *ring;    // [2][J][33] snapshots of packed display rows (33: rows of neighbours in other banks)
   uint8_t *done;     // [2][J] done flags of the end-of-step message
   uint64_t *full;    // [2]
   uint64_t *empty;   // [2]
 };
+constexpr int kRingPitch = 33;
 
-// base layout | ring | done flags | barriers
-__device__ __forceinline__ WsSmem carve_ws(uint8_t *smem, int J) {
+// behind the records and registers: ring | done flags | barriers
+__device__ __forceinline__ WsSmem carve_ws(uint32_t n_uops, int J, int emu_warps) {
   WsSmem w;
-  w.base = carve<false, false>(smem, J);
-  w.ring = reinterpret_cast<uint64_t *>(w.base.V + 16 * J);
-  w.done = reinterpret_cast<uint8_t *>(w.ring + 2 * 32 * J);
+  uint8_t *p = reinterpret_cast<uint8_t *>(smem_recs(n_uops) + J * Rec<false>::kWords) + emu_warps * 32 * kLaneBytes;
+  w.ring = reinterpret_cast<uint64_t *>(p);
+  w.done = reinterpret_cast<uint8_t *>(w.ring + 2 * kRingPitch * J);
   w.full = reinterpret_cast<uint64_t *>(w.done + ((2 * J + 15) & ~15));
   w.empty = w.full + 2;
   return w;
 }
 
+// The rows this lane owns into slot b of the ring.
+__device__ __forceinline__ void ring_put(const WsSmem &W, const Ctx &C, int J, int j, uint32_t b) {
+  uint64_t *dst = W.ring + (b * J + j) * kRingPitch;
+  for (uint32_t r = C.sub; r < 32u; r += C.L) dst[r] = disp_of(C)[r];
+}
+
 // Emulator side of one group. `msg` counts messages of this CTA.
-__device__ void run_group_emu(const StepLaunch &p, const Group &g, const WsSmem &W, uint32_t &msg,
+__device__ void run_group_emu(const StepLaunch &p, const Group &g, const Warp &W, const WsSmem &X, uint32_t &msg,
                               bool &failed) {
-  const Smem &S = W.base;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, ipw = p.ipw;
-  const int E = (int)(blockDim.x >> 5) - p.writers;
-  const int J = E * ipw;
-  const int j = w * ipw + lane;
   const DevState &st = p.st;
-  const int64_t n = st.n;
-  const GameDev &G = *S.game;
-  const bool mine = lane < ipw;
-  const bool active = mine && j < (int)g.count;
-  const int64_t slot = (int64_t)g.slot0 + (active ? j : 0);
+  const GameDev &G = smem_game();
+  const int64_t slot = (int64_t)g.slot0 + (W.active ? W.j : 0);
   const IO io = p.io_table ? p.io_table[g.io] : p.io0;
   const uint32_t quirks = p.quirks;
-
+  const Ctx C = make_ctx<false>(W, st, slot, (uint32_t)p.n_uops);
   Regs R;
-  load_regs<false>(R, st, slot);
-  const int64_t row = active ? (int64_t)st.out_row[slot] : 0;
-  uint32_t ep = st.ep[slot];
-  int32_t prev = st.prev_score[slot];
-  if (mine) {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) S.stack[i * J + j] = st.stack[i * n + slot];
-#pragma unroll 8
-    for (int r = 0; r < 32; ++r) S.disp[r * J + j] = st.disp[r * n + slot];
-  }
-  const Ctx C{S.disp + (mine ? j : 0), S.stack + (mine ? j : 0), S.V + (mine ? j : 0),
-              st.ram + slot * (int64_t)kRamBytes, J, S.uops, S.alu, st.rpl + slot * 16};
-  if (mine) load_V(C, st, slot);
+  load_regs<false>(R, C);
+  const int64_t row = (int64_t)C.rec[Rec<false>::kRow];
+  uint32_t ep = C.rec[Rec<false>::kEp];
+  int32_t prev = W.active ? score(R, C, G) : 0;
   const uint32_t K = G.K, FS = G.frameskip, first_kept = FS - (uint32_t)p.S;
 
   for (int s = 0; s < p.steps && !failed; ++s) {
     const int64_t io_row = (int64_t)(p.step0 + s) * io.rows + row;
     int key = -1;
-    if (active) {
-      uint32_t a = io.actions[io_row];
-      // sticky actions (§3.2): repeat the previous step's action with probability sticky / 2^32
-      if (G.sticky != 0u && philox_w0(R.uid, R.env_steps, 0u, 2u, R.key0, R.key1) < G.sticky) a = R.last_act;
-      R.last_act = a;
-      if (a < G.n_actions) key = G.action_set[a] & 15;
-      else if (a > G.n_actions) R.status |= OCTAX_STATUS_BAD_ACTION;
-    }
+    if (W.active) key = key_of(R, G, applied_action<true, false>(R, C, G, io.actions[io_row]));
     R.draws = 0;
     R.phase = 0;
     for (uint32_t f = 0; f < FS && !failed; ++f) {
-      if (active) {
-        run_instrs<false, false>(R, C, key, quirks, K);
-        tick(R);
+      if (W.active) {
+        run_instrs<false>(R, C, key, quirks, K);
+        tick(C);
       }
       if (f >= first_kept) {  // hand the frame to the writers
         const uint32_t b = msg & 1u, use = msg >> 1;
-        if (!mbar_wait(W.empty + b, (use & 1u) ^ 1u, p.err)) {
+        if (!mbar_wait(X.empty + b, (use & 1u) ^ 1u, p.err)) {
           failed = true;
           break;
         }
-        if (mine) {
-          uint64_t *dst = W.ring + b * 32 * J + j;
-#pragma unroll 8
-          for (int r = 0; r < 32; ++r) dst[r * J] = S.disp[r * J + j];
-        }
-        mbar_arrive(W.full + b);
+        if (W.active) ring_put(X, C, W.J, W.j, b);
+        mbar_arrive(X.full + b);
         ++msg;
       }
     }
     if (failed) break;
     bool done = false;
-    if (active) {
+    if (W.active) {
       const int32_t sc = score(R, C, G);
       ep += 1;
       R.env_steps += 1;
       done = terminated(R, C, G) || (G.max_steps != 0 && ep >= G.max_steps);
-      io.reward[io_row] = (float)(sc - prev);
-      io.done[io_row] = done ? 1 : 0;
+      if (C.sub == 0) {
+        io.reward[io_row] = (float)(sc - prev);
+        io.done[io_row] = done ? 1 : 0;
+      }
       if (done) {
-        reset_instance<true, false, false>(R, C, G, quirks);
+        reset_instance<true, false>(R, C, G, quirks);
         ep = 0;
         prev = score(R, C, G);
       } else {
@@ -1225,33 +1249,22 @@ __device__ void run_group_emu(const StepLaunch &p, const Group &g, const WsSmem 
     }
     // end-of-step message: done flags and the reset displays
     const uint32_t b = msg & 1u, use = msg >> 1;
-    if (!mbar_wait(W.empty + b, (use & 1u) ^ 1u, p.err)) {
+    if (!mbar_wait(X.empty + b, (use & 1u) ^ 1u, p.err)) {
       failed = true;
       break;
     }
-    if (mine) {
-      W.done[b * J + j] = done ? 1 : 0;
-      if (done) {
-        uint64_t *dst = W.ring + b * 32 * J + j;
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) dst[r * J] = S.disp[r * J + j];
-      }
+    if (W.active) {
+      X.done[b * W.J + W.j] = done ? 1 : 0;
+      if (done) ring_put(X, C, W.J, W.j, b);
     }
-    mbar_arrive(W.full + b);
+    mbar_arrive(X.full + b);
     ++msg;
   }
 
-  if (active && !failed) {
-    store_regs<false>(R, st, slot);
-    store_V(C, st, slot);
-    st.wrange[slot] = R.wrange;
-    st.ep[slot] = ep;
-    st.prev_score[slot] = prev;
-#pragma unroll
-    for (int i = 0; i < 16; ++i) st.stack[i * n + slot] = (uint16_t)S.stack[i * J + j];
-#pragma unroll 8
-    for (int r = 0; r < 32; ++r) st.disp[r * n + slot] = S.disp[r * J + j];
-  }
+  // a failed wait fails the whole warp's group: its records stay as they were
+  const bool ok = __all_sync(kFull, !failed);
+  if (ok && W.active) store_regs<false>(R, C, ep);
+  if (ok) return_records<false>(W, st, g, kFull);
 }
 
 // Writer side of one group: writer warp ww owns instances
@@ -1273,9 +1286,9 @@ __device__ void run_group_writer(const StepLaunch &p, const Group &g, const WsSm
   for (int m = 0; m < 4; ++m) {
     jj[m] = ww * per + 8 * m + (lane >> 2);
     const bool act = m < passes && jj[m] < (int)g.count;
-    orow[m] = act ? (int64_t)p.st.out_row[(int64_t)g.slot0 + jj[m]] : -1;
+    orow[m] = act ? (int64_t)p.st.rec[((int64_t)g.slot0 + jj[m]) * Rec<false>::kWords + Rec<false>::kRow] : -1;
   }
-  const GameDev &G = *W.base.game;
+  const GameDev &G = smem_game();
   const uint32_t FS = G.frameskip, first_kept = FS - (uint32_t)S_;
   for (int s = 0; s < p.steps && !failed; ++s) {
     const int64_t step_row = (int64_t)(p.step0 + s) * io.rows;
@@ -1285,20 +1298,18 @@ __device__ void run_group_writer(const StepLaunch &p, const Group &g, const WsSm
         failed = true;
         break;
       }
-      const uint64_t *ring = W.ring + b * 32 * J;
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         if (m >= passes || orow[m] < 0) continue;
         uint8_t *obs = io.obs + (step_row + orow[m]) * (int64_t)S_ * kFrameBytes + q * 16u;
-        const uint64_t *col = ring + jj[m];
+        const uint64_t *rows = W.ring + (b * J + jj[m]) * kRingPitch;
         if (f < FS) {
           uint8_t *dst = obs + (f - first_kept) * kFrameBytes;
 #pragma unroll 8
-          for (int r = 0; r < 32; ++r)
-            __stcs(reinterpret_cast<uint4 *>(dst + r * 64), expand16(col[r * J], q, W.base.lut));
+          for (int r = 0; r < 32; ++r) __stcs(reinterpret_cast<uint4 *>(dst + r * 64), expand16(rows[r], q));
         } else if (W.done[b * J + jj[m]]) {
           for (int r = 0; r < 32; ++r) {
-            const uint4 o = expand16(col[r * J], q, W.base.lut);
+            const uint4 o = expand16(rows[r], q);
             for (int k = 0; k < S_; ++k)
               __stcs(reinterpret_cast<uint4 *>(obs + k * kFrameBytes + r * 64), o);
           }
@@ -1311,16 +1322,14 @@ __device__ void run_group_writer(const StepLaunch &p, const Group &g, const WsSm
 }
 
 __global__ void step_kernel_ws(const StepLaunch p) {
-  uint8_t *const smem = g_smem;
   const int E = (int)(blockDim.x >> 5) - p.writers;
-  const int J = E * p.ipw;
-  const WsSmem W = carve_ws(smem, J);
+  const WsSmem X = carve_ws((uint32_t)p.n_uops, E * p.ipw, E);
   __shared__ int s_group;
   if (threadIdx.x == 0) {
-    mbar_init(W.full + 0, (uint32_t)E * 32u);
-    mbar_init(W.full + 1, (uint32_t)E * 32u);
-    mbar_init(W.empty + 0, (uint32_t)p.writers * 32u);
-    mbar_init(W.empty + 1, (uint32_t)p.writers * 32u);
+    mbar_init(X.full + 0, (uint32_t)E * 32u);
+    mbar_init(X.full + 1, (uint32_t)E * 32u);
+    mbar_init(X.empty + 0, (uint32_t)p.writers * 32u);
+    mbar_init(X.empty + 1, (uint32_t)p.writers * 32u);
   }
   __syncthreads();
   const bool writer = (int)(threadIdx.x >> 5) >= E;
@@ -1336,14 +1345,17 @@ __global__ void step_kernel_ws(const StepLaunch p) {
     }
     if (gi >= p.n_groups) break;
     const Group g = p.groups[gi];
+    const Warp W = make_warp(p.ipw, E, g, (uint32_t)p.n_uops, Rec<false>::kWords);
+    if (!writer) fetch_records<false>(W, p.st, g);
     if ((int)g.game != cur_game) {
-      stage_game<false>(W.base, p.games, p.images, g.game, p.quirks, J);
+      stage_game(p.blobs, p.stride, g.game, (uint32_t)p.n_uops);
       cur_game = g.game;
     }
+    copy_wait();
     __syncthreads();
     if (!failed) {
-      if (writer) run_group_writer(p, g, W, msg, failed);
-      else run_group_emu(p, g, W, msg, failed);
+      if (writer) run_group_writer(p, g, X, msg, failed);
+      else run_group_emu(p, g, W, X, msg, failed);
     }
     __syncthreads();  // shared memory is reused by the next group
     if (!p.work_counter) break;
@@ -1351,64 +1363,47 @@ __global__ void step_kernel_ws(const StepLaunch p) {
 }
 
 template <bool kS>
-__global__ void __launch_bounds__(kMaxBlock) reset_kernel(const ResetLaunch p) {
-  uint8_t *const smem = g_smem;
-  const int t = threadIdx.x, lane = t & 31, w = t >> 5, ipw = p.ipw;
-  const int J = (blockDim.x >> 5) * ipw;
-  const int j = w * ipw + lane;
-  const Smem S = carve<kS, false>(smem, J);
+__global__ void __launch_bounds__(kMaxBlock, 2) reset_kernel(const ResetLaunch p) {
+  using T = Rec<kS>;
   const Group g = p.groups[blockIdx.x];
-  stage_game<false>(S, p.games, p.images, g.game, p.quirks, J);
+  const Warp W = make_warp(p.ipw, blockDim.x >> 5, g, (uint32_t)p.n_uops, T::kWords);
+  if (!p.init) fetch_records<kS>(W, p.st, g);
+  stage_game(p.blobs, p.stride, g.game, (uint32_t)p.n_uops);
+  copy_wait();
   __syncthreads();
   const DevState &st = p.st;
-  const int64_t n = st.n;
-  const GameDev &G = *S.game;
-  const bool mine = lane < ipw;
-  const bool active = mine && j < (int)g.count;
-  const int64_t slot = (int64_t)g.slot0 + (active ? j : 0);
-  const int64_t row = !active ? 0 : (p.init && p.set_rows) ? (int64_t)(g.row0 + j) : (int64_t)st.out_row[slot];
-  const bool doit = active && (p.mask == nullptr || p.mask[row] != 0);
+  const GameDev &G = smem_game();
+  const int64_t slot = (int64_t)g.slot0 + (W.active ? W.j : 0);
+  const Ctx C = make_ctx<kS>(W, st, slot, (uint32_t)p.n_uops);
   Regs R;
   if (p.init) {
     const uint64_t seed = p.seed_of_group ? p.seed_of_group[blockIdx.x] : p.seed;
     R.status = 0;
     R.env_steps = 0;
-    R.key0 = (uint32_t)(seed & 0xFFFFFFFFu);
-    R.key1 = (uint32_t)(seed >> 32);
-    R.uid = p.uid_of_slot ? p.uid_of_slot[slot] : (uint32_t)row;
+    if (W.active) {
+      const uint32_t row = p.row_of_slot ? p.row_of_slot[slot] : g.row0 + (uint32_t)W.j;
+      for (int k = T::kRow + 1; k < T::kWords; ++k) C.rec[k] = 0;
+      C.rec[T::kMisc] = (uint32_t)g.game << 16;
+      C.rec[T::kKey] = (uint32_t)(seed & 0xFFFFFFFFu);
+      C.rec[T::kKey + 1] = (uint32_t)(seed >> 32);
+      C.rec[T::kUid] = p.uid_of_slot ? p.uid_of_slot[slot] : row;
+      C.rec[T::kRow] = row;
+    }
+    __syncwarp();
   } else {
-    load_regs<kS>(R, st, slot);
+    load_regs<kS>(R, C);
   }
-  const Ctx C{S.disp + (mine ? j : 0), S.stack + (mine ? j : 0), S.V + (mine ? j : 0),
-              st.ram + slot * (int64_t)kRamBytes, J, S.uops, S.alu, st.rpl + slot * 16};
-  if (doit) reset_instance<true, kS, false>(R, C, G, p.quirks);
-  const unsigned which = __ballot_sync(kFull, doit);
+  const uint32_t row = C.rec[T::kRow];
+  const bool doit = W.active && (p.mask == nullptr || p.mask[row] != 0);
+  if (doit) reset_instance<true, kS>(R, C, G, p.quirks);
+  const unsigned which = __ballot_sync(kFull, doit && C.sub == 0);
   if (p.obs && which) {
     __syncwarp();
-    write_reset_obs<kS>(S.disp + w * ipw, J, doit ? p.obs + row * (int64_t)p.S * Disp<kS>::kFrame : nullptr,
-                        p.S, which, lane, S.lut);
-    __syncwarp();
+    write_reset_obs<kS>(W.recs, doit ? p.obs + (int64_t)row * p.S * Disp<kS>::kFrame : nullptr, p.S, which, W.lane, W.sh);
   }
-  if (doit) {
-    store_regs<kS>(R, st, slot);
-    store_V(C, st, slot);
-    st.wrange[slot] = R.wrange;
-    st.ep[slot] = 0;
-    st.prev_score[slot] = score(R, C, G);
-    if (p.init) {
-      st.key[slot] = R.key0;
-      st.key[n + slot] = R.key1;
-      st.uid[slot] = R.uid;
-      if (p.set_rows) {
-        st.out_row[slot] = (uint32_t)row;
-        st.game[slot] = g.game;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) st.stack[i * n + slot] = (uint16_t)S.stack[i * J + j];
-#pragma unroll 8
-    for (int r = 0; r < Disp<kS>::kWords; ++r) st.disp[r * n + slot] = S.disp[r * J + j];
-  }
+  __syncwarp();
+  if (doit) store_regs<kS>(R, C, 0u);
+  return_records<kS>(W, st, g, which);
 }
 
 // RAM byte of a slot as the program sees it.
@@ -1420,105 +1415,98 @@ __device__ __forceinline__ uint8_t ram_byte(const DevState &st, const uint8_t *i
 __device__ __forceinline__ uint64_t fnv_byte(uint64_t h, uint32_t b) {
   return (h ^ (uint64_t)(b & 0xFFu)) * 1099511628211ull;
 }
+__device__ __forceinline__ uint64_t fnv_word(uint64_t h, uint32_t w) {
+  for (int b = 0; b < 4; ++b) h = fnv_byte(h, w >> (8 * b));
+  return h;
+}
 
-__global__ void hash_kernel(const DevState st, const uint8_t *images, const uint32_t *slot_of_row,
+__global__ void hash_kernel(const DevState st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
                             int64_t rows, uint64_t *out) {
   const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (row >= rows) return;
   const int64_t slot = slot_of_row[row];
-  const int64_t n = st.n;
-  const uint8_t *img = images + (size_t)st.game[slot] * kRamBytes;
+  const uint32_t *rec = st.rec + slot * rec_words(st.schip);
+  const uint32_t *t = rec + 2 * disp_words(st.schip);  // the words behind the display
+  const uint32_t misc = t[6];
+  const uint8_t *img = blobs + (misc >> 16) * stride;
   uint64_t h = 14695981039346656037ull;
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t w = st.v[j * n + slot];
-    for (int b = 0; b < 4; ++b) h = fnv_byte(h, w >> (8 * b));
-  }
-  const uint32_t pcI = st.pcI[slot], misc = st.misc[slot];
-  const uint32_t I = pcI >> 16, PC = pcI & 0xFFFFu;
-  h = fnv_byte(h, I);
-  h = fnv_byte(h, I >> 8);
-  h = fnv_byte(h, PC);
-  h = fnv_byte(h, PC >> 8);
-  for (int b = 0; b < 4; ++b) h = fnv_byte(h, misc >> (8 * b));  // SP DT ST status
-  for (int i = 0; i < 16; ++i) {
-    const uint32_t e = st.stack[i * n + slot];
-    h = fnv_byte(h, e);
-    h = fnv_byte(h, e >> 8);
-  }
-  for (int r = 0; r < disp_words(st.schip); ++r) {  // SCHIP words run [y][h], as in the record
-    const uint64_t w = st.disp[r * n + slot];
-    for (int b = 0; b < 8; ++b) h = fnv_byte(h, (uint32_t)(w >> (8 * b)));
-  }
-  const uint64_t dirty = st.dirty[slot];
+  for (int j = 0; j < 4; ++j) h = fnv_word(h, t[j]);
+  const uint32_t I = t[5] >> 16, PC = t[5] & 0xFFFFu;
+  h = fnv_word(h, I | PC << 16);
+  h = fnv_word(h, (misc & 0x7Fu) | (t[4] & 0xFFu) << 8 | (t[4] & 0xFF0000u) | (misc & 0xFF00u) << 16);  // SP DT ST status
+  for (int i = 0; i < 8; ++i) h = fnv_word(h, t[12 + i]);
+  for (int r = 0; r < 2 * disp_words(st.schip); ++r) h = fnv_word(h, rec[r]);  // SCHIP words run [y][h], as in the record
+  const uint64_t dirty = t[8] | (uint64_t)t[9] << 32;
   for (uint32_t a = 0; a < (uint32_t)kRamBytes; ++a) h = fnv_byte(h, ram_byte(st, img, slot, dirty, a));
-  const uint32_t ep = st.ep[slot], es = st.env_steps[slot];
-  for (int b = 0; b < 4; ++b) h = fnv_byte(h, ep >> (8 * b));
-  for (int b = 0; b < 4; ++b) h = fnv_byte(h, es >> (8 * b));
-  h = fnv_byte(h, st.last_act[slot]);
+  h = fnv_word(h, t[10]);
+  h = fnv_word(h, t[11]);
+  h = fnv_byte(h, t[4] >> 8);
   if (st.schip) {
-    h = fnv_byte(h, st.mode[slot]);
-    for (int i = 0; i < 16; ++i) h = fnv_byte(h, st.rpl[slot * 16 + i]);
+    h = fnv_byte(h, (misc >> 7) & 1u);
+    for (int i = 0; i < 4; ++i) h = fnv_word(h, t[24 + i]);
   }
   out[row] = h;
 }
 
-__global__ void records_kernel(const DevState st, const uint8_t *images, const uint32_t *slot_of_row,
+__global__ void records_kernel(const DevState st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
                                int64_t first, int64_t count, octax_state_record *out) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int64_t slot = slot_of_row[first + i];
-  const int64_t n = st.n;
+  const uint32_t *w = st.rec + slot * rec_words(st.schip);
+  const uint32_t *t = w + 2 * disp_words(st.schip);
   octax_state_record &rec = out[i];
-  for (int j = 0; j < 4; ++j) {
-    const uint32_t w = st.v[j * n + slot];
-    for (int b = 0; b < 4; ++b) rec.V[4 * j + b] = (uint8_t)(w >> (8 * b));
-  }
-  const uint32_t pcI = st.pcI[slot], misc = st.misc[slot];
+  for (int j = 0; j < 16; ++j) rec.V[j] = (uint8_t)(t[j >> 2] >> (8 * (j & 3)));
+  const uint32_t pcI = t[5], misc = t[6], timers = t[4];
   rec.PC = (uint16_t)(pcI & 0xFFFFu);
   rec.I = (uint16_t)(pcI >> 16);
-  rec.SP = (uint8_t)misc;
-  rec.DT = (uint8_t)(misc >> 8);
-  rec.ST = (uint8_t)(misc >> 16);
-  rec.status = (uint8_t)(misc >> 24);
-  for (int k = 0; k < 16; ++k) rec.stack[k] = st.stack[k * n + slot];
+  rec.SP = (uint8_t)(misc & 0x7Fu);
+  rec.DT = (uint8_t)timers;
+  rec.ST = (uint8_t)(timers >> 16);
+  rec.status = (uint8_t)(misc >> 8);
+  for (int k = 0; k < 16; ++k) rec.stack[k] = (uint16_t)(t[12 + (k >> 1)] >> (16 * (k & 1)));
+  const uint64_t *disp = reinterpret_cast<const uint64_t *>(w);
   for (int y = 0; y < 64; ++y)
     for (int hw = 0; hw < 2; ++hw)
-      rec.display[y][hw] = st.schip ? st.disp[(2 * y + hw) * n + slot]
-                                    : (y < 32 && hw == 0 ? st.disp[y * n + slot] : 0ull);
-  const uint8_t *img = images + (size_t)st.game[slot] * kRamBytes;
-  const uint64_t dirty = st.dirty[slot];
+      rec.display[y][hw] = st.schip ? disp[2 * y + hw] : (y < 32 && hw == 0 ? disp[y] : 0ull);
+  const uint8_t *img = blobs + (misc >> 16) * stride;
+  const uint64_t dirty = t[8] | (uint64_t)t[9] << 32;
   for (uint32_t a = 0; a < (uint32_t)kRamBytes; ++a) rec.ram[a] = ram_byte(st, img, slot, dirty, a);
-  rec.episode_steps = st.ep[slot];
-  rec.env_steps = st.env_steps[slot];
-  rec.last_action = st.last_act[slot];
-  rec.hires = st.schip ? st.mode[slot] : 0;
+  rec.episode_steps = t[10];
+  rec.env_steps = t[11];
+  rec.last_action = (uint8_t)(timers >> 8);
+  rec.hires = st.schip ? (misc >> 7) & 1u : 0;
   for (int k = 0; k < 6; ++k) rec.pad[k] = 0;
-  for (int k = 0; k < 16; ++k) rec.rpl[k] = st.schip ? st.rpl[slot * 16 + k] : 0;
+  for (int k = 0; k < 16; ++k) rec.rpl[k] = st.schip ? (uint8_t)(t[24 + (k >> 2)] >> (8 * (k & 3))) : 0;
 }
 
-__global__ void set_records_kernel(const DevState st, const GameDev *games, const uint8_t *images,
+__global__ void set_records_kernel(const DevState st, const uint8_t *blobs, size_t stride,
                                    const uint32_t *slot_of_row, int64_t first, int64_t count,
                                    const octax_state_record *in) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= count) return;
   const int64_t slot = slot_of_row[first + i];
-  const int64_t n = st.n;
   const octax_state_record &rec = in[i];
+  uint32_t *w = st.rec + slot * rec_words(st.schip);
+  uint32_t *t = w + 2 * disp_words(st.schip);
   for (int j = 0; j < 4; ++j) {
-    uint32_t w = 0;
-    for (int b = 0; b < 4; ++b) w |= (uint32_t)rec.V[4 * j + b] << (8 * b);
-    st.v[j * n + slot] = w;
+    uint32_t v = 0;
+    for (int b = 0; b < 4; ++b) v |= (uint32_t)rec.V[4 * j + b] << (8 * b);
+    t[j] = v;
   }
-  st.pcI[slot] = (uint32_t)(rec.PC & 0xFFFu) | ((uint32_t)rec.I << 16);
-  st.misc[slot] = (uint32_t)rec.SP | ((uint32_t)rec.DT << 8) | ((uint32_t)rec.ST << 16) |
-                  ((uint32_t)rec.status << 24);
-  for (int k = 0; k < 16; ++k) st.stack[k * n + slot] = rec.stack[k];
-  for (int r = 0; r < disp_words(st.schip); ++r)
-    st.disp[r * n + slot] = st.schip ? rec.display[r >> 1][r & 1] : rec.display[r][0];
-  st.mode[slot] = st.schip ? rec.hires : 0;
-  for (int k = 0; k < 16; ++k) st.rpl[slot * 16 + k] = st.schip ? rec.rpl[k] : 0;
-  const int game = st.game[slot];
-  const uint8_t *img = images + (size_t)game * kRamBytes;
+  t[4] = (uint32_t)rec.DT | (uint32_t)rec.last_action << 8 | (uint32_t)rec.ST << 16 | 15u << 24;
+  t[5] = (uint32_t)(rec.PC & 0xFFFu) | ((uint32_t)rec.I << 16);
+  t[6] = (t[6] & 0xFFFF0000u) | (uint32_t)rec.status << 8 | (st.schip && rec.hires ? 0x80u : 0u) | (uint32_t)rec.SP;
+  for (int k = 0; k < 8; ++k) t[12 + k] = (uint32_t)rec.stack[2 * k] | (uint32_t)rec.stack[2 * k + 1] << 16;
+  uint64_t *disp = reinterpret_cast<uint64_t *>(w);
+  for (int r = 0; r < disp_words(st.schip); ++r) disp[r] = st.schip ? rec.display[r >> 1][r & 1] : rec.display[r][0];
+  if (st.schip)
+    for (int k = 0; k < 4; ++k) {
+      uint32_t v = 0;
+      for (int b = 0; b < 4; ++b) v |= (uint32_t)rec.rpl[4 * k + b] << (8 * b);
+      t[24 + k] = v;
+    }
+  const uint8_t *img = blobs + (t[6] >> 16) * stride;
   uint64_t dirty = 0;
   uint32_t lo = 0xFFFu, hi = 0u;
   uint8_t *ram = st.ram + slot * (int64_t)kRamBytes;
@@ -1537,40 +1525,20 @@ __global__ void set_records_kernel(const DevState st, const GameDev *games, cons
       for (int b = 0; b < (1 << kPageShift); ++b) ram[(page << kPageShift) + b] = rec.ram[(page << kPageShift) + b];
     }
   }
-  st.dirty[slot] = dirty;
-  st.wrange[slot] = lo | hi << 16;  // the bytes that differ from the image lie in [lo, hi]
-  st.ep[slot] = rec.episode_steps;
-  st.env_steps[slot] = rec.env_steps;
-  st.last_act[slot] = rec.last_action;
-  // score of the restored state (the next step's reward baseline)
-  const GameDev &G = games[game];
-  int32_t s = 0;
-  for (uint32_t k = 0; k < G.n_score; ++k) {
-    const TermDev &t = G.score[k];
-    const int32_t v = t.src == OCTAX_SRC_REG ? (int32_t)rec.V[t.idx & 15] : (int32_t)rec.ram[t.idx & 0xFFF];
-    switch (t.xform) {
-      case OCTAX_X_RAW: s += v; break;
-      case OCTAX_X_NEG: s -= v; break;
-      case OCTAX_X_DEC_TENS: s += v / 10; break;
-      case OCTAX_X_DEC_ONES: s += v % 10; break;
-      case OCTAX_X_DEC_TENS_MINUS_ONES: s += v / 10 - v % 10; break;
-      case OCTAX_X_NIB_HI_MINUS_LO: s += (v >> 4) - (v & 15); break;
-      case OCTAX_X_ZERO_IF_GT: s += v > t.arg ? 0 : v; break;
-      default: break;
-    }
-  }
-  st.prev_score[slot] = s;
+  t[7] = lo | hi << 16;  // the bytes that differ from the image lie in [lo, hi]
+  t[8] = (uint32_t)dirty;
+  t[9] = (uint32_t)(dirty >> 32);
+  t[10] = rec.episode_steps;
+  t[11] = rec.env_steps;
 }
 
 }  // namespace
 
-size_t step_smem_bytes(int block, int ipw, int schip, int wide) {
+size_t step_smem_bytes(int block, int ipw, int schip, int n_uops) {
   const size_t J = (size_t)(block / 32) * ipw;
-  return (size_t)kRamBytes + kGameSmem + (wide ? kUopSmemWide : kUopSmemNarrow) + kLutSmem + kAluSmem +
-         J * (disp_words(schip) * sizeof(uint64_t) + 32 * sizeof(uint32_t));
+  return blob_bytes(n_uops) + J * 4 * rec_words(schip) + (size_t)block * kLaneBytes;
 }
 
-// Dynamic shared memory a CTA may opt into, less room for static shared data.
 // Opt-in dynamic shared memory limit of the current device (less 1 KB for
 // static shared memory), queried once per device ordinal.
 size_t max_dynamic_smem() {
@@ -1588,9 +1556,28 @@ size_t max_dynamic_smem() {
   return v;
 }
 
-size_t step_ws_smem_bytes(int block, int ipw) {
+size_t step_ws_smem_bytes(int block, int ipw, int n_uops) {
   const size_t J = (size_t)(block / 32) * ipw;
-  return step_smem_bytes(block, ipw, 0) + 2 * 32 * 8 * J + ((2 * J + 15) & ~(size_t)15) + 4 * 8;
+  return step_smem_bytes(block, ipw, 0, n_uops) + 2 * kRingPitch * 8 * J + ((2 * J + 15) & ~(size_t)15) + 4 * 8;
+}
+
+// The accepted shapes: 23,232 bytes for the game and 384 (SCHIP 1,152) per
+// instance, with the writers' ring 512 more and the hand-over's flags. The
+// kernels need less than that, or run without the micro-op table
+// (launch_uops).
+bool shape_fits(int block, int ipw, int schip, int writers) {
+  const size_t J = (size_t)(block / 32) * ipw;
+  size_t need = 23232 + J * (schip ? 1152 : 384);
+  if (writers > 0) need += 512 * J + ((2 * J + 15) & ~(size_t)15) + 32;
+  return need <= max_dynamic_smem();
+}
+
+// Micro-ops staged by a launch: the table, or none where it does not fit
+// beside the records (SCHIP, a 3.5 KB ROM and more than 160 instances per
+// CTA): every instruction then takes the switch.
+static int launch_uops(int block, int ipw, int schip, int writers, int n_uops) {
+  const size_t need = writers > 0 ? step_ws_smem_bytes(block, ipw, n_uops) : step_smem_bytes(block, ipw, schip, n_uops);
+  return need <= max_dynamic_smem() ? n_uops : 0;
 }
 
 // The dynamic shared memory attribute of a kernel applies to the current
@@ -1604,64 +1591,28 @@ static cudaError_t ensure_smem_attr() {
   if (de != cudaSuccess) return de;
   std::lock_guard<std::mutex> lk(mu);
   if (done[dev]) return cudaSuccess;
-  const size_t cap = max_dynamic_smem();
-  auto lim = [&](int schip, int wide) { return (int)std::min(step_smem_bytes(kMaxBlock, 32, schip, wide), cap); };
-  const struct {
-    const void *fn;
-    int smem;
-  } fns[] = {
-      {(const void *)step_kernel_chip8<true>, lim(0, 1)},       {(const void *)step_kernel_chip8<false>, lim(0, 0)},
-      {(const void *)step_kernel<true, false, true>, lim(0, 1)}, {(const void *)step_kernel<true, false, false>, lim(0, 0)},
-      {(const void *)step_kernel<false, true, false>, lim(1, 0)}, {(const void *)step_kernel<true, true, false>, lim(1, 0)},
-      {(const void *)reset_kernel<false>, lim(0, 0)},            {(const void *)reset_kernel<true>, lim(1, 0)},
-      {(const void *)step_kernel_ws, (int)cap}};
-  for (const auto &f : fns) {
-    cudaError_t e = cudaFuncSetAttribute(f.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem);
+  const int cap = (int)max_dynamic_smem();
+  const void *fns[] = {(const void *)step_kernel<false, false>, (const void *)step_kernel<true, false>,
+                       (const void *)step_kernel<false, true>,  (const void *)step_kernel<true, true>,
+                       (const void *)reset_kernel<false>,       (const void *)reset_kernel<true>,
+                       (const void *)step_kernel_ws};
+  for (const void *f : fns) {
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
     if (e != cudaSuccess) return e;
   }
   done[dev] = true;
   return cudaSuccess;
 }
 
-// CHIP-8 step kernel (no writer warps) for a shape: the 16-byte micro-op
-// table when it fits and keeps the narrow table's resident CTAs per SM.
-static bool use_wide(int block, int ipw, int wrappers) {
-  static std::mutex mu;
-  static std::map<std::tuple<int, int, int, int>, bool> memo;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  std::lock_guard<std::mutex> lk(mu);
-  const auto key = std::make_tuple(dev, block, ipw, wrappers);
-  auto it = memo.find(key);
-  if (it != memo.end()) return it->second;
-  const size_t sw = step_smem_bytes(block, ipw, 0, 1), sn = step_smem_bytes(block, ipw, 0, 0);
-  bool wide = false;
-  if (sw <= max_dynamic_smem()) {
-    int ow = 0, on = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &ow, wrappers ? (const void *)step_kernel<true, false, true> : (const void *)step_kernel_chip8<true>, block, sw);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &on, wrappers ? (const void *)step_kernel<true, false, false> : (const void *)step_kernel_chip8<false>, block, sn);
-    wide = ow >= on && ow > 0;
-  }
-  memo[key] = wide;
-  return wide;
-}
-
 // The step kernel instantiation for a launch (null: writer warps on SCHIP).
-static const void *step_fn(const StepLaunch &p, int block) {
-  if (p.writers > 0) return p.st.schip ? nullptr : (const void *)step_kernel_ws;
-  if (p.st.schip)
-    return p.wrappers ? (const void *)step_kernel<true, true, false> : (const void *)step_kernel<false, true, false>;
-  if (use_wide(block, p.ipw, p.wrappers))
-    return p.wrappers ? (const void *)step_kernel<true, false, true> : (const void *)step_kernel_chip8<true>;
-  return p.wrappers ? (const void *)step_kernel<true, false, false> : (const void *)step_kernel_chip8<false>;
+static const void *step_fn(int writers, int wrappers, int schip) {
+  if (writers > 0) return schip ? nullptr : (const void *)step_kernel_ws;
+  if (schip) return wrappers ? (const void *)step_kernel<true, true> : (const void *)step_kernel<false, true>;
+  return wrappers ? (const void *)step_kernel<true, false> : (const void *)step_kernel<false, false>;
 }
 
-static size_t step_fn_smem(const StepLaunch &p, int block) {
-  if (p.writers > 0) return step_ws_smem_bytes(block, p.ipw);
-  const int wide = !p.st.schip && use_wide(block, p.ipw, p.wrappers);
-  return step_smem_bytes(block, p.ipw, p.st.schip, wide);
+static size_t launch_smem(int block, int ipw, int schip, int writers, int n_uops) {
+  return writers > 0 ? step_ws_smem_bytes(block, ipw, n_uops) : step_smem_bytes(block, ipw, schip, n_uops);
 }
 
 cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s) {
@@ -1669,12 +1620,14 @@ cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s
   cudaError_t e = ensure_smem_attr();
   if (e != cudaSuccess) return e;
   if (grid <= 0) return cudaSuccess;
-  const void *fn = step_fn(p, block);
+  const void *fn = step_fn(p.writers, p.wrappers, p.st.schip);
   if (!fn) return cudaErrorInvalidValue;
   StepLaunch copy = p;
+  copy.n_uops = launch_uops(block, p.ipw, p.st.schip, p.writers, p.n_uops);
   void *args[] = {&copy};
   const int threads = p.writers > 0 ? block + 32 * p.writers : block;
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args, step_fn_smem(p, block), s);
+  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args,
+                          launch_smem(block, p.ipw, p.st.schip, p.writers, copy.n_uops), s);
 }
 
 cudaError_t launch_reset(const ResetLaunch &p, int block, cudaStream_t s) {
@@ -1682,40 +1635,44 @@ cudaError_t launch_reset(const ResetLaunch &p, int block, cudaStream_t s) {
   cudaError_t e = ensure_smem_attr();
   if (e != cudaSuccess) return e;
   if (p.n_groups <= 0) return cudaSuccess;
-  if (p.st.schip)
-    reset_kernel<true><<<p.n_groups, block, step_smem_bytes(block, p.ipw, 1), s>>>(p);
-  else
-    reset_kernel<false><<<p.n_groups, block, step_smem_bytes(block, p.ipw, 0), s>>>(p);
+  ResetLaunch copy = p;
+  copy.n_uops = launch_uops(block, p.ipw, p.st.schip, 0, p.n_uops);
+  const size_t smem = step_smem_bytes(block, p.ipw, p.st.schip, copy.n_uops);
+  if (p.st.schip) reset_kernel<true><<<p.n_groups, block, smem, s>>>(copy);
+  else reset_kernel<false><<<p.n_groups, block, smem, s>>>(copy);
   return cudaGetLastError();
 }
 
-cudaError_t launch_hash(const DevState &st, const uint8_t *images, const uint32_t *slot_of_row,
+cudaError_t launch_tables(uint8_t *blobs, size_t stride, int n_games, int n_uops, int schip, uint32_t quirks,
+                          cudaStream_t s) {
+  tables_kernel<<<n_games, 256, 0, s>>>(blobs, stride, (uint32_t)n_uops, schip, quirks);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_hash(const DevState &st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
                         int64_t rows, uint64_t *out, cudaStream_t s) {
   if (rows <= 0) return cudaSuccess;
   if (!state_complete(st)) return cudaErrorInvalidValue;
   const int tb = 128;
-  hash_kernel<<<(unsigned)((rows + tb - 1) / tb), tb, 0, s>>>(st, images, slot_of_row, rows, out);
+  hash_kernel<<<(unsigned)((rows + tb - 1) / tb), tb, 0, s>>>(st, blobs, stride, slot_of_row, rows, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_records(const DevState &st, const uint8_t *images, const uint32_t *slot_of_row,
+cudaError_t launch_records(const DevState &st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
                            int64_t first, int64_t count, octax_state_record *out, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   if (!state_complete(st)) return cudaErrorInvalidValue;
   const int tb = 128;
-  records_kernel<<<(unsigned)((count + tb - 1) / tb), tb, 0, s>>>(st, images, slot_of_row, first, count,
-                                                                   out);
+  records_kernel<<<(unsigned)((count + tb - 1) / tb), tb, 0, s>>>(st, blobs, stride, slot_of_row, first, count, out);
   return cudaGetLastError();
 }
 
-cudaError_t launch_set_records(const DevState &st, const GameDev *games, const uint8_t *images,
-                               const uint32_t *slot_of_row, int64_t first, int64_t count,
-                               const octax_state_record *in, cudaStream_t s) {
+cudaError_t launch_set_records(const DevState &st, const uint8_t *blobs, size_t stride, const uint32_t *slot_of_row,
+                               int64_t first, int64_t count, const octax_state_record *in, cudaStream_t s) {
   if (count <= 0) return cudaSuccess;
   if (!state_complete(st)) return cudaErrorInvalidValue;
   const int tb = 128;
-  set_records_kernel<<<(unsigned)((count + tb - 1) / tb), tb, 0, s>>>(st, games, images, slot_of_row,
-                                                                       first, count, in);
+  set_records_kernel<<<(unsigned)((count + tb - 1) / tb), tb, 0, s>>>(st, blobs, stride, slot_of_row, first, count, in);
   return cudaGetLastError();
 }
 
@@ -1724,41 +1681,29 @@ cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t 
   if (!state_complete(p.st)) return cudaErrorInvalidValue;
   cudaError_t e = ensure_smem_attr();
   if (e != cudaSuccess) return e;
-  const void *fn = step_fn(p, block);
+  const void *fn = step_fn(p.writers, p.wrappers, p.st.schip);
   if (!fn) return cudaErrorInvalidValue;
   StepLaunch copy = p;
+  copy.n_uops = launch_uops(block, p.ipw, p.st.schip, p.writers, p.n_uops);
   void *args[] = {&copy};
   cudaKernelNodeParams kp;
   memset(&kp, 0, sizeof kp);
   kp.func = const_cast<void *>(fn);
   kp.gridDim = dim3((unsigned)grid);
   kp.blockDim = dim3((unsigned)(p.writers > 0 ? block + 32 * p.writers : block));
-  kp.sharedMemBytes = (unsigned)step_fn_smem(p, block);
+  kp.sharedMemBytes = (unsigned)launch_smem(block, p.ipw, p.st.schip, p.writers, copy.n_uops);
   kp.kernelParams = args;
   return cudaGraphAddKernelNode(node, g, dep ? &dep : nullptr, dep ? 1 : 0, &kp);
 }
 
 cudaError_t alloc_state(DevState &st, int64_t n, int schip, void **block_out, size_t *bytes_out) {
-  const size_t N = (size_t)n;
-  // every array starts on a 256-byte boundary
-  auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-  const size_t sizes[] = {16 * N, 4 * N, 4 * N, 32 * N, 8 * (size_t)disp_words(schip) * N, 8 * N, 4096 * N,
-                          4 * N,  4 * N, 4 * N, 8 * N,  4 * N,   4 * N, 2 * N, N, N, 16 * N, 4 * N};
-  size_t total = 0;
-  for (size_t b : sizes) total += up(b);
+  const size_t rec = ((size_t)n * 4 * rec_words(schip) + 255) & ~(size_t)255;
+  const size_t total = rec + (size_t)n * kRamBytes;
   uint8_t *base = nullptr;
   cudaError_t e = cudaMalloc(&base, total);
   if (e != cudaSuccess) return e;
-  size_t off = 0;
-  void **dst[] = {(void **)&st.v,   (void **)&st.pcI,        (void **)&st.misc,      (void **)&st.stack,
-                  (void **)&st.disp, (void **)&st.dirty,     (void **)&st.ram,       (void **)&st.ep,
-                  (void **)&st.env_steps, (void **)&st.prev_score, (void **)&st.key, (void **)&st.uid,
-                  (void **)&st.out_row, (void **)&st.game, (void **)&st.last_act, (void **)&st.mode,
-                  (void **)&st.rpl, (void **)&st.wrange};
-  for (int i = 0; i < 18; ++i) {
-    *dst[i] = base + off;
-    off += up(sizes[i]);
-  }
+  st.rec = reinterpret_cast<uint32_t *>(base);
+  st.ram = base + rec;
   st.n = n;
   st.schip = schip;
   *block_out = base;
@@ -1766,22 +1711,16 @@ cudaError_t alloc_state(DevState &st, int64_t n, int schip, void **block_out, si
   return cudaSuccess;
 }
 
-int max_resident_ctas(int block, int ipw, int writers, int wrappers, int schip) {
+int max_resident_ctas(int block, int ipw, int writers, int wrappers, int schip, int n_uops) {
   if (ensure_smem_attr() != cudaSuccess) return 0;
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (writers > 0)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel_ws, block + 32 * writers,
-                                                  step_ws_smem_bytes(block, ipw));
-  else {
-    StepLaunch p;
-    memset(&p, 0, sizeof p);
-    p.st.schip = schip;
-    p.wrappers = wrappers;
-    p.ipw = ipw;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_fn(p, block), block, step_fn_smem(p, block));
-  }
+  const void *fn = step_fn(writers, wrappers, schip);
+  if (!fn) return 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &per_sm, fn, block + 32 * writers,
+      launch_smem(block, ipw, schip, writers, launch_uops(block, ipw, schip, writers, n_uops)));
   return sms * per_sm;
 }
 

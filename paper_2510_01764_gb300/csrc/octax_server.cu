@@ -111,8 +111,8 @@ struct octax_server {
   uint32_t quirks = 0;
   uint32_t capacity = 0;
   std::vector<GameDev> games_h;
-  GameDev *games_d = nullptr;
-  uint8_t *images_d = nullptr;
+  uint8_t *blobs_d = nullptr;
+  int n_uops = 0;
   DevState st{};
   void *state_block = nullptr;
   uint8_t *act_arena = nullptr;  // [capacity * kMaxSteps]
@@ -235,8 +235,9 @@ bool tick(octax_server *s) {
     ResetLaunch p;
     memset(&p, 0, sizeof p);
     p.st = s->st;
-    p.games = s->games_d;
-    p.images = s->images_d;
+    p.blobs = s->blobs_d;
+    p.n_uops = s->n_uops;
+    p.stride = (uint32_t)blob_stride(s->n_uops);
     p.groups = t.d_rgroups;
     p.n_groups = (int)k;
     p.S = s->S;
@@ -244,7 +245,6 @@ bool tick(octax_server *s) {
     p.ipw = s->ipw;
     p.init = 1;
     p.seed_of_group = t.d_seeds;
-    p.set_rows = 1;
     if (r == cudaSuccess) r = launch_reset(p, s->block, s->stream);
   }
   // ---- one batched step over every running request
@@ -264,8 +264,9 @@ bool tick(octax_server *s) {
   StepLaunch p;
   memset(&p, 0, sizeof p);
   p.st = s->st;
-  p.games = s->games_d;
-  p.images = s->images_d;
+  p.blobs = s->blobs_d;
+  p.n_uops = s->n_uops;
+  p.stride = (uint32_t)blob_stride(s->n_uops);
   p.groups = t.d_groups;
   p.n_groups = (int)g;
   p.io_table = t.d_io;
@@ -361,7 +362,7 @@ int octax_server_create(const octax_game *games, int n_games, uint32_t quirks,
     return OCTAX_EINVAL;
   }
   const int schip = games[0].variant == OCTAX_VARIANT_SCHIP;
-  if (step_smem_bytes(B, ipw, schip) > max_dynamic_smem()) {
+  if (!shape_fits(B, ipw, schip, 0)) {
     set_error("octax_server_create: too many instances per CTA for shared memory");
     return OCTAX_EINVAL;
   }
@@ -396,11 +397,9 @@ int octax_server_create(const octax_game *games, int n_games, uint32_t quirks,
   if (r == cudaSuccess) r = cudaMalloc(&s->act_arena, (size_t)s->capacity * kMaxSteps);
   if (r == cudaSuccess) r = cudaMalloc(&s->err_d, sizeof(unsigned int));
   if (r == cudaSuccess) r = cudaMemset(s->err_d, 0, sizeof(unsigned int));
-  if (r == cudaSuccess) r = cudaMalloc(&s->games_d, s->games_h.size() * sizeof(GameDev));
-  if (r == cudaSuccess) r = cudaMalloc(&s->images_d, images.size());
-  if (r == cudaSuccess)
-    r = cudaMemcpy(s->games_d, s->games_h.data(), s->games_h.size() * sizeof(GameDev), cudaMemcpyHostToDevice);
-  if (r == cudaSuccess) r = cudaMemcpy(s->images_d, images.data(), images.size(), cudaMemcpyHostToDevice);
+  s->n_uops = table_uops(games, n_games);
+  if (r == cudaSuccess) r = cudaMalloc(&s->blobs_d, s->games_h.size() * blob_stride(s->n_uops));
+  if (r == cudaSuccess) r = upload_blobs(s->games_h, images, s->n_uops, schip, quirks, s->blobs_d, s->stream);
   s->ticks.resize(depth);
   for (auto &t : s->ticks)
     if (r == cudaSuccess) r = cudaEventCreateWithFlags(&t.ev, cudaEventDisableTiming);
@@ -612,8 +611,7 @@ void octax_server_destroy(octax_server *s) {
   cudaFree(s->state_block);
   cudaFree(s->act_arena);
   cudaFree(s->err_d);
-  cudaFree(s->games_d);
-  cudaFree(s->images_d);
+  cudaFree(s->blobs_d);
   if (s->stream) cudaStreamDestroy(s->stream);
   delete s;
 }

@@ -7,8 +7,8 @@
 // allocation (which may synchronise the device) would break the timing
 // budget. For them this file keeps everything the kernels need besides the
 // caller's inputs and outputs -- the emulator state of up to
-// kStaticMaxEnvs instances, the game descriptor, its 4 KB RAM image and the
-// CTA group table -- in one file-scope __device__ array. Each loaded device
+// kStaticMaxEnvs instances, the game's blob (RAM image, descriptor, micro-ops)
+// and the CTA group table -- in one file-scope __device__ array. Each loaded device
 // holds that array (about 4.6 MB) until the process exits.
 //
 // The array's name is only a host-side stand-in in host code; the device
@@ -30,18 +30,10 @@ constexpr int kStaticPerCta = kStaticBlock / 32 * kStaticIpw;
 constexpr int kStaticMaxGroups = (int)((kStaticMaxEnvs + kStaticPerCta - 1) / kStaticPerCta);
 
 constexpr size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr size_t N = (size_t)kStaticMaxEnvs;
-// per-slot arrays, in the order of the pointer list in octax_rollout_static
-constexpr size_t kArr[18] = {16 * N, 4 * N, 4 * N, 32 * N, 256 * N, 8 * N, 4096 * N,
-                             4 * N,  4 * N, 4 * N, 8 * N,  4 * N,   4 * N, 2 * N, N, N, 16 * N, 4 * N};
-constexpr size_t state_bytes() {
-  size_t t = 0;
-  for (size_t b : kArr) t += up256(b);
-  return t;
-}
-constexpr size_t kOffGame = state_bytes();
-constexpr size_t kOffImage = kOffGame + up256(sizeof(GameDev));
-constexpr size_t kOffGroups = kOffImage + kRamBytes;
+constexpr int kMaxUops = 3584 / 2;
+constexpr size_t kOffRam = up256((size_t)kStaticMaxEnvs * 4 * Rec<false>::kWords);
+constexpr size_t kOffBlob = kOffRam + (size_t)kStaticMaxEnvs * kRamBytes;
+constexpr size_t kOffGroups = kOffBlob + up256(blob_bytes(kMaxUops));
 constexpr size_t kScratchBytes = kOffGroups + up256(kStaticMaxGroups * sizeof(Group));
 
 static __device__ __align__(256) uint8_t g_scratch[kScratchBytes];
@@ -57,10 +49,10 @@ struct SetupArgs {
 };
 
 __global__ void static_setup_kernel(const SetupArgs a) {
-  uint8_t *img = g_scratch + kOffImage + a.half * (kRamBytes / 2);
+  uint8_t *img = g_scratch + kOffBlob + a.half * (kRamBytes / 2);
   for (int i = threadIdx.x; i < kRamBytes / 2; i += blockDim.x) img[i] = a.image_half[i];
   if (a.half != 0) return;
-  if (threadIdx.x == 0) *reinterpret_cast<GameDev *>(g_scratch + kOffGame) = a.game;
+  if (threadIdx.x == 0) *reinterpret_cast<GameDev *>(g_scratch + kOffBlob + kRamBytes) = a.game;
   Group *groups = reinterpret_cast<Group *>(g_scratch + kOffGroups);
   for (int gi = threadIdx.x; gi < a.n_groups; gi += blockDim.x) {
     const uint32_t s0 = (uint32_t)gi * kStaticPerCta;
@@ -128,19 +120,11 @@ extern "C" int octax_rollout_static(const octax_game *game, int64_t n_envs, uint
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
 
   DevState st{};
-  size_t off = 0;
-  void **dst[] = {(void **)&st.v,        (void **)&st.pcI,        (void **)&st.misc, (void **)&st.stack,
-                  (void **)&st.disp,     (void **)&st.dirty,      (void **)&st.ram,  (void **)&st.ep,
-                  (void **)&st.env_steps, (void **)&st.prev_score, (void **)&st.key,  (void **)&st.uid,
-                  (void **)&st.out_row,  (void **)&st.game,   (void **)&st.last_act,
-                  (void **)&st.mode,     (void **)&st.rpl,    (void **)&st.wrange};
-  for (int i = 0; i < 18; ++i) {
-    *dst[i] = base + off;
-    off += up256(kArr[i]);
-  }
-  st.n = kStaticMaxEnvs;  // array stride; slots [0, n_envs) are used
-  const GameDev *game_d = reinterpret_cast<const GameDev *>(base + kOffGame);
-  const uint8_t *image_d = base + kOffImage;
+  st.n = kStaticMaxEnvs;  // slots [0, n_envs) are used
+  st.rec = reinterpret_cast<uint32_t *>(base);
+  st.ram = base + kOffRam;
+  uint8_t *blob_d = base + kOffBlob;
+  const int n_uops = table_uops(game, 1);
   const Group *groups_d = reinterpret_cast<const Group *>(base + kOffGroups);
   const int n_groups = (int)((n_envs + kStaticPerCta - 1) / kStaticPerCta);
 
@@ -155,6 +139,7 @@ extern "C" int octax_rollout_static(const octax_game *game, int64_t n_envs, uint
     static_setup_kernel<<<1, 256, 0, s>>>(a);
   }
   cudaError_t r = cudaGetLastError();
+  if (r == cudaSuccess) r = launch_tables(blob_d, blob_stride(n_uops), 1, n_uops, 0, quirks, s);
   if (r != cudaSuccess) return cuda_fail(r, "octax_rollout_static: setup launch");
 
   // reset every instance (this clears all state a step reads; RAM pages are
@@ -162,8 +147,9 @@ extern "C" int octax_rollout_static(const octax_game *game, int64_t n_envs, uint
   ResetLaunch rp;
   memset(&rp, 0, sizeof rp);
   rp.st = st;
-  rp.games = game_d;
-  rp.images = image_d;
+  rp.blobs = blob_d;
+  rp.n_uops = n_uops;
+  rp.stride = (uint32_t)blob_stride(n_uops);
   rp.groups = groups_d;
   rp.n_groups = n_groups;
   rp.S = game->stack_frames;
@@ -171,7 +157,6 @@ extern "C" int octax_rollout_static(const octax_game *game, int64_t n_envs, uint
   rp.ipw = kStaticIpw;
   rp.init = 1;
   rp.seed = seed;
-  rp.set_rows = 1;
   r = launch_reset(rp, kStaticBlock, s);
   if (r != cudaSuccess) return cuda_fail(r, "octax_rollout_static: reset launch");
 
@@ -180,8 +165,9 @@ extern "C" int octax_rollout_static(const octax_game *game, int64_t n_envs, uint
     StepLaunch p;
     memset(&p, 0, sizeof p);
     p.st = st;
-    p.games = game_d;
-    p.images = image_d;
+    p.blobs = blob_d;
+    p.n_uops = n_uops;
+    p.stride = (uint32_t)blob_stride(n_uops);
     p.groups = groups_d;
     p.n_groups = n_groups;
     p.io0 = IO{actions_dev, obs_dev, reward_dev, done_dev, n_envs};
