@@ -64,6 +64,7 @@ struct octax_policy {
   int sms = 0;
   void *w1 = nullptr, *w2 = nullptr, *w3 = nullptr, *wh = nullptr;  // packed bf16
   float *fp = nullptr;        // biases and output layers (fp32), see FpLayout
+  uint8_t *act2 = nullptr;    // conv2 output, batches of 8 instances
   uint8_t *act3 = nullptr;    // flattened features, heads' A-operand tiles
   uint64_t *ring = nullptr;   // rollout: two packed observation slots [2][max_envs][4][32]
   unsigned int *err = nullptr;
@@ -78,54 +79,47 @@ int env_device(const octax_env *e);
 namespace {
 
 constexpr int kP = 8;            // instances per conv batch
-constexpr int kThreads = 256;      // heads kernel: two warps per TMEM lane quarter
-constexpr int kConvWork = 256;               // conv kernel: 8 warps build / drain (two per TMEM lane quarter)
-constexpr int kConvThreads = kConvWork + 96; // + three warps whose first lanes issue the MMAs and bulk copies
-constexpr int kIssuer = kConvWork;           // conv1's even pairs, conv3, the W1 / W2 copies and W3's first taps
-constexpr int kIssuer2 = kConvWork + 32;     // conv2's tiles and the rest of W3
-constexpr int kIssuer3 = kConvWork + 64;     // conv1's odd pairs
+constexpr int kThreads = 256;    // heads kernel: two warps per TMEM lane quarter
+// conv1 / conv2 kernel: warps by role; a draining warp reads the TMEM lane quarter warp & 3
+constexpr int kDrain1Warps = 8, kDrain2Warps = 4, kBuildWarps = 4, kIssueWarps = 3;
+constexpr int kIssueWarp = kDrain1Warps + kDrain2Warps + kBuildWarps;  // the first of them
+constexpr int kConvThreads = 32 * (kIssueWarp + kIssueWarps);
+// conv3 kernel: draining warps, a warp for the copies, a warp for the MMAs
+constexpr int kDrain3Warps = 8, kConv3Threads = 32 * (kDrain3Warps + 2);
 constexpr int kMaxLogits = 17;   // 16 keys + the no-op
 constexpr uint64_t kMaxWaitNs = 1000000000ull;
 constexpr uint32_t kMaxPolls = 1u << 24;
 
-// ---- conv kernel shared memory (bytes) -------------------------------------
+// ---- conv1 / conv2 kernel shared memory (bytes) ------------------------------
 constexpr uint32_t kW1Off = 0;                             // conv1 B: [j 3][dx 2][chunk 4][n 64][8]
 constexpr uint32_t kW1Bytes = 6 * 4 * 64 * 16;
 constexpr uint32_t kW2Off = kW1Off + kW1Bytes;             // conv2 B: [ky 4][kx & 1][chunk 4][n 128][8]
 constexpr uint32_t kW2Bytes = 4 * 2 * 4 * 128 * 16;
-constexpr uint32_t kW3Bytes = 3 * 8 * 192 * 16;            // conv3 B: [ky 3][chunk 8][n = 64 kx + o][8]
-constexpr uint32_t kSubPos = 33;                           // band: 4 grid rows of 8 + 1 pad position
-constexpr uint32_t kSubBytes = kSubPos * 512;              // position: 4 chunks x 8 instances x 16 B
-constexpr uint32_t kAct1Bytes = 4 * kSubBytes;             // 4 parity sub-grids
-constexpr uint32_t kW3Off = kW2Off + kW2Bytes;             // W3 overlays frames + band (dead by then)
-constexpr uint32_t kFrOff = kW3Off;                        // frames [32 rows][4][8] u64 during conv1
-constexpr uint32_t kAct1Off = kW3Off + 8192;
-constexpr uint32_t kW3RegionBytes = kW3Bytes > 8192 + kAct1Bytes ? kW3Bytes : 8192 + kAct1Bytes;
-constexpr uint32_t kXOff = kW3Off + kW3RegionBytes;        // blocks (conv1) | conv2 output
-constexpr uint32_t kBlkOff = kXOff;                        // 2 buffers x 49 block positions x 512 B
-constexpr uint32_t kBlkBytes = 49 * 512;
-constexpr uint32_t kAct2Off = kXOff;                       // 50 positions x (8 chunks x 8 x 16 B)
-constexpr uint32_t kAct2Bytes = 50 * 1024;
-constexpr uint32_t kXBytes = kAct2Bytes > 2 * kBlkBytes ? kAct2Bytes : 2 * kBlkBytes;
-// conv2 / conv3 drain exchange: rows g + 1 and g + 2 of the warps that hold
-// the last positions of a TMEM lane quarter come from the next quarter's
-// warp: [supplier 2][channel half 2][lane 8 | 16][36 floats] (rows padded to
-// 144 B: 16-byte aligned, and 8 lanes' rows start in distinct bank groups);
-// conv2 tiles alternate between the two parts.
+constexpr uint32_t kAct1Off = kW2Off + kW2Bytes;           // band: 4 parity sub-grids of five grid rows of 8
+constexpr uint32_t kSubBytes = 5 * 8 * 512;                // position: 4 chunks x 8 instances x 16 B
+constexpr uint32_t kAct1Bytes = 4 * kSubBytes;
+constexpr uint32_t kBlkRows = 5;                           // ring of block rows; a batch's 15 go round it three times
+constexpr uint32_t kBlkOff = kAct1Off + kAct1Bytes;        // 16 positions each, and one that only discarded rows read
+constexpr uint32_t kBlkBytes = (kBlkRows * 16 + 1) * 512;
+constexpr uint32_t kFrOff = kBlkOff + kBlkBytes;           // frames [32 rows][4][8] u64
+constexpr uint32_t kXbOff = kFrOff + 8192;
+// conv2 drain exchange: row g + 1 of the warps that hold the last positions
+// of a TMEM lane quarter comes from the next quarter's warp: [supplier 2]
+// [channel half 2][lane 8][36 floats] (rows padded to 144 B: 16-byte
+// aligned, and 8 lanes' rows start in distinct bank groups).
 constexpr int kXbPitch = 36;
-constexpr uint32_t kXbRow = kXbPitch * 4;
-constexpr uint32_t kXb1Off = kXOff + kXBytes;              // part kx = 1: lanes 0..7
-constexpr uint32_t kXb2Off = kXb1Off + 2 * 2 * 8 * kXbRow;  // part kx = 2: lanes 0..15
-constexpr uint32_t kConvSmem = kXb2Off + 2 * 2 * 16 * kXbRow;
-constexpr uint32_t kW3EarlyBytes = 8192;                   // W3 tap 0: loaded once the frames are dead
-static_assert(kAct1Off + kAct1Bytes <= kXOff && kW3Off + kW3Bytes <= kXOff, "band and W3 inside their region");
-static_assert(kFrOff + 8192 <= kAct1Off && kW3Off + kW3EarlyBytes <= kAct1Off, "frames / early W3 below the band");
+constexpr uint32_t kConvSmem = kXbOff + 2 * 2 * 8 * kXbPitch * 4;
 static_assert(kConvSmem + 1024 <= 227 * 1024, "conv kernel shared memory (with 1 KB of static shared data)");
+constexpr uint32_t kAct2Bytes = 36 * 1024;                 // conv2 output of a batch: position: 8 chunks x 8 x 16 B
+// TMEM columns (fp32): conv1: 2 buffers x 2 output rows x 32; conv2: 2 buffers x 128
+constexpr uint32_t kD1Col = 0, kD2Col = 128, kConvTmemCols = 512;
 
-// TMEM columns (fp32) of the conv kernel's accumulators.
-// conv1: 2 buffers x 2 output rows x 32; conv2: 3 tiles x 128; conv3: 2 tiles x 192
-// (over conv1's and conv2's columns, all drained before conv3 is issued).
-constexpr uint32_t kD1Col = 0, kD2Col = 128, kD3Col = 0, kConvTmemCols = 512;
+// ---- conv3 kernel -------------------------------------------------------------
+constexpr uint32_t kW3Bytes = 3 * 8 * 192 * 16;            // conv3 B: [ky 3][chunk 8][n = 64 kx + o][8]
+constexpr int kStages3 = 6;                                // ring of one kx each: 6 rows x 4 positions x 1 KB
+constexpr uint32_t kStage3Bytes = 24 * 1024;
+constexpr uint32_t kConv3Smem = kW3Bytes + kStages3 * kStage3Bytes;
+static_assert(kConv3Smem + 1024 <= 227 * 1024, "conv3 kernel shared memory (with 1 KB of static shared data)");
 
 // ---- heads kernel -----------------------------------------------------------
 constexpr int kHeadStages = 3;
@@ -154,16 +148,20 @@ __device__ __forceinline__ uint64_t global_ns() {
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  if (mbar_try(bar, parity)) return true;
   const uint64_t t0 = global_ns();
   for (uint32_t i = 0; i < kMaxPolls; ++i) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    if (ok) return true;
+    if (mbar_try(bar, parity)) return true;
     if (global_ns() - t0 > kMaxWaitNs) break;
   }
   return false;
@@ -304,20 +302,43 @@ __device__ __forceinline__ void xrow_get(const float *row, float (&v)[32]) {
     v[4 * c + 3] = f.w;
   }
 }
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);  // .x = a (low half)
-  return *reinterpret_cast<uint32_t *>(&h);
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
 }
-// bias + ReLU on 8 values, packed to one 16-byte chunk of 8 bf16.
-// (bias: 16-byte aligned shared memory, read as two vectors)
-__device__ __forceinline__ uint4 relu_chunk(const float *v, const float *bias) {
-  const float4 b0 = reinterpret_cast<const float4 *>(bias)[0], b1 = reinterpret_cast<const float4 *>(bias)[1];
-  const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-  float o[8];
+// bias (pairs) + ReLU on 8 values, packed to one 16-byte chunk of 8 bf16.
+// Rounding keeps order and sign, so the maximum with 0 may follow it, two
+// values at a time.
+__device__ __forceinline__ uint4 relu_chunk(const float *v, const uint64_t *bias) {
+  uint32_t o[4];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) o[j] = fmaxf(v[j] + bb[j], 0.0f);
-  return make_uint4(pack_bf16(o[0], o[1]), pack_bf16(o[2], o[3]), pack_bf16(o[4], o[5]), pack_bf16(o[6], o[7]));
+  for (int j = 0; j < 4; ++j) {
+    uint64_t s;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(s) : "l"(f32x2(v[2 * j], v[2 * j + 1])), "l"(bias[j]));
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(s));
+    const __nv_bfloat162 h = __hmax2(__floats2bfloat162_rn(lo, hi), __floats2bfloat162_rn(0.0f, 0.0f));
+    o[j] = *reinterpret_cast<const uint32_t *>(&h);
+  }
+  return make_uint4(o[0], o[1], o[2], o[3]);
 }
+// Barrier `id` of kN threads that also says whether all of them are ok.
+template <int kN>
+__device__ __forceinline__ bool all_ok(int id, bool ok) {
+  uint32_t any_fail;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.eq.u32 p, %1, 0;\n\tbarrier.red.or.pred q, %2, %3, p;\n\t"
+      "selp.u32 %0, 1, 0, q;\n\t}"
+      : "=r"(any_fail)
+      : "r"((uint32_t)ok), "r"(id), "r"(kN)
+      : "memory");
+  return !any_fail;
+}
+// Programmatic dependent launch: the next kernel of the stream may start its
+// set-up; what it reads of this grid's results waits for the grid's end.
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 __device__ __forceinline__ uint32_t philox_w0(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
                                               uint32_t k1) {
@@ -342,46 +363,55 @@ struct ConvArgs {
   const uint64_t *obs_words;  // [n][4][32] packed frames (or null)
   const uint8_t *obs_u8;      // [n][4][32][64] uint8 frames (or null)
   int64_t n;
-  const uint8_t *w1, *w2, *w3;  // packed bf16 B operands
-  const float *fp;              // FpLayout
-  uint8_t *act3;                // [tiles][16][8][128][16 B]
+  const uint8_t *w1, *w2;     // packed bf16 B operands
+  const float *fp;            // FpLayout
+  uint8_t *act2;              // [batches][6 py][6 px][8 chunks][8 instances][16 B]
   unsigned int *err;
-  int stall;                    // diagnostic: the first conv1 commit is skipped (its wait runs out)
+  int stall;                  // diagnostic: the first conv1 commit is skipped (its wait runs out)
 };
 
-// One 32-column conv1 tile or 64-column conv2/conv3 tile: issue `taps` x
-// `kks` MMAs (M = 128) accumulating into TMEM column `col`.
-struct TileSpec {
-  uint32_t a_base, a_lbo, a_sbo;
-  uint32_t b_base, b_lbo, b_sbo;
-};
-
+// conv1 and conv2 of batches blockIdx.x, blockIdx.x + gridDim.x, ... Every
+// role runs its own loop over the batches' steps and meets the others through
+// mbarriers only, so that the roles work on different steps (and, around a
+// batch's end, on different batches) at the same time:
+//   builders     wait c1[P & 1] (pair P - 2's MMAs: its block rows are free)  arrive blk[P & 1]
+//   conv1 issue  wait blk[P & 1], d1f[P & 1] (accumulator drained)           commit c1[P & 1]
+//   conv1 drain  wait c1[P & 1], c2[.] where band rows are rewritten         arrive d1f[P & 1], band
+//   conv2 issue  wait band, d2f[T & 1]                                       commit c2[T & 1]
+//   conv2 drain  wait c2[T & 1]                                              arrive d2f[T & 1]
+// P counts conv1 pairs (7 per batch), T conv2 tiles (3 per batch). A barrier
+// never gets two phases ahead of any of its waiters: pair P + 2 needs pair P
+// drained and its blocks rebuilt, tile T + 2 needs tile T drained, and the
+// conv1 drain waits for every tile before it writes the rows that the tile
+// after next needs. Every wait is bounded; a role whose wait runs out leaves
+// its loop, and the others run into their own limits.
 template <bool kU8>
-__global__ void __launch_bounds__(kConvThreads, 1) policy_conv_kernel(const ConvArgs a) {
+__global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const ConvArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  // MMA completion: conv1 x2, conv2, conv3 x2; bulk copies: W1 + W2, W3 x2; the final
-  // drain on the error path (bars[8], [12], [13], one per issuing thread); conv1 blocks
-  // built x2 (per block buffer), band rows written (worker arrivals)
-  __shared__ __align__(8) uint64_t bars[14];
+  __shared__ __align__(8) uint64_t bars[15];
   __shared__ uint32_t tmem_s;
-  __shared__ __align__(16) float sb[160];    // b1 | b2 | b3 (offsets used are multiples of 8)
+  __shared__ __align__(16) float sb[96];     // b1 | b2
   __shared__ uint2 nib[16];                  // 4 pixel bits -> 4 bf16 0 / 1 (element k = bit k)
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const uint32_t sbase = smem_u32(sm);
-  const uint32_t bar_c1_0 = smem_u32(&bars[0]), bar_c1_1 = smem_u32(&bars[1]);
-  const uint32_t bar_c2 = smem_u32(&bars[2]), bar_c3a = smem_u32(&bars[3]), bar_c3b = smem_u32(&bars[7]);
-  const uint32_t bar_w = smem_u32(&bars[4]), bar_w3a = smem_u32(&bars[5]), bar_w3b = smem_u32(&bars[6]);
-  const uint32_t bar_blk0 = smem_u32(&bars[9]), bar_blk1 = smem_u32(&bars[11]), bar_band = smem_u32(&bars[10]);
+  auto bar = [&](int j) { return smem_u32(&bars[j]); };
+  // pairs of barriers, by the parity of the pair / tile
+  constexpr int kBarC1 = 0, kBarBlk = 2, kBarD1f = 4, kBarC2 = 6, kBarD2f = 8, kBarBand = 10, kBarW = 11, kBarFin = 12;
 
-  for (int j = t; j < 160; j += kConvThreads) sb[j] = a.fp[j];
+  for (int j = t; j < 96; j += kConvThreads) sb[j] = a.fp[j];
   if (t < 16)  // 1.0 in bf16 is 0x3F80
     nib[t] = make_uint2((t & 1) * 0x3F80u | ((t >> 1) & 1) * 0x3F800000u,
                         ((t >> 2) & 1) * 0x3F80u | ((t >> 3) & 1) * 0x3F800000u);
   if (t == 0) {
-    for (int j = 0; j < 9; ++j) mbar_init(smem_u32(&bars[j]), 1);
-    for (int j = 9; j < 12; ++j) mbar_init(smem_u32(&bars[j]), kConvWork);
-    mbar_init(smem_u32(&bars[12]), 1);
-    mbar_init(smem_u32(&bars[13]), 1);
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(bar(kBarC1 + j), 1);
+      mbar_init(bar(kBarBlk + j), kBuildWarps);
+      mbar_init(bar(kBarD1f + j), kDrain1Warps);
+      mbar_init(bar(kBarC2 + j), 1);
+      mbar_init(bar(kBarD2f + j), kDrain2Warps);
+    }
+    mbar_init(bar(kBarBand), kDrain1Warps);
+    for (int j = kBarW; j < 15; ++j) mbar_init(bar(j), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -393,381 +423,427 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv_kernel(const Conv
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_s;
-  if (t == kIssuer) {
-    mbar_expect_tx(bar_w, kW1Bytes + kW2Bytes);
-    bulk_g2s(sbase + kW1Off, a.w1, kW1Bytes, bar_w);
-    for (uint32_t o = 0; o < kW2Bytes; o += 16384) bulk_g2s(sbase + kW2Off + o, a.w2 + o, 16384, bar_w);
-  }
-  // every exit from the batch loop tests ok right after a block-wide
-  // reduction of every thread's outcome, so all threads leave it together
-  bool ok = !__syncthreads_or(!mbar_wait(bar_w, 0));
-  uint32_t ph_c1_0 = 0, ph_c1_1 = 0, ph_c2 = 0, ph_c3a = 0, ph_c3b = 0, ph_w3 = 0;  // ph_w3: both W3 barriers
-  uint32_t ph_blk0 = 0, ph_blk1 = 0, ph_band = 0;  // issuing threads: conv1 blocks built, band rows written
-  uint32_t w3_pend = 0;  // issuing threads: W3 copies issued and not yet waited for (bit 0 early, bit 1 rest)
+  grid_dependents_launch();  // the next kernel's CTAs may set up where there is room; they wait for this grid's end
   const int64_t n_batches = (a.n + kP - 1) / kP;
-  static_assert(kP * 64 == 2 * kConvWork, "two packed-frame pieces per worker");
-  // a worker's two pieces of a batch's packed frames (q = t, t + 256:
-  // instance q & 7, frame (q >> 7) & 3, rows 2 y2 and 2 y2 + 1, y2 = (q >> 3) & 15)
-  auto load_frames = [&](int64_t first, uint4 &v0, uint4 &v1) {
-    uint4 v[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int q = t + kConvWork * k, i = q & 7, c = (q >> 7) & 3, y2 = (q >> 3) & 15;
-      if (first + i < a.n)
-        v[k] = __ldg(reinterpret_cast<const uint4 *>(a.obs_words + (first + i) * 128 + c * 32 + 2 * y2));
-    }
-    v0 = v[0];
-    v1 = v[1];
-  };
-  uint4 pf[2] = {make_uint4(0, 0, 0, 0), make_uint4(0, 0, 0, 0)};
-  bool pf_ok = false;
-  // warps w and w + 4 read the same TMEM lane quarter (rows 32 (w & 3) ..), each
-  // one half of the accumulator's columns
-  const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-  const int half = warp >> 2;
-  const bool issuer = warp >= kConvWork / 32;  // the MMA-issuing warps take no part in building / draining
-  const int r = 32 * (warp & 3) + lane;  // M-tile row of this thread (TMEM lane)
-  // base descriptors of every MMA operand (the issuing loops add constant offsets)
-  const uint64_t a1d0 = sdesc(sbase + kBlkOff, 128, 512), a1d1 = sdesc(sbase + kBlkOff + kBlkBytes, 128, 512);
-  const uint64_t b1d = sdesc(sbase + kW1Off, 1024, 128);
-  const uint64_t a2d = sdesc(sbase + kAct1Off, 128, 512), b2d = sdesc(sbase + kW2Off, 2048, 128);
-  const uint64_t a3d = sdesc(sbase + kAct2Off, 128, 1024), b3d = sdesc(sbase + kW3Off, 3072, 128);
-  const int g = r >> 3, ri = r & 7;      // grid position in the tile, instance in the batch
+  const int my_batches = (int)((n_batches - blockIdx.x + gridDim.x - 1) / gridDim.x);
+  const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;  // a warp reads TMEM lane quarter warp & 3
+  const int g = 4 * (warp & 3) + (lane >> 3), ri = lane & 7;     // grid position in the M tile, instance in the batch
+  bool ok = true;
 
-  // wait for the next phase of a barrier (block-uniform outcome; also a block barrier)
-  auto wait_all = [&](uint32_t bar, uint32_t &phase) -> bool {
-    const bool w_ok = mbar_wait(bar, phase);
-    phase ^= 1u;
-    return !__syncthreads_or(!w_ok);
-  };
-  // the same among the 8 worker warps only (named barrier 1), so that they
-  // need not wait for the issuing thread while it is issuing
-  auto wait_workers = [&](uint32_t bar, uint32_t &phase) -> bool {
-    const uint32_t w_ok = mbar_wait(bar, phase);
-    phase ^= 1u;
-    uint32_t any_fail;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\tsetp.eq.u32 p, %1, 0;\n\tbarrier.red.or.pred q, 1, %2, p;\n\t"
-        "selp.u32 %0, 1, 0, q;\n\t}"
-        : "=r"(any_fail)
-        : "r"(w_ok), "r"(kConvWork)
-        : "memory");
-    return !any_fail;
-  };
-
-  for (int64_t batch = blockIdx.x; batch < n_batches && ok; batch += gridDim.x) {
-    const int64_t i0 = batch * kP;
-    // ---- frames of the batch, packed (bit x of row word y = pixel (x, y)),
-    // stored [row y][frame c][instance i] so that the 32 lanes of a warp
-    // building one block position read 32 consecutive words
-    uint64_t *fr = reinterpret_cast<uint64_t *>(sm + kFrOff);
-    if (!kU8) {
-      // each worker's two 16-byte pieces (q = t, t + 256): loaded during the
-      // previous batch's last drain (pf_ok), else here
-      if (!issuer && !pf_ok) {
-        load_frames(i0, pf[0], pf[1]);
-      }
-      pf_ok = false;
-      for (int k = 0; k < 2 && !issuer; ++k) {  // instance i, frame c, rows 2 y2, 2 y2 + 1
-        const int q = t + kConvWork * k, i = q & 7, c = (q >> 7) & 3, y2 = (q >> 3) & 15;
-        fr[((2 * y2) * 4 + c) * 8 + i] = (uint64_t)pf[k].x | (uint64_t)pf[k].y << 32;
-        fr[((2 * y2 + 1) * 4 + c) * 8 + i] = (uint64_t)pf[k].z | (uint64_t)pf[k].w << 32;
-      }
-    } else {
-      for (int q = issuer ? kP * 128 : t; q < kP * 128; q += kConvWork) {  // one 64-byte row each
-        const int i = q & 7, c = (q >> 8) & 3, y = (q >> 3) & 31;
-        uint64_t bits = 0;
-        if (i0 + i < a.n) {
-          const uint4 *src = reinterpret_cast<const uint4 *>(a.obs_u8 + ((i0 + i) * 128 + c * 32 + y) * 64);
+  if (warp < kDrain1Warps) {
+    // ---- conv1 drain: warps w and w + 4 read the same lane quarter, each 16
+    // channels of both output rows of a pair; bias, ReLU, bf16, band
+    const int half = warp >> 2, ox = g;
+    uint64_t bias[8];
 #pragma unroll
-          for (int k4 = 0; k4 < 4; ++k4) {
-            const uint4 v = __ldg(src + k4);
-            const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int k = 0; k < 4; ++k)
-#pragma unroll
-              for (int bb = 0; bb < 4; ++bb)
-                bits |= (uint64_t)(((w4[k] >> (8 * bb)) & 0xFFu) != 0u) << (16 * k4 + 4 * k + bb);
-          }
+    for (int j = 0; j < 8; ++j) bias[j] = f32x2(sb[16 * half + 2 * j], sb[16 * half + 2 * j + 1]);
+    uint8_t *const dst0 = sm + kAct1Off + (ox & 1) * kSubBytes + (ox >> 1) * 512 + ri * 16 + 2 * half * 128;
+    uint32_t P = 0;
+    for (int bi = 0; bi < my_batches && ok; ++bi) {
+      for (int pr = 0; pr < 7; ++pr, ++P) {
+        ok = mbar_wait(bar(kBarC1 + (P & 1)), (P >> 1) & 1);
+        // the conv2 tile that read the slot this pair's rows go to: the previous
+        // batch's last tile, then tiles 0 and 1
+        if ((pr == 0 && bi > 0) || pr == 4 || pr == 6) {
+          const uint32_t T = 3 * bi + (pr == 0 ? -1 : (pr - 4) >> 1);
+          ok = ok && mbar_wait(bar(kBarC2 + (T & 1)), (T >> 1) & 1);
         }
-        fr[(y * 4 + c) * 8 + i] = bits;
-      }
-    }
-    __syncthreads();
-
-    // ---- conv1 rows 0..13 (row 14 is never read by conv2) in 7 pairs,
-    // software-pipelined: the blocks of pair p + 1 are built and its 16 MMAs
-    // issued (second block buffer, second pair of TMEM accumulators) before
-    // pair p's epilogue; conv2 runs on each completed band of three grid rows
-    // while conv1 continues.
-    // Blocks of block rows 2p .. 2p + 2 (position b = bx + 16 (by - 2p)); the
-    // pad position 48 is read by discarded rows only. Warp w builds positions
-    // 6w .. 6w + 5; lane = frame * 8 + instance; a 16-entry table turns 4
-    // pixel bits into 4 bf16 elements.
-    auto build = [&](int pr, int buf) {
-      if (issuer) return;
-      uint8_t *blk = sm + kBlkOff + buf * kBlkBytes;
-      // a warp's 6 positions span at most two block rows: load their row words once
-      const int r0 = (6 * warp) >> 4, r1 = (6 * warp + 5) >> 4;
-      const int y0 = 2 * (2 * pr + r0), y1 = 2 * (2 * pr + r1);
-      const uint64_t a0 = fr[y0 * 32 + lane], a1 = fr[(y0 + 1) * 32 + lane];
-      const uint64_t b0 = fr[y1 * 32 + lane], b1 = fr[(y1 + 1) * 32 + lane];
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        const int b = 6 * warp + j, bx = b & 15;
-        const bool first = (b >> 4) == r0;
-        const uint2 lo = nib[(uint32_t)((first ? a0 : b0) >> (4 * bx)) & 15u];
-        const uint2 hi = nib[(uint32_t)((first ? a1 : b1) >> (4 * bx)) & 15u];
-        *reinterpret_cast<uint4 *>(blk + b * 512 + lane * 16) = make_uint4(lo.x, lo.y, hi.x, hi.y);
-      }
-    };
-    // Both output rows of the pair in one N = 64 accumulator: block row j
-    // (shift dx) feeds row 2p through tap (dx, dy = j) and row 2p + 1 through
-    // tap (dx, dy = j - 1); W1 holds, per (j, dx), those two taps stacked
-    // over n (zeros where a tap does not apply), so each MMA reads its A tile
-    // once for 64 outputs.
-    auto issue_c1 = [&](int buf, bool first) {  // the issuing thread: output rows 2p, 2p + 1
-      tc_fence_after();
-      for (int j = 0; j < 3; ++j)
-        for (int dx = 0; dx < 2; ++dx)
-          for (int kk = 0; kk < 2; ++kk) {
-            const uint64_t ad = sdesc_at(buf ? a1d1 : a1d0, (16 * j + dx) * 512 + kk * 256);
-            const uint64_t bd = sdesc_at(b1d, (2 * j + dx) * 4096 + kk * 2048);
-            mma_bf16(tmem + kD1Col + 64 * buf, ad, bd, idesc_bf16(128, 64), (j | dx | kk) != 0);
-          }
-      if (!(a.stall && first)) mma_commit(buf ? bar_c1_1 : bar_c1_0);
-    };
-    auto issue_c2 = [&](int tt) {  // the issuing thread: conv2 tile tt (output rows 2tt, 2tt + 1)
-      tc_fence_after();
-      for (int ky = 0; ky < 4; ++ky)
-        for (int px = 0; px < 2; ++px) {  // taps (px, ky) and (px + 2, ky)
-          const uint32_t sg = px + 2 * (ky & 1), shift = 8 * (ky >> 1);
-          for (int kk = 0; kk < 2; ++kk) {
-            const uint64_t ad = sdesc_at(a2d, sg * kSubBytes + shift * 512 + kk * 256);
-            const uint64_t bd = sdesc_at(b2d, (ky * 2 + px) * 8192 + kk * 4096);
-            mma_bf16(tmem + kD2Col + 128 * tt, ad, bd, idesc_bf16(128, 128), (ky | px | kk) != 0);
-          }
-        }
-      mma_commit(bar_c2);
-    };
-    // The workers and the two issuing threads meet only through mbarriers
-    // here. The workers arrive on blk[p & 1] when pair p's blocks are built,
-    // which also says that pair p - 2 has been drained, so its TMEM buffer is
-    // free (one barrier per block buffer: the next arrival on it needs pair
-    // p's MMAs, issued only after the issuing thread of pairs p & 1 has
-    // waited, so it never falls two phases behind a parity wait). They arrive on band
-    // when the band rows of pairs 2, 4 and 6 are written; conv2's issuing
-    // thread waits for it (the next arrival needs a conv1 pair whose MMAs come
-    // after the tile's wait in the tensor pipe's order, through the slide's
-    // wait for the tile). Each worker waits for the MMAs itself, so the
-    // workers go on while an issuing thread sits in a full MMA queue. Every
-    // wait is bounded; one that runs out only clears r_ok, and each side still
-    // runs its whole schedule (no other side waits on it for long).
-    bool r_ok = true;
-    if (!issuer) {
-      build(0, 0);
-      fence_async_smem();
-      mbar_arrive(bar_blk0);
-      for (int pr = 0; pr < 7; ++pr) {
-        const int cb = pr & 1, nb = cb ^ 1;
-        if (pr + 1 < 7) {  // buffer nb: pair pr - 1's MMAs done (waited for last iteration)
-          build(pr + 1, nb);
-          fence_async_smem();
-          mbar_arrive(nb ? bar_blk1 : bar_blk0);
-        }
-        r_ok &= mbar_wait(cb ? bar_c1_1 : bar_c1_0, cb ? ph_c1_1 : ph_c1_0);
-        if (cb) ph_c1_1 ^= 1u; else ph_c1_0 ^= 1u;
-        if (pr == 4 || pr == 6) {  // the previous tile must finish before its rows are rewritten
-          r_ok &= mbar_wait(bar_c2, ph_c2);
-          ph_c2 ^= 1u;
-          asm volatile("bar.sync 1, %0;" ::"r"(kConvWork) : "memory");  // every worker's rows written
-          // slide: grid rows 2, 3 -> 0, 1 (4 sub-grids x 16 positions x 512 B)
-          for (int q = t; q < 4 * 16 * 32; q += kConvWork) {
-            const int sgq = q >> 9, rem = q & 511;
-            uint4 *base = reinterpret_cast<uint4 *>(sm + kAct1Off + sgq * kSubBytes);
-            base[rem] = base[16 * 32 + rem];
-          }
-          asm volatile("bar.sync 1, %0;" ::"r"(kConvWork) : "memory");
+        if (!__all_sync(0xFFFFFFFFu, ok)) {
+          ok = false;
+          break;
         }
         tc_fence_after();
-        {
-          float v[32];  // columns 16 half .. of row 2p (v[0..15]) and of row 2p + 1 (v[16..31])
-          const uint32_t d = tmem + lane_base + kD1Col + 64 * cb + 16 * half;
-          tmem_ld16x2(d, d + 32, v);
-          const int ox = g;
+        float v[32];  // columns 16 half .. of row 2 pr (v[0..15]) and of row 2 pr + 1 (v[16..31])
+        const uint32_t d = tmem + lane_base + kD1Col + 64 * (P & 1) + 16 * half;
+        tmem_ld16x2(d, d + 32, v);
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(kBarD1f + (P & 1)));
+        if (ox <= 13) {  // conv2 reads x <= 13
+          // grid row pr in slot pr of the band's five, rows 5 and 6 in slots 1 and
+          // 2, row 4 in slots 4 and 0: each tile's three rows are neighbours
+          uint8_t *const dst = dst0 + (pr < 5 ? pr : pr - 4) * 4096;
 #pragma unroll
-          for (int s2 = 0; s2 < 2; ++s2) {
-            const int oy = 2 * pr + s2;
-            if (ox <= 13) {  // conv2 reads x <= 13
-              const int band = pr < 4 ? 0 : (pr < 6 ? 1 : 2);  // band b holds grid rows 2b .. 2b + 3
-              const int slot = pr - 2 * band;                   // this pair's grid row is oy >> 1 = pr
-              const int sg = (ox & 1) + 2 * (oy & 1);
-              uint8_t *dst = sm + kAct1Off + sg * kSubBytes + ((ox >> 1) + 8 * slot) * 512 + ri * 16;
+          for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
-              for (int c = 0; c < 2; ++c)
-                *reinterpret_cast<uint4 *>(dst + (2 * half + c) * 128) =
-                    relu_chunk(v + 16 * s2 + 8 * c, sb + 16 * half + 8 * c);
+            for (int c = 0; c < 2; ++c) {
+              const uint4 o = relu_chunk(v + 16 * s2 + 8 * c, bias + 4 * c);
+              uint8_t *const q = dst + 2 * s2 * kSubBytes + c * 128;
+              *reinterpret_cast<uint4 *>(q) = o;
+              if (pr == 4) *reinterpret_cast<uint4 *>(q - 4 * 4096) = o;
+            }
+        }
+        if (pr == 2 || pr == 4 || pr == 6) {  // three rows of a tile are there
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar(kBarBand));
+        }
+      }
+    }
+  } else if (warp < kDrain1Warps + kDrain2Warps) {
+    // ---- conv2 drain: output g (valid for px = g & 7 < 6) adds row g + 1's
+    // second half: by a shuffle, or for g = 3, 11 from the next lane quarter
+    // (rows 4, 12) through the exchange buffer, which each half of the
+    // channels has its own part of
+    const int px = g & 7, qt = warp & 3;
+    uint32_t T = 0;
+    for (int bi = 0; bi < my_batches && ok; ++bi) {
+      const int64_t batch = blockIdx.x + (int64_t)bi * gridDim.x;
+      for (int tt = 0; tt < 3 && ok; ++tt, ++T) {
+        ok = all_ok<kDrain2Warps * 32>(1, mbar_wait(bar(kBarC2 + (T & 1)), (T >> 1) & 1));
+        if (!ok) break;
+        tc_fence_after();
+        uint8_t *const dst = a.act2 + batch * (int64_t)kAct2Bytes + (px + 6 * (2 * tt + (g >> 3))) * 1024 + ri * 16;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float *const xb = reinterpret_cast<float *>(sm + kXbOff) + ((qt >> 1) * 2 + h) * 8 * kXbPitch;
+          float v[32], w[32];
+          const uint32_t d = tmem + lane_base + kD2Col + 128 * (T & 1) + 32 * h;
+          tmem_ld32x2(d, d + 64, v, w);
+          if (h == 1) {  // accumulator read: tile T + 2 may have it
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(kBarD2f + (T & 1)));
+          }
+          if ((qt & 1) && lane < 8) xrow_put(xb + lane * kXbPitch, w);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) w[c] = __shfl_down_sync(0xFFFFFFFFu, w[c], 8);
+          asm volatile("bar.sync 1, %0;" ::"r"(kDrain2Warps * 32) : "memory");
+          if (!(qt & 1) && lane >= 24) xrow_get(xb + (lane - 24) * kXbPitch, w);
+#pragma unroll
+          for (int c = 0; c < 32; ++c) v[c] += w[c];
+          if (px < 6) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const ulonglong2 *const b2 = reinterpret_cast<const ulonglong2 *>(sb + 32 + 32 * h + 8 * c);
+              const uint64_t bias[4] = {b2[0].x, b2[0].y, b2[1].x, b2[1].y};
+              *reinterpret_cast<uint4 *>(dst + (4 * h + c) * 128) = relu_chunk(v + 8 * c, bias);
             }
           }
         }
-        tc_fence_before();
-        if (pr == 2 || pr == 4 || pr == 6) {
-          fence_async_smem();
-          mbar_arrive(bar_band);
-        }
-      }
-      // (the issuing warps skip the waits on conv2 tiles 0 and 1: two parity
-      // flips, so their ph_c2 agrees with the workers' again here)
-    } else if (t == kIssuer || t == kIssuer3) {  // conv1's even / odd pairs
-      for (int pr = t == kIssuer ? 0 : 1; pr < 7; pr += 2) {
-        const int b = pr & 1;
-        r_ok &= mbar_wait(b ? bar_blk1 : bar_blk0, b ? ph_blk1 : ph_blk0);
-        if (b) ph_blk1 ^= 1u; else ph_blk0 ^= 1u;
-        issue_c1(pr & 1, pr == 0);
-        if (pr == 6) {  // the frames are dead: W3 taps 0-1 into their place
-          mbar_expect_tx(bar_w3a, kW3EarlyBytes);
-          bulk_g2s(sbase + kW3Off, a.w3, kW3EarlyBytes, bar_w3a);
-          w3_pend |= 1u;
-        }
-      }
-    } else if (t == kIssuer2) {  // conv2 tiles as the band fills (rows of pairs 2, 4 and 6)
-      for (int tt = 0; tt < 3; ++tt) {
-        r_ok &= mbar_wait(bar_band, ph_band);
-        ph_band ^= 1u;
-        issue_c2(tt);
       }
     }
-    // (no block barrier here: the drains of conv2 tiles 0 and 1 below need
-    // only the workers' own waits, and conv2's issuing thread may still be
-    // issuing tile 2; r_ok joins the block-wide wait on tile 2)
-    // ---- conv2 epilogues into region X: tiles 0 and 1 (done) while tile 2
-    // computes; conv2's issuing thread loads the rest of W3 over the band as soon
-    // as tile 2 is done
-    // Output g (valid for px = g & 7 < 6) adds row g + 1's second half: by a
-    // shuffle, or for g = 3, 11 from the next lane quarter (rows 4, 12)
-    // through the exchange buffer.
-    auto drain_c2 = [&](int tt) {
-      const int px = g & 7, py = 2 * tt + (g >> 3), h = half, qt = warp & 3;
-      float *xb = reinterpret_cast<float *>(sm + ((tt & 1) ? kXb2Off : kXb1Off)) + ((qt >> 1) * 2 + h) * 8 * kXbPitch;
-      float v[32], w[32];
-      const uint32_t d = tmem + lane_base + kD2Col + 128 * tt + 32 * h;
-      tmem_ld32x2(d, d + 64, v, w);
-      if ((qt & 1) && lane < 8) xrow_put(xb + lane * kXbPitch, w);
+  } else if (warp < kIssueWarp) {
+    // ---- builders. A batch's frames lie in shared memory as packed rows (bit
+    // x of row word y = pixel (x, y)), [row y][frame c][instance i], so that
+    // the 32 lanes of a warp building one block position read 32 consecutive
+    // words. Thread tb holds rows 2 y2, 2 y2 + 1 of all four frames of one
+    // instance of the next batch in registers.
+    const int bw = warp - kDrain1Warps - kDrain2Warps, tb = 32 * bw + lane, fi = tb & 7, y2 = tb >> 3;
+    uint64_t *const fr = reinterpret_cast<uint64_t *>(sm + kFrOff);
+    uint8_t *const blk = sm + kBlkOff + 4 * bw * 512 + lane * 16;
+    uint64_t pf[8];  // [frame c][row 2 y2, 2 y2 + 1]
+    auto load_words = [&](int64_t first) {
 #pragma unroll
-      for (int c = 0; c < 32; ++c) w[c] = __shfl_down_sync(0xFFFFFFFFu, w[c], 8);
-      asm volatile("bar.sync 1, %0;" ::"r"(kConvWork) : "memory");
-      if (!(qt & 1) && lane >= 24) xrow_get(xb + (lane - 24) * kXbPitch, w);
-#pragma unroll
-      for (int c = 0; c < 32; ++c) v[c] += w[c];
-      if (px < 6) {
-        uint8_t *dst = sm + kAct2Off + (px + 8 * py) * 1024 + ri * 16;
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          *reinterpret_cast<uint4 *>(dst + (4 * h + c) * 128) = relu_chunk(v + 8 * c, sb + 32 + 32 * h + 8 * c);
+      for (int c = 0; c < 4; ++c) {
+        ulonglong2 v = make_ulonglong2(0, 0);
+        if (first + fi < a.n)
+          v = __ldg(reinterpret_cast<const ulonglong2 *>(a.obs_words + (first + fi) * 128 + c * 32 + 2 * y2));
+        pf[2 * c] = v.x;
+        pf[2 * c + 1] = v.y;
       }
     };
-    if (issuer) {
-      if (t == kIssuer2 && mbar_wait(bar_c2, ph_c2)) {  // (a timeout here shows in the waits below)
-        fence_async_smem();
-        mbar_expect_tx(bar_w3b, kW3Bytes - kW3EarlyBytes);
-        for (uint32_t o = kW3EarlyBytes; o < kW3Bytes; o += 16384)
-          bulk_g2s(sbase + kW3Off + o, a.w3 + o, 16384, bar_w3b);
-        w3_pend |= 2u;
+    // uint8 frames: frame c's two rows are 128 bytes, on their way while the
+    // pairs between are built, then packed (nonzero -> 1)
+    uint4 raw[8];
+    auto load_bytes = [&](int64_t first, int c) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        raw[q] = first + fi < a.n
+                     ? __ldg(reinterpret_cast<const uint4 *>(a.obs_u8 + ((first + fi) * 128 + c * 32 + 2 * y2) * 64) + q)
+                     : make_uint4(0, 0, 0, 0);
+    };
+    auto pack_bytes = [&](int c) {
+#pragma unroll
+      for (int y = 0; y < 2; ++y) {
+        uint32_t bits[2] = {0, 0};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const uint4 r = raw[4 * y + q];
+          const uint32_t w4[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            // bit 0 of each byte that is not zero; the product gathers the four in its top byte
+            const uint32_t m = ((((w4[e] & 0x7F7F7F7Fu) + 0x7F7F7F7Fu) | w4[e]) >> 7) & 0x01010101u;
+            bits[q >> 1] |= ((m * 0x01020408u) >> 24) << (16 * (q & 1) + 4 * e);
+          }
+        }
+        pf[2 * c + y] = (uint64_t)bits[0] | (uint64_t)bits[1] << 32;
+      }
+    };
+    auto build_row = [&](int row, int slot) {  // block row: pixel rows 2 row, 2 row + 1; this warp's 4 of 16 positions
+      const uint32_t u0 = (uint32_t)(fr[2 * row * 32 + lane] >> (16 * bw));
+      const uint32_t u1 = (uint32_t)(fr[(2 * row + 1) * 32 + lane] >> (16 * bw));
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const uint2 lo = nib[(u0 >> (4 * j)) & 15u], hi = nib[(u1 >> (4 * j)) & 15u];
+        *reinterpret_cast<uint4 *>(blk + (16 * slot + j) * 512) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+      }
+    };
+    if (kU8) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        load_bytes((int64_t)blockIdx.x * kP, c);
+        pack_bytes(c);
       }
     } else {
-      tc_fence_after();
-      drain_c2(0);
-      drain_c2(1);
+      load_words((int64_t)blockIdx.x * kP);
     }
-    {  // conv2 tile 2, and every thread's outcome so far
-      const bool w_ok = mbar_wait(bar_c2, ph_c2) && ok && r_ok;
-      ph_c2 ^= 1u;
-      ok = !__syncthreads_or(!w_ok);
-    }
-    if (!ok) break;
-    tc_fence_after();
-    if (!issuer) drain_c2(2);
-    tc_fence_before();
-    fence_async_smem();
-    ok = !__syncthreads_or(!(mbar_wait(bar_w3a, ph_w3) && mbar_wait(bar_w3b, ph_w3)));
-    ph_w3 ^= 1u;
-    w3_pend = 0;
-    if (!ok) break;
-
-    // ---- conv3: two tiles of 16 positions (qx + 8 qy, qy in {2u, 2u + 1}),
-    // 3 kernel rows x 4 k-steps of N = 192 each (one completion barrier per
-    // tile, so the first tile drains while the second computes)
-    if (t == kIssuer) {
-      tc_fence_after();
-      for (int u = 0; u < 2; ++u) {
-        for (int ky = 0; ky < 3; ++ky)
-          for (int kk = 0; kk < 4; ++kk) {
-            const uint64_t ad = sdesc_at(a3d, (16 * u + 8 * ky) * 1024 + kk * 256);
-            const uint64_t bd = sdesc_at(b3d, ky * 24576 + kk * 6144);
-            mma_bf16(tmem + kD3Col + 192 * u, ad, bd, idesc_bf16(128, 192), (ky | kk) != 0);
-          }
-        mma_commit(u ? bar_c3b : bar_c3a);
-      }
-    }
-    // Drain: the outputs (qx < 4) lie in lane quarters 0 and 2 (positions
-    // g = 0..3, 8..11); rows g + 1 and g + 2 come from the same warp by
-    // shuffles, or, past the quarter's end, from quarters 1 and 3 (positions
-    // 4, 5 and 12, 13, no outputs of their own) through the exchange buffer.
-    // (the issuing warps go on to the batch's closing barrier; the workers'
-    // outcome joins it there)
-    for (int u = 0; u < 2 && !issuer; ++u) {
-      ok = (u ? wait_workers(bar_c3b, ph_c3b) : wait_workers(bar_c3a, ph_c3a)) && ok;
-      if (!ok) continue;  // uniform among the workers
-      if (!kU8 && u == 1 && batch + gridDim.x < n_batches) {  // the next batch's frames, in flight during this drain
-        load_frames((batch + gridDim.x) * kP, pf[0], pf[1]);
-        pf_ok = true;
-      }
-      tc_fence_after();
-      const int qt = warp & 3, h = half, sup = qt >> 1;
-      const uint32_t d = tmem + lane_base + kD3Col + 192 * u + 32 * h;
-      float *xb1 = reinterpret_cast<float *>(sm + kXb1Off) + (sup * 2 + h) * 8 * kXbPitch;
-      float *xb2 = reinterpret_cast<float *>(sm + kXb2Off) + (sup * 2 + h) * 16 * kXbPitch;
-      float v[32], w[32], x[32];
-      if (qt & 1) {  // supplier: rows 4 qt + 0, 1 for the previous quarter
-        tmem_ld32x2(d + 64, d + 128, v, w);
-        if (lane < 8) xrow_put(xb1 + lane * kXbPitch, v);
-        if (lane < 16) xrow_put(xb2 + lane * kXbPitch, w);
-        asm volatile("bar.sync 1, %0;" ::"r"(kConvWork) : "memory");
-        continue;
-      }
-      tmem_ld32x2(d + 64, d + 128, w, x);
+    uint32_t P = 0;
+    for (int bi = 0; bi < my_batches; ++bi) {
+      const int64_t next = (blockIdx.x + (int64_t)(bi + 1) * gridDim.x) * kP;  // past the end: rows of zeros
+      ok = all_ok<kBuildWarps * 32>(2, ok);  // every builder has read the previous frames
+      if (!ok) break;
 #pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        w[c] = __shfl_down_sync(0xFFFFFFFFu, w[c], 8);
-        x[c] = __shfl_down_sync(0xFFFFFFFFu, x[c], 16);
+      for (int k = 0; k < 8; ++k) fr[((2 * y2 + (k & 1)) * 4 + (k >> 1)) * 8 + fi] = pf[k];
+      asm volatile("bar.sync 2, %0;" ::"r"(kBuildWarps * 32) : "memory");
+      if (!kU8) load_words(next);
+#pragma unroll
+      for (int pr = 0; pr < 7; ++pr, ++P) {
+        // rows 2 pr + 1 and 2 pr + 2 take the places of rows that pair P - 2 read
+        // last, a batch's rows 0 .. 2 those of the previous batch's last two pairs
+        if (ok && P >= 2) ok = mbar_wait(bar(kBarC1 + (P & 1)), ((P - 2) >> 1) & 1);
+        if (pr == 0) {
+          if (ok && P >= 1) ok = mbar_wait(bar(kBarC1 + ((P - 1) & 1)), ((P - 1) >> 1) & 1);
+          build_row(0, 0);
+        }
+        build_row(2 * pr + 1, (2 * pr + 1) % kBlkRows);
+        build_row(2 * pr + 2, (2 * pr + 2) % kBlkRows);
+        fence_async_smem();
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (ok && lane == 0) mbar_arrive(bar(kBarBlk + (P & 1)));
+        if (kU8) {
+          if (pr == 2) pack_bytes(0);
+          if (pr == 4) pack_bytes(1);
+          if (pr == 5) pack_bytes(2);
+          if (pr == 0) load_bytes(next, 0);
+          if (pr == 2) load_bytes(next, 1);
+          if (pr == 4) load_bytes(next, 2);
+          if (pr == 5) load_bytes(next, 3);
+        }
       }
+      if (kU8) pack_bytes(3);
+    }
+  } else if (lane == 0) {
+    // ---- issuing threads (one per warp)
+    const int who = warp - kIssueWarp;  // 0, 1: conv1 pairs of that parity; 2: conv2
+    if (who == 0) {
+      mbar_expect_tx(bar(kBarW), kW1Bytes + kW2Bytes);
+      bulk_g2s(sbase + kW1Off, a.w1, kW1Bytes, bar(kBarW));
+      for (uint32_t o = 0; o < kW2Bytes; o += 16384) bulk_g2s(sbase + kW2Off + o, a.w2 + o, 16384, bar(kBarW));
+    }
+    ok = mbar_wait(bar(kBarW), 0);
+    if (who < 2) {
+      // Both output rows of a pair in one N = 64 accumulator: block row j (shift
+      // dx) feeds row 2p through tap (dx, dy = j) and row 2p + 1 through tap (dx,
+      // dy = j - 1); W1 holds, per (j, dx), those two taps stacked over n (zeros
+      // where a tap does not apply), so each MMA reads its A tile once for 64
+      // outputs.
+      const uint64_t a1d = sdesc(sbase + kBlkOff, 128, 512), b1d = sdesc(sbase + kW1Off, 1024, 128);
+      const uint32_t d = tmem + kD1Col + 64 * who;
+      uint32_t pr = who;
+      const uint32_t pairs = 7 * (uint32_t)my_batches;
+      for (uint32_t P = who; P < pairs && ok; P += 2) {
+        uint64_t ad[3];
+        uint32_t slot = 2 * pr % kBlkRows;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          ad[j] = sdesc_at(a1d, slot * 16 * 512);
+          slot = slot + 1 == kBlkRows ? 0 : slot + 1;
+        }
+        ok = (P < 2 || mbar_wait(bar(kBarD1f + who), ((P >> 1) - 1) & 1)) && mbar_wait(bar(kBarBlk + who), (P >> 1) & 1);
+        if (!ok) break;
+        tc_fence_after();
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+#pragma unroll
+          for (int dx = 0; dx < 2; ++dx)
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+              mma_bf16(d, sdesc_at(ad[j], dx * 512 + kk * 256), sdesc_at(b1d, (2 * j + dx) * 4096 + kk * 2048),
+                       idesc_bf16(128, 64), (j | dx | kk) != 0);
+        if (!(a.stall && P == 0)) mma_commit(bar(kBarC1 + who));
+        pr = pr >= 5 ? pr - 5 : pr + 2;
+      }
+    } else {
+      const uint64_t a2d = sdesc(sbase + kAct1Off, 128, 512), b2d = sdesc(sbase + kW2Off, 2048, 128);
+      const uint32_t tiles = 3 * (uint32_t)my_batches;
+      uint32_t tt = 0;
+      for (uint32_t T = 0; T < tiles && ok; ++T) {
+        ok = (T < 2 || mbar_wait(bar(kBarD2f + (T & 1)), ((T >> 1) - 1) & 1)) && mbar_wait(bar(kBarBand), T & 1);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t at = sdesc_at(a2d, tt == 1 ? 2 * 4096 : 0);  // tile 1 from slot 2 on, tiles 0 and 2 from slot 0
+        const uint32_t d = tmem + kD2Col + 128 * (T & 1);
+#pragma unroll
+        for (int ky = 0; ky < 4; ++ky)
+#pragma unroll
+          for (int px = 0; px < 2; ++px)  // taps (px, ky) and (px + 2, ky)
+#pragma unroll
+            for (int kk = 0; kk < 2; ++kk)
+              mma_bf16(d, sdesc_at(at, (px + 2 * (ky & 1)) * kSubBytes + (ky >> 1) * 4096 + kk * 256),
+                       sdesc_at(b2d, (ky * 2 + px) * 8192 + kk * 4096), idesc_bf16(128, 128), (ky | px | kk) != 0);
+        mma_commit(bar(kBarC2 + (T & 1)));
+        tt = tt == 2 ? 0 : tt + 1;
+      }
+    }
+  }
+  ok = !__syncthreads_or(!ok);
+  if (!ok && t == 0) atomicOr(a.err, 1u);
+  if (!ok && warp >= kIssueWarp && lane == 0) {  // let this thread's MMAs and copies land
+    mma_commit(bar(kBarFin + warp - kIssueWarp));
+    mbar_wait(bar(kBarFin + warp - kIssueWarp), 0);
+    if (warp == kIssueWarp) mbar_wait(bar(kBarW), 0);
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kConvTmemCols));
+}
+
+struct Conv3Args {
+  const uint8_t *act2;
+  int64_t n;
+  const uint8_t *w3;          // packed bf16 B operand
+  const float *fp;            // FpLayout
+  uint8_t *act3;              // [tiles][16][8][128][16 B]
+  unsigned int *err;
+};
+
+// conv3 of batches blockIdx.x, blockIdx.x + gridDim.x, ...: the M tile is the
+// 4 x 4 output positions of 8 instances exactly. Tap (kx, ky) reads input
+// positions (qx + kx, qy + ky): the ring's stages hold, for one kx, columns
+// kx .. kx + 3 of the six rows (24 positions; each row is one bulk copy of 4
+// KB), and ky shifts the start by one row of them.
+__global__ void __launch_bounds__(kConv3Threads, 1) policy_conv3_kernel(const Conv3Args a) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ __align__(8) uint64_t full[kStages3], empty[kStages3], done[2], freed[2], bar_w, fin;
+  __shared__ uint32_t tmem_s;
+  __shared__ __align__(16) float sb[64];
+  __shared__ int s_issued, s_landed;  // stages whose copies were issued / waited for
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const uint32_t sbase = smem_u32(sm);
+  if (t < 64) sb[t] = a.fp[FpLayout::b3 + t];
+  if (t == 0) {
+    for (int s = 0; s < kStages3; ++s) {
+      mbar_init(smem_u32(&full[s]), 1);
+      mbar_init(smem_u32(&empty[s]), 1);
+    }
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(smem_u32(&done[j]), 1);
+      mbar_init(smem_u32(&freed[j]), kDrain3Warps);
+    }
+    mbar_init(smem_u32(&bar_w), 1);
+    mbar_init(smem_u32(&fin), 1);
+    s_issued = s_landed = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
+                 "r"(kConvTmemCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_s;
+  grid_dependents_launch();
+  const int64_t n_batches = (a.n + kP - 1) / kP;
+  const int my_batches = (int)((n_batches - blockIdx.x + gridDim.x - 1) / gridDim.x);
+  bool ok = true;
+  if (warp < kDrain3Warps) {
+    // drain: warps w and w + 4 read lane quarter w & 3 (four positions), 32 of the 64 channels each
+    const int half = warp >> 2, m = 4 * (warp & 3) + (lane >> 3), ri = lane & 7;  // m = qx + 4 qy
+    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
+    for (int bi = 0; bi < my_batches; ++bi) {
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&done[bi & 1]), (bi >> 1) & 1));
+      if (!ok) break;
+      tc_fence_after();
+      float v[32], w[32], x[32];
+      const uint32_t d = tmem + lane_base + 256 * (bi & 1) + 32 * half;
+      tmem_ld32x2(d + 64, d + 128, w, x);
       tmem_ld32(d, v);
-      asm volatile("bar.sync 1, %0;" ::"r"(kConvWork) : "memory");
-      if (lane >= 24) xrow_get(xb1 + (lane - 24) * kXbPitch, w);
-      if (lane >= 16) xrow_get(xb2 + (lane - 16) * kXbPitch, x);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&freed[bi & 1]));
 #pragma unroll
       for (int c = 0; c < 32; ++c) v[c] += w[c] + x[c];
-      const int m = 16 * u + g, qx = m & 7, qy = m >> 3;
-      const int64_t inst = i0 + ri;
-      if (qx < 4 && inst < a.n) {
-        const int q = qx + 4 * qy;  // feature slice: k = 64 q + channel
-        uint8_t *dst = a.act3 + (inst >> 7) * (int64_t)kAct3TileBytes + q * 16384 + (inst & 127) * 16;
+      const int64_t inst = (blockIdx.x + (int64_t)bi * gridDim.x) * kP + ri;
+      if (inst < a.n) {
+        // feature slice m: k = 64 m + channel
+        uint8_t *dst = a.act3 + (inst >> 7) * (int64_t)kAct3TileBytes + m * 16384 + (inst & 127) * 16;
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          *reinterpret_cast<uint4 *>(dst + (4 * h + c) * 2048) = relu_chunk(v + 8 * c, sb + 96 + 32 * h + 8 * c);
+        for (int c = 0; c < 4; ++c) {
+          const ulonglong2 *const b3 = reinterpret_cast<const ulonglong2 *>(sb + 32 * half + 8 * c);
+          const uint64_t bias[4] = {b3[0].x, b3[0].y, b3[1].x, b3[1].y};
+          *reinterpret_cast<uint4 *>(dst + (4 * half + c) * 2048) = relu_chunk(v + 8 * c, bias);
+        }
       }
     }
-    tc_fence_before();
-    ok = !__syncthreads_or(!ok);  // region X and the W3 region are rewritten by the next batch
+  } else if (t == kDrain3Warps * 32) {  // copies
+    mbar_expect_tx(smem_u32(&bar_w), kW3Bytes);
+    for (uint32_t o = 0; o < kW3Bytes; o += 24576) bulk_g2s(sbase + o, a.w3 + o, 24576, smem_u32(&bar_w));
+    grid_dependency_wait();  // conv2's output
+    const int total = 3 * my_batches;
+    int kx = 0, st = 0, use = 0, issued = 0;
+    const uint8_t *src = a.act2 + (int64_t)blockIdx.x * kAct2Bytes;
+    for (int q = 0; q < total; ++q) {
+      if (use > 0) ok = mbar_wait(smem_u32(&empty[st]), (use - 1) & 1);  // the stage's previous MMAs are done
+      if (!ok) break;
+      const uint32_t f = smem_u32(&full[st]), dst = sbase + kW3Bytes + st * kStage3Bytes;
+      mbar_expect_tx(f, kStage3Bytes);
+#pragma unroll
+      for (int py = 0; py < 6; ++py) bulk_g2s(dst + py * 4096, src + (kx + 6 * py) * 1024, 4096, f);
+      issued = q + 1;
+      if (++kx == 3) {
+        kx = 0;
+        src += (int64_t)gridDim.x * kAct2Bytes;
+      }
+      if (++st == kStages3) {
+        st = 0;
+        ++use;
+      }
+    }
+    s_issued = issued;
+  } else if (t == kDrain3Warps * 32 + 32) {  // MMAs
+    const uint64_t a3d = sdesc(sbase + kW3Bytes, 128, 1024), b3d = sdesc(sbase, 3072, 128);
+    ok = mbar_wait(smem_u32(&bar_w), 0);
+    int st = 0, use = 0, landed = 0;
+    for (int bi = 0; bi < my_batches && ok; ++bi) {
+      if (bi >= 2) ok = mbar_wait(smem_u32(&freed[bi & 1]), ((bi >> 1) - 1) & 1);
+      for (int kx = 0; kx < 3 && ok; ++kx) {
+        ok = mbar_wait(smem_u32(&full[st]), use & 1);
+        if (!ok) break;
+        ++landed;
+        tc_fence_after();
+        const uint64_t at = sdesc_at(a3d, st * kStage3Bytes), bt = sdesc_at(b3d, kx * 1024);
+        const uint32_t d = tmem + 256 * (bi & 1) + 64 * kx;  // an accumulator per kx, summed by the drain
+#pragma unroll
+        for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            mma_bf16(d, sdesc_at(at, ky * 4096 + kk * 256), sdesc_at(bt, ky * 24576 + kk * 6144), idesc_bf16(128, 64),
+                     (ky | kk) != 0);
+        mma_commit(smem_u32(&empty[st]));
+        if (++st == kStages3) {
+          st = 0;
+          ++use;
+        }
+      }
+      if (ok) mma_commit(smem_u32(&done[bi & 1]));
+    }
+    s_landed = landed;
   }
-  if (!ok && t == 0) atomicOr(a.err, 1u);
-  if (!ok && (t == kIssuer || t == kIssuer2 || t == kIssuer3)) {  // let this thread's MMAs and copies land
-    const uint32_t fin = smem_u32(&bars[t == kIssuer ? 8 : (t == kIssuer2 ? 12 : 13)]);
-    mma_commit(fin);
-    mbar_wait(fin, 0);
-    if (t == kIssuer) mbar_wait(bar_w, 0);
-    if (w3_pend & 1u) mbar_wait(bar_w3a, ph_w3);
-    if (w3_pend & 2u) mbar_wait(bar_w3b, ph_w3);
+  ok = !__syncthreads_or(!ok);
+  if (!ok && t == 0) {
+    atomicOr(a.err, 1u);
+    // copies issued but never waited for land before shared memory goes
+    mbar_wait(smem_u32(&bar_w), 0);
+    for (int q = s_landed; q < s_issued; ++q) mbar_wait(smem_u32(&full[q % kStages3]), (q / kStages3) & 1);
+  }
+  if (!ok && t == kDrain3Warps * 32 + 32) {  // let this thread's MMAs land before TMEM goes
+    mma_commit(smem_u32(&fin));
+    mbar_wait(smem_u32(&fin), 0);
   }
   tc_fence_before();
   __syncthreads();
@@ -833,6 +909,7 @@ __global__ void __launch_bounds__(kThreads, 1) policy_heads_kernel(const HeadsAr
   __shared__ int s_landed;  // slices whose copies the MMA thread has waited for
   int loaded = 0;           // thread 0: slices whose copies were issued
   if (t == 0) {
+    grid_dependency_wait();  // conv3's features
     for (int s = 0; s < kSlices && ok; ++s) {
       const int st = s % kHeadStages;
       // stage st last held slice s - kHeadStages: its MMAs must be done
@@ -976,26 +1053,42 @@ uint16_t bf16_bits(float f) {
   return b;
 }
 
+// dependent: the kernel may be set up before the one ahead of it in the
+// stream has ended; it waits for that itself (grid_dependency_wait).
+template <class Args>
+cudaError_t launch(void (*kernel)(const Args), dim3 grid, int block, size_t smem, cudaStream_t s, bool dependent,
+                   const Args &args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
 int launch_forward(octax_policy *p, int64_t n, const uint64_t *obs_words, const uint8_t *obs_u8, uint64_t seed,
                    uint32_t step, float *logits, float *value, uint8_t *actions, cudaStream_t s) {
   if (n < 1 || n > p->max_envs) {
     set_error("octax_policy: need 1 <= n_envs <= max_envs of the policy");
     return OCTAX_EINVAL;
   }
-  ConvArgs c{obs_words, obs_u8, n, (const uint8_t *)p->w1, (const uint8_t *)p->w2, (const uint8_t *)p->w3, p->fp,
-             p->act3, p->err, p->stall};
-  const int64_t batches = (n + kP - 1) / kP;
-  const int grid = (int)std::min<int64_t>(batches, p->sms);
-  if (obs_u8)
-    policy_conv_kernel<true><<<grid, kConvThreads, kConvSmem, s>>>(c);
-  else
-    policy_conv_kernel<false><<<grid, kConvThreads, kConvSmem, s>>>(c);
-  cudaError_t r = cudaGetLastError();
-  if (r != cudaSuccess) return cuda_fail(r, "policy conv launch");
+  ConvArgs c{obs_words, obs_u8, n, (const uint8_t *)p->w1, (const uint8_t *)p->w2, p->fp, p->act2, p->err, p->stall};
+  Conv3Args c3{p->act2, n, (const uint8_t *)p->w3, p->fp, p->act3, p->err};
   HeadsArgs h{p->act3, n, (const uint8_t *)p->wh, p->fp, p->n_logits, logits, value, actions,
               (uint32_t)seed, (uint32_t)(seed >> 32), step, p->err};
-  policy_heads_kernel<<<dim3((unsigned)((n + 127) / 128), 2), kThreads, kHeadSmem, s>>>(h);
-  r = cudaGetLastError();
+  const int64_t batches = (n + kP - 1) / kP;
+  const unsigned grid = (unsigned)std::min<int64_t>(batches, p->sms);
+  cudaError_t r = obs_u8 ? launch(policy_conv12_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, false, c)
+                         : launch(policy_conv12_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, false, c);
+  if (r != cudaSuccess) return cuda_fail(r, "policy conv launch");
+  r = launch(policy_conv3_kernel, dim3(grid), kConv3Threads, kConv3Smem, s, true, c3);
+  if (r != cudaSuccess) return cuda_fail(r, "policy conv3 launch");
+  r = launch(policy_heads_kernel, dim3((unsigned)((n + 127) / 128), 2), kThreads, kHeadSmem, s, true, h);
   if (r != cudaSuccess) return cuda_fail(r, "policy heads launch");
   return OCTAX_OK;
 }
@@ -1105,6 +1198,9 @@ int octax_policy_create(const octax_policy_params *prm, int64_t max_envs, int de
   if ((r = cudaMalloc(&p->w3, w3p.size() * 2)) != cudaSuccess) return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc(&p->wh, whp.size() * 2)) != cudaSuccess) return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc((void **)&p->fp, fp.size() * 4)) != cudaSuccess) return fail(r, "octax_policy_create: alloc");
+  const int64_t batches = (max_envs + kP - 1) / kP;
+  if ((r = cudaMalloc((void **)&p->act2, (size_t)batches * kAct2Bytes)) != cudaSuccess)
+    return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc((void **)&p->act3, (size_t)tiles * kAct3TileBytes)) != cudaSuccess)
     return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc((void **)&p->ring, (size_t)2 * max_envs * 1024)) != cudaSuccess)
@@ -1126,9 +1222,11 @@ int octax_policy_create(const octax_policy_params *prm, int64_t max_envs, int de
   if (r == cudaSuccess) r = cudaMemset(p->ring, 0, (size_t)2 * max_envs * 1024);
   if (r == cudaSuccess) r = cudaMemset(p->err, 0, 4);
   if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(policy_conv_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
+    r = cudaFuncSetAttribute(policy_conv12_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
   if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(policy_conv_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
+    r = cudaFuncSetAttribute(policy_conv12_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
+  if (r == cudaSuccess)
+    r = cudaFuncSetAttribute(policy_conv3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kConv3Smem);
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(policy_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadSmem);
   if (r != cudaSuccess) return fail(r, "octax_policy_create: upload");
@@ -1231,7 +1329,7 @@ void octax_policy_destroy(octax_policy *p) {
   if (!p) return;
   cudaSetDevice(p->device);
   if (p->stream) cudaStreamSynchronize(p->stream);
-  for (void *q : {p->w1, p->w2, p->w3, p->wh, (void *)p->fp, (void *)p->act3, (void *)p->ring, (void *)p->err})
+  for (void *q : {p->w1, p->w2, p->w3, p->wh, (void *)p->fp, (void *)p->act2, (void *)p->act3, (void *)p->ring, (void *)p->err})
     if (q) cudaFree(q);
   if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
   delete p;
