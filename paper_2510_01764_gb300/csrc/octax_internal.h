@@ -197,6 +197,34 @@ int table_uops(const octax_game *games, int n_games);
 cudaError_t upload_blobs(const std::vector<GameDev> &games, const std::vector<uint8_t> &images, int n_uops, int schip,
                          uint32_t quirks, uint8_t *blobs, cudaStream_t s);
 
+// Programmatic dependent launch: a kernel launched with `dependent` may be set
+// up before the one ahead of it in the stream has ended. It touches nothing
+// that another kernel may write before its grid_dependency_wait(), which
+// returns when the kernels ahead have ended, and lets its own successor be set
+// up (grid_dependents_launch()) only after that, or where all it writes follows
+// from data read after that: so no two kernels of a stream run side by side
+// but for their set-up.
+#ifdef __CUDACC__
+__device__ __forceinline__ void grid_dependents_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+#endif
+inline cudaError_t launch_kernel(const void *fn, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t s,
+                                 bool dependent) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelExC(&cfg, fn, args);
+}
+
 // Error reporting (thread-local message).
 void set_error(const std::string &msg);
 int cuda_fail(cudaError_t e, const char *what);

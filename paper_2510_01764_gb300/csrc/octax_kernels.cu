@@ -1049,6 +1049,9 @@ __device__ void run_group(const StepLaunch &p, const Group &g, const Warp &W) {
         __syncwarp();
       }
     }
+    // little is left of the launch: its successor may be set up (earlier, its
+    // waiting CTAs would keep the SMs from other streams' kernels)
+    if (s + 1 == p.steps) grid_dependents_launch();
     bool done = false;
     if (W.active) {
       const int32_t sc = score(R, C, G);
@@ -1098,11 +1101,12 @@ __global__ void __launch_bounds__(kMaxBlock, 2) step_kernel(const StepLaunch p) 
     if (gi >= p.n_groups) break;
     const Group g = p.groups[gi];
     const Warp W = make_warp(p.ipw, blockDim.x >> 5, g, (uint32_t)p.n_uops, Rec<kS>::kWords);
-    fetch_records<kS>(W, p.st, g);
     if ((int)g.game != cur_game) {
       stage_game(p.blobs, p.stride, g.game, (uint32_t)p.n_uops);
       cur_game = g.game;
     }
+    grid_dependency_wait();  // states, actions and output buffers from here on
+    fetch_records<kS>(W, p.st, g);
     copy_wait();
     __syncthreads();
     run_group<kWrap, kS>(p, g, W);
@@ -1346,11 +1350,12 @@ __global__ void step_kernel_ws(const StepLaunch p) {
     if (gi >= p.n_groups) break;
     const Group g = p.groups[gi];
     const Warp W = make_warp(p.ipw, E, g, (uint32_t)p.n_uops, Rec<false>::kWords);
-    if (!writer) fetch_records<false>(W, p.st, g);
     if ((int)g.game != cur_game) {
       stage_game(p.blobs, p.stride, g.game, (uint32_t)p.n_uops);
       cur_game = g.game;
     }
+    grid_dependency_wait();  // states, actions and output buffers from here on
+    if (!writer) fetch_records<false>(W, p.st, g);
     copy_wait();
     __syncthreads();
     if (!failed) {
@@ -1626,8 +1631,8 @@ cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s
   copy.n_uops = launch_uops(block, p.ipw, p.st.schip, p.writers, p.n_uops);
   void *args[] = {&copy};
   const int threads = p.writers > 0 ? block + 32 * p.writers : block;
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args,
-                          launch_smem(block, p.ipw, p.st.schip, p.writers, copy.n_uops), s);
+  return launch_kernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args,
+                       launch_smem(block, p.ipw, p.st.schip, p.writers, copy.n_uops), s, !p.work_counter);
 }
 
 cudaError_t launch_reset(const ResetLaunch &p, int block, cudaStream_t s) {

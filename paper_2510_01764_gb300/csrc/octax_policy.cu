@@ -79,13 +79,12 @@ int env_device(const octax_env *e);
 namespace {
 
 constexpr int kP = 8;            // instances per conv batch
-constexpr int kThreads = 256;    // heads kernel: two warps per TMEM lane quarter
 // conv1 / conv2 kernel: warps by role; a draining warp reads the TMEM lane quarter warp & 3
 constexpr int kDrain1Warps = 8, kDrain2Warps = 4, kBuildWarps = 4, kIssueWarps = 3;
 constexpr int kIssueWarp = kDrain1Warps + kDrain2Warps + kBuildWarps;  // the first of them
 constexpr int kConvThreads = 32 * (kIssueWarp + kIssueWarps);
-// conv3 kernel: draining warps, a warp for the copies, a warp for the MMAs
-constexpr int kDrain3Warps = 8, kConv3Threads = 32 * (kDrain3Warps + 2);
+// conv3 kernel: draining warps, then a warp each for the copies and the MMAs of even and of odd batches
+constexpr int kDrain3Warps = 8, kConv3Threads = 32 * (kDrain3Warps + 4);
 constexpr int kMaxLogits = 17;   // 16 keys + the no-op
 constexpr uint64_t kMaxWaitNs = 1000000000ull;
 constexpr uint32_t kMaxPolls = 1u << 24;
@@ -95,8 +94,9 @@ constexpr uint32_t kW1Off = 0;                             // conv1 B: [j 3][dx 
 constexpr uint32_t kW1Bytes = 6 * 4 * 64 * 16;
 constexpr uint32_t kW2Off = kW1Off + kW1Bytes;             // conv2 B: [ky 4][kx & 1][chunk 4][n 128][8]
 constexpr uint32_t kW2Bytes = 4 * 2 * 4 * 128 * 16;
-constexpr uint32_t kAct1Off = kW2Off + kW2Bytes;           // band: 4 parity sub-grids of five grid rows of 8
-constexpr uint32_t kSubBytes = 5 * 8 * 512;                // position: 4 chunks x 8 instances x 16 B
+constexpr uint32_t kAct1Off = kW2Off + kW2Bytes;           // band: 4 parity sub-grids of six grid rows of 7
+constexpr uint32_t kBandSlots = 6, kSlotBytes = 7 * 512;   // position: 4 chunks x 8 instances x 16 B
+constexpr uint32_t kSubBytes = kBandSlots * kSlotBytes;
 constexpr uint32_t kAct1Bytes = 4 * kSubBytes;
 constexpr uint32_t kBlkRows = 5;                           // ring of block rows; a batch's 15 go round it three times
 constexpr uint32_t kBlkOff = kAct1Off + kAct1Bytes;        // 16 positions each, and one that only discarded rows read
@@ -104,11 +104,11 @@ constexpr uint32_t kBlkBytes = (kBlkRows * 16 + 1) * 512;
 constexpr uint32_t kFrOff = kBlkOff + kBlkBytes;           // frames [32 rows][4][8] u64
 constexpr uint32_t kXbOff = kFrOff + 8192;
 // conv2 drain exchange: row g + 1 of the warps that hold the last positions
-// of a TMEM lane quarter comes from the next quarter's warp: [supplier 2]
-// [channel half 2][lane 8][36 floats] (rows padded to 144 B: 16-byte
-// aligned, and 8 lanes' rows start in distinct bank groups).
+// of a TMEM lane quarter comes from the next quarter's warp: [supplier 3]
+// [lane 8][36 floats] (rows padded to 144 B: 16-byte aligned, and 8 lanes'
+// rows start in distinct bank groups).
 constexpr int kXbPitch = 36;
-constexpr uint32_t kConvSmem = kXbOff + 2 * 2 * 8 * kXbPitch * 4;
+constexpr uint32_t kConvSmem = kXbOff + 3 * 8 * kXbPitch * 4;
 static_assert(kConvSmem + 1024 <= 227 * 1024, "conv kernel shared memory (with 1 KB of static shared data)");
 constexpr uint32_t kAct2Bytes = 36 * 1024;                 // conv2 output of a batch: position: 8 chunks x 8 x 16 B
 // TMEM columns (fp32): conv1: 2 buffers x 2 output rows x 32; conv2: 2 buffers x 128
@@ -122,12 +122,12 @@ constexpr uint32_t kConv3Smem = kW3Bytes + kStages3 * kStage3Bytes;
 static_assert(kConv3Smem + 1024 <= 227 * 1024, "conv3 kernel shared memory (with 1 KB of static shared data)");
 
 // ---- heads kernel -----------------------------------------------------------
-constexpr int kHeadStages = 3;
-constexpr uint32_t kHA = 128 * 32 * 2;      // A slice: 128 rows x 32 K (bf16) = 4 chunk planes
-constexpr uint32_t kHB = 256 * 32 * 2;      // B slice: 256 rows x 32 K
-constexpr uint32_t kHeadOutOff = kHeadStages * (kHA + kHB);
-constexpr uint32_t kHeadPartOff = kHeadOutOff + (kMaxLogits + 1) * 256 * 4 + 2 * 256 * 4;
-constexpr uint32_t kHeadSmem = kHeadPartOff + 128 * (kMaxLogits + 1) * 4;  // + partial outputs of warps 4-7
+constexpr uint32_t kHA = 128 * 64 * 2;                // A slice: 128 rows x 64 K (bf16) = 8 chunk planes
+constexpr uint32_t kHB = 256 * 64 * 2;                // B slice: 256 rows x 64 K
+constexpr uint32_t kHeadRing = 192 * 1024;            // stages | output layer [output][256] | biases, hidden and output
+constexpr uint32_t kHeadSmem = kHeadRing + kMaxLogits * 256 * 4 + (256 + 32) * 4;
+static_assert(kHeadSmem + 1024 <= 227 * 1024, "heads kernel shared memory (with 1 KB of static shared data)");
+static_assert(2 * 8 * kMaxLogits * 128 * 4 <= kHeadRing, "the sums fit the ring");
 constexpr uint32_t kAct3TileBytes = 128 * 1024 * 2;   // [slice 16][chunk 8][row 128][16 B]
 
 // fp32 parameter block: b1 32 | b2 64 | b3 64 | bh [2][256] | wa2 [17][256] | ba2 [17] | wc2 [256] | bc2
@@ -158,11 +158,16 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+  // the timer is read rarely: a read takes longer than the waits of a pipeline that runs
   if (mbar_try(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
+  uint64_t t0 = 0;
   for (uint32_t i = 0; i < kMaxPolls; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if (global_ns() - t0 > kMaxWaitNs) break;
+#pragma unroll 1
+    for (int k = 0; k < 32; ++k)
+      if (mbar_try(bar, parity)) return true;
+    const uint64_t now = global_ns();
+    if (i == 0) t0 = now;
+    if (now - t0 > kMaxWaitNs) break;
   }
   return false;
 }
@@ -203,6 +208,22 @@ __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+// The same from a whole warp in step: one lane issues. All operands are the
+// same in every lane and known to be, so they need no moves to uniform
+// registers behind every instruction.
+__device__ __forceinline__ void mma_bf16_warp(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n\t.reg .pred p, e;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|e, 0xFFFFFFFF;\n\t"
+      "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ __forceinline__ void mma_commit_warp(uint32_t bar) {
+  asm volatile(
+      "{\n\t.reg .pred e;\n\telect.sync _|e, 0xFFFFFFFF;\n\t"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -335,11 +356,11 @@ __device__ __forceinline__ bool all_ok(int id, bool ok) {
       : "memory");
   return !any_fail;
 }
-// Programmatic dependent launch: the next kernel of the stream may start its
-// set-up; what it reads of this grid's results waits for the grid's end.
-__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
+// The band slot of the row after row pr (of a batch's seven): past the last
+// slot comes the first, or, if that holds row pr again, the second.
+__device__ __forceinline__ uint32_t next_slot(uint32_t slot, int pr) {
+  return slot < kBandSlots - 1 ? slot + 1 : pr < 6 ? 1 : 0;
+}
 __device__ __forceinline__ uint32_t philox_w0(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3, uint32_t k0,
                                               uint32_t k1) {
 #pragma unroll
@@ -376,32 +397,35 @@ struct ConvArgs {
 // batch's end, on different batches) at the same time:
 //   builders     wait c1[P & 1] (pair P - 2's MMAs: its block rows are free)  arrive blk[P & 1]
 //   conv1 issue  wait blk[P & 1], d1f[P & 1] (accumulator drained)           commit c1[P & 1]
-//   conv1 drain  wait c1[P & 1], c2[.] where band rows are rewritten         arrive d1f[P & 1], band
-//   conv2 issue  wait band, d2f[T & 1]                                       commit c2[T & 1]
+//   conv1 drain  wait c1[P & 1], c2[.] where band rows are rewritten         arrive d1f[P & 1], band[T & 1]
+//   conv2 issue  wait band[T & 1], d2f[T & 1]                                commit c2[T & 1]
 //   conv2 drain  wait c2[T & 1]                                              arrive d2f[T & 1]
 // P counts conv1 pairs (7 per batch), T conv2 tiles (3 per batch). A barrier
 // never gets two phases ahead of any of its waiters: pair P + 2 needs pair P
 // drained and its blocks rebuilt, tile T + 2 needs tile T drained, and the
-// conv1 drain waits for every tile before it writes the rows that the tile
-// after next needs. Every wait is bounded; a role whose wait runs out leaves
+// conv1 drain waits for every tile before it completes the rows of the tile
+// after next.
+// The band: each conv1 grid row goes to the next of six slots, round and
+// round. A tile reads its three rows as two pairs of neighbours, so a row that
+// falls on the last slot is also written to the first, where its pair with the
+// row after it is. A slot is rewritten five rows later at the earliest: when
+// rows 0, 2 and 5 of a batch are written the tiles before last have to be done
+// (the previous batch's 1 and 2, this one's 0), which leaves a tile two pairs'
+// time. Every wait is bounded; a role whose wait runs out leaves
 // its loop, and the others run into their own limits.
 template <bool kU8>
 __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const ConvArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  __shared__ __align__(8) uint64_t bars[15];
+  __shared__ __align__(8) uint64_t bars[16];
   __shared__ uint32_t tmem_s;
   __shared__ __align__(16) float sb[96];     // b1 | b2
-  __shared__ uint2 nib[16];                  // 4 pixel bits -> 4 bf16 0 / 1 (element k = bit k)
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const uint32_t sbase = smem_u32(sm);
   auto bar = [&](int j) { return smem_u32(&bars[j]); };
   // pairs of barriers, by the parity of the pair / tile
-  constexpr int kBarC1 = 0, kBarBlk = 2, kBarD1f = 4, kBarC2 = 6, kBarD2f = 8, kBarBand = 10, kBarW = 11, kBarFin = 12;
+  constexpr int kBarC1 = 0, kBarBlk = 2, kBarD1f = 4, kBarC2 = 6, kBarD2f = 8, kBarBand = 10, kBarW = 12, kBarFin = 13;
 
   for (int j = t; j < 96; j += kConvThreads) sb[j] = a.fp[j];
-  if (t < 16)  // 1.0 in bf16 is 0x3F80
-    nib[t] = make_uint2((t & 1) * 0x3F80u | ((t >> 1) & 1) * 0x3F800000u,
-                        ((t >> 2) & 1) * 0x3F80u | ((t >> 3) & 1) * 0x3F800000u);
   if (t == 0) {
     for (int j = 0; j < 2; ++j) {
       mbar_init(bar(kBarC1 + j), 1);
@@ -409,9 +433,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
       mbar_init(bar(kBarD1f + j), kDrain1Warps);
       mbar_init(bar(kBarC2 + j), 1);
       mbar_init(bar(kBarD2f + j), kDrain2Warps);
+      mbar_init(bar(kBarBand + j), kDrain1Warps);
     }
-    mbar_init(bar(kBarBand), kDrain1Warps);
-    for (int j = kBarW; j < 15; ++j) mbar_init(bar(j), 1);
+    for (int j = kBarW; j < 16; ++j) mbar_init(bar(j), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -423,7 +447,6 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_s;
-  grid_dependents_launch();  // the next kernel's CTAs may set up where there is room; they wait for this grid's end
   const int64_t n_batches = (a.n + kP - 1) / kP;
   const int my_batches = (int)((n_batches - blockIdx.x + gridDim.x - 1) / gridDim.x);
   const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;  // a warp reads TMEM lane quarter warp & 3
@@ -438,14 +461,12 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
 #pragma unroll
     for (int j = 0; j < 8; ++j) bias[j] = f32x2(sb[16 * half + 2 * j], sb[16 * half + 2 * j + 1]);
     uint8_t *const dst0 = sm + kAct1Off + (ox & 1) * kSubBytes + (ox >> 1) * 512 + ri * 16 + 2 * half * 128;
-    uint32_t P = 0;
+    uint32_t P = 0, slot = 0;
     for (int bi = 0; bi < my_batches && ok; ++bi) {
       for (int pr = 0; pr < 7; ++pr, ++P) {
         ok = mbar_wait(bar(kBarC1 + (P & 1)), (P >> 1) & 1);
-        // the conv2 tile that read the slot this pair's rows go to: the previous
-        // batch's last tile, then tiles 0 and 1
-        if ((pr == 0 && bi > 0) || pr == 4 || pr == 6) {
-          const uint32_t T = 3 * bi + (pr == 0 ? -1 : (pr - 4) >> 1);
+        if (bi > 0 ? pr == 0 || pr == 2 || pr == 5 : pr == 5) {  // the last tile that read the slot
+          const uint32_t T = 3 * bi + (pr == 0 ? -2 : pr == 2 ? -1 : 0);
           ok = ok && mbar_wait(bar(kBarC2 + (T & 1)), (T >> 1) & 1);
         }
         if (!__all_sync(0xFFFFFFFFu, ok)) {
@@ -460,9 +481,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(kBarD1f + (P & 1)));
         if (ox <= 13) {  // conv2 reads x <= 13
-          // grid row pr in slot pr of the band's five, rows 5 and 6 in slots 1 and
-          // 2, row 4 in slots 4 and 0: each tile's three rows are neighbours
-          uint8_t *const dst = dst0 + (pr < 5 ? pr : pr - 4) * 4096;
+          uint8_t *const dst = dst0 + slot * kSlotBytes;
+          const bool twice = slot == kBandSlots - 1 && pr < 6;
 #pragma unroll
           for (int s2 = 0; s2 < 2; ++s2)
 #pragma unroll
@@ -470,22 +490,24 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
               const uint4 o = relu_chunk(v + 16 * s2 + 8 * c, bias + 4 * c);
               uint8_t *const q = dst + 2 * s2 * kSubBytes + c * 128;
               *reinterpret_cast<uint4 *>(q) = o;
-              if (pr == 4) *reinterpret_cast<uint4 *>(q - 4 * 4096) = o;
+              if (twice) *reinterpret_cast<uint4 *>(q - (kBandSlots - 1) * kSlotBytes) = o;
             }
         }
+        slot = next_slot(slot, pr);
         if (pr == 2 || pr == 4 || pr == 6) {  // three rows of a tile are there
           fence_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(bar(kBarBand));
+          if (lane == 0) mbar_arrive(bar(kBarBand + ((3 * bi + (pr >> 1) - 1) & 1)));
         }
       }
     }
   } else if (warp < kDrain1Warps + kDrain2Warps) {
-    // ---- conv2 drain: output g (valid for px = g & 7 < 6) adds row g + 1's
-    // second half: by a shuffle, or for g = 3, 11 from the next lane quarter
-    // (rows 4, 12) through the exchange buffer, which each half of the
-    // channels has its own part of
-    const int px = g & 7, qt = warp & 3;
+    // ---- conv2 drain: positions g = px + 7 (row of the tile), outputs at px <
+    // 6, which add position g + 1's second half: by a shuffle, or from the next
+    // lane quarter through the exchange buffer
+    const int px = g % 7, qt = warp & 3;
+    const bool valid = px < 6 && g < 14;
+    float *const xb = reinterpret_cast<float *>(sm + kXbOff) + (lane & 7) * kXbPitch;
     uint32_t T = 0;
     for (int bi = 0; bi < my_batches && ok; ++bi) {
       const int64_t batch = blockIdx.x + (int64_t)bi * gridDim.x;
@@ -493,10 +515,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
         ok = all_ok<kDrain2Warps * 32>(1, mbar_wait(bar(kBarC2 + (T & 1)), (T >> 1) & 1));
         if (!ok) break;
         tc_fence_after();
-        uint8_t *const dst = a.act2 + batch * (int64_t)kAct2Bytes + (px + 6 * (2 * tt + (g >> 3))) * 1024 + ri * 16;
+        uint8_t *const dst = a.act2 + batch * (int64_t)kAct2Bytes + (px + 6 * (2 * tt + g / 7)) * 1024 + ri * 16;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          float *const xb = reinterpret_cast<float *>(sm + kXbOff) + ((qt >> 1) * 2 + h) * 8 * kXbPitch;
           float v[32], w[32];
           const uint32_t d = tmem + lane_base + kD2Col + 128 * (T & 1) + 32 * h;
           tmem_ld32x2(d, d + 64, v, w);
@@ -504,15 +525,16 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kBarD2f + (T & 1)));
+            asm volatile("bar.sync 1, %0;" ::"r"(kDrain2Warps * 32) : "memory");  // the other half's rows were read
           }
-          if ((qt & 1) && lane < 8) xrow_put(xb + lane * kXbPitch, w);
+          if (qt > 0 && lane < 8) xrow_put(xb + (qt - 1) * 8 * kXbPitch, w);
 #pragma unroll
           for (int c = 0; c < 32; ++c) w[c] = __shfl_down_sync(0xFFFFFFFFu, w[c], 8);
           asm volatile("bar.sync 1, %0;" ::"r"(kDrain2Warps * 32) : "memory");
-          if (!(qt & 1) && lane >= 24) xrow_get(xb + (lane - 24) * kXbPitch, w);
+          if (qt < 3 && lane >= 24) xrow_get(xb + qt * 8 * kXbPitch, w);
 #pragma unroll
           for (int c = 0; c < 32; ++c) v[c] += w[c];
-          if (px < 6) {
+          if (valid) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
               const ulonglong2 *const b2 = reinterpret_cast<const ulonglong2 *>(sb + 32 + 32 * h + 8 * c);
@@ -571,15 +593,25 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
         pf[2 * c + y] = (uint64_t)bits[0] | (uint64_t)bits[1] << 32;
       }
     };
-    auto build_row = [&](int row, int slot) {  // block row: pixel rows 2 row, 2 row + 1; this warp's 4 of 16 positions
-      const uint32_t u0 = (uint32_t)(fr[2 * row * 32 + lane] >> (16 * bw));
-      const uint32_t u1 = (uint32_t)(fr[(2 * row + 1) * 32 + lane] >> (16 * bw));
+    // block row: pixel rows 2 row, 2 row + 1; this warp's 4 of 16 positions
+    auto expand_row = [&](int row, uint4(&o)[4]) {
+      // 16 pixels of either pixel row: the even ones stay, the odd ones move up
+      // to bit 16 and on, so a mask and a product give two bf16 (1.0 is 0x3F80)
+      const uint16_t *const px = reinterpret_cast<const uint16_t *>(fr + 2 * row * 32 + lane) + bw;
+      const uint32_t u0 = px[0], u1 = px[4 * 32];
+      const uint32_t s0 = (u0 & 0x5555u) | (u0 & 0xAAAAu) << 15, s1 = (u1 & 0x5555u) | (u1 & 0xAAAAu) << 15;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const uint2 lo = nib[(u0 >> (4 * j)) & 15u], hi = nib[(u1 >> (4 * j)) & 15u];
-        *reinterpret_cast<uint4 *>(blk + (16 * slot + j) * 512) = make_uint4(lo.x, lo.y, hi.x, hi.y);
+        const uint32_t e0 = s0 >> (8 * (j >> 1)), e1 = s1 >> (8 * (j >> 1));
+        const uint32_t m = 0x00010001u << (4 * (j & 1)), one = 0x3F80u >> (4 * (j & 1));
+        o[j] = make_uint4((e0 & m) * one, (e0 & (m << 2)) * (one >> 2), (e1 & m) * one, (e1 & (m << 2)) * (one >> 2));
       }
     };
+    auto put_row = [&](int row, const uint4(&o)[4]) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) *reinterpret_cast<uint4 *>(blk + (16 * (row % (int)kBlkRows) + j) * 512) = o[j];
+    };
+    grid_dependency_wait();  // the observations
     if (kU8) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
@@ -597,21 +629,30 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
 #pragma unroll
       for (int k = 0; k < 8; ++k) fr[((2 * y2 + (k & 1)) * 4 + (k >> 1)) * 8 + fi] = pf[k];
       asm volatile("bar.sync 2, %0;" ::"r"(kBuildWarps * 32) : "memory");
-      if (!kU8) load_words(next);
 #pragma unroll
       for (int pr = 0; pr < 7; ++pr, ++P) {
         // rows 2 pr + 1 and 2 pr + 2 take the places of rows that pair P - 2 read
         // last, a batch's rows 0 .. 2 those of the previous batch's last two pairs
+        // (the pixels are expanded before the wait: what follows it delays the
+        // pair's MMAs, and with them the pair after next)
+        uint4 o0[4], o1[4], o2[4];
+        if (pr == 0) expand_row(0, o0);
+        expand_row(2 * pr + 1, o1);
+        expand_row(2 * pr + 2, o2);
         if (ok && P >= 2) ok = mbar_wait(bar(kBarC1 + (P & 1)), ((P - 2) >> 1) & 1);
         if (pr == 0) {
+          put_row(0, o0);
+          put_row(1, o1);
           if (ok && P >= 1) ok = mbar_wait(bar(kBarC1 + ((P - 1) & 1)), ((P - 1) >> 1) & 1);
-          build_row(0, 0);
+        } else {
+          put_row(2 * pr + 1, o1);
         }
-        build_row(2 * pr + 1, (2 * pr + 1) % kBlkRows);
-        build_row(2 * pr + 2, (2 * pr + 2) % kBlkRows);
+        put_row(2 * pr + 2, o2);
         fence_async_smem();
         ok = __all_sync(0xFFFFFFFFu, ok);
         if (ok && lane == 0) mbar_arrive(bar(kBarBlk + (P & 1)));
+        // (not before the first pair's fence, which would wait for them)
+        if (!kU8 && pr == 1) load_words(next);
         if (kU8) {
           if (pr == 2) pack_bytes(0);
           if (pr == 4) pack_bytes(1);
@@ -623,24 +664,30 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
         }
       }
       if (kU8) pack_bytes(3);
+      // what is left is two pairs and a tile: about the time the next kernel's
+      // set-up takes (earlier, its waiting CTAs would keep the SMs from other streams)
+      if (bi + 1 == my_batches) grid_dependents_launch();
     }
-  } else if (lane == 0) {
-    // ---- issuing threads (one per warp)
-    const int who = warp - kIssueWarp;  // 0, 1: conv1 pairs of that parity; 2: conv2
-    if (who == 0) {
+  } else {
+    // ---- issuing warps: whole warps in step, one lane of which issues
+    const int who = __shfl_sync(0xFFFFFFFFu, warp - kIssueWarp, 0);  // 0, 1: conv1 pairs of that parity; 2: conv2
+    if (who == 0 && lane == 0) {
       mbar_expect_tx(bar(kBarW), kW1Bytes + kW2Bytes);
       bulk_g2s(sbase + kW1Off, a.w1, kW1Bytes, bar(kBarW));
       for (uint32_t o = 0; o < kW2Bytes; o += 16384) bulk_g2s(sbase + kW2Off + o, a.w2 + o, 16384, bar(kBarW));
     }
-    ok = mbar_wait(bar(kBarW), 0);
+    __syncwarp();
+    const uint32_t tm = __shfl_sync(0xFFFFFFFFu, tmem, 0);
+    ok = __all_sync(0xFFFFFFFFu, mbar_wait(bar(kBarW), 0));
     if (who < 2) {
       // Both output rows of a pair in one N = 64 accumulator: block row j (shift
       // dx) feeds row 2p through tap (dx, dy = j) and row 2p + 1 through tap (dx,
       // dy = j - 1); W1 holds, per (j, dx), those two taps stacked over n (zeros
-      // where a tap does not apply), so each MMA reads its A tile once for 64
-      // outputs.
+      // where a tap does not apply), so the MMAs of j = 1 read their A tile once
+      // for 64 outputs. Those of j = 0 and 2 take the half that is not zero,
+      // but for the first, which also clears row 2p + 1.
       const uint64_t a1d = sdesc(sbase + kBlkOff, 128, 512), b1d = sdesc(sbase + kW1Off, 1024, 128);
-      const uint32_t d = tmem + kD1Col + 64 * who;
+      const uint32_t d = tm + kD1Col + 64 * who;
       uint32_t pr = who;
       const uint32_t pairs = 7 * (uint32_t)my_batches;
       for (uint32_t P = who; P < pairs && ok; P += 2) {
@@ -651,7 +698,8 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
           ad[j] = sdesc_at(a1d, slot * 16 * 512);
           slot = slot + 1 == kBlkRows ? 0 : slot + 1;
         }
-        ok = (P < 2 || mbar_wait(bar(kBarD1f + who), ((P >> 1) - 1) & 1)) && mbar_wait(bar(kBarBlk + who), (P >> 1) & 1);
+        ok = __all_sync(0xFFFFFFFFu, (P < 2 || mbar_wait(bar(kBarD1f + who), ((P >> 1) - 1) & 1)) &&
+                                         mbar_wait(bar(kBarBlk + who), (P >> 1) & 1));
         if (!ok) break;
         tc_fence_after();
 #pragma unroll
@@ -660,38 +708,50 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
           for (int dx = 0; dx < 2; ++dx)
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              mma_bf16(d, sdesc_at(ad[j], dx * 512 + kk * 256), sdesc_at(b1d, (2 * j + dx) * 4096 + kk * 2048),
-                       idesc_bf16(128, 64), (j | dx | kk) != 0);
-        if (!(a.stall && P == 0)) mma_commit(bar(kBarC1 + who));
+              mma_bf16_warp(d + (j == 2 ? 32 : 0), sdesc_at(ad[j], dx * 512 + kk * 256),
+                       sdesc_at(b1d, (2 * j + dx) * 4096 + kk * 2048 + (j == 2 ? 32 * 16 : 0)),
+                       idesc_bf16(128, j == 1 || (j | dx | kk) == 0 ? 64 : 32), (j | dx | kk) != 0);
+        if (!(a.stall && P == 0)) mma_commit_warp(bar(kBarC1 + who));
         pr = pr >= 5 ? pr - 5 : pr + 2;
       }
     } else {
       const uint64_t a2d = sdesc(sbase + kAct1Off, 128, 512), b2d = sdesc(sbase + kW2Off, 2048, 128);
       const uint32_t tiles = 3 * (uint32_t)my_batches;
-      uint32_t tt = 0;
+      int tt = 0;
+      uint32_t slot = 0, s0 = 0, s1 = 0, s2 = 0;  // the next row's, and those of the tile's rows 0 .. 2
       for (uint32_t T = 0; T < tiles && ok; ++T) {
-        ok = (T < 2 || mbar_wait(bar(kBarD2f + (T & 1)), ((T >> 1) - 1) & 1)) && mbar_wait(bar(kBarBand), T & 1);
+        s0 = s2;
+        if (tt == 0) {
+          s0 = slot;
+          slot = next_slot(slot, 0);
+        }
+        s1 = slot;
+        slot = next_slot(slot, 2 * tt + 1);
+        s2 = slot;
+        slot = next_slot(slot, 2 * tt + 2);
+        const uint64_t at[2] = {sdesc_at(a2d, s0 % (kBandSlots - 1) * kSlotBytes), sdesc_at(a2d, s1 % (kBandSlots - 1) * kSlotBytes)};
+        ok = __all_sync(0xFFFFFFFFu, (T < 2 || mbar_wait(bar(kBarD2f + (T & 1)), ((T >> 1) - 1) & 1)) &&
+                                         mbar_wait(bar(kBarBand + (T & 1)), (T >> 1) & 1));
         if (!ok) break;
         tc_fence_after();
-        const uint64_t at = sdesc_at(a2d, tt == 1 ? 2 * 4096 : 0);  // tile 1 from slot 2 on, tiles 0 and 2 from slot 0
-        const uint32_t d = tmem + kD2Col + 128 * (T & 1);
+        const uint32_t d = tm + kD2Col + 128 * (T & 1);
 #pragma unroll
         for (int ky = 0; ky < 4; ++ky)
 #pragma unroll
           for (int px = 0; px < 2; ++px)  // taps (px, ky) and (px + 2, ky)
 #pragma unroll
             for (int kk = 0; kk < 2; ++kk)
-              mma_bf16(d, sdesc_at(at, (px + 2 * (ky & 1)) * kSubBytes + (ky >> 1) * 4096 + kk * 256),
+              mma_bf16_warp(d, sdesc_at(at[ky >> 1], (px + 2 * (ky & 1)) * kSubBytes + kk * 256),
                        sdesc_at(b2d, (ky * 2 + px) * 8192 + kk * 4096), idesc_bf16(128, 128), (ky | px | kk) != 0);
-        mma_commit(bar(kBarC2 + (T & 1)));
+        mma_commit_warp(bar(kBarC2 + (T & 1)));
         tt = tt == 2 ? 0 : tt + 1;
       }
     }
   }
   ok = !__syncthreads_or(!ok);
   if (!ok && t == 0) atomicOr(a.err, 1u);
-  if (!ok && warp >= kIssueWarp && lane == 0) {  // let this thread's MMAs and copies land
-    mma_commit(bar(kBarFin + warp - kIssueWarp));
+  if (!ok && warp >= kIssueWarp) {  // let this warp's MMAs and copies land
+    mma_commit_warp(bar(kBarFin + warp - kIssueWarp));
     mbar_wait(bar(kBarFin + warp - kIssueWarp), 0);
     if (warp == kIssueWarp) mbar_wait(bar(kBarW), 0);
   }
@@ -711,16 +771,17 @@ struct Conv3Args {
 };
 
 // conv3 of batches blockIdx.x, blockIdx.x + gridDim.x, ...: the M tile is the
-// 4 x 4 output positions of 8 instances exactly. Tap (kx, ky) reads input
+// 4 x 4 output positions of 8 instances exactly. Even and odd batches have
+// three stages, an accumulator buffer, a copying and an issuing thread each. Tap (kx, ky) reads input
 // positions (qx + kx, qy + ky): the ring's stages hold, for one kx, columns
 // kx .. kx + 3 of the six rows (24 positions; each row is one bulk copy of 4
 // KB), and ky shifts the start by one row of them.
 __global__ void __launch_bounds__(kConv3Threads, 1) policy_conv3_kernel(const Conv3Args a) {
   extern __shared__ __align__(1024) uint8_t sm[];
-  __shared__ __align__(8) uint64_t full[kStages3], empty[kStages3], done[2], freed[2], bar_w, fin;
+  __shared__ __align__(8) uint64_t full[kStages3], empty[kStages3], done[2], freed[2], bar_w, fin[2];
   __shared__ uint32_t tmem_s;
   __shared__ __align__(16) float sb[64];
-  __shared__ int s_issued, s_landed;  // stages whose copies were issued / waited for
+  __shared__ int s_issued[2], s_landed[2];  // stages whose copies were issued / waited for, even and odd batches
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const uint32_t sbase = smem_u32(sm);
   if (t < 64) sb[t] = a.fp[FpLayout::b3 + t];
@@ -732,10 +793,10 @@ __global__ void __launch_bounds__(kConv3Threads, 1) policy_conv3_kernel(const Co
     for (int j = 0; j < 2; ++j) {
       mbar_init(smem_u32(&done[j]), 1);
       mbar_init(smem_u32(&freed[j]), kDrain3Warps);
+      mbar_init(smem_u32(&fin[j]), 1);
+      s_issued[j] = s_landed[j] = 0;
     }
     mbar_init(smem_u32(&bar_w), 1);
-    mbar_init(smem_u32(&fin), 1);
-    s_issued = s_landed = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
@@ -747,7 +808,6 @@ __global__ void __launch_bounds__(kConv3Threads, 1) policy_conv3_kernel(const Co
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = tmem_s;
-  grid_dependents_launch();
   const int64_t n_batches = (a.n + kP - 1) / kP;
   const int my_batches = (int)((n_batches - blockIdx.x + gridDim.x - 1) / gridDim.x);
   bool ok = true;
@@ -780,70 +840,67 @@ __global__ void __launch_bounds__(kConv3Threads, 1) policy_conv3_kernel(const Co
         }
       }
     }
-  } else if (t == kDrain3Warps * 32) {  // copies
-    mbar_expect_tx(smem_u32(&bar_w), kW3Bytes);
-    for (uint32_t o = 0; o < kW3Bytes; o += 24576) bulk_g2s(sbase + o, a.w3 + o, 24576, smem_u32(&bar_w));
+  } else if (lane == 0 && warp < kDrain3Warps + 2) {  // copies of this thread's batches: even or odd
+    const int who = warp - kDrain3Warps;
+    if (who == 0) {
+      mbar_expect_tx(smem_u32(&bar_w), kW3Bytes);
+      for (uint32_t o = 0; o < kW3Bytes; o += 24576) bulk_g2s(sbase + o, a.w3 + o, 24576, smem_u32(&bar_w));
+    }
     grid_dependency_wait();  // conv2's output
-    const int total = 3 * my_batches;
-    int kx = 0, st = 0, use = 0, issued = 0;
-    const uint8_t *src = a.act2 + (int64_t)blockIdx.x * kAct2Bytes;
-    for (int q = 0; q < total; ++q) {
-      if (use > 0) ok = mbar_wait(smem_u32(&empty[st]), (use - 1) & 1);  // the stage's previous MMAs are done
-      if (!ok) break;
-      const uint32_t f = smem_u32(&full[st]), dst = sbase + kW3Bytes + st * kStage3Bytes;
-      mbar_expect_tx(f, kStage3Bytes);
+    int issued = 0;
+    for (int bi = who; bi < my_batches && ok; bi += 2) {
+      const uint8_t *const src = a.act2 + (blockIdx.x + (int64_t)bi * gridDim.x) * kAct2Bytes;
+      for (int kx = 0; kx < 3; ++kx) {
+        const int st = 3 * who + kx;
+        if (bi >= 2) ok = mbar_wait(smem_u32(&empty[st]), ((bi >> 1) - 1) & 1);  // the stage's previous MMAs are done
+        if (!ok) break;
+        const uint32_t f = smem_u32(&full[st]), dst = sbase + kW3Bytes + st * kStage3Bytes;
+        mbar_expect_tx(f, kStage3Bytes);
 #pragma unroll
-      for (int py = 0; py < 6; ++py) bulk_g2s(dst + py * 4096, src + (kx + 6 * py) * 1024, 4096, f);
-      issued = q + 1;
-      if (++kx == 3) {
-        kx = 0;
-        src += (int64_t)gridDim.x * kAct2Bytes;
-      }
-      if (++st == kStages3) {
-        st = 0;
-        ++use;
+        for (int py = 0; py < 6; ++py) bulk_g2s(dst + py * 4096, src + (kx + 6 * py) * 1024, 4096, f);
+        ++issued;
       }
     }
-    s_issued = issued;
-  } else if (t == kDrain3Warps * 32 + 32) {  // MMAs
-    const uint64_t a3d = sdesc(sbase + kW3Bytes, 128, 1024), b3d = sdesc(sbase, 3072, 128);
+    grid_dependents_launch();
+    s_issued[who] = issued;
+  } else if (lane == 0) {  // MMAs of this thread's batches
+    const int who = warp - kDrain3Warps - 2;
+    const uint64_t a3d = sdesc(sbase + kW3Bytes + 3 * who * kStage3Bytes, 128, 1024), b3d = sdesc(sbase, 3072, 128);
     ok = mbar_wait(smem_u32(&bar_w), 0);
-    int st = 0, use = 0, landed = 0;
-    for (int bi = 0; bi < my_batches && ok; ++bi) {
-      if (bi >= 2) ok = mbar_wait(smem_u32(&freed[bi & 1]), ((bi >> 1) - 1) & 1);
+    int landed = 0;
+    for (int bi = who; bi < my_batches && ok; bi += 2) {
+      if (bi >= 2) ok = mbar_wait(smem_u32(&freed[who]), ((bi >> 1) - 1) & 1);
       for (int kx = 0; kx < 3 && ok; ++kx) {
-        ok = mbar_wait(smem_u32(&full[st]), use & 1);
+        ok = mbar_wait(smem_u32(&full[3 * who + kx]), (bi >> 1) & 1);
         if (!ok) break;
         ++landed;
         tc_fence_after();
-        const uint64_t at = sdesc_at(a3d, st * kStage3Bytes), bt = sdesc_at(b3d, kx * 1024);
-        const uint32_t d = tmem + 256 * (bi & 1) + 64 * kx;  // an accumulator per kx, summed by the drain
+        const uint64_t at = sdesc_at(a3d, kx * kStage3Bytes), bt = sdesc_at(b3d, kx * 1024);
+        const uint32_t d = tmem + 256 * who + 64 * kx;  // an accumulator per kx, summed by the drain
 #pragma unroll
         for (int ky = 0; ky < 3; ++ky)
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
             mma_bf16(d, sdesc_at(at, ky * 4096 + kk * 256), sdesc_at(bt, ky * 24576 + kk * 6144), idesc_bf16(128, 64),
                      (ky | kk) != 0);
-        mma_commit(smem_u32(&empty[st]));
-        if (++st == kStages3) {
-          st = 0;
-          ++use;
-        }
+        mma_commit(smem_u32(&empty[3 * who + kx]));
       }
-      if (ok) mma_commit(smem_u32(&done[bi & 1]));
+      if (ok) mma_commit(smem_u32(&done[who]));
     }
-    s_landed = landed;
+    s_landed[who] = landed;
   }
   ok = !__syncthreads_or(!ok);
   if (!ok && t == 0) {
     atomicOr(a.err, 1u);
     // copies issued but never waited for land before shared memory goes
     mbar_wait(smem_u32(&bar_w), 0);
-    for (int q = s_landed; q < s_issued; ++q) mbar_wait(smem_u32(&full[q % kStages3]), (q / kStages3) & 1);
+    for (int who = 0; who < 2; ++who)
+      for (int q = s_landed[who]; q < s_issued[who]; ++q)
+        mbar_wait(smem_u32(&full[3 * who + q % 3]), (q / 3) & 1);
   }
-  if (!ok && t == kDrain3Warps * 32 + 32) {  // let this thread's MMAs land before TMEM goes
-    mma_commit(smem_u32(&fin));
-    mbar_wait(smem_u32(&fin), 0);
+  if (!ok && warp >= kDrain3Warps + 2 && lane == 0) {  // let this thread's MMAs land before TMEM goes
+    mma_commit(smem_u32(&fin[warp - kDrain3Warps - 2]));
+    mbar_wait(smem_u32(&fin[warp - kDrain3Warps - 2]), 0);
   }
   tc_fence_before();
   __syncthreads();
@@ -864,27 +921,25 @@ struct HeadsArgs {
   unsigned int *err;
 };
 
-// blockIdx.x: 128-instance tile; blockIdx.y: 0 actor, 1 critic.
-__global__ void __launch_bounds__(kThreads, 1) policy_heads_kernel(const HeadsArgs a) {
+// MT tiles of 128 instances by a head's 256 hidden units per CTA; blockIdx.y: 0
+// actor, 1 critic. K = 1024 comes in slices of 64 through a ring of stages (one
+// thread issues the copies, another the MMAs).
+template <int MT>
+__global__ void __launch_bounds__(256 * MT, 1) policy_heads_kernel(const HeadsArgs a) {
+  constexpr uint32_t kStage = MT * kHA + kHB, kCols = MT * 256;
+  constexpr int kStages = kHeadRing / kStage, kSlices = 16, kThreads = 256 * MT;
   extern __shared__ __align__(1024) uint8_t sm[];
-  __shared__ __align__(8) uint64_t full[kHeadStages], empty[kHeadStages], fin;
+  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], fin;
   __shared__ uint32_t tmem_s;
+  __shared__ int s_landed;  // slices whose copies the MMA thread has waited for
   const int t = threadIdx.x, warp = t >> 5;
   const int head = blockIdx.y;
-  const int64_t tile = blockIdx.x;
+  const int64_t tile = (int64_t)blockIdx.x * MT;
   const uint32_t sbase = smem_u32(sm);
-  float *wout = reinterpret_cast<float *>(sm + kHeadOutOff);      // actor [L][256] or critic [256]
-  float *bias = wout + (kMaxLogits + 1) * 256;                     // [256] hidden biases, then outputs'
-  if (head == 0) {
-    for (int j = t; j < a.L * 256; j += kThreads) wout[j] = a.fp[FpLayout::wa2 + j];
-    for (int j = t; j < a.L; j += kThreads) bias[256 + j] = a.fp[FpLayout::ba2 + j];
-  } else {
-    for (int j = t; j < 256; j += kThreads) wout[j] = a.fp[FpLayout::wc2 + j];
-    if (t == 0) bias[256] = a.fp[FpLayout::bc2];
-  }
-  for (int j = t; j < 256; j += kThreads) bias[j] = a.fp[FpLayout::bh + 256 * head + j];
+  float *wout = reinterpret_cast<float *>(sm + kHeadRing);        // actor [L][256] or critic [256]
+  float *bias = wout + kMaxLogits * 256;                           // [256] hidden biases, then outputs'
   if (t == 0) {
-    for (int s = 0; s < kHeadStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(smem_u32(&full[s]), 1);
       mbar_init(smem_u32(&empty[s]), 1);
     }
@@ -892,7 +947,8 @@ __global__ void __launch_bounds__(kThreads, 1) policy_heads_kernel(const HeadsAr
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&tmem_s)));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
+                 "r"(kCols));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc_fence_before();
@@ -900,149 +956,160 @@ __global__ void __launch_bounds__(kThreads, 1) policy_heads_kernel(const HeadsAr
   tc_fence_after();
   const uint32_t tmem = tmem_s;
   const uint8_t *A = a.act3 + tile * (int64_t)kAct3TileBytes;
-  const uint8_t *B = a.wh + (int64_t)head * (16 * 8 * 256 * 16);
-  constexpr int kSlices = 32;  // K = 1024 in slices of 32 (4 chunks)
+  const uint8_t *B = a.wh + (int64_t)head * kSlices * kHB;
   bool ok = true;
   // Thread 0 issues the copies, thread 32 the MMAs: each runs its own chain of
   // waits and issues (a bulk copy or an MMA costs far more latency on the
   // issuing thread than its bytes or its share of the tensor pipe).
-  __shared__ int s_landed;  // slices whose copies the MMA thread has waited for
   int loaded = 0;           // thread 0: slices whose copies were issued
   if (t == 0) {
+    // the first slices' weights need not wait for conv3
+    for (int s = 0; s < kStages && s < kSlices; ++s) {
+      const uint32_t f = smem_u32(&full[s]);
+      mbar_expect_tx(f, kStage);
+      bulk_g2s(sbase + s * kStage + MT * kHA, B + (int64_t)s * kHB, kHB, f);
+    }
     grid_dependency_wait();  // conv3's features
     for (int s = 0; s < kSlices && ok; ++s) {
-      const int st = s % kHeadStages;
-      // stage st last held slice s - kHeadStages: its MMAs must be done
-      if (s >= kHeadStages) ok = mbar_wait(smem_u32(&empty[st]), ((s / kHeadStages) - 1) & 1);
-      if (!ok) break;
+      const int st = s % kStages;
       const uint32_t f = smem_u32(&full[st]);
-      mbar_expect_tx(f, kHA + kHB);
-      bulk_g2s(sbase + st * (kHA + kHB), A + (int64_t)s * kHA, kHA, f);
-      bulk_g2s(sbase + st * (kHA + kHB) + kHA, B + (int64_t)s * kHB, kHB, f);
+      if (s >= kStages) {  // stage st last held slice s - kStages: its MMAs must be done
+        ok = mbar_wait(smem_u32(&empty[st]), ((s / kStages) - 1) & 1);
+        if (!ok) break;
+        mbar_expect_tx(f, kStage);
+        bulk_g2s(sbase + st * kStage + MT * kHA, B + (int64_t)s * kHB, kHB, f);
+      }
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+        bulk_g2s(sbase + st * kStage + m * kHA, A + m * (int64_t)kAct3TileBytes + (int64_t)s * kHA, kHA, f);
       loaded = s + 1;
     }
   } else if (t == 32) {
     int landed = 0;
     for (int s = 0; s < kSlices && ok; ++s) {
-      const int st = s % kHeadStages;
-      ok = mbar_wait(smem_u32(&full[st]), (s / kHeadStages) & 1);
+      const int st = s % kStages;
+      ok = mbar_wait(smem_u32(&full[st]), (s / kStages) & 1);
       if (!ok) break;
       landed = s + 1;
       tc_fence_after();
-      const uint32_t a0 = sbase + st * (kHA + kHB), b0 = a0 + kHA;
-      for (int kk = 0; kk < 2; ++kk)
-        mma_bf16(tmem, sdesc(a0 + kk * 2 * 2048, 2048, 128), sdesc(b0 + kk * 2 * 4096, 4096, 128),
-                 idesc_bf16(128, 256), (s | kk) != 0);
+      const uint64_t a0 = sdesc(sbase + st * kStage, 2048, 128);
+      const uint64_t b0 = sdesc(sbase + st * kStage + MT * kHA, 256 * 16, 128);
+#pragma unroll
+      for (int m = 0; m < MT; ++m)
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk)
+          mma_bf16(tmem + m * 256, sdesc_at(a0, m * kHA + kk * 2 * 2048), sdesc_at(b0, kk * 2 * 256 * 16),
+                   idesc_bf16(128, 256), (s | kk) != 0);
       mma_commit(smem_u32(&empty[st]));
     }
     // the last slice's MMAs complete -> every earlier one has too
-    if (ok) ok = mbar_wait(smem_u32(&empty[(kSlices - 1) % kHeadStages]), ((kSlices - 1) / kHeadStages) & 1);
+    if (ok) ok = mbar_wait(smem_u32(&empty[(kSlices - 1) % kStages]), ((kSlices - 1) / kStages) & 1);
     if (!ok) {  // let this thread's MMAs land before TMEM goes
       mma_commit(smem_u32(&fin));
       mbar_wait(smem_u32(&fin), 0);
     }
     s_landed = landed;
+  } else if (warp >= 2) {  // meanwhile the output layers
+    const int outs = head == 0 ? a.L : 1;
+    const float *const w = a.fp + (head == 0 ? FpLayout::wa2 : FpLayout::wc2);
+    const float *const b = a.fp + (head == 0 ? FpLayout::ba2 : FpLayout::bc2);
+    for (int j = t - 64; j < outs * 256; j += kThreads - 64) wout[j] = w[j];
+    for (int j = t - 64; j < 256; j += kThreads - 64) bias[j] = a.fp[FpLayout::bh + 256 * head + j];
+    for (int j = t - 64; j < outs; j += kThreads - 64) bias[256 + j] = b[j];
   }
   ok = !__syncthreads_or(!ok);
   if (!ok && t == 0)  // copies issued but never waited for land before shared memory goes
-    for (int q = s_landed; q < loaded; ++q) mbar_wait(smem_u32(&full[q % kHeadStages]), (q / kHeadStages) & 1);
+    for (int q = s_landed; q < loaded; ++q) mbar_wait(smem_u32(&full[q % kStages]), (q / kStages) & 1);
   tc_fence_after();
-  // warps w and w + 4 read TMEM lane quarter w & 3 (instance t & 127), each
-  // one half of the 256 hidden units; warps 4-7 hand their partial outputs
-  // over through shared memory
-  const int row = t & 127, hh = warp >> 2;
-  const int64_t inst = tile * 128 + row;
-  float *part = reinterpret_cast<float *>(sm + kHeadPartOff) + row * (kMaxLogits + 1);
-  float acc[kMaxLogits];
-#pragma unroll
-  for (int j = 0; j < kMaxLogits; ++j) acc[j] = 0.0f;
+  // A TMEM lane quarter (warp & 3) and half of the hidden units per warp;
+  // the products of 32 hidden units with an output's weights meet in the stages'
+  // shared memory, [tile][32 units][output][row]. Loops stay rolled: every
+  // instruction here runs a few times only, so fetching it is what it costs
+  // (unrolled over the outputs this took 10 K cycles of a tile pair's 33 K).
+  const int row = t & 127, hh = (warp >> 2) & 1, m = warp >> 3;
+  const int64_t inst = (tile + m) * 128 + row;
+  const int outs = head == 0 ? a.L : 1;
+  float *const sums = reinterpret_cast<float *>(sm) + m * (8 * kMaxLogits * 128) + row;
   if (ok) {
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    // one output's dot product over 32 hidden units: the weights as 8 vector
-    // loads, four independent partial sums
-    auto dot32 = [&](const float(&h)[32], const float *w) -> float {
-      const float4 *w4 = reinterpret_cast<const float4 *>(w);
-      float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
+#pragma unroll 1
+    for (int c = 0; c < 4; ++c) {
+      const int unit = 128 * hh + 32 * c;
+      float h[32];
+      tmem_ld32(tmem + lane_base + m * 256 + unit, h);
+      const float4 *const b4 = reinterpret_cast<const float4 *>(bias + unit);
 #pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const float4 ww = w4[q];
-        s0 = fmaf(h[4 * q], ww.x, s0);
-        s1 = fmaf(h[4 * q + 1], ww.y, s1);
-        s2 = fmaf(h[4 * q + 2], ww.z, s2);
-        s3 = fmaf(h[4 * q + 3], ww.w, s3);
+      for (int j = 0; j < 8; ++j) {
+        const float4 b = b4[j];
+        h[4 * j] = fmaxf(h[4 * j] + b.x, 0.0f);
+        h[4 * j + 1] = fmaxf(h[4 * j + 1] + b.y, 0.0f);
+        h[4 * j + 2] = fmaxf(h[4 * j + 2] + b.z, 0.0f);
+        h[4 * j + 3] = fmaxf(h[4 * j + 3] + b.w, 0.0f);
       }
-      return (s0 + s1) + (s2 + s3);
-    };
-    auto chunk = [&](float(&h)[32], int c0) {
+#pragma unroll 1
+      for (int o = 0; o < outs; ++o) {  // the weights as 8 vector loads, four independent partial sums
+        const float4 *const w4 = reinterpret_cast<const float4 *>(wout + o * 256 + unit);
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, s3 = 0.0f;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) h[j] = fmaxf(h[j] + bias[c0 + j], 0.0f);
-      if (head == 0) {
-#pragma unroll
-        for (int o = 0; o < kMaxLogits; ++o)
-          if (o < a.L) acc[o] += dot32(h, wout + o * 256 + c0);
-      } else {
-        acc[0] += dot32(h, wout + c0);
+        for (int q = 0; q < 8; ++q) {
+          const float4 ww = w4[q];
+          s0 = fmaf(h[4 * q], ww.x, s0);
+          s1 = fmaf(h[4 * q + 1], ww.y, s1);
+          s2 = fmaf(h[4 * q + 2], ww.z, s2);
+          s3 = fmaf(h[4 * q + 3], ww.w, s3);
+        }
+        sums[((unit >> 5) * kMaxLogits + o) * 128] = (s0 + s1) + (s2 + s3);
       }
-    };
-    for (int c0 = 128 * hh; c0 < 128 * hh + 128; c0 += 64) {  // two 32-column TMEM loads behind one wait
-      float v[32], w[32];
-      tmem_ld32x2(tmem + lane_base + c0, tmem + lane_base + c0 + 32, v, w);
-      chunk(v, c0);
-      chunk(w, c0 + 32);
-    }
-    if (hh) {
-#pragma unroll
-      for (int o = 0; o < kMaxLogits; ++o) part[o] = acc[o];
     }
   }
   __syncthreads();
-  if (ok && !hh) {
+  if (ok && !hh && inst < a.n) {
+    float top = -INFINITY;
+#pragma unroll 1
+    for (int o = 0; o < outs; ++o) {
+      float lo = 0.0f, hi = 0.0f;
 #pragma unroll
-    for (int o = 0; o < kMaxLogits; ++o) acc[o] += part[o];
-    if (inst < a.n) {
-      if (head == 0) {
-        float m = -INFINITY;
-#pragma unroll
-        for (int o = 0; o < kMaxLogits; ++o)
-          if (o < a.L) {
-            acc[o] += bias[256 + o];
-            m = fmaxf(m, acc[o]);
-            if (a.logits) a.logits[inst * a.L + o] = acc[o];
-          }
-        if (a.actions) {
-          // inverse CDF: the first index whose cumulative weight exceeds u * total
-          const uint32_t w = philox_w0((uint32_t)inst, a.step, 0u, 0u, a.key0, a.key1);
-          const float u = (float)(w >> 8) * 5.9604644775390625e-08f;  // 2^-24
-          float e[kMaxLogits], tot = 0.0f;
-#pragma unroll
-          for (int o = 0; o < kMaxLogits; ++o) {
-            e[o] = o < a.L ? expf(acc[o] - m) : 0.0f;
-            tot += e[o];
-          }
-          const float target = u * tot;
-          float run = 0.0f;
-          int pick = a.L - 1;
-          bool found = false;
-#pragma unroll
-          for (int o = 0; o < kMaxLogits; ++o) {
-            run += e[o];
-            if (o < a.L && !found && target < run) {
-              pick = o;
-              found = true;
-            }
-          }
-          a.actions[inst] = (uint8_t)pick;
-        }
-      } else if (a.value) {
-        a.value[inst] = acc[0] + bias[256];
+      for (int c = 0; c < 4; ++c) {
+        lo += sums[(c * kMaxLogits + o) * 128];
+        hi += sums[((4 + c) * kMaxLogits + o) * 128];
       }
+      lo += hi;
+      lo += bias[256 + o];
+      top = fmaxf(top, lo);
+      sums[o * 128] = lo;  // (this thread's own)
+      if (head == 0) {
+        if (a.logits) a.logits[inst * a.L + o] = lo;
+      } else if (a.value) {
+        a.value[inst] = lo;
+      }
+    }
+    if (head == 0 && a.actions) {
+      // inverse CDF: the first index whose cumulative weight exceeds u * total
+      const uint32_t w = philox_w0((uint32_t)inst, a.step, 0u, 0u, a.key0, a.key1);
+      const float u = (float)(w >> 8) * 5.9604644775390625e-08f;  // 2^-24
+      float tot = 0.0f, run = 0.0f;
+#pragma unroll 1
+      for (int o = 0; o < outs; ++o) {
+        const float e = expf(sums[o * 128] - top);
+        sums[o * 128] = e;
+        tot += e;
+      }
+      const float target = u * tot;
+      int pick = 0;
+#pragma unroll 1
+      for (; pick < outs - 1; ++pick) {
+        run += sums[pick * 128];
+        if (target < run) break;
+      }
+      a.actions[inst] = (uint8_t)pick;
     }
   }
   if (!ok && t == 0) atomicOr(a.err, 1u);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols));
 }
 
 // ---- host: weight packing ----------------------------------------------------
@@ -1053,22 +1120,10 @@ uint16_t bf16_bits(float f) {
   return b;
 }
 
-// dependent: the kernel may be set up before the one ahead of it in the
-// stream has ended; it waits for that itself (grid_dependency_wait).
 template <class Args>
-cudaError_t launch(void (*kernel)(const Args), dim3 grid, int block, size_t smem, cudaStream_t s, bool dependent,
-                   const Args &args) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = dependent ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args);
+cudaError_t launch(void (*kernel)(const Args), dim3 grid, int block, size_t smem, cudaStream_t s, Args &args) {
+  void *list[] = {&args};
+  return launch_kernel((const void *)kernel, grid, dim3((unsigned)block), list, smem, s, true);
 }
 
 int launch_forward(octax_policy *p, int64_t n, const uint64_t *obs_words, const uint8_t *obs_u8, uint64_t seed,
@@ -1083,12 +1138,17 @@ int launch_forward(octax_policy *p, int64_t n, const uint64_t *obs_words, const 
               (uint32_t)seed, (uint32_t)(seed >> 32), step, p->err};
   const int64_t batches = (n + kP - 1) / kP;
   const unsigned grid = (unsigned)std::min<int64_t>(batches, p->sms);
-  cudaError_t r = obs_u8 ? launch(policy_conv12_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, false, c)
-                         : launch(policy_conv12_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, false, c);
+  cudaError_t r = obs_u8 ? launch(policy_conv12_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, c)
+                         : launch(policy_conv12_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, c);
   if (r != cudaSuccess) return cuda_fail(r, "policy conv launch");
-  r = launch(policy_conv3_kernel, dim3(grid), kConv3Threads, kConv3Smem, s, true, c3);
+  r = launch(policy_conv3_kernel, dim3(grid), kConv3Threads, kConv3Smem, s, c3);
   if (r != cudaSuccess) return cuda_fail(r, "policy conv3 launch");
-  r = launch(policy_heads_kernel, dim3((unsigned)((n + 127) / 128), 2), kThreads, kHeadSmem, s, true, h);
+  // A CTA holds an SM's shared memory, so they run in waves of one per SM: one
+  // tile each as long as that makes one wave, else two (the weights then come
+  // in once for both).
+  const unsigned tiles = (unsigned)((n + 127) / 128);
+  r = 2 * (int64_t)tiles <= p->sms ? launch(policy_heads_kernel<1>, dim3(tiles, 2), 256, kHeadSmem, s, h)
+                                   : launch(policy_heads_kernel<2>, dim3((tiles + 1) / 2, 2), 512, kHeadSmem, s, h);
   if (r != cudaSuccess) return cuda_fail(r, "policy heads launch");
   return OCTAX_OK;
 }
@@ -1188,7 +1248,7 @@ int octax_policy_create(const octax_policy_params *prm, int64_t max_envs, int de
   p->max_envs = max_envs;
   cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, device);
   if (p->sms < 1) p->sms = 1;
-  const int64_t tiles = (max_envs + 127) / 128;
+  const int64_t tiles = (max_envs + 255) / 256 * 2;  // (the heads kernel reads them in pairs)
   auto fail = [&](cudaError_t e, const char *what) {
     octax_policy_destroy(p);
     return cuda_fail(e, what);
@@ -1228,7 +1288,9 @@ int octax_policy_create(const octax_policy_params *prm, int64_t max_envs, int de
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(policy_conv3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kConv3Smem);
   if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(policy_heads_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadSmem);
+    r = cudaFuncSetAttribute(policy_heads_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadSmem);
+  if (r == cudaSuccess)
+    r = cudaFuncSetAttribute(policy_heads_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadSmem);
   if (r != cudaSuccess) return fail(r, "octax_policy_create: upload");
   *out = p;
   return OCTAX_OK;
