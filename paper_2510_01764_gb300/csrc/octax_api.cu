@@ -76,6 +76,8 @@ struct octax_env {
   std::vector<void *> allocs;
   size_t bytes = 0;
   octax_launch cfg{64, 8, 4, 0, 1, 0, 0};
+  octax_launch own_cfg{64, 8, 4, 0, 1, 0, 0};  // launched until a configuration is set or tuned (own_shape)
+  bool cfg_set = false;
   std::map<std::pair<int, int>, GroupTable> groups;  // by (instances per CTA, wave)
   unsigned int *counters_d = nullptr;
   int counters_cap = 0;
@@ -179,6 +181,30 @@ GameDev to_dev(const octax_game &g) {
 int block_ok(int b) { return b == 32 || b == 64 || b == 128 || b == 256; }
 int ipw_ok(int v) { return v >= 1 && v <= 32; }
 int per_cta(const octax_launch &c) { return c.block / 32 * c.inst_per_warp; }
+
+// The shape an environment of n instances runs in when none was set. Few
+// instances per warp keep its lanes on one path (a warp takes the datapath, a
+// sprite and the switch one after the other when its instances are at
+// different instructions); many of them cost fewer warps and fewer
+// instructions. So as few as the instances per SM allow, four warps to a CTA
+// where several share the game's tables. Measured against 64 x 8 x 4 (us, one
+// call after another / three environments in turn on their streams): one step
+// of 64 template instances 14.7 / 6.7 -> 9.1 / 6.4; of 4,096 19.9 / 9.0 ->
+// 16.8 / 8.0; 16 packed steps of 512 shooters 232 / 78 -> 118 / 46, of 2,048
+// 235 / 84 -> 152 / 70, of 30,000 539 / 397 -> 398 / 301; 8 steps of 100,000
+// random programs 1,962 / 1,702 -> 1,635 / 1,134; 8 Super-CHIP steps of 1,024
+// 358 / 121 -> 180 / 71. The lines: 8,192 template instances take 20.8 / 13.2
+// with 4 to a warp and 22.7 / 11.9 with 8; 12,289 shooters 275 / 168 with 8 and
+// 367 / 148 with 16. Launches of 16 steps save three of four state round trips
+// (16 steps of 12,289: 275 -> 249).
+octax_launch own_shape(int64_t n, int sms, int schip) {
+  const int64_t per_sm = (n + sms - 1) / sms;
+  int ipw = per_sm <= 8 ? 1 : per_sm <= 16 ? 2 : per_sm <= 32 ? 4 : 8;
+  if (!schip && per_sm > 128) ipw = 16;
+  return octax_launch{ipw <= 2 ? 64 : 128, ipw, 16, 0, 1, 0, 0};
+}
+
+const octax_launch &shape_of(const octax_env *e) { return e->cfg_set ? e->cfg : e->own_cfg; }
 
 // Resident CTAs of one wave for a balanced launch (0 = not balanced).
 int wave_of(const octax_env *e, const octax_launch &c) {
@@ -334,7 +360,7 @@ StepLaunch base_launch(octax_env *e, const GroupTable *gt) {
   p.n_groups = gt->count;
   p.S = e->S;
   p.quirks = e->quirks;
-  p.ipw = e->cfg.inst_per_warp;
+  p.ipw = shape_of(e).inst_per_warp;
   p.err = e->err_d;
   p.wrappers = uses_wrappers(e->games_h.data(), e->games_h.size());
   p.stall_writers = e->stall_writers;
@@ -555,8 +581,11 @@ int octax_create(const octax_game *games, int n_games, const uint16_t *game_of_e
     free_env(e);
     return rc;
   }
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
+  e->own_cfg = own_shape(n_envs, std::max(sms, 1), e->schip);
   GroupTable *gt = nullptr;
-  int rc = get_groups(e, per_cta(e->cfg), wave_of(e, e->cfg), &gt);
+  int rc = get_groups(e, per_cta(shape_of(e)), wave_of(e, shape_of(e)), &gt);
   if (rc) {
     free_env(e);
     return rc;
@@ -571,12 +600,12 @@ int octax_create(const octax_game *games, int n_games, const uint16_t *game_of_e
   p.n_groups = gt->count;
   p.S = e->S;
   p.quirks = quirks;
-  p.ipw = e->cfg.inst_per_warp;
+  p.ipw = shape_of(e).inst_per_warp;
   p.init = 1;
   p.seed = seed;
   p.row_of_slot = row_tmp;
   p.uid_of_slot = uid_tmp;
-  r = launch_reset(p, e->cfg.block, e->stream);
+  r = launch_reset(p, shape_of(e).block, e->stream);
   if (r == cudaSuccess) r = cudaStreamSynchronize(e->stream);
   if (r != cudaSuccess) {
     rc = cuda_fail(r, "octax_create reset");
@@ -597,7 +626,7 @@ int octax_reset(octax_env *e, const uint8_t *mask_dev, uint8_t *obs_dev) {
     return OCTAX_EINVAL;
   }
   GroupTable *gt = nullptr;
-  int rc = get_groups(e, per_cta(e->cfg), wave_of(e, e->cfg), &gt);
+  int rc = get_groups(e, per_cta(shape_of(e)), wave_of(e, shape_of(e)), &gt);
   if (rc) return rc;
   ResetLaunch p;
   memset(&p, 0, sizeof p);
@@ -611,8 +640,8 @@ int octax_reset(octax_env *e, const uint8_t *mask_dev, uint8_t *obs_dev) {
   p.obs = obs_dev;
   p.S = e->S;
   p.quirks = e->quirks;
-  p.ipw = e->cfg.inst_per_warp;
-  cudaError_t r = launch_reset(p, e->cfg.block, e->stream);
+  p.ipw = shape_of(e).inst_per_warp;
+  cudaError_t r = launch_reset(p, shape_of(e).block, e->stream);
   return r == cudaSuccess ? OCTAX_OK : cuda_fail(r, "octax_reset");
 }
 
@@ -625,7 +654,7 @@ int octax_step(octax_env *e, const uint8_t *actions_dev, uint8_t *obs_dev, float
   int rc = check_io(actions_dev, obs_dev, reward_dev, done_dev);
   if (rc) return rc;
   IO io{actions_dev, obs_dev, reward_dev, done_dev, e->n};
-  octax_launch cfg = e->cfg;
+  octax_launch cfg = shape_of(e);
   cfg.steps_per_launch = 1;
   cfg.use_graph = 0;
   return enqueue_steps(e, cfg, 1, io);
@@ -640,7 +669,7 @@ int octax_step_n(octax_env *e, int n_steps, const uint8_t *actions_dev, uint8_t 
   int rc = check_io(actions_dev, obs_dev, reward_dev, done_dev);
   if (rc) return rc;
   IO io{actions_dev, obs_dev, reward_dev, done_dev, e->n};
-  return enqueue_steps(e, e->cfg, n_steps, io);
+  return enqueue_steps(e, shape_of(e), n_steps, io);
 }
 
 int octax_step_n_packed(octax_env *e, int n_steps, const uint8_t *actions_dev, uint64_t *obs_words_dev,
@@ -653,7 +682,7 @@ int octax_step_n_packed(octax_env *e, int n_steps, const uint8_t *actions_dev, u
   int rc = check_io(actions_dev, obs, reward_dev, done_dev);
   if (rc) return rc;
   IO io{actions_dev, obs, reward_dev, done_dev, e->n, 1, 0};
-  octax_launch cfg = e->cfg;
+  octax_launch cfg = shape_of(e);
   cfg.writer_warps = 0;  // the writer warps write uint8 frames only
   return enqueue_steps(e, cfg, n_steps, io);
 }
@@ -676,7 +705,7 @@ int step_once(octax_env *e, const uint8_t *actions_dev, uint8_t *obs_dev, float 
   int rc = check_io(actions_dev, obs_dev, reward_dev, done_dev);
   if (rc) return rc;
   IO io{actions_dev, obs_dev, reward_dev, done_dev, e->n, packed, 0};
-  octax_launch cfg = e->cfg;
+  octax_launch cfg = shape_of(e);
   cfg.steps_per_launch = 1;
   cfg.use_graph = 0;
   if (packed) cfg.writer_warps = 0;
@@ -850,6 +879,7 @@ int octax_set_launch(octax_env *e, const octax_launch *cfg) {
     return OCTAX_EINVAL;
   }
   e->cfg = *cfg;
+  e->cfg_set = true;
   return OCTAX_OK;
 }
 
@@ -956,10 +986,11 @@ int octax_autotune(octax_env *e, int n_steps, const uint8_t *actions_dev, float 
   // plain kernel, up to 32 steps per launch (long launches rank shapes as
   // they will run)
   for (int b : {32, 64, 128, 256})
-    for (int ipw : {32, 16, 8, 7, 6, 4})
+    for (int ipw : {32, 16, 8, 7, 6, 4, 2, 1})
       for (int bal : {0, 1}) {
         const int J = b / 32 * ipw;
-        if (J >= 8 && J <= 256) trial(octax_launch{b, ipw, std::min(32, n_steps), 0, 1, 0, bal});
+        if (ipw <= 2 && e->own_cfg.inst_per_warp > 4) continue;  // far too many warps
+        if ((J >= 8 || ipw <= 2) && J <= 256) trial(octax_launch{b, ipw, std::min(32, n_steps), 0, 1, 0, bal});
       }
   // stage 2: writer warps, persistence and steps per launch around the best
   // shape. Launches up to 256 steps and the call length itself are
@@ -992,6 +1023,7 @@ int octax_autotune(octax_env *e, int n_steps, const uint8_t *actions_dev, float 
     return cuda_fail(r, "octax_autotune");
   }
   e->cfg = best;
+  e->cfg_set = true;
   if (best_ms_out) *best_ms_out = best_ms;
   return OCTAX_OK;
 }
