@@ -182,25 +182,12 @@ int block_ok(int b) { return b == 32 || b == 64 || b == 128 || b == 256; }
 int ipw_ok(int v) { return v >= 1 && v <= 32; }
 int per_cta(const octax_launch &c) { return c.block / 32 * c.inst_per_warp; }
 
-// The shape an environment of n instances runs in when none was set. Few
-// instances per warp keep its lanes on one path (a warp takes the datapath, a
-// sprite and the switch one after the other when its instances are at
-// different instructions); many of them cost fewer warps and fewer
-// instructions. So as few as the instances per SM allow, four warps to a CTA
-// where several share the game's tables. Measured against 64 x 8 x 4 (us, one
-// call after another / three environments in turn on their streams): one step
-// of 64 template instances 14.7 / 6.7 -> 9.1 / 6.4; of 4,096 19.9 / 9.0 ->
-// 16.8 / 8.0; 16 packed steps of 512 shooters 232 / 78 -> 118 / 46, of 2,048
-// 235 / 84 -> 152 / 70, of 30,000 539 / 397 -> 398 / 301; 8 steps of 100,000
-// random programs 1,962 / 1,702 -> 1,635 / 1,134; 8 Super-CHIP steps of 1,024
-// 358 / 121 -> 180 / 71. The lines: 8,192 template instances take 20.8 / 13.2
-// with 4 to a warp and 22.7 / 11.9 with 8; 12,289 shooters 275 / 168 with 8 and
-// 367 / 148 with 16. Launches of 16 steps save three of four state round trips
-// (16 steps of 12,289: 275 -> 249).
+// The shape an environment of n instances runs in when none was set: four warps
+// to a CTA where several instances a warp share the game's tables, launches of
+// 16 steps (three of four state round trips saved: 16 packed steps of 12,289
+// shooters 275 -> 249 us).
 octax_launch own_shape(int64_t n, int sms, int schip) {
-  const int64_t per_sm = (n + sms - 1) / sms;
-  int ipw = per_sm <= 8 ? 1 : per_sm <= 16 ? 2 : per_sm <= 32 ? 4 : 8;
-  if (!schip && per_sm > 128) ipw = 16;
+  const int ipw = spread_ipw(n, sms, schip);
   return octax_launch{ipw <= 2 ? 64 : 128, ipw, 16, 0, 1, 0, 0};
 }
 
@@ -234,6 +221,26 @@ const char *launch_problem(const octax_launch &c, int schip) {
 }
 
 }  // namespace
+
+// Few instances per warp keep its lanes on one path (a warp takes the datapath,
+// a sprite and the switch one after the other when its instances are at
+// different instructions); many of them cost fewer warps and fewer
+// instructions. So as few as the instances per SM allow. Measured against 64
+// threads x 8 x 4 steps (us, one call after another / three environments in
+// turn on their streams): one step of 64 template instances 14.7 / 6.7 -> 9.1 /
+// 6.4; of 4,096 19.9 / 9.0 -> 16.8 / 8.0; 16 packed steps of 512 shooters 232 /
+// 78 -> 118 / 46, of 2,048 235 / 84 -> 152 / 70, of 30,000 539 / 397 -> 398 /
+// 301; 8 steps of 100,000 random programs 1,962 / 1,702 -> 1,635 / 1,134; 8
+// Super-CHIP steps of 1,024 358 / 121 -> 180 / 71. The lines: 8,192 template
+// instances (54 per SM) take 20.8 / 13.2 with 4 to a warp and 22.7 / 11.9 with
+// 8; 25,000 (164) of 16 ROMs 434 / 342 with 8 and 630 / 305 with 16, 30,000
+// shooters (197) 486 / 394 and 398 / 301; 8,192 Super-CHIP 436 / 307 with 8,
+// 644 / 311 with 16.
+int octax::spread_ipw(int64_t n, int sms, int schip) {
+  const int64_t per_sm = (n + sms - 1) / sms;
+  if (!schip && per_sm > 192) return 16;
+  return per_sm <= 8 ? 1 : per_sm <= 16 ? 2 : per_sm <= 32 ? 4 : 8;
+}
 
 // Validate the descriptors and build the device descriptors + initial RAM images.
 int octax::build_games(const octax_game *games, int n_games, std::vector<GameDev> &dev,

@@ -197,6 +197,9 @@ int table_uops(const octax_game *games, int n_games);
 cudaError_t upload_blobs(const std::vector<GameDev> &games, const std::vector<uint8_t> &images, int n_uops, int schip,
                          uint32_t quirks, uint8_t *blobs, cudaStream_t s);
 
+// Instances per warp for n instances on `sms` SMs.
+int spread_ipw(int64_t n, int sms, int schip);
+
 // Programmatic dependent launch: a kernel launched with `dependent` may be set
 // up before the one ahead of it in the stream has ended. It touches nothing
 // that another kernel may write before its grid_dependency_wait(), which

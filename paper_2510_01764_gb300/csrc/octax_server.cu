@@ -88,6 +88,8 @@ struct TickBuf {
   IO *h_io = nullptr, *d_io = nullptr;
   uint64_t *h_seeds = nullptr, *d_seeds = nullptr;
   Group *h_rgroups = nullptr, *d_rgroups = nullptr;  // reset groups of admissions
+  uint8_t *h_acts = nullptr;                         // their actions
+  size_t cap_acts = 0;
   size_t cap_groups = 0, cap_io = 0;
   cudaEvent_t ev = nullptr;
   bool pending = false;
@@ -103,8 +105,8 @@ struct octax_server {
   int device = 0;
   cudaStream_t stream = nullptr;
   int block = 64;   // threads per CTA
-  int ipw = 8;      // instances per warp
-  int J = 16;       // instances per CTA
+  int ipw = 8;      // instances per warp, at most
+  int sms = 1;
   int depth = 2;
   int n_games = 0, S = 4;
   int schip = 0;  // OCTAX_VARIANT_SCHIP games
@@ -135,7 +137,17 @@ struct octax_server {
 
 namespace {
 
-int grow_tick(octax_server *s, TickBuf &t, size_t groups, size_t ios) {
+int grow_tick(octax_server *s, TickBuf &t, size_t groups, size_t ios, size_t acts) {
+  if (acts > t.cap_acts) {
+    cudaStreamSynchronize(s->stream);  // no copy may still read the old buffer
+    cudaFreeHost(t.h_acts);
+    t.h_acts = nullptr;
+    t.cap_acts = 0;
+    const size_t cap = std::max<size_t>(2 * acts, 1 << 16);
+    const cudaError_t r = cudaMallocHost(&t.h_acts, cap);
+    if (r != cudaSuccess) return cuda_fail(r, "server actions buffer");
+    t.cap_acts = cap;
+  }
   if (groups <= t.cap_groups && ios <= t.cap_io) return OCTAX_OK;
   cudaStreamSynchronize(s->stream);  // no tick may still read the old tables
   const size_t g = std::max(groups, 2 * t.cap_groups) + 64, io = std::max(ios, 2 * t.cap_io) + 16;
@@ -206,11 +218,20 @@ bool tick(octax_server *s) {
   if (run.empty()) return false;
   uint32_t k_steps = kMaxSteps;  // steps of this tick
   for (Req *q : run) k_steps = std::min<uint32_t>(k_steps, q->r.n_steps - q->steps_done);
-  const int B = s->J;  // instances per CTA
-  size_t n_groups = 0, n_rgroups = 0;
+  // A tick of few instances takes fewer per warp than configured (see
+  // spread_ipw): the last ticks of a wave, with 1,600 instances left, took 40
+  // us at 16 to a warp, as long as ones of 19,000.
+  int64_t active = 0;
+  for (Req *q : run) active += q->r.n_envs;
+  const int ipw = std::min(s->ipw, spread_ipw(active, s->sms, s->schip));
+  const int B = s->block / 32 * ipw;  // instances per CTA
+  size_t n_groups = 0, n_rgroups = 0, acts = 0;
   for (Req *q : run) n_groups += (q->r.n_envs + B - 1) / B;
-  for (Req *q : admitted) n_rgroups += (q->r.n_envs + B - 1) / B;
-  if (grow_tick(s, t, std::max(n_groups, n_rgroups), run.size())) {
+  for (Req *q : admitted) {
+    n_rgroups += (q->r.n_envs + B - 1) / B;
+    acts += (size_t)q->r.n_envs * kMaxSteps;
+  }
+  if (grow_tick(s, t, std::max(n_groups, n_rgroups), run.size(), acts)) {
     std::lock_guard<std::mutex> lk(s->mu);
     s->fatal = "server tick: table allocation failed";
     s->stop = true;
@@ -220,16 +241,29 @@ bool tick(octax_server *s) {
   cudaError_t r = cudaSuccess;
   // ---- admissions: actions into the arena, reset the slots
   if (!admitted.empty()) {
-    size_t k = 0;
+    // requests on neighbouring slots share one copy from page-locked memory (a
+    // copy from each request's own pageable memory held this thread ~3 us)
+    size_t k = 0, from = 0, len = 0;  // the run of requests not yet copied: its place in h_acts
+    uint32_t first = 0;               // and its first slot
+    auto flush = [&] {
+      if (len && r == cudaSuccess)
+        r = cudaMemcpyAsync(s->act_arena + (size_t)first * kMaxSteps, t.h_acts + from, len, cudaMemcpyHostToDevice,
+                            s->stream);
+      from += len;
+      len = 0;
+    };
     for (Req *q : admitted) {
-      r = cudaMemcpyAsync(s->act_arena + (size_t)q->slot0 * kMaxSteps, q->actions.data(),
-                          q->actions.size(), cudaMemcpyHostToDevice, s->stream);
+      if (q->slot0 != first + len / kMaxSteps) flush();
+      if (!len) first = q->slot0;
+      memcpy(t.h_acts + from + len, q->actions.data(), q->actions.size());
+      len += (size_t)q->r.n_envs * kMaxSteps;
       for (uint32_t c = 0; c < q->r.n_envs; c += B) {
         t.h_rgroups[k] = Group{q->slot0 + c, (uint16_t)std::min<uint32_t>(B, q->r.n_envs - c), q->r.game, 0u, c};
         t.h_seeds[k] = q->r.seed;
         ++k;
       }
     }
+    flush();
     if (r == cudaSuccess) r = cudaMemcpyAsync(t.d_rgroups, t.h_rgroups, k * sizeof(Group), cudaMemcpyHostToDevice, s->stream);
     if (r == cudaSuccess) r = cudaMemcpyAsync(t.d_seeds, t.h_seeds, k * sizeof(uint64_t), cudaMemcpyHostToDevice, s->stream);
     ResetLaunch p;
@@ -242,7 +276,7 @@ bool tick(octax_server *s) {
     p.n_groups = (int)k;
     p.S = s->S;
     p.quirks = s->quirks;
-    p.ipw = s->ipw;
+    p.ipw = ipw;
     p.init = 1;
     p.seed_of_group = t.d_seeds;
     if (r == cudaSuccess) r = launch_reset(p, s->block, s->stream);
@@ -274,7 +308,7 @@ bool tick(octax_server *s) {
   p.steps = (int)k_steps;
   p.S = s->S;
   p.quirks = s->quirks;
-  p.ipw = s->ipw;
+  p.ipw = ipw;
   p.err = s->err_d;
   p.wrappers = uses_wrappers(s->games_h.data(), s->games_h.size());
   if (r == cudaSuccess) r = launch_step(p, (int)g, s->block, s->stream);
@@ -382,7 +416,8 @@ int octax_server_create(const octax_game *games, int n_games, uint32_t quirks,
   cudaGetDevice(&s->device);
   s->block = B;
   s->ipw = ipw;
-  s->J = B / 32 * ipw;
+  cudaDeviceGetAttribute(&s->sms, cudaDevAttrMultiProcessorCount, s->device);
+  if (s->sms < 1) s->sms = 1;
   s->depth = depth;
   s->n_games = n_games;
   s->S = games[0].stack_frames;
@@ -602,6 +637,7 @@ void octax_server_destroy(octax_server *s) {
     cudaFreeHost(t.h_io);
     cudaFreeHost(t.h_seeds);
     cudaFreeHost(t.h_rgroups);
+    cudaFreeHost(t.h_acts);
     cudaFree(t.d_groups);
     cudaFree(t.d_io);
     cudaFree(t.d_seeds);

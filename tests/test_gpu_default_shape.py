@@ -22,7 +22,7 @@ def _built():
     oracle.build()
 
 
-@pytest.mark.parametrize("per_sm,over", [(0, 1), (0, 5), (8, 0), (8, 1), (16, 0), (16, 1), (32, 0), (32, 1), (128, 0), (128, 1)])
+@pytest.mark.parametrize("per_sm,over", [(0, 1), (0, 5), (8, 0), (8, 1), (16, 0), (16, 1), (32, 0), (32, 1), (192, 0), (192, 1)])
 def test_chip8(per_sm, over):
     n = per_sm * torch.cuda.get_device_properties(0).multi_processor_count + over
     games = [W.replace(g, max_episode_steps=7, sticky_prob=0.25, max_noops=3) for g in W.cfg_shooter().games]
