@@ -79,17 +79,17 @@ int env_device(const octax_env *e);
 namespace {
 
 constexpr int kP = 8;            // instances per conv batch
-// conv1 / conv2 kernel: warps by role; a draining warp reads the TMEM lane quarter warp & 3
+// conv kernel, conv1 and conv2: warps by role; a draining warp reads the TMEM lane quarter warp & 3
 constexpr int kDrain1Warps = 8, kDrain2Warps = 4, kBuildWarps = 4, kIssueWarps = 3;
 constexpr int kIssueWarp = kDrain1Warps + kDrain2Warps + kBuildWarps;  // the first of them
 constexpr int kConvThreads = 32 * (kIssueWarp + kIssueWarps);
-// conv3 kernel: draining warps, then a warp each for the copies and the MMAs of even and of odd batches
-constexpr int kDrain3Warps = 8, kConv3Threads = 32 * (kDrain3Warps + 4);
+// conv3, by the same warps: draining, then a warp each for the copies and the MMAs of even and of odd batches
+constexpr int kDrain3Warps = 8;
 constexpr int kMaxLogits = 17;   // 16 keys + the no-op
 constexpr uint64_t kMaxWaitNs = 1000000000ull;
 constexpr uint32_t kMaxPolls = 1u << 24;
 
-// ---- conv1 / conv2 kernel shared memory (bytes) ------------------------------
+// ---- conv1 / conv2 shared memory (bytes) ------------------------------
 constexpr uint32_t kW1Off = 0;                             // conv1 B: [j 3][dx 2][chunk 4][n 64][8]
 constexpr uint32_t kW1Bytes = 6 * 4 * 64 * 16;
 constexpr uint32_t kW2Off = kW1Off + kW1Bytes;             // conv2 B: [ky 4][kx & 1][chunk 4][n 128][8]
@@ -114,12 +114,11 @@ constexpr uint32_t kAct2Bytes = 36 * 1024;                 // conv2 output of a 
 // TMEM columns (fp32): conv1: 2 buffers x 2 output rows x 32; conv2: 2 buffers x 128
 constexpr uint32_t kD1Col = 0, kD2Col = 128, kConvTmemCols = 512;
 
-// ---- conv3 kernel -------------------------------------------------------------
+// ---- conv3 --------------------------------------------------------------------
 constexpr uint32_t kW3Bytes = 3 * 8 * 192 * 16;            // conv3 B: [ky 3][chunk 8][n = 64 kx + o][8]
 constexpr int kStages3 = 6;                                // ring of one kx each: 6 rows x 4 positions x 1 KB
 constexpr uint32_t kStage3Bytes = 24 * 1024;
-constexpr uint32_t kConv3Smem = kW3Bytes + kStages3 * kStage3Bytes;
-static_assert(kConv3Smem + 1024 <= 227 * 1024, "conv3 kernel shared memory (with 1 KB of static shared data)");
+static_assert(kW3Bytes + kStages3 * kStage3Bytes <= kConvSmem, "conv3's weights and stages over the others' operands");
 
 // ---- heads kernel -----------------------------------------------------------
 constexpr uint32_t kHA = 128 * 64 * 2;                // A slice: 128 rows x 64 K (bf16) = 8 chunk planes
@@ -384,14 +383,116 @@ struct ConvArgs {
   const uint64_t *obs_words;  // [n][4][32] packed frames (or null)
   const uint8_t *obs_u8;      // [n][4][32][64] uint8 frames (or null)
   int64_t n;
-  const uint8_t *w1, *w2;     // packed bf16 B operands
+  const uint8_t *w1, *w2, *w3;  // packed bf16 B operands
   const float *fp;            // FpLayout
   uint8_t *act2;              // [batches][6 py][6 px][8 chunks][8 instances][16 B]
+  uint8_t *act3;              // [tiles][16][8][128][16 B]
   unsigned int *err;
   int stall;                  // diagnostic: the first conv1 commit is skipped (its wait runs out)
 };
 
-// conv1 and conv2 of batches blockIdx.x, blockIdx.x + gridDim.x, ... Every
+struct Conv3Smem {
+  uint64_t full[kStages3], empty[kStages3], done[2], freed[2], bar_w, fin[2];
+  int issued[2], landed[2];  // stages whose copies were issued / waited for, even and odd batches
+};
+
+// conv3 of the CTA's batches, from conv2's output as this CTA wrote it: the M
+// tile is the 4 x 4 output positions of 8 instances exactly. Tap (kx, ky) reads
+// input positions (qx + kx, qy + ky): the stages hold, for one kx, columns kx ..
+// kx + 3 of the six rows (24 positions; each row is one bulk copy of 4 KB), and
+// ky shifts the start by one row of them. Even and odd batches have three
+// stages, an accumulator buffer, a copying and an issuing thread each: the
+// MMAs of one accumulator run at one per ~85 cycles, of two side by side at
+// one per 42. Returns this thread's outcome.
+__device__ __forceinline__ bool conv3_batches(const ConvArgs &a, uint8_t *sm, Conv3Smem &S, const float *bias3,
+                                              uint32_t tmem, int my_batches) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t sbase = smem_u32(sm);
+  bool ok = true;
+  if (warp < kDrain3Warps) {
+    // drain: warps w and w + 4 read lane quarter w & 3 (four positions), 32 of the 64 channels each
+    const int half = warp >> 2, m = 4 * (warp & 3) + (lane >> 3), ri = lane & 7;  // m = qx + 4 qy
+    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
+    for (int bi = 0; bi < my_batches; ++bi) {
+      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&S.done[bi & 1]), (bi >> 1) & 1));
+      if (!ok) break;
+      tc_fence_after();
+      float v[32], w[32];
+      const uint32_t d = tmem + lane_base + 256 * (bi & 1) + 32 * half;
+      tmem_ld32x2(d + 64, d + 128, v, w);
+#pragma unroll
+      for (int c = 0; c < 32; ++c) w[c] += v[c];
+      tmem_ld32(d, v);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&S.freed[bi & 1]));
+#pragma unroll
+      for (int c = 0; c < 32; ++c) v[c] += w[c];
+      const int64_t inst = (blockIdx.x + (int64_t)bi * gridDim.x) * kP + ri;
+      if (inst < a.n) {
+        // feature slice m: k = 64 m + channel
+        uint8_t *dst = a.act3 + (inst >> 7) * (int64_t)kAct3TileBytes + m * 16384 + (inst & 127) * 16;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const ulonglong2 *const b3 = reinterpret_cast<const ulonglong2 *>(bias3 + 32 * half + 8 * c);
+          const uint64_t bias[4] = {b3[0].x, b3[0].y, b3[1].x, b3[1].y};
+          *reinterpret_cast<uint4 *>(dst + (4 * half + c) * 2048) = relu_chunk(v + 8 * c, bias);
+        }
+      }
+    }
+  } else if (lane == 0 && warp < kDrain3Warps + 2) {  // copies of this thread's batches: even or odd
+    const int who = warp - kDrain3Warps;
+    if (who == 0) {
+      mbar_expect_tx(smem_u32(&S.bar_w), kW3Bytes);
+      for (uint32_t o = 0; o < kW3Bytes; o += 24576) bulk_g2s(sbase + o, a.w3 + o, 24576, smem_u32(&S.bar_w));
+    }
+    int issued = 0;
+    for (int bi = who; bi < my_batches && ok; bi += 2) {
+      const uint8_t *const src = a.act2 + (blockIdx.x + (int64_t)bi * gridDim.x) * kAct2Bytes;
+      for (int kx = 0; kx < 3; ++kx) {
+        const int st = 3 * who + kx;
+        if (bi >= 2) ok = mbar_wait(smem_u32(&S.empty[st]), ((bi >> 1) - 1) & 1);  // the stage's previous MMAs are done
+        if (!ok) break;
+        const uint32_t f = smem_u32(&S.full[st]), dst = sbase + kW3Bytes + st * kStage3Bytes;
+        mbar_expect_tx(f, kStage3Bytes);
+#pragma unroll
+        for (int py = 0; py < 6; ++py) bulk_g2s(dst + py * 4096, src + (kx + 6 * py) * 1024, 4096, f);
+        ++issued;
+      }
+    }
+    grid_dependents_launch();  // (earlier, the next kernel's waiting CTAs would keep the SMs from other streams)
+    S.issued[who] = issued;
+  } else if (lane == 0 && warp < kDrain3Warps + 4) {  // MMAs of this thread's batches
+    const int who = warp - kDrain3Warps - 2;
+    const uint64_t a3d = sdesc(sbase + kW3Bytes + 3 * who * kStage3Bytes, 128, 1024), b3d = sdesc(sbase, 3072, 128);
+    ok = mbar_wait(smem_u32(&S.bar_w), 0);
+    int landed = 0;
+    for (int bi = who; bi < my_batches && ok; bi += 2) {
+      if (bi >= 2) ok = mbar_wait(smem_u32(&S.freed[who]), ((bi >> 1) - 1) & 1);
+      for (int kx = 0; kx < 3 && ok; ++kx) {
+        ok = mbar_wait(smem_u32(&S.full[3 * who + kx]), (bi >> 1) & 1);
+        if (!ok) break;
+        ++landed;
+        tc_fence_after();
+        const uint64_t at = sdesc_at(a3d, kx * kStage3Bytes), bt = sdesc_at(b3d, kx * 1024);
+        const uint32_t d = tmem + 256 * who + 64 * kx;  // an accumulator per kx, summed by the drain
+#pragma unroll
+        for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            mma_bf16(d, sdesc_at(at, ky * 4096 + kk * 256), sdesc_at(bt, ky * 24576 + kk * 6144), idesc_bf16(128, 64),
+                     (ky | kk) != 0);
+        mma_commit(smem_u32(&S.empty[3 * who + kx]));
+      }
+      if (ok) mma_commit(smem_u32(&S.done[who]));
+    }
+    S.landed[who] = landed;
+  }
+  return ok;
+}
+
+// The convolutions of batches blockIdx.x, blockIdx.x + gridDim.x, ...: conv1 and
+// conv2 of all of them, then conv3 (conv3_batches). In the first part every
 // role runs its own loop over the batches' steps and meets the others through
 // mbarriers only, so that the roles work on different steps (and, around a
 // batch's end, on different batches) at the same time:
@@ -414,18 +515,19 @@ struct ConvArgs {
 // time. Every wait is bounded; a role whose wait runs out leaves
 // its loop, and the others run into their own limits.
 template <bool kU8>
-__global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const ConvArgs a) {
+__global__ void __launch_bounds__(kConvThreads, 1) policy_conv_kernel(const ConvArgs a) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ __align__(8) uint64_t bars[16];
   __shared__ uint32_t tmem_s;
-  __shared__ __align__(16) float sb[96];     // b1 | b2
+  __shared__ __align__(16) float sb[160];    // b1 | b2 | b3
+  __shared__ __align__(8) Conv3Smem s3;
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const uint32_t sbase = smem_u32(sm);
   auto bar = [&](int j) { return smem_u32(&bars[j]); };
   // pairs of barriers, by the parity of the pair / tile
   constexpr int kBarC1 = 0, kBarBlk = 2, kBarD1f = 4, kBarC2 = 6, kBarD2f = 8, kBarBand = 10, kBarW = 12, kBarFin = 13;
 
-  for (int j = t; j < 96; j += kConvThreads) sb[j] = a.fp[j];
+  for (int j = t; j < 160; j += kConvThreads) sb[j] = a.fp[j];
   if (t == 0) {
     for (int j = 0; j < 2; ++j) {
       mbar_init(bar(kBarC1 + j), 1);
@@ -435,6 +537,17 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
       mbar_init(bar(kBarD2f + j), kDrain2Warps);
       mbar_init(bar(kBarBand + j), kDrain1Warps);
     }
+    for (int s = 0; s < kStages3; ++s) {
+      mbar_init(smem_u32(&s3.full[s]), 1);
+      mbar_init(smem_u32(&s3.empty[s]), 1);
+    }
+    for (int j = 0; j < 2; ++j) {
+      mbar_init(smem_u32(&s3.done[j]), 1);
+      mbar_init(smem_u32(&s3.freed[j]), kDrain3Warps);
+      mbar_init(smem_u32(&s3.fin[j]), 1);
+      s3.issued[j] = s3.landed[j] = 0;
+    }
+    mbar_init(smem_u32(&s3.bar_w), 1);
     for (int j = kBarW; j < 16; ++j) mbar_init(bar(j), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -664,9 +777,6 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
         }
       }
       if (kU8) pack_bytes(3);
-      // what is left is two pairs and a tile: about the time the next kernel's
-      // set-up takes (earlier, its waiting CTAs would keep the SMs from other streams)
-      if (bi + 1 == my_batches) grid_dependents_launch();
     }
   } else {
     // ---- issuing warps: whole warps in step, one lane of which issues
@@ -748,159 +858,31 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv12_kernel(const Co
       }
     }
   }
-  ok = !__syncthreads_or(!ok);
-  if (!ok && t == 0) atomicOr(a.err, 1u);
-  if (!ok && warp >= kIssueWarp) {  // let this warp's MMAs and copies land
-    mma_commit_warp(bar(kBarFin + warp - kIssueWarp));
-    mbar_wait(bar(kBarFin + warp - kIssueWarp), 0);
-    if (warp == kIssueWarp) mbar_wait(bar(kBarW), 0);
-  }
+  // conv2's output, written above, is read by bulk copies below, into shared
+  // memory that was written and read above
+  asm volatile("fence.proxy.async;" ::: "memory");
   tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kConvTmemCols));
-}
-
-struct Conv3Args {
-  const uint8_t *act2;
-  int64_t n;
-  const uint8_t *w3;          // packed bf16 B operand
-  const float *fp;            // FpLayout
-  uint8_t *act3;              // [tiles][16][8][128][16 B]
-  unsigned int *err;
-};
-
-// conv3 of batches blockIdx.x, blockIdx.x + gridDim.x, ...: the M tile is the
-// 4 x 4 output positions of 8 instances exactly. Even and odd batches have
-// three stages, an accumulator buffer, a copying and an issuing thread each. Tap (kx, ky) reads input
-// positions (qx + kx, qy + ky): the ring's stages hold, for one kx, columns
-// kx .. kx + 3 of the six rows (24 positions; each row is one bulk copy of 4
-// KB), and ky shifts the start by one row of them.
-__global__ void __launch_bounds__(kConv3Threads, 1) policy_conv3_kernel(const Conv3Args a) {
-  extern __shared__ __align__(1024) uint8_t sm[];
-  __shared__ __align__(8) uint64_t full[kStages3], empty[kStages3], done[2], freed[2], bar_w, fin[2];
-  __shared__ uint32_t tmem_s;
-  __shared__ __align__(16) float sb[64];
-  __shared__ int s_issued[2], s_landed[2];  // stages whose copies were issued / waited for, even and odd batches
-  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  const uint32_t sbase = smem_u32(sm);
-  if (t < 64) sb[t] = a.fp[FpLayout::b3 + t];
-  if (t == 0) {
-    for (int s = 0; s < kStages3; ++s) {
-      mbar_init(smem_u32(&full[s]), 1);
-      mbar_init(smem_u32(&empty[s]), 1);
-    }
-    for (int j = 0; j < 2; ++j) {
-      mbar_init(smem_u32(&done[j]), 1);
-      mbar_init(smem_u32(&freed[j]), kDrain3Warps);
-      mbar_init(smem_u32(&fin[j]), 1);
-      s_issued[j] = s_landed[j] = 0;
-    }
-    mbar_init(smem_u32(&bar_w), 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_s)),
-                 "r"(kConvTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = tmem_s;
-  const int64_t n_batches = (a.n + kP - 1) / kP;
-  const int my_batches = (int)((n_batches - blockIdx.x + gridDim.x - 1) / gridDim.x);
-  bool ok = true;
-  if (warp < kDrain3Warps) {
-    // drain: warps w and w + 4 read lane quarter w & 3 (four positions), 32 of the 64 channels each
-    const int half = warp >> 2, m = 4 * (warp & 3) + (lane >> 3), ri = lane & 7;  // m = qx + 4 qy
-    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    for (int bi = 0; bi < my_batches; ++bi) {
-      ok = __all_sync(0xFFFFFFFFu, mbar_wait(smem_u32(&done[bi & 1]), (bi >> 1) & 1));
-      if (!ok) break;
-      tc_fence_after();
-      float v[32], w[32], x[32];
-      const uint32_t d = tmem + lane_base + 256 * (bi & 1) + 32 * half;
-      tmem_ld32x2(d + 64, d + 128, w, x);
-      tmem_ld32(d, v);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&freed[bi & 1]));
-#pragma unroll
-      for (int c = 0; c < 32; ++c) v[c] += w[c] + x[c];
-      const int64_t inst = (blockIdx.x + (int64_t)bi * gridDim.x) * kP + ri;
-      if (inst < a.n) {
-        // feature slice m: k = 64 m + channel
-        uint8_t *dst = a.act3 + (inst >> 7) * (int64_t)kAct3TileBytes + m * 16384 + (inst & 127) * 16;
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const ulonglong2 *const b3 = reinterpret_cast<const ulonglong2 *>(sb + 32 * half + 8 * c);
-          const uint64_t bias[4] = {b3[0].x, b3[0].y, b3[1].x, b3[1].y};
-          *reinterpret_cast<uint4 *>(dst + (4 * half + c) * 2048) = relu_chunk(v + 8 * c, bias);
-        }
-      }
-    }
-  } else if (lane == 0 && warp < kDrain3Warps + 2) {  // copies of this thread's batches: even or odd
-    const int who = warp - kDrain3Warps;
-    if (who == 0) {
-      mbar_expect_tx(smem_u32(&bar_w), kW3Bytes);
-      for (uint32_t o = 0; o < kW3Bytes; o += 24576) bulk_g2s(sbase + o, a.w3 + o, 24576, smem_u32(&bar_w));
-    }
-    grid_dependency_wait();  // conv2's output
-    int issued = 0;
-    for (int bi = who; bi < my_batches && ok; bi += 2) {
-      const uint8_t *const src = a.act2 + (blockIdx.x + (int64_t)bi * gridDim.x) * kAct2Bytes;
-      for (int kx = 0; kx < 3; ++kx) {
-        const int st = 3 * who + kx;
-        if (bi >= 2) ok = mbar_wait(smem_u32(&empty[st]), ((bi >> 1) - 1) & 1);  // the stage's previous MMAs are done
-        if (!ok) break;
-        const uint32_t f = smem_u32(&full[st]), dst = sbase + kW3Bytes + st * kStage3Bytes;
-        mbar_expect_tx(f, kStage3Bytes);
-#pragma unroll
-        for (int py = 0; py < 6; ++py) bulk_g2s(dst + py * 4096, src + (kx + 6 * py) * 1024, 4096, f);
-        ++issued;
-      }
-    }
-    grid_dependents_launch();
-    s_issued[who] = issued;
-  } else if (lane == 0) {  // MMAs of this thread's batches
-    const int who = warp - kDrain3Warps - 2;
-    const uint64_t a3d = sdesc(sbase + kW3Bytes + 3 * who * kStage3Bytes, 128, 1024), b3d = sdesc(sbase, 3072, 128);
-    ok = mbar_wait(smem_u32(&bar_w), 0);
-    int landed = 0;
-    for (int bi = who; bi < my_batches && ok; bi += 2) {
-      if (bi >= 2) ok = mbar_wait(smem_u32(&freed[who]), ((bi >> 1) - 1) & 1);
-      for (int kx = 0; kx < 3 && ok; ++kx) {
-        ok = mbar_wait(smem_u32(&full[3 * who + kx]), (bi >> 1) & 1);
-        if (!ok) break;
-        ++landed;
-        tc_fence_after();
-        const uint64_t at = sdesc_at(a3d, kx * kStage3Bytes), bt = sdesc_at(b3d, kx * 1024);
-        const uint32_t d = tmem + 256 * who + 64 * kx;  // an accumulator per kx, summed by the drain
-#pragma unroll
-        for (int ky = 0; ky < 3; ++ky)
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_bf16(d, sdesc_at(at, ky * 4096 + kk * 256), sdesc_at(bt, ky * 24576 + kk * 6144), idesc_bf16(128, 64),
-                     (ky | kk) != 0);
-        mma_commit(smem_u32(&empty[3 * who + kx]));
-      }
-      if (ok) mma_commit(smem_u32(&done[who]));
-    }
-    s_landed[who] = landed;
-  }
   ok = !__syncthreads_or(!ok);
-  if (!ok && t == 0) {
-    atomicOr(a.err, 1u);
-    // copies issued but never waited for land before shared memory goes
-    mbar_wait(smem_u32(&bar_w), 0);
-    for (int who = 0; who < 2; ++who)
-      for (int q = s_landed[who]; q < s_issued[who]; ++q)
-        mbar_wait(smem_u32(&full[3 * who + q % 3]), (q / 3) & 1);
-  }
-  if (!ok && warp >= kDrain3Warps + 2 && lane == 0) {  // let this thread's MMAs land before TMEM goes
-    mma_commit(smem_u32(&fin[warp - kDrain3Warps - 2]));
-    mbar_wait(smem_u32(&fin[warp - kDrain3Warps - 2]), 0);
+  tc_fence_after();
+  const bool third = ok;
+  if (third) ok = conv3_batches(a, sm, s3, sb + 96, tmem, my_batches);
+  ok = !__syncthreads_or(!ok);
+  if (!ok) {  // the MMAs and copies of every issuing thread land before TMEM and shared memory go
+    if (t == 0) atomicOr(a.err, 1u);
+    if (warp >= kIssueWarp) {
+      mma_commit_warp(bar(kBarFin + warp - kIssueWarp));
+      mbar_wait(bar(kBarFin + warp - kIssueWarp), 0);
+      if (warp == kIssueWarp) mbar_wait(bar(kBarW), 0);
+    }
+    if (third && warp >= kDrain3Warps && warp < kDrain3Warps + 2 && lane == 0) {
+      const int who = warp - kDrain3Warps;
+      mbar_wait(smem_u32(&s3.bar_w), 0);
+      for (int q = s3.landed[who]; q < s3.issued[who]; ++q) mbar_wait(smem_u32(&s3.full[3 * who + q % 3]), (q / 3) & 1);
+    }
+    if (third && warp >= kDrain3Warps + 2 && warp < kDrain3Warps + 4 && lane == 0) {
+      mma_commit(smem_u32(&s3.fin[warp - kDrain3Warps - 2]));
+      mbar_wait(smem_u32(&s3.fin[warp - kDrain3Warps - 2]), 0);
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -1132,17 +1114,15 @@ int launch_forward(octax_policy *p, int64_t n, const uint64_t *obs_words, const 
     set_error("octax_policy: need 1 <= n_envs <= max_envs of the policy");
     return OCTAX_EINVAL;
   }
-  ConvArgs c{obs_words, obs_u8, n, (const uint8_t *)p->w1, (const uint8_t *)p->w2, p->fp, p->act2, p->err, p->stall};
-  Conv3Args c3{p->act2, n, (const uint8_t *)p->w3, p->fp, p->act3, p->err};
+  ConvArgs c{obs_words, obs_u8, n, (const uint8_t *)p->w1, (const uint8_t *)p->w2, (const uint8_t *)p->w3, p->fp,
+             p->act2, p->act3, p->err, p->stall};
   HeadsArgs h{p->act3, n, (const uint8_t *)p->wh, p->fp, p->n_logits, logits, value, actions,
               (uint32_t)seed, (uint32_t)(seed >> 32), step, p->err};
   const int64_t batches = (n + kP - 1) / kP;
   const unsigned grid = (unsigned)std::min<int64_t>(batches, p->sms);
-  cudaError_t r = obs_u8 ? launch(policy_conv12_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, c)
-                         : launch(policy_conv12_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, c);
+  cudaError_t r = obs_u8 ? launch(policy_conv_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, c)
+                         : launch(policy_conv_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, c);
   if (r != cudaSuccess) return cuda_fail(r, "policy conv launch");
-  r = launch(policy_conv3_kernel, dim3(grid), kConv3Threads, kConv3Smem, s, c3);
-  if (r != cudaSuccess) return cuda_fail(r, "policy conv3 launch");
   // A CTA holds an SM's shared memory, so they run in waves of one per SM: one
   // tile each as long as that makes one wave, else two (the weights then come
   // in once for both).
@@ -1282,11 +1262,9 @@ int octax_policy_create(const octax_policy_params *prm, int64_t max_envs, int de
   if (r == cudaSuccess) r = cudaMemset(p->ring, 0, (size_t)2 * max_envs * 1024);
   if (r == cudaSuccess) r = cudaMemset(p->err, 0, 4);
   if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(policy_conv12_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
+    r = cudaFuncSetAttribute(policy_conv_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
   if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(policy_conv12_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
-  if (r == cudaSuccess)
-    r = cudaFuncSetAttribute(policy_conv3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kConv3Smem);
+    r = cudaFuncSetAttribute(policy_conv_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kConvSmem);
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(policy_heads_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kHeadSmem);
   if (r == cudaSuccess)
