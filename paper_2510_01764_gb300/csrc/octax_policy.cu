@@ -8,11 +8,7 @@
 // VALID convolutions; weights and stored activations in bfloat16, products
 // accumulated in fp32 (TMEM), heads' output layers in fp32 on the CUDA cores.
 //
-// Conv kernel (persistent, one CTA per SM: 8 warps that build operands and
-// drain accumulators, and three threads in three more warps that issue the
-// MMAs and bulk copies: an MMA costs its issuing thread more time than its
-// share of the tensor pipe, so conv1's even pairs, its odd pairs and conv2's
-// tiles come from different threads). A batch of kP = 8
+// Conv kernel (persistent, one CTA per SM). A batch of kP = 8
 // instances is processed at a time; the rows of every GEMM are
 // (grid position, instance) with the instance fastest, so one 8-row core
 // matrix of the tcgen05 no-swizzle K-major layout is one grid position of
@@ -24,28 +20,37 @@
 //    covers 2 x 2 blocks, so it is 4 taps of K = 32 (4 frames x 8 pixels)
 //    over a 16 x 16 grid of blocks, expanded from the packed frame bits to
 //    bf16 0/1; two output rows (16 positions x 8 instances = 128 rows each)
-//    share one N = 64 accumulator fed by the three block rows they read.
+//    share one accumulator fed by the three block rows they read.
 //  - conv2 (stride 2) reads conv1's output split by the parity of x and y:
 //    tap (kx, ky) reads sub-grid (kx & 1, ky & 1) at offset (kx >> 1,
-//    ky >> 1) of an 8-wide grid. The taps kx and kx + 2 read the same
+//    ky >> 1) of a 7-wide grid. The taps kx and kx + 2 read the same
 //    sub-grid one position apart, so they are stacked along N (N = 128) and
 //    the drain adds columns 64..127 of row g + 1 to columns 0..63 of row g.
-//    The sub-grids are kept as a band of four grid rows that slides down by
-//    two with conv1's output rows; each M tile covers two output rows and
-//    reads three grid rows, so the next conv1 pair writes the fourth while
-//    the tile computes.
-//  - conv3 (stride 1) reads conv2's output on an 8-wide grid. The three taps
-//    kx of a kernel row ky read the same rows shifted by kx positions, so
-//    they are stacked along N (N = 192: one MMA per ky and k-step reads its A
-//    tile once for all three) and the shift is applied when draining: the
-//    output at position g sums columns 0..63 of row g, 64..127 of row g + 1
-//    and 128..191 of row g + 2.
-//  Rows whose grid position lies outside the layer's output are computed
+//    The sub-grids are a band of six grid rows, written round and round; each M
+//    tile covers two output rows and reads three grid rows.
+//  - conv3 (stride 1) follows when the CTA's batches are through conv2; its A
+//    operand is conv2's output in three copies, shifted by kx, so that the M
+//    tile is the 16 output positions and nothing else.
+//  Rows whose grid position lies outside conv1's or conv2's output are computed
 //  and discarded (they read padding or neighbouring positions, always inside
 //  the buffers).
-// Heads kernel: one CTA per (128-instance tile, head); K = 1024 streamed in
-// 32-wide slices through a 3-stage ring (one thread issues the copies,
-// another the MMAs); the actor CTA also draws the action.
+// What bounds it: the chains of MMAs that add into one accumulator (12 of conv1
+// per pair of rows, 16 of conv2 per tile; each link takes 85-105 cycles whatever
+// N <= 128) and their hand-overs; 9.6 K cycles a batch for conv1 and conv2,
+// of which the tensor pipe needs 5.8 K, and 2.4 K for conv3 (1.7 K of operand
+// reads). Against the form before it (a CTA took each batch through all
+// phases, conv3's output positions 22 of 32 rows; 150 us for 16,384
+// instances): 75 us for conv1 and conv2 and about 18 us for conv3. Its steps:
+// roles that run ahead of each other, also over a batch's end (forward 173.5
+// -> 126.5 us); a wait that seldom reads the timer, blocks expanded before the
+// wait, a band whose rows are rewritten five rows later (112.5); MMAs issued
+// by whole warps, whose operands need no moves to uniform registers (12 MMAs
+// in 1.25 K -> 0.75 K cycles; 101.8); conv3 in the same kernel (99.2). No
+// gain: a ring of 7 block rows with four accumulators; conv1's A operand in
+// TMEM; conv1's two rows as separate chains.
+// Heads kernel: a head of one or two 128-instance tiles per CTA; K = 1024
+// streamed in 64-wide slices; the actor CTA also draws the action. Bound by the
+// MMAs (16.4 K cycles for two tiles) and the first slice's arrival (2.4 K).
 #include <cuda_bf16.h>
 
 #include <algorithm>
