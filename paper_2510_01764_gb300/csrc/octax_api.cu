@@ -339,7 +339,8 @@ int get_groups(octax_env *e, int cap, int wave, GroupTable **out) {
   t.count = (int)gs.size();
   cudaError_t r = dalloc(e, &t.dev, gs.size());
   if (r != cudaSuccess) return cuda_fail(r, "group table");
-  r = cudaMemcpy(t.dev, gs.data(), gs.size() * sizeof(Group), cudaMemcpyHostToDevice);
+  // in the stream, ahead of the launch that reads it (a kernel set up early reads its groups before it waits)
+  r = cudaMemcpyAsync(t.dev, gs.data(), gs.size() * sizeof(Group), cudaMemcpyHostToDevice, e->stream);
   if (r != cudaSuccess) return cuda_fail(r, "group table upload");
   e->groups[gkey] = t;
   *out = &e->groups[gkey];
