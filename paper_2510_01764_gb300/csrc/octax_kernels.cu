@@ -751,8 +751,12 @@ __device__ __forceinline__ bool terminated(const Regs &R, const Ctx &C, const Ga
 // K), then the no-op reset wrapper (§3.2): a drawn number of no-key env steps
 // of frameskip frames each, unobserved. The previous action becomes the no-op.
 // kWrap = false compiles the wrapper out (no game of the launch uses it).
+// The lanes of the instance meet here first: the stack and the flag registers
+// are one copy for all of them, and a lane behind may still be at the last
+// instructions of its step (a return reads the stack).
 template <bool kWrap, bool kS>
 __device__ __forceinline__ void reset_instance(Regs &R, const Ctx &C, const GameDev &G, uint32_t quirks) {
+  __syncwarp(C.gmask);
   uint32_t *const V = reinterpret_cast<uint32_t *>(C.V);
 #pragma unroll
   for (int i = 0; i < 4; ++i) V[i] = 0;
