@@ -1132,8 +1132,9 @@ __global__ void __launch_bounds__(kMaxBlock, 2) step_kernel(const StepLaunch p) 
 // ordered. Slots hand over through mbarriers (full: all emulator threads
 // arrive; empty: all writer threads arrive); every wait polls a bounded
 // number of times for at most kMaxWaitNs of the global timer and, if it
-// gives up, records the failure in p.err and stops the thread's work instead
-// of hanging.
+// gives up, records the failure in p.err. The lanes of a warp decide together
+// whether a wait ran out (those of an instance meet in the interpreter, which
+// has no limit), and what one warp gave up ends the CTA's work on later groups.
 
 constexpr uint32_t kMaxPolls = 1u << 22;
 constexpr uint64_t kMaxWaitNs = 1000000000ull;  // one second
@@ -1227,10 +1228,8 @@ __device__ void run_group_emu(const StepLaunch &p, const Group &g, const Warp &W
       }
       if (f >= first_kept) {  // hand the frame to the writers
         const uint32_t b = msg & 1u, use = msg >> 1;
-        if (!mbar_wait(X.empty + b, (use & 1u) ^ 1u, p.err)) {
-          failed = true;
-          break;
-        }
+        failed = !__all_sync(kFull, mbar_wait(X.empty + b, (use & 1u) ^ 1u, p.err));
+        if (failed) break;
         if (W.active) ring_put(X, C, W.J, W.j, b);
         mbar_arrive(X.full + b);
         ++msg;
@@ -1257,10 +1256,8 @@ __device__ void run_group_emu(const StepLaunch &p, const Group &g, const Warp &W
     }
     // end-of-step message: done flags and the reset displays
     const uint32_t b = msg & 1u, use = msg >> 1;
-    if (!mbar_wait(X.empty + b, (use & 1u) ^ 1u, p.err)) {
-      failed = true;
-      break;
-    }
+    failed = !__all_sync(kFull, mbar_wait(X.empty + b, (use & 1u) ^ 1u, p.err));
+    if (failed) break;
     if (W.active) {
       X.done[b * W.J + W.j] = done ? 1 : 0;
       if (done) ring_put(X, C, W.J, W.j, b);
@@ -1270,9 +1267,9 @@ __device__ void run_group_emu(const StepLaunch &p, const Group &g, const Warp &W
   }
 
   // a failed wait fails the whole warp's group: its records stay as they were
-  const bool ok = __all_sync(kFull, !failed);
-  if (ok && W.active) store_regs<false>(R, C, ep);
-  if (ok) return_records<false>(W, st, g, kFull);
+  if (failed) return;
+  if (W.active) store_regs<false>(R, C, ep);
+  return_records<false>(W, st, g, kFull);
 }
 
 // Writer side of one group: writer warp ww owns instances
@@ -1302,10 +1299,8 @@ __device__ void run_group_writer(const StepLaunch &p, const Group &g, const WsSm
     const int64_t step_row = (int64_t)(p.step0 + s) * io.rows;
     for (uint32_t f = first_kept; f <= FS; ++f) {  // FS - S frames, then the end-of-step message
       const uint32_t b = msg & 1u, use = msg >> 1;
-      if (!mbar_wait(W.full + b, use & 1u, p.err)) {
-        failed = true;
-        break;
-      }
+      failed = !__all_sync(kFull, mbar_wait(W.full + b, use & 1u, p.err));
+      if (failed) break;
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
         if (m >= passes || orow[m] < 0) continue;
@@ -1366,7 +1361,7 @@ __global__ void step_kernel_ws(const StepLaunch p) {
       if (writer) run_group_writer(p, g, X, msg, failed);
       else run_group_emu(p, g, W, X, msg, failed);
     }
-    __syncthreads();  // shared memory is reused by the next group
+    failed = __syncthreads_or(failed);  // (and shared memory is reused by the next group)
     if (!p.work_counter) break;
   }
 }
