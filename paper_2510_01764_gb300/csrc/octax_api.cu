@@ -339,8 +339,17 @@ int get_groups(octax_env *e, int cap, int wave, GroupTable **out) {
   t.count = (int)gs.size();
   cudaError_t r = dalloc(e, &t.dev, gs.size());
   if (r != cudaSuccess) return cuda_fail(r, "group table");
-  // in the stream, ahead of the launch that reads it (a kernel set up early reads its groups before it waits)
-  r = cudaMemcpyAsync(t.dev, gs.data(), gs.size() * sizeof(Group), cudaMemcpyHostToDevice, e->stream);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  r = cudaStreamIsCapturing(e->stream, &capture);
+  if (r == cudaSuccess && capture != cudaStreamCaptureStatusNone) {
+    // while the stream is captured (in a mode that allows the allocation): now, and not as a node of the graph,
+    // which would copy from this call's memory at each replay and leave the table empty until the first
+    r = cudaMemcpy(t.dev, gs.data(), gs.size() * sizeof(Group), cudaMemcpyHostToDevice);
+    if (r == cudaSuccess) r = cudaStreamSynchronize(cudaStreamLegacy);
+  } else if (r == cudaSuccess) {
+    // in the stream, ahead of the launch that reads it (a kernel set up early reads its groups before it waits)
+    r = cudaMemcpyAsync(t.dev, gs.data(), gs.size() * sizeof(Group), cudaMemcpyHostToDevice, e->stream);
+  }
   if (r != cudaSuccess) return cuda_fail(r, "group table upload");
   e->groups[gkey] = t;
   *out = &e->groups[gkey];
