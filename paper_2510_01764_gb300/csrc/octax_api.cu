@@ -193,6 +193,12 @@ octax_launch own_shape(int64_t n, int sms, int schip) {
 
 const octax_launch &shape_of(const octax_env *e) { return e->cfg_set ? e->cfg : e->own_cfg; }
 
+// What is launched for a configuration.
+octax_launch fitted(const octax_env *e, octax_launch c) {
+  c.inst_per_warp = fit_ipw(c.block, c.inst_per_warp, e->schip, c.writer_warps, e->n_uops);
+  return c;
+}
+
 // Resident CTAs of one wave for a balanced launch (0 = not balanced).
 int wave_of(const octax_env *e, const octax_launch &c) {
   if (!c.balance) return 0;
@@ -377,7 +383,6 @@ StepLaunch base_launch(octax_env *e, const GroupTable *gt) {
   p.n_groups = gt->count;
   p.S = e->S;
   p.quirks = e->quirks;
-  p.ipw = shape_of(e).inst_per_warp;
   p.err = e->err_d;
   p.wrappers = uses_wrappers(e->games_h.data(), e->games_h.size());
   p.stall_writers = e->stall_writers;
@@ -399,7 +404,8 @@ int check_io(const uint8_t *actions, const uint8_t *obs, const float *reward, co
 }
 
 // Enqueue n_steps steps as a chain of launches of `spl` steps each.
-int enqueue_steps(octax_env *e, const octax_launch &cfg, int n_steps, const IO &io) {
+int enqueue_steps(octax_env *e, const octax_launch &shape, int n_steps, const IO &io) {
+  const octax_launch cfg = fitted(e, shape);
   GroupTable *gt = nullptr;
   int rc = get_groups(e, per_cta(cfg), wave_of(e, cfg), &gt);
   if (rc) return rc;
@@ -642,8 +648,9 @@ int octax_reset(octax_env *e, const uint8_t *mask_dev, uint8_t *obs_dev) {
     set_error("octax_reset: obs must be 16-byte aligned");
     return OCTAX_EINVAL;
   }
+  const octax_launch cfg = fitted(e, shape_of(e));
   GroupTable *gt = nullptr;
-  int rc = get_groups(e, per_cta(shape_of(e)), wave_of(e, shape_of(e)), &gt);
+  int rc = get_groups(e, per_cta(cfg), wave_of(e, cfg), &gt);
   if (rc) return rc;
   ResetLaunch p;
   memset(&p, 0, sizeof p);
@@ -657,8 +664,8 @@ int octax_reset(octax_env *e, const uint8_t *mask_dev, uint8_t *obs_dev) {
   p.obs = obs_dev;
   p.S = e->S;
   p.quirks = e->quirks;
-  p.ipw = shape_of(e).inst_per_warp;
-  cudaError_t r = launch_reset(p, shape_of(e).block, e->stream);
+  p.ipw = cfg.inst_per_warp;
+  cudaError_t r = launch_reset(p, cfg.block, e->stream);
   return r == cudaSuccess ? OCTAX_OK : cuda_fail(r, "octax_reset");
 }
 

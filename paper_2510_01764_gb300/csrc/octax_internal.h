@@ -115,7 +115,7 @@ struct IO {
 struct StepLaunch {
   DevState st;
   const uint8_t *blobs;    // [n_games][blob_stride(n_uops)]
-  int n_uops;              // micro-ops per game (0 in a launch without room for the table)
+  int n_uops;              // micro-ops per game
   uint32_t stride;         // blob_stride of the table as built
   const Group *groups;
   int n_groups;
@@ -159,6 +159,8 @@ size_t step_ws_smem_bytes(int block, int ipw, int n_uops);
 size_t max_dynamic_smem();
 // The launch shapes that are accepted: what a CTA's instances may take of shared memory.
 bool shape_fits(int block, int ipw, int schip, int writers);
+// Instances per warp, at most ipw, that an accepted shape launches beside a table of n_uops micro-ops.
+int fit_ipw(int block, int ipw, int schip, int writers, int n_uops);
 // Fills the pixel table and the micro-ops of every blob from its RAM image.
 cudaError_t launch_tables(uint8_t *blobs, size_t stride, int n_games, int n_uops, int schip, uint32_t quirks,
                           cudaStream_t s);

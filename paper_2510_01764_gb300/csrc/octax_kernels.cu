@@ -903,10 +903,7 @@ __device__ __forceinline__ const GameDev &smem_game() { return *reinterpret_cast
 // Starts the copy of a game's blob (all threads; copy_wait and a barrier follow).
 __device__ __forceinline__ void stage_game(const uint8_t *blobs, uint32_t stride, int game, uint32_t n_uops) {
   const uint8_t *src = blobs + (size_t)game * stride;
-  const uint32_t bytes = n_uops ? blob_bytes(n_uops) : (uint32_t)kBlobUops;
-  for (uint32_t i = 16 * threadIdx.x; i < bytes; i += 16 * blockDim.x) copy16_async(g_smem + i, src + i);
-  // no room for the table: only the sentinel
-  if (!n_uops && threadIdx.x < 3) reinterpret_cast<uint32_t *>(g_smem + kBlobUops)[threadIdx.x] = threadIdx.x ? kKindRaw : kUSlow;
+  for (uint32_t i = 16 * threadIdx.x; i < blob_bytes(n_uops); i += 16 * blockDim.x) copy16_async(g_smem + i, src + i);
 }
 
 // The lanes of a warp and what it emulates: ipw instances, each by 1 << sh lanes.
@@ -1566,9 +1563,7 @@ size_t step_ws_smem_bytes(int block, int ipw, int n_uops) {
 }
 
 // The accepted shapes: 23,232 bytes for the game and 384 (SCHIP 1,152) per
-// instance, with the writers' ring 512 more and the hand-over's flags. The
-// kernels need less than that, or run without the micro-op table
-// (launch_uops).
+// instance, with the writers' ring 512 more and the hand-over's flags.
 bool shape_fits(int block, int ipw, int schip, int writers) {
   const size_t J = (size_t)(block / 32) * ipw;
   size_t need = 23232 + J * (schip ? 1152 : 384);
@@ -1576,12 +1571,16 @@ bool shape_fits(int block, int ipw, int schip, int writers) {
   return need <= max_dynamic_smem();
 }
 
-// Micro-ops staged by a launch: the table, or none where it does not fit
-// beside the records (SCHIP, a 3.5 KB ROM and more than 160 instances per
-// CTA): every instruction then takes the switch.
-static int launch_uops(int block, int ipw, int schip, int writers, int n_uops) {
-  const size_t need = writers > 0 ? step_ws_smem_bytes(block, ipw, n_uops) : step_smem_bytes(block, ipw, schip, n_uops);
-  return need <= max_dynamic_smem() ? n_uops : 0;
+static size_t launch_smem(int block, int ipw, int schip, int writers, int n_uops) {
+  return writers > 0 ? step_ws_smem_bytes(block, ipw, n_uops) : step_smem_bytes(block, ipw, schip, n_uops);
+}
+
+// Most instances per warp, up to ipw, whose records fit a CTA's shared memory
+// beside the game's table. Of the accepted shapes one can lose some: 256 x 22
+// of Super-CHIP games with a ROM over 3,326 bytes run as 256 x 21.
+int fit_ipw(int block, int ipw, int schip, int writers, int n_uops) {
+  while (ipw > 1 && launch_smem(block, ipw, schip, writers, n_uops) > max_dynamic_smem()) --ipw;
+  return ipw;
 }
 
 // The dynamic shared memory attribute of a kernel applies to the current
@@ -1615,10 +1614,6 @@ static const void *step_fn(int writers, int wrappers, int schip) {
   return wrappers ? (const void *)step_kernel<true, false> : (const void *)step_kernel<false, false>;
 }
 
-static size_t launch_smem(int block, int ipw, int schip, int writers, int n_uops) {
-  return writers > 0 ? step_ws_smem_bytes(block, ipw, n_uops) : step_smem_bytes(block, ipw, schip, n_uops);
-}
-
 cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s) {
   if (!state_complete(p.st)) return cudaErrorInvalidValue;
   cudaError_t e = ensure_smem_attr();
@@ -1627,11 +1622,10 @@ cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s
   const void *fn = step_fn(p.writers, p.wrappers, p.st.schip);
   if (!fn) return cudaErrorInvalidValue;
   StepLaunch copy = p;
-  copy.n_uops = launch_uops(block, p.ipw, p.st.schip, p.writers, p.n_uops);
   void *args[] = {&copy};
   const int threads = p.writers > 0 ? block + 32 * p.writers : block;
   return launch_kernel(fn, dim3((unsigned)grid), dim3((unsigned)threads), args,
-                       launch_smem(block, p.ipw, p.st.schip, p.writers, copy.n_uops), s, !p.work_counter);
+                       launch_smem(block, p.ipw, p.st.schip, p.writers, p.n_uops), s, !p.work_counter);
 }
 
 cudaError_t launch_reset(const ResetLaunch &p, int block, cudaStream_t s) {
@@ -1639,11 +1633,9 @@ cudaError_t launch_reset(const ResetLaunch &p, int block, cudaStream_t s) {
   cudaError_t e = ensure_smem_attr();
   if (e != cudaSuccess) return e;
   if (p.n_groups <= 0) return cudaSuccess;
-  ResetLaunch copy = p;
-  copy.n_uops = launch_uops(block, p.ipw, p.st.schip, 0, p.n_uops);
-  const size_t smem = step_smem_bytes(block, p.ipw, p.st.schip, copy.n_uops);
-  if (p.st.schip) reset_kernel<true><<<p.n_groups, block, smem, s>>>(copy);
-  else reset_kernel<false><<<p.n_groups, block, smem, s>>>(copy);
+  const size_t smem = step_smem_bytes(block, p.ipw, p.st.schip, p.n_uops);
+  if (p.st.schip) reset_kernel<true><<<p.n_groups, block, smem, s>>>(p);
+  else reset_kernel<false><<<p.n_groups, block, smem, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -1688,14 +1680,13 @@ cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t 
   const void *fn = step_fn(p.writers, p.wrappers, p.st.schip);
   if (!fn) return cudaErrorInvalidValue;
   StepLaunch copy = p;
-  copy.n_uops = launch_uops(block, p.ipw, p.st.schip, p.writers, p.n_uops);
   void *args[] = {&copy};
   cudaKernelNodeParams kp;
   memset(&kp, 0, sizeof kp);
   kp.func = const_cast<void *>(fn);
   kp.gridDim = dim3((unsigned)grid);
   kp.blockDim = dim3((unsigned)(p.writers > 0 ? block + 32 * p.writers : block));
-  kp.sharedMemBytes = (unsigned)launch_smem(block, p.ipw, p.st.schip, p.writers, copy.n_uops);
+  kp.sharedMemBytes = (unsigned)launch_smem(block, p.ipw, p.st.schip, p.writers, p.n_uops);
   kp.kernelParams = args;
   return cudaGraphAddKernelNode(node, g, dep ? &dep : nullptr, dep ? 1 : 0, &kp);
 }
@@ -1722,9 +1713,8 @@ int max_resident_ctas(int block, int ipw, int writers, int wrappers, int schip, 
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const void *fn = step_fn(writers, wrappers, schip);
   if (!fn) return 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-      &per_sm, fn, block + 32 * writers,
-      launch_smem(block, ipw, schip, writers, launch_uops(block, ipw, schip, writers, n_uops)));
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block + 32 * writers,
+                                                launch_smem(block, ipw, schip, writers, n_uops));
   return sms * per_sm;
 }
 
