@@ -279,7 +279,8 @@ int octax::build_games(const octax_game *games, int n_games, std::vector<GameDev
 int octax::table_uops(const octax_game *games, int n_games) {
   uint32_t len = 0;
   for (int g = 0; g < n_games; ++g) len = std::max(len, games[g].rom_len);
-  return (int)((len + 1) / 2);
+  const int n = (int)((len + 1) / 2);
+  return n > kLongTable ? n + 0x200 / 2 : n;  // from address 0 on (table_base)
 }
 
 cudaError_t octax::upload_blobs(const std::vector<GameDev> &games, const std::vector<uint8_t> &images, int n_uops,

@@ -51,14 +51,26 @@ constexpr int kGameSmem = 192;
 constexpr int kLutSmem = 256 * 8;            // byte of pixels -> 8 output bytes
 // What a CTA stages of its game, one contiguous blob per game in device
 // memory, in this order: RAM image | descriptor | pixel table | coefficients |
-// micro-ops (one per even address of the ROM and a sentinel; 8 bytes of each,
-// then 4 bytes of each).
+// micro-ops (one per even address from table_base on, to the end of the longest
+// ROM, and a sentinel; 8 bytes of each, then 4 bytes of each).
 constexpr int kBlobLut = kRamBytes + kGameSmem;
 constexpr int kBlobCoef = kBlobLut + kLutSmem;
 constexpr int kBlobUops = kBlobCoef + 64;
 __host__ __device__ constexpr uint32_t blob_bytes(uint32_t n_uops) {
   return ((uint32_t)kBlobUops + 12 * (n_uops + 1) + 15) & ~15u;
 }
+// First address of a table of n_uops micro-ops: that of the ROM, or 0 where the
+// longest ROM has more than 3,072 bytes. Programs that fall through into the
+// memory below the ROM (random ones end up there: 7 of 10 of their instructions
+// after 200 steps) then leave the datapath no more; the 3 KB this takes are a
+// seventh of what such an environment's CTAs stage. 262,144 random programs of
+// 3,584 bytes, 2,000 steps: 414 us a step with the ROM's addresses alone, 400
+// with all; 16,384 and 65,536 of them 1-5 % faster, template programs padded to
+// that length 0.7 % faster to 1 % slower. At 3,072 bytes neither side leads
+// (0.94-1.04); at 1,024, where a CTA of 32 instances loses one of eight resident
+// ones, template programs lose 5 %.
+constexpr int kLongTable = 3072 / 2;
+__host__ __device__ constexpr uint32_t table_base(uint32_t n_uops) { return n_uops > (uint32_t)kLongTable ? 0u : 0x200u; }
 inline size_t blob_stride(int n_uops) { return ((size_t)blob_bytes((uint32_t)n_uops) + 255) & ~(size_t)255; }
 
 // Emulator state: one record of 32-bit words per slot (slot = index), the same
@@ -193,7 +205,7 @@ cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t 
 // Validate game descriptors; build device descriptors and 4 KB RAM images.
 int build_games(const octax_game *games, int n_games, std::vector<GameDev> &dev,
                 std::vector<uint8_t> &images);
-// Micro-op table length for these games (entries for every address of the longest ROM).
+// Micro-op table length for these games (entries to the end of the longest ROM).
 int table_uops(const octax_game *games, int n_games);
 // Upload the blobs of `games` (device memory of n * blob_stride bytes) and build their tables.
 cudaError_t upload_blobs(const std::vector<GameDev> &games, const std::vector<uint8_t> &images, int n_uops, int schip,

@@ -26,7 +26,8 @@
 //    the result, whose bit 8 is the flag and which decides a skip by being
 //    zero; the next PC is one of two that the micro-op carries. Micro-ops are
 //    decoded once per environment (tables_kernel) for every even address of
-//    the ROM and staged with the image. DXYN has a branch of its own; the
+//    the ROM (of a long ROM, from address 0 on: table_base) and staged with the
+//    image. DXYN has a branch of its own; the
 //    rest (CXNN, calls and returns, 00E0, BCD and bulk memory ops, odd or
 //    written addresses, undefined encodings, the Super-CHIP forms) takes a
 //    divergent switch;
@@ -89,6 +90,7 @@ struct Ctx {
   uint32_t *rec;       // shared: this instance's record
   uint8_t *ram;        // global: this instance's 4 KB RAM (dirty pages)
   uint32_t n_uops;     // entries of the micro-op table (the sentinel follows)
+  uint32_t base;       // address of the first one
   uint32_t sub, L;     // this lane among the L of its instance
   uint32_t gmask;      // those lanes
 };
@@ -114,18 +116,18 @@ __device__ __forceinline__ uint32_t dirty_bit(uint64_t dirty, uint32_t a) {
 
 // Micro-op offset (8 bytes per even address) of a PC; the sentinel's for an
 // odd PC or one outside the table.
-__device__ __forceinline__ uint32_t to_off(uint32_t pc, uint32_t n_uops) {
-  const uint32_t d = pc - 0x200u;
-  return min(__funnelshift_r(d, d, 1), n_uops) << 3;
+__device__ __forceinline__ uint32_t to_off(uint32_t pc, const Ctx &C) {
+  const uint32_t d = pc - C.base;
+  return min(__funnelshift_r(d, d, 1), C.n_uops) << 3;
 }
-__device__ __forceinline__ uint32_t off_pc(uint32_t off) { return 0x200u + (off >> 2); }
+__device__ __forceinline__ uint32_t off_pc(uint32_t off, const Ctx &C) { return C.base + (off >> 2); }
 
 // A fetch at offset o reads the two bytes from off_pc(o) on; the range starts
 // one byte early for that. Nothing written: an offset no fetch has.
-__device__ __forceinline__ void set_range(Regs &R, uint32_t wrange) {
+__device__ __forceinline__ void set_range(Regs &R, const Ctx &C, uint32_t wrange) {
   const uint32_t lo = wrange & 0xFFFFu, hi = wrange >> 16;
   R.wrange = wrange;
-  R.wbase = lo > hi ? 0x40000000u : (lo - 1u - 0x200u) << 2;
+  R.wbase = lo > hi ? 0x40000000u : (lo - 1u - C.base) << 2;
   R.wspan = lo > hi ? 0u : ((hi - lo + 1u) << 2) + 3u;
 }
 
@@ -161,7 +163,7 @@ __device__ __forceinline__ void wr8(Regs &R, const Ctx &C, uint32_t a, uint32_t 
     R.dirty |= 1ull << page;
     __syncwarp(C.gmask);
   }
-  set_range(R, min(R.wrange & 0xFFFFu, a) | max(R.wrange >> 16, a) << 16);
+  set_range(R, C, min(R.wrange & 0xFFFFu, a) | max(R.wrange >> 16, a) << 16);
   C.ram[a] = (uint8_t)val;
 }
 
@@ -344,7 +346,8 @@ __constant__ const uint32_t kCoefs[16] = {
 
 // Micro-op of `op` at table entry e. Successors and jump targets outside the
 // table leave the instruction to the switch, which sets PC itself.
-__device__ __forceinline__ uint3 make_uop(uint32_t op, uint32_t e, uint32_t n_uops, uint32_t quirks, bool schip) {
+__device__ __forceinline__ uint3 make_uop(uint32_t op, uint32_t e, uint32_t base, uint32_t n_uops, uint32_t quirks,
+                                          bool schip) {
   const uint32_t cls = op >> 12, x = (op >> 8) & 15u, y = (op >> 4) & 15u, n = op & 15u, nn = op & 0xFFu;
   const uint32_t nnn = op & 0xFFFu;
   const uint32_t next = (e + 1) << 3, skip = (e + 2) << 3;
@@ -362,8 +365,8 @@ __device__ __forceinline__ uint3 make_uop(uint32_t op, uint32_t e, uint32_t n_uo
                 (schip && ((op & 0xFFF0u) == 0x00C0u || (op >= 0x00FBu && op <= 0x00FFu))));
       break;
     case 0x1:
-      fast = nnn >= 0x200u && !(nnn & 1u) && ((nnn - 0x200u) >> 1) < n_uops;
-      t = f = (nnn - 0x200u) << 2;
+      fast = nnn >= base && !(nnn & 1u) && ((nnn - base) >> 1) < n_uops;
+      t = f = (nnn - base) << 2;
       break;
     case 0x3:
     case 0x4:
@@ -450,10 +453,11 @@ __global__ void tables_kernel(uint8_t *blobs, uint64_t stride, uint32_t n_uops, 
   if (threadIdx.x < 16) reinterpret_cast<uint32_t *>(b + kBlobCoef)[threadIdx.x] = kCoefs[threadIdx.x];
   uint2 *xy = reinterpret_cast<uint2 *>(b + kBlobUops);
   uint32_t *z = reinterpret_cast<uint32_t *>(xy + n_uops + 1);
+  const uint32_t base = table_base(n_uops);
   for (uint32_t e = threadIdx.x; e <= n_uops; e += blockDim.x) {
     uint3 u = make_uint3(kUSlow, kKindRaw, 0u);  // the sentinel
     if (e < n_uops)
-      u = make_uop((uint32_t)b[0x200 + 2 * e] << 8 | b[0x201 + 2 * e], e, n_uops, quirks, schip != 0);
+      u = make_uop((uint32_t)b[base + 2 * e] << 8 | b[base + 2 * e + 1], e, base, n_uops, quirks, schip != 0);
     xy[e] = make_uint2(u.x, u.y);
     z[e] = u.z;
   }
@@ -674,14 +678,14 @@ __device__ __forceinline__ void run_instrs(Regs &R, const Ctx &C, int key, uint3
   const uint32_t sentinel = C.n_uops << 3;
   const uint8_t *const imms = uops + sentinel + 8;
   const int32_t keyterm = key >= 0 ? -key : 256;
-  uint32_t off = to_off(R.pc, C.n_uops);
+  uint32_t off = to_off(R.pc, C);
   // Not unrolled: on divergent programs a second copy of the datapath costs
   // more in instruction fetch than the loop overhead it saves.
 #pragma unroll 1
   for (uint32_t k = 0; k < count; ++k) {
     uint2 u = *reinterpret_cast<const uint2 *>(uops + off);
     const uint32_t z = *reinterpret_cast<const uint32_t *>(imms + (off >> 1));
-    if (off - R.wbase <= R.wspan && dirty_bit(R.dirty, off_pc(off))) u = make_uint2(kUSlow, kKindRaw);  // written
+    if (off - R.wbase <= R.wspan && dirty_bit(R.dirty, off_pc(off, C))) u = make_uint2(kUSlow, kKindRaw);  // written
     const uint32_t vx = C.V[(u.x >> 8) & 0xFFu], vy = C.V[(u.x >> 16) & 0xFFu];
     if (!(u.x & kUSlow)) {
       const uint32_t c = *reinterpret_cast<const uint32_t *>(g_smem + kBlobCoef + (u.x & 0xFFu));
@@ -694,7 +698,7 @@ __device__ __forceinline__ void run_instrs(Regs &R, const Ctx &C, int key, uint3
       if (u.x & kUFlag) C.V[15] = (uint8_t)((((uint32_t)res >> 8) ^ ((u.x & kUBit0) ? vx : 0u)) & 1u);
       if (u.x & kUIndex) R.I = (uint32_t)res;
     } else {
-      const uint32_t pc = off == sentinel ? R.pc : off_pc(off);
+      const uint32_t pc = off == sentinel ? R.pc : off_pc(off, C);
       R.pc = (pc + 2u) & 0xFFFu;
       if (u.y & kKindDraw) {
         if (kS) draw_schip(R, C, vx, vy, u.y & 15u, quirks);
@@ -703,10 +707,10 @@ __device__ __forceinline__ void run_instrs(Regs &R, const Ctx &C, int key, uint3
         const uint32_t op = (u.y & kKindRaw) ? rd8(R, C, pc) << 8 | rd8(R, C, pc + 1u) : u.y;
         exec_slow<kS>(R, C, op, pc, key, quirks);
       }
-      off = to_off(R.pc, C.n_uops);
+      off = to_off(R.pc, C);
     }
   }
-  if (off != sentinel) R.pc = off_pc(off);
+  if (off != sentinel) R.pc = off_pc(off, C);
 }
 
 __device__ __forceinline__ int32_t term_value(const Regs &R, const Ctx &C, const TermDev &t) {
@@ -765,7 +769,7 @@ __device__ __forceinline__ void reset_instance(Regs &R, const Ctx &C, const Game
   R.I = 0;
   R.sp = 0;
   R.dirty = 0;
-  set_range(R, kNoWrites);
+  set_range(R, C, kNoWrites);
 #pragma unroll
   for (int i = 0; i < 8; ++i) C.rec[Rec<kS>::kStack + i] = 0;
   clear_display<kS>(C);
@@ -938,6 +942,7 @@ __device__ __forceinline__ Ctx make_ctx(const Warp &W, const DevState &st, int64
   C.V = reinterpret_cast<uint8_t *>(smem_recs(n_uops) + W.J * Rec<kS>::kWords) + threadIdx.x * kLaneBytes;
   C.ram = st.ram + slot * (int64_t)kRamBytes;
   C.n_uops = n_uops;
+  C.base = table_base(n_uops);
   C.L = 1u << W.sh;
   C.sub = W.lane & (C.L - 1u);
   C.gmask = (W.sh == 5 ? kFull : (1u << C.L) - 1u) << (W.lane - C.sub);
@@ -960,7 +965,7 @@ __device__ __forceinline__ void load_regs(Regs &R, const Ctx &C) {
   R.hires = kS ? (misc >> 7) & 1u : 0u;
   R.status = (misc >> 8) & 0xFFu;
   R.dirty = *reinterpret_cast<const uint64_t *>(C.rec + Rec<kS>::kDirty);
-  set_range(R, C.rec[Rec<kS>::kWrange]);
+  set_range(R, C, C.rec[Rec<kS>::kWrange]);
   R.env_steps = C.rec[Rec<kS>::kEnv];
   R.draws = 0;
   R.phase = 0;
@@ -1577,7 +1582,7 @@ static size_t launch_smem(int block, int ipw, int schip, int writers, int n_uops
 
 // Most instances per warp, up to ipw, whose records fit a CTA's shared memory
 // beside the game's table. Of the accepted shapes one can lose some: 256 x 22
-// of Super-CHIP games with a ROM over 3,326 bytes run as 256 x 21.
+// of Super-CHIP games with a ROM over 3,072 bytes run as 256 x 21.
 int fit_ipw(int block, int ipw, int schip, int writers, int n_uops) {
   while (ipw > 1 && launch_smem(block, ipw, schip, writers, n_uops) > max_dynamic_smem()) --ipw;
   return ipw;

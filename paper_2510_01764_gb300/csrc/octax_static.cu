@@ -30,7 +30,7 @@ constexpr int kStaticPerCta = kStaticBlock / 32 * kStaticIpw;
 constexpr int kStaticMaxGroups = (int)((kStaticMaxEnvs + kStaticPerCta - 1) / kStaticPerCta);
 
 constexpr size_t up256(size_t b) { return (b + 255) & ~(size_t)255; }
-constexpr int kMaxUops = 3584 / 2;
+constexpr int kMaxUops = kRamBytes / 2;
 constexpr size_t kOffRam = up256((size_t)kStaticMaxEnvs * 4 * Rec<false>::kWords);
 constexpr size_t kOffBlob = kOffRam + (size_t)kStaticMaxEnvs * kRamBytes;
 constexpr size_t kOffGroups = kOffBlob + up256(blob_bytes(kMaxUops));
