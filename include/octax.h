@@ -154,7 +154,8 @@ typedef struct {
                                 all [64][2] row-major), ram, episode_steps, env_steps,
                                 last_action, and for SCHIP hires and rpl            */
 
-/* Launch configuration (chosen by octax_autotune or set by hand). A CTA of
+/* Launch configuration: chosen from the environment's size when it is created,
+ * until octax_autotune or octax_set_launch give another. A CTA of
  * `block` emulator threads runs block/32 * inst_per_warp instances of one
  * game; with writer_warps > 0 it also has that many warps that only write
  * observations (block/32 * inst_per_warp / writer_warps must be 8, 16 or 32;
@@ -272,7 +273,11 @@ int octax_sync(octax_env *env, int timeout_ms);
 int octax_debug_stall_writers(octax_env *env, int on);
 
 /* Read / set the launch configuration (the paper defines no counterpart:
- * XLA picks its own launches). EINVAL for unsupported values. */
+ * XLA picks its own launches). octax_get_launch gives the configuration that
+ * the next call runs in, the one chosen from the size included, so a caller may
+ * change one field of it and set the result (writer warps need a shape that
+ * divides among them: 64 threads of 8 instances per warp take one or two). EINVAL
+ * for unsupported values. */
 int octax_get_launch(const octax_env *env, octax_launch *out);
 int octax_set_launch(octax_env *env, const octax_launch *cfg);
 

@@ -890,7 +890,7 @@ int octax_get_launch(const octax_env *e, octax_launch *out) {
     set_error("octax_get_launch: null argument");
     return OCTAX_EINVAL;
   }
-  *out = e->cfg;
+  *out = shape_of(e);
   return OCTAX_OK;
 }
 
@@ -974,8 +974,7 @@ int octax_autotune(octax_env *e, int n_steps, const uint8_t *actions_dev, float 
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   if (r == cudaSuccess) r = cudaEventCreate(&t0);
   if (r == cudaSuccess) r = cudaEventCreate(&t1);
-  const octax_launch saved = e->cfg;
-  octax_launch best = saved;
+  octax_launch best = shape_of(e);
   float best_ms = 1e30f;
   int rc = r == cudaSuccess ? OCTAX_OK : cuda_fail(r, "octax_autotune setup");
   // Every candidate runs the same n_steps from the caller's state (restored
@@ -983,7 +982,6 @@ int octax_autotune(octax_env *e, int n_steps, const uint8_t *actions_dev, float 
   // see the same phase of the workload (episode ends, resets).
   auto trial = [&](const octax_launch &c) {
     if (rc != OCTAX_OK || launch_problem(c, e->schip) || c.steps_per_launch > n_steps) return;
-    e->cfg = c;
     cudaError_t q = copy_state(false);
     rc = q == cudaSuccess ? enqueue_steps(e, c, n_steps, io) : cuda_fail(q, "octax_autotune");  // warm-up
     float ms_min = 1e30f;
@@ -1039,14 +1037,8 @@ int octax_autotune(octax_env *e, int n_steps, const uint8_t *actions_dev, float 
   cudaFree(obs);
   cudaFree(rew);
   cudaFree(done);
-  if (rc) {
-    e->cfg = saved;
-    return rc;
-  }
-  if (r != cudaSuccess) {
-    e->cfg = saved;
-    return cuda_fail(r, "octax_autotune");
-  }
+  if (rc) return rc;
+  if (r != cudaSuccess) return cuda_fail(r, "octax_autotune");
   e->cfg = best;
   e->cfg_set = true;
   if (best_ms_out) *best_ms_out = best_ms;

@@ -258,6 +258,7 @@ class Env:
                              C.byref(h)))
         self._h = h
         self._keep = keep
+        self._size_shape = True  # no launch shape was set or tuned yet
 
     # ------------------------------------------------------------------ helpers
     def _u8(self, *shape):
@@ -409,11 +410,24 @@ class Env:
                 "use_graph": c.use_graph, "writer_warps": c.writer_warps, "balance": c.balance}
 
     def set_launch(self, **kw) -> None:
+        """Set the launch configuration (octax_launch); fields not given stay
+        as in ``launch``. Writer warps on a shape that was chosen from the size
+        and does not divide among them: of its fields not given, the instances
+        per warp become 8 and, if need be, the block 64."""
         cur = self.launch
         cur.update(kw)
+        if self._size_shape and cur["writer_warps"] > 0:
+            def fits():
+                per_cta = cur["block"] // 32 * cur["inst_per_warp"]
+                return per_cta % cur["writer_warps"] == 0 and per_cta // cur["writer_warps"] in (8, 16, 32)
+            if not fits() and "inst_per_warp" not in kw:
+                cur["inst_per_warp"] = 8
+            if not fits() and "block" not in kw:
+                cur["block"] = 64
         c = CLaunch(cur["block"], cur["inst_per_warp"], cur["steps_per_launch"], cur["persistent"],
                     cur["use_graph"], cur["writer_warps"], cur["balance"])
         check(load_library().octax_set_launch(self._h, C.byref(c)))
+        self._size_shape = False
 
     def autotune(self, n_steps: int = 8, actions=None) -> float:
         """Pick the fastest launch configuration for step_n calls of n_steps
@@ -422,6 +436,7 @@ class Env:
             self._check_dev(actions, self._torch.uint8, (n_steps, self.n), "actions")
         ms = C.c_float()
         check(load_library().octax_autotune(self._h, n_steps, _ptr(actions), C.byref(ms)))
+        self._size_shape = False
         return ms.value
 
     @property
