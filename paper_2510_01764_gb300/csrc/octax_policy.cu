@@ -69,7 +69,7 @@ struct octax_policy {
   int sms = 0;
   void *w1 = nullptr, *w2 = nullptr, *w3 = nullptr, *wh = nullptr;  // packed bf16
   float *fp = nullptr;        // biases and output layers (fp32), see FpLayout
-  uint8_t *act2 = nullptr;    // conv2 output, batches of 8 instances
+  uint8_t *act2 = nullptr;    // conv2 output of one conv launch, batches of 8 instances
   uint8_t *act3 = nullptr;    // flattened features, heads' A-operand tiles
   uint64_t *ring = nullptr;   // rollout: two packed observation slots [2][max_envs][4][32]
   unsigned int *err = nullptr;
@@ -116,6 +116,15 @@ constexpr int kXbPitch = 36;
 constexpr uint32_t kConvSmem = kXbOff + 3 * 8 * kXbPitch * 4;
 static_assert(kConvSmem + 1024 <= 227 * 1024, "conv kernel shared memory (with 1 KB of static shared data)");
 constexpr uint32_t kAct2Bytes = 36 * 1024;                 // conv2 output of a batch: position: 8 chunks x 8 x 16 B
+// Most batches per CTA of one conv launch; more instances take several launches
+// over the same act2, which so stays within 350 MB (without a limit it took 4.6
+// KB of each instance, more than all else that a policy keeps of one). A launch
+// costs its weights' copy and the pipeline's start: 131,072 instances 798 us in
+// one launch, 809 in two of 54 batches, 841 with at most 24 and 846 with at most
+// 16, whose act2 (88 MB) stays in L2: that gains nothing. A multiple of 16, so
+// that a launch of the most begins at a tile of the features.
+constexpr int kMaxRounds = 64;
+static_assert(kMaxRounds * kP % 128 == 0, "launches begin at a tile of 128 instances");
 // TMEM columns (fp32): conv1: 2 buffers x 2 output rows x 32; conv2: 2 buffers x 128
 constexpr uint32_t kD1Col = 0, kD2Col = 128, kConvTmemCols = 512;
 
@@ -1123,15 +1132,23 @@ int launch_forward(octax_policy *p, int64_t n, const uint64_t *obs_words, const 
     set_error("octax_policy: need 1 <= n_envs <= max_envs of the policy");
     return OCTAX_EINVAL;
   }
-  ConvArgs c{obs_words, obs_u8, n, (const uint8_t *)p->w1, (const uint8_t *)p->w2, (const uint8_t *)p->w3, p->fp,
-             p->act2, p->act3, p->err, p->stall};
   HeadsArgs h{p->act3, n, (const uint8_t *)p->wh, p->fp, p->n_logits, logits, value, actions,
               (uint32_t)seed, (uint32_t)(seed >> 32), step, p->err};
-  const int64_t batches = (n + kP - 1) / kP;
-  const unsigned grid = (unsigned)std::min<int64_t>(batches, p->sms);
-  cudaError_t r = obs_u8 ? launch(policy_conv_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, c)
-                         : launch(policy_conv_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, c);
-  if (r != cudaSuccess) return cuda_fail(r, "policy conv launch");
+  // launches of about the same number of whole rounds, which begin at a tile of 128 instances
+  const int64_t round = (int64_t)p->sms * kP, launches = (n + kMaxRounds * round - 1) / (kMaxRounds * round);
+  const int64_t rounds = (n + launches * round - 1) / (launches * round);
+  const int64_t per = std::min(((rounds + 1) / 2 * 2 * round + 127) / 128 * 128, kMaxRounds * round);  // instances of one
+  cudaError_t r = cudaSuccess;
+  for (int64_t i = 0; i < n; i += per) {
+    const int64_t m = std::min(per, n - i);
+    ConvArgs c{obs_words ? obs_words + i * 128 : nullptr, obs_u8 ? obs_u8 + i * 8192 : nullptr, m,
+               (const uint8_t *)p->w1, (const uint8_t *)p->w2, (const uint8_t *)p->w3, p->fp, p->act2,
+               p->act3 + i / 128 * (int64_t)kAct3TileBytes, p->err, p->stall};
+    const unsigned grid = (unsigned)std::min<int64_t>((m + kP - 1) / kP, p->sms);
+    r = obs_u8 ? launch(policy_conv_kernel<true>, dim3(grid), kConvThreads, kConvSmem, s, c)
+               : launch(policy_conv_kernel<false>, dim3(grid), kConvThreads, kConvSmem, s, c);
+    if (r != cudaSuccess) return cuda_fail(r, "policy conv launch");
+  }
   // A CTA holds an SM's shared memory, so they run in waves of one per SM: one
   // tile each as long as that makes one wave, else two (the weights then come
   // in once for both).
@@ -1247,7 +1264,7 @@ int octax_policy_create(const octax_policy_params *prm, int64_t max_envs, int de
   if ((r = cudaMalloc(&p->w3, w3p.size() * 2)) != cudaSuccess) return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc(&p->wh, whp.size() * 2)) != cudaSuccess) return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc((void **)&p->fp, fp.size() * 4)) != cudaSuccess) return fail(r, "octax_policy_create: alloc");
-  const int64_t batches = (max_envs + kP - 1) / kP;
+  const int64_t batches = std::min<int64_t>((max_envs + kP - 1) / kP, (int64_t)kMaxRounds * p->sms);
   if ((r = cudaMalloc((void **)&p->act2, (size_t)batches * kAct2Bytes)) != cudaSuccess)
     return fail(r, "octax_policy_create: alloc");
   if ((r = cudaMalloc((void **)&p->act3, (size_t)tiles * kAct3TileBytes)) != cudaSuccess)
