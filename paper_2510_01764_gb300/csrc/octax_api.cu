@@ -186,9 +186,23 @@ int per_cta(const octax_launch &c) { return c.block / 32 * c.inst_per_warp; }
 // to a CTA where several instances a warp share the game's tables, launches of
 // 16 steps (three of four state round trips saved: 16 packed steps of 12,289
 // shooters 275 -> 249 us).
-octax_launch own_shape(int64_t n, int sms, int schip) {
-  const int ipw = spread_ipw(n, sms, schip);
-  return octax_launch{ipw <= 2 ? 64 : 128, ipw, 16, 0, 1, 0, 0};
+// A CTA runs one game and stages its tables, however few instances of it there
+// are. Where a game has at most half of what the CTA takes (n / games, rounded
+// up), its warps share those. 16 steps of 2,000 random programs x 16 instances
+// 2,674 us with 16 to a warp, 1,417 with 4 (2,172 in 64 x 8, which every
+// environment ran in before); x 8 1,639 and 1,104; x 4 1,381 and 809; of 4,000
+// x 24 4,488 and 3,323, x 2 1,718 and 941; of 2,000 template programs x 16 1,386
+// and 804. Above half it depends: x 40 2,992 with 16 to a warp and 3,126 with
+// 10, x 48 3,604 and 3,328, x 60 4,344 and 4,411.
+octax_launch own_shape(int64_t n, int games, int sms, int schip) {
+  octax_launch c{64, spread_ipw(n, sms, schip), 16, 0, 1, 0, 0};
+  if (c.inst_per_warp > 2) c.block = 128;
+  const int64_t each = (n + games - 1) / games;
+  if (games > 1 && 2 * each <= per_cta(c)) {
+    c.block = each >= 4 ? 128 : each >= 2 ? 64 : 32;
+    c.inst_per_warp = (int)((each + c.block / 32 - 1) / (c.block / 32));
+  }
+  return c;
 }
 
 const octax_launch &shape_of(const octax_env *e) { return e->cfg_set ? e->cfg : e->own_cfg; }
@@ -607,7 +621,9 @@ int octax_create(const octax_game *games, int n_games, const uint16_t *game_of_e
   }
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
-  e->own_cfg = own_shape(n_envs, std::max(sms, 1), e->schip);
+  int used = 1;  // games with instances
+  for (int64_t s = 1; s < n_envs; ++s) used += e->game_of_slot[s] != e->game_of_slot[s - 1];
+  e->own_cfg = own_shape(n_envs, used, std::max(sms, 1), e->schip);
   GroupTable *gt = nullptr;
   int rc = get_groups(e, per_cta(shape_of(e)), wave_of(e, shape_of(e)), &gt);
   if (rc) {

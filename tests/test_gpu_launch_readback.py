@@ -84,3 +84,27 @@ def test_a_failed_autotune_leaves_the_chosen_shape():
     with pytest.raises(o.OctaxError):
         env.autotune(0)
     assert env.launch == before
+
+
+@pytest.mark.parametrize("games,each,block,ipw", [(64, 1, 32, 1), (700, 2, 64, 1), (700, 3, 64, 2), (700, 4, 128, 1),
+                                                  (700, 16, 128, 4), (700, 17, 128, 8), (1200, 32, 128, 8),
+                                                  (1200, 33, 128, 16)])
+def test_many_games(games, each, block, ipw):
+    """CTAs of one game each, cut to the instances it has where these are at most
+    half of what the size alone gives a CTA; the results stay those of any shape."""
+    import numpy as np
+
+    from paper_2510_01764_gb300 import octax as o
+
+    rng = np.random.default_rng(games + each)
+    gs = [W.random_game(900 + r) for r in range(8)]
+    n = games * each
+    goe = rng.permutation(np.arange(n) % games).astype(np.uint16)
+    env = o.Env([gs[g % 8] for g in range(games)], n, game_of_env=goe, seed=2)
+    assert (env.launch["block"], env.launch["inst_per_warp"]) == (block, ipw)
+    ref = o.Env(gs, n, game_of_env=goe % 8, seed=2)
+    ref.set_launch(block=64, inst_per_warp=8, steps_per_launch=4)
+    acts = torch.from_numpy(W.actions(4, 0, 12, n)).cuda()
+    for x, y in zip(env.step_n_packed(acts), ref.step_n_packed(acts)):
+        assert torch.equal(x, y)
+    assert torch.equal(env.state_hash(), ref.state_hash())
