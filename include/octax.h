@@ -324,7 +324,9 @@ typedef struct {
                                   (4,468 B of state and 8 B of per-step
                                   buffers each; Super-CHIP: budget / 5,244)   */
   int32_t block;               /* threads per CTA: 32, 64, 128, 256 (0 = 64)    */
-  int32_t inst_per_warp;       /* 1, 2, 4, 8, 16, 32 (0 = 8)                    */
+  int32_t inst_per_warp;       /* 1, 2, 4, 8, 16, 32 (0 = 8): of ticks that fill
+                                  the device; the most of one with fewer
+                                  instances, which spreads them over more warps */
   int32_t max_inflight_ticks;  /* batched launches enqueued ahead, 1..8 (0 = 2) */
   int32_t reserved;
 } octax_server_config;

@@ -258,7 +258,7 @@ const char *launch_problem(const octax_launch &c, int schip) {
 // 644 / 311 with 16.
 int octax::spread_ipw(int64_t n, int sms, int schip) {
   const int64_t per_sm = (n + sms - 1) / sms;
-  if (!schip && per_sm > 192) return 16;
+  if (!schip && per_sm > 192) return most_spread_ipw(schip);
   return per_sm <= 8 ? 1 : per_sm <= 16 ? 2 : per_sm <= 32 ? 4 : 8;
 }
 

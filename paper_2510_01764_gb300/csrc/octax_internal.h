@@ -213,6 +213,8 @@ cudaError_t upload_blobs(const std::vector<GameDev> &games, const std::vector<ui
 
 // Instances per warp for n instances on `sms` SMs.
 int spread_ipw(int64_t n, int sms, int schip);
+// The most it gives.
+inline int most_spread_ipw(int schip) { return schip ? 8 : 16; }
 
 // Programmatic dependent launch: a kernel launched with `dependent` may be set
 // up before the one ahead of it in the stream has ended. It touches nothing

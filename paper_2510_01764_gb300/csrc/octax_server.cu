@@ -220,10 +220,12 @@ bool tick(octax_server *s) {
   for (Req *q : run) k_steps = std::min<uint32_t>(k_steps, q->r.n_steps - q->steps_done);
   // A tick of few instances takes fewer per warp than configured (see
   // spread_ipw): the last ticks of a wave, with 1,600 instances left, took 40
-  // us at 16 to a warp, as long as ones of 19,000.
+  // us at 16 to a warp, as long as ones of 19,000. One that fills the device
+  // runs as configured, also above what spread_ipw ever gives.
   int64_t active = 0;
   for (Req *q : run) active += q->r.n_envs;
-  const int ipw = std::min(s->ipw, spread_ipw(active, s->sms, s->schip));
+  const int spread = spread_ipw(active, s->sms, s->schip);
+  const int ipw = spread == most_spread_ipw(s->schip) ? s->ipw : std::min(s->ipw, spread);
   const int B = s->block / 32 * ipw;  // instances per CTA
   size_t n_groups = 0, n_rgroups = 0, acts = 0;
   for (Req *q : run) n_groups += (q->r.n_envs + B - 1) / B;
