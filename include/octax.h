@@ -441,7 +441,8 @@ typedef struct {
 
 /* Create a policy on `device` for batches of up to max_envs instances (its
  * device buffers: packed weights 1.2 MB, features 2 KB and a two-slot packed
- * observation ring 2 KB per instance). cuda_stream: the stream of
+ * observation ring 2 KB per instance, and 4.6 KB more of each of at most 512
+ * instances per SM: what one conv launch takes). cuda_stream: the stream of
  * octax_policy_forward calls (NULL = a stream of its own). Synchronous.
  * EINVAL: a NULL array, n_logits outside 1..17, max_envs outside 1..2^31. */
 int octax_policy_create(const octax_policy_params *params, int64_t max_envs, int device, void *cuda_stream,
