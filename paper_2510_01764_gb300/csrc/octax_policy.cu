@@ -682,16 +682,17 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv_kernel(const Conv
     uint64_t *const fr = reinterpret_cast<uint64_t *>(sm + kFrOff);
     uint8_t *const blk = sm + kBlkOff + 4 * bw * 512 + lane * 16;
     // The observations may have been written by the kernel ahead in the stream
-    // while this one was set up, so they are read with volatile loads through L2,
-    // which stay behind the dependency wait; the read-only path is for memory
-    // that nothing writes during the whole kernel.
+    // while this one was set up, so they are read with ordinary loads, which stay
+    // behind the dependency wait; the read-only path is for memory that nothing
+    // writes during the whole kernel. (Not past L1: a thread's eight 16-byte
+    // loads of uint8 rows share a line.)
     uint64_t pf[8];  // [frame c][row 2 y2, 2 y2 + 1]
     auto load_words = [&](int64_t first) {
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         ulonglong2 v = make_ulonglong2(0, 0);
         if (first + fi < a.n)
-          v = __ldcg(reinterpret_cast<const ulonglong2 *>(a.obs_words + (first + fi) * 128 + c * 32 + 2 * y2));
+          v = *reinterpret_cast<const ulonglong2 *>(a.obs_words + (first + fi) * 128 + c * 32 + 2 * y2);
         pf[2 * c] = v.x;
         pf[2 * c + 1] = v.y;
       }
@@ -703,7 +704,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) policy_conv_kernel(const Conv
 #pragma unroll
       for (int q = 0; q < 8; ++q)
         raw[q] = first + fi < a.n
-                     ? __ldcg(reinterpret_cast<const uint4 *>(a.obs_u8 + ((first + fi) * 128 + c * 32 + 2 * y2) * 64) + q)
+                     ? reinterpret_cast<const uint4 *>(a.obs_u8 + ((first + fi) * 128 + c * 32 + 2 * y2) * 64)[q]
                      : make_uint4(0, 0, 0, 0);
     };
     auto pack_bytes = [&](int c) {
