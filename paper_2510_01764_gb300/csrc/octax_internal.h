@@ -64,7 +64,7 @@ __host__ __device__ constexpr uint32_t blob_bytes(uint32_t n_uops) {
 // memory below the ROM (random ones end up there: 7 of 10 of their instructions
 // after 200 steps) then leave the datapath no more; the 3 KB this takes are a
 // seventh of what such an environment's CTAs stage. 262,144 random programs of
-// 3,584 bytes, 2,000 steps: 414 us a step with the ROM's addresses alone, 400
+// 3,584 bytes, 2,000 steps: 414 us a step with the ROM's addresses alone, 397
 // with all; 16,384 and 65,536 of them 1-5 % faster, template programs padded to
 // that length 0.7 % faster to 1 % slower. At 3,072 bytes neither side leads
 // (0.94-1.04); at 1,024, where a CTA of 32 instances loses one of eight resident

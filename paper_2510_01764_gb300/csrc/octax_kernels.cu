@@ -50,7 +50,7 @@
 // 6.2 us, of 16,384 34.2 -> 20.9 us (7.0 TB/s), 16 packed steps of 12,289
 // shooter instances 352 -> 163 us, 8 Super-CHIP steps of 8,192 492 -> 303 us,
 // 8 steps of 65,536 over 16 ROMs 978 -> 836 us, 4 steps of 262,144 random
-// programs 1,472 -> 1,452 us. The micro-ops take 12 bytes and not 16 so that
+// programs 1,472 -> 1,391 us. The micro-ops take 12 bytes and not 16 so that
 // a CTA of 64 instances with a 3.5 KB ROM keeps four CTAs per SM (random
 // programs 1,683 us with 16); the pixel table stays because expanding by
 // multiplication costs the issue-bound cases 1 % (it gains 7 % on one step of
@@ -936,13 +936,13 @@ __device__ __forceinline__ Warp make_warp(int ipw, int emu_warps, const Group &g
 }
 
 template <bool kS>
-__device__ __forceinline__ Ctx make_ctx(const Warp &W, const DevState &st, int64_t slot, uint32_t n_uops) {
+__device__ __forceinline__ Ctx make_ctx(const Warp &W, const DevState &st, int64_t slot, uint32_t n_uops, uint32_t base) {
   Ctx C;
   C.rec = W.recs + (W.active ? W.i : 0) * Rec<kS>::kWords;
   C.V = reinterpret_cast<uint8_t *>(smem_recs(n_uops) + W.J * Rec<kS>::kWords) + threadIdx.x * kLaneBytes;
   C.ram = st.ram + slot * (int64_t)kRamBytes;
   C.n_uops = n_uops;
-  C.base = table_base(n_uops);
+  C.base = base;
   C.L = 1u << W.sh;
   C.sub = W.lane & (C.L - 1u);
   C.gmask = (W.sh == 5 ? kFull : (1u << C.L) - 1u) << (W.lane - C.sub);
@@ -1013,14 +1013,14 @@ __device__ __forceinline__ uint32_t applied_action(const Regs &R, const Ctx &C, 
   return a;
 }
 
-template <bool kWrap, bool kS>
+template <bool kWrap, bool kS, uint32_t kBase>
 __device__ void run_group(const StepLaunch &p, const Group &g, const Warp &W) {
   const DevState &st = p.st;
   const GameDev &G = smem_game();
   const int64_t slot = (int64_t)g.slot0 + (W.active ? W.j : 0);
   const IO io = p.io_table ? p.io_table[g.io] : p.io0;
   const uint32_t quirks = p.quirks;
-  const Ctx C = make_ctx<kS>(W, st, slot, (uint32_t)p.n_uops);
+  const Ctx C = make_ctx<kS>(W, st, slot, (uint32_t)p.n_uops, kBase);
   const int frame = io.packed ? 8 * Disp<kS>::kWords : Disp<kS>::kFrame;
   Regs R;
   load_regs<kS>(R, C);
@@ -1092,8 +1092,10 @@ __device__ void run_group(const StepLaunch &p, const Group &g, const Warp &W) {
 // One CTA's loop over groups (a persistent CTA pulls them off the queue).
 // Every step kernel is held to 128 registers (two 256-thread CTAs per SM).
 // kWrap: the sticky-action / no-op-reset variant (games without the wrappers
-// run the kernel without them); kS: the Super-CHIP display layout.
-template <bool kWrap, bool kS>
+// run the kernel without them); kS: the Super-CHIP display layout; kBase: the
+// table's first address (computed in the kernel it costs the issue-bound cases
+// 0.3-0.7 % and random programs 0.9 %).
+template <bool kWrap, bool kS, uint32_t kBase>
 __global__ void __launch_bounds__(kMaxBlock, 2) step_kernel(const StepLaunch p) {
   __shared__ int s_group;
   int cur_game = -1;
@@ -1115,7 +1117,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) step_kernel(const StepLaunch p) 
     fetch_records<kS>(W, p.st, g);
     copy_wait();
     __syncthreads();
-    run_group<kWrap, kS>(p, g, W);
+    run_group<kWrap, kS, kBase>(p, g, W);
     if (!p.work_counter) break;
     __syncthreads();  // shared memory is reused by the next group
   }
@@ -1209,7 +1211,7 @@ __device__ void run_group_emu(const StepLaunch &p, const Group &g, const Warp &W
   const int64_t slot = (int64_t)g.slot0 + (W.active ? W.j : 0);
   const IO io = p.io_table ? p.io_table[g.io] : p.io0;
   const uint32_t quirks = p.quirks;
-  const Ctx C = make_ctx<false>(W, st, slot, (uint32_t)p.n_uops);
+  const Ctx C = make_ctx<false>(W, st, slot, (uint32_t)p.n_uops, table_base((uint32_t)p.n_uops));
   Regs R;
   load_regs<false>(R, C);
   const int64_t row = (int64_t)C.rec[Rec<false>::kRow];
@@ -1380,7 +1382,7 @@ __global__ void __launch_bounds__(kMaxBlock, 2) reset_kernel(const ResetLaunch p
   const DevState &st = p.st;
   const GameDev &G = smem_game();
   const int64_t slot = (int64_t)g.slot0 + (W.active ? W.j : 0);
-  const Ctx C = make_ctx<kS>(W, st, slot, (uint32_t)p.n_uops);
+  const Ctx C = make_ctx<kS>(W, st, slot, (uint32_t)p.n_uops, table_base((uint32_t)p.n_uops));
   Regs R;
   if (p.init) {
     const uint64_t seed = p.seed_of_group ? p.seed_of_group[blockIdx.x] : p.seed;
@@ -1588,6 +1590,17 @@ int fit_ipw(int block, int ipw, int schip, int writers, int n_uops) {
   return ipw;
 }
 
+// The step kernel instantiation for a launch (null: writer warps on SCHIP).
+template <uint32_t kBase>
+static const void *plain_fn(int wrappers, int schip) {
+  if (schip) return wrappers ? (const void *)step_kernel<true, true, kBase> : (const void *)step_kernel<false, true, kBase>;
+  return wrappers ? (const void *)step_kernel<true, false, kBase> : (const void *)step_kernel<false, false, kBase>;
+}
+static const void *step_fn(int writers, int wrappers, int schip, int n_uops) {
+  if (writers > 0) return schip ? nullptr : (const void *)step_kernel_ws;
+  return table_base((uint32_t)n_uops) == 0u ? plain_fn<0u>(wrappers, schip) : plain_fn<0x200u>(wrappers, schip);
+}
+
 // The dynamic shared memory attribute of a kernel applies to the current
 // device only, so it is set once per device ordinal (under a lock: the
 // serving thread and user threads launch concurrently).
@@ -1600,10 +1613,11 @@ static cudaError_t ensure_smem_attr() {
   std::lock_guard<std::mutex> lk(mu);
   if (done[dev]) return cudaSuccess;
   const int cap = (int)max_dynamic_smem();
-  const void *fns[] = {(const void *)step_kernel<false, false>, (const void *)step_kernel<true, false>,
-                       (const void *)step_kernel<false, true>,  (const void *)step_kernel<true, true>,
-                       (const void *)reset_kernel<false>,       (const void *)reset_kernel<true>,
-                       (const void *)step_kernel_ws};
+  const int kShort = 0, kLong = kLongTable + 1;  // micro-ops of tables at either base
+  const void *fns[] = {step_fn(0, 0, 0, kShort),          step_fn(0, 1, 0, kShort), step_fn(0, 0, 1, kShort),
+                       step_fn(0, 1, 1, kShort),          step_fn(0, 0, 0, kLong),  step_fn(0, 1, 0, kLong),
+                       step_fn(0, 0, 1, kLong),           step_fn(0, 1, 1, kLong),  (const void *)reset_kernel<false>,
+                       (const void *)reset_kernel<true>, (const void *)step_kernel_ws};
   for (const void *f : fns) {
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
     if (e != cudaSuccess) return e;
@@ -1612,19 +1626,12 @@ static cudaError_t ensure_smem_attr() {
   return cudaSuccess;
 }
 
-// The step kernel instantiation for a launch (null: writer warps on SCHIP).
-static const void *step_fn(int writers, int wrappers, int schip) {
-  if (writers > 0) return schip ? nullptr : (const void *)step_kernel_ws;
-  if (schip) return wrappers ? (const void *)step_kernel<true, true> : (const void *)step_kernel<false, true>;
-  return wrappers ? (const void *)step_kernel<true, false> : (const void *)step_kernel<false, false>;
-}
-
 cudaError_t launch_step(const StepLaunch &p, int grid, int block, cudaStream_t s) {
   if (!state_complete(p.st)) return cudaErrorInvalidValue;
   cudaError_t e = ensure_smem_attr();
   if (e != cudaSuccess) return e;
   if (grid <= 0) return cudaSuccess;
-  const void *fn = step_fn(p.writers, p.wrappers, p.st.schip);
+  const void *fn = step_fn(p.writers, p.wrappers, p.st.schip, p.n_uops);
   if (!fn) return cudaErrorInvalidValue;
   StepLaunch copy = p;
   void *args[] = {&copy};
@@ -1682,7 +1689,7 @@ cudaError_t add_step_node(cudaGraph_t g, cudaGraphNode_t *node, cudaGraphNode_t 
   if (!state_complete(p.st)) return cudaErrorInvalidValue;
   cudaError_t e = ensure_smem_attr();
   if (e != cudaSuccess) return e;
-  const void *fn = step_fn(p.writers, p.wrappers, p.st.schip);
+  const void *fn = step_fn(p.writers, p.wrappers, p.st.schip, p.n_uops);
   if (!fn) return cudaErrorInvalidValue;
   StepLaunch copy = p;
   void *args[] = {&copy};
@@ -1716,7 +1723,7 @@ int max_resident_ctas(int block, int ipw, int writers, int wrappers, int schip, 
   int dev = 0, sms = 0, per_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const void *fn = step_fn(writers, wrappers, schip);
+  const void *fn = step_fn(writers, wrappers, schip, n_uops);
   if (!fn) return 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, block + 32 * writers,
                                                 launch_smem(block, ipw, schip, writers, n_uops));
