@@ -35,8 +35,9 @@
 //  and discarded (they read padding or neighbouring positions, always inside
 //  the buffers).
 // What bounds it: the chains of MMAs that add into one accumulator (12 of conv1
-// per pair of rows, 16 of conv2 per tile; each link takes 85-105 cycles whatever
-// N <= 128) and their hand-overs; 9.6 K cycles a batch for conv1 and conv2,
+// per pair of rows, 16 of conv2 per tile; links of one chain alone were seen 85
+// cycles apart, 12 of conv3's N = 64 in 1,010, and two chains side by side gave
+// an MMA every 42) and their hand-overs; 9.6 K cycles a batch for conv1 and conv2,
 // of which the tensor pipe needs 5.8 K, and 2.4 K for conv3 (1.7 K of operand
 // reads). Against the form before it (a CTA took each batch through all
 // phases, conv3's output positions 22 of 32 rows; 150 us for 16,384
@@ -44,8 +45,10 @@
 // roles that run ahead of each other, also over a batch's end (forward 173.5
 // -> 126.5 us); a wait that seldom reads the timer, blocks expanded before the
 // wait, a band whose rows are rewritten five rows later (112.5); MMAs issued
-// by whole warps, whose operands need no moves to uniform registers (12 MMAs
-// in 1.25 K -> 0.75 K cycles; 101.8); conv3 in the same kernel (99.2). No
+// by whole warps, whose operands need no moves to uniform registers (issuing 12
+// took 1.25 K, now 0.75 K cycles of the warp; 101.8); conv3 in the same kernel
+// (99.2). The microseconds of a forward here are of three policies in turn; one
+// after another it takes 108 us (174 and 195 before all of them). No
 // gain: a ring of 7 block rows with four accumulators; conv1's A operand in
 // TMEM; conv1's two rows as separate chains.
 // Heads kernel: a head of one or two 128-instance tiles per CTA; K = 1024
@@ -281,7 +284,7 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t a0, uint32_t a1, float (&v)
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
-// 32 columns at each of a0, a1 (and a2) of this thread's TMEM lane, behind one wait.
+// 32 columns at each of a0 and a1 of this thread's TMEM lane, behind one wait.
 __device__ __forceinline__ void tmem_ld32x2(uint32_t a0, uint32_t a1, float (&v)[32], float (&w)[32]) {
   uint32_t r[32], q[32];
   asm volatile(
